@@ -143,9 +143,11 @@ struct tim_ctx {
     DevBuf ld_in_r, ld_in_d, ld_in_w;  // device copies of tim_load_graph's host arrays
 
     // forward cascades (spread.cu): G as out-records {in-CSR position, destination},
-    // built from G^T on first use; per-block visited bitmaps (kept all-zero between
-    // calls) and queues; cascade counts, seeds, counters
-    DevBuf out_rowptr, out_rec, mc_bitmap, mc_queue, mc_counts, mc_seeds, mc_scal;
+    // built from G^T on first use, with the out-record of every in-CSR position;
+    // per-block visited bitmaps (kept all-zero between calls), queues and live-edge bits;
+    // cascade counts, seeds, counters
+    DevBuf out_rowptr, out_row, out_rec, out_pos, mc_bitmap, mc_queue, mc_live, mc_counts, mc_seeds,
+        mc_scal;
     bool have_out = false, mc_clean = false;
 
     // generic scratch for scans and sorts

@@ -12,17 +12,35 @@
 // of sid is then exactly the set of nodes that reach its root in this cascade's world.
 //
 // The walk needs G itself: out-records {in-CSR position, destination} grouped by
-// source, built from G^T on first use. One block per cascade: its visited bitmap (n
-// bits) and queue (the activated nodes, n slots) live in global memory, one pair per
-// resident block; the block expands the queue round by round (warps claim queued nodes
-// and stride over their out-records) until a round adds nothing.
+// source, and the inverse (out-record index of every in-CSR position), built from G^T on
+// first use. One block per cascade. Its visited bitmap (n bits) sits in shared memory
+// when it fits there, its queue (the activated nodes, n slots) and the live-edge bits
+// (below) in global memory, one set per resident block. A round expands the nodes the
+// round before added; a round that adds nothing ends the cascade.
+//
+// A round runs in one of two ways. Walking tests every out-edge of the round's nodes by
+// its own draw (a Philox block per edge: the in-CSR positions of one node's out-edges are
+// scattered). Drawing evaluates the cascade's whole world once: IC draws the coins of
+// four consecutive in-CSR positions with one Philox block and 16 contiguous bytes of
+// thresholds, LT and triggering models make one pick per unvisited node, and every live
+// edge sets one bit at its out-record; from then on a node's live out-edges are read 32
+// to a word. A cascade starts walking and draws its world as soon as the out-edges it
+// would have walked by the end of the next round pass a fixed share (MC_WALK) of the draws
+// that the world takes (m / 4 blocks for IC, n picks otherwise): small cascades never pay
+// for a world, large ones walk little before they do. Against walking alone (one 256-thread
+// block per cascade, one warp per node): 50 seeds on R-MAT 18, 2000 IC cascades 42.2 -> 10.9
+// ms, 1000 LT cascades 70.4 -> 7.4 ms. Drawing is bound by issue (Philox) and by the one L1
+// sector per clock of scattered out-record indexes and bit updates, the rounds by their
+// chains of dependent loads.
 #include <algorithm>
 
 #include "common.cuh"
 
 namespace {
 
-constexpr int MC_THREADS = 256;
+// largest visited bitmaps kept in shared memory, one and two per SM (n up to 1.55 million
+// and 0.65 million nodes), beside the blocks' stages
+constexpr uint64_t MC_SMEM_MAX = 190 * 1024, MC_SMEM_TWO = 80 * 1024;
 
 __global__ void out_count_kernel(const uint32_t* __restrict__ src, uint64_t m,
                                  uint32_t* __restrict__ cnt) {
@@ -31,11 +49,20 @@ __global__ void out_count_kernel(const uint32_t* __restrict__ src, uint64_t m,
         atomicAdd(&cnt[__ldg(src + j)], 1u);
 }
 
+// Rows of the out-records as one 8-byte word per node (m < 2^32): one load per node.
+__global__ void out_rows_kernel(const uint64_t* __restrict__ out_rowptr, uint64_t n,
+                                uint2* __restrict__ out_row) {
+    for (uint64_t v = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; v < n;
+         v += (uint64_t)gridDim.x * blockDim.x)
+        out_row[v] = make_uint2((uint32_t)out_rowptr[v], (uint32_t)out_rowptr[v + 1]);
+}
+
 // One warp per destination v: each in-edge j = (u -> v) becomes out-record {j, v} of u.
 __global__ void out_scatter_kernel(const uint64_t* __restrict__ rowptr,
                                    const uint32_t* __restrict__ src, uint64_t n,
                                    const uint64_t* __restrict__ out_rowptr,
-                                   uint32_t* __restrict__ cursor, uint2* __restrict__ out_rec) {
+                                   uint32_t* __restrict__ cursor, uint2* __restrict__ out_rec,
+                                   uint32_t* __restrict__ out_pos) {
     const int lane = threadIdx.x & 31;
     const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     for (uint64_t v = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5; v < n; v += nw) {
@@ -43,7 +70,9 @@ __global__ void out_scatter_kernel(const uint64_t* __restrict__ rowptr,
         for (uint64_t j = b + lane; j < e; j += 32) {
             const uint32_t u = __ldg(src + j);
             const uint32_t slot = atomicAdd(&cursor[u], 1u);
-            out_rec[out_rowptr[u] + slot] = make_uint2((uint32_t)j, (uint32_t)v);
+            const uint64_t at = out_rowptr[u] + slot;
+            out_rec[at] = make_uint2((uint32_t)j, (uint32_t)v);
+            if (out_pos) out_pos[j] = (uint32_t)at;
         }
     }
 }
@@ -52,17 +81,21 @@ struct McArgs {
     const uint64_t* rowptr;
     const uint32_t* thr;
     const unsigned long long* node_thr;
-    const uint64_t* out_rowptr;
+    const uint2* out_row;
     const uint2* out_rec;
+    const uint32_t* out_pos;
     int model;
-    uint64_t n;
+    uint64_t n, m;
     PhiloxKeys K;
     uint64_t sid0, count;
     const int32_t* seeds;
     int k;
-    uint32_t* bitmap;  // slots * words
+    uint32_t* bitmap;  // slots * words (unless the bitmaps sit in shared memory)
     uint32_t* queue;   // slots * n
     uint64_t words;
+    uint32_t* live;    // slots * live_words: bit e = out-record e is live
+    uint64_t live_words;          // a multiple of 4
+    unsigned long long draw_at;   // out-edges a cascade walks at most; ~0: never draws
     uint32_t* counts;              // per cascade
     unsigned long long* scal;      // [0] next cascade, [1] total activated
     // triggering model: options per node, cumulative thresholds, sorted in-CSR positions
@@ -72,44 +105,224 @@ struct McArgs {
     const uint32_t* opt_pos;
 };
 
-// Does v keep in-edge j in the world of sid (LT)?
-__device__ __forceinline__ bool lt_kept(const McArgs& a, uint32_t s0, uint32_t s1, uint32_t v,
-                                        uint32_t j) {
+// The in-edge node v keeps in the world of sid (LT), or the end of its in-list for none.
+__device__ __forceinline__ uint64_t lt_pick(const McArgs& a, uint32_t s0, uint32_t s1, uint32_t v,
+                                            uint64_t* end_out) {
     const uint64_t beg = __ldg(a.rowptr + v), end = __ldg(a.rowptr + v + 1);
     const uint32_t x = philox4x32_10(s0, s1, v, TIM_TAG_LT, a.K).x;
     const unsigned long long nt = __ldg(a.node_thr + v);
-    const uint64_t p = (nt >> 32) ? lt_uniform_pick(nt, beg, end, x)
-                                  : lane_lt_search(a.thr, beg, end, x);
-    return p == (uint64_t)j;
+    *end_out = end;
+    return (nt >> 32) ? lt_uniform_pick(nt, beg, end, x) : lane_lt_search(a.thr, beg, end, x);
 }
 
-// Does v keep in-edge j in the world of sid (triggering model)? v picks its option with
-// the RR walk's draw; j is kept iff it is among the option's positions (ascending).
-__device__ __forceinline__ bool trig_kept(const McArgs& a, uint32_t s0, uint32_t s1, uint32_t v,
-                                          uint32_t j) {
+// The option node v picks in the world of sid (triggering model): its positions are
+// opt_pos[*lo .. *hi), none when they are equal.
+__device__ __forceinline__ void trig_pick(const McArgs& a, uint32_t s0, uint32_t s1, uint32_t v,
+                                          uint64_t* lo, uint64_t* hi) {
+    *lo = *hi = 0;
     const uint64_t o0 = __ldg(a.node_opt + v), o1 = __ldg(a.node_opt + v + 1);
-    if (o1 == o0) return false;
+    if (o1 == o0) return;
     const uint32_t x = philox4x32_10(s0, s1, v, TIM_TAG_LT, a.K).x;
     const uint64_t o = lane_lt_search(a.opt_cum, o0, o1, x);
-    if (o >= o1) return false;
-    uint64_t lo = __ldg(a.opt_off + o), hi = __ldg(a.opt_off + o + 1);
-    for (int it = 0; it < 40 && lo < hi; it++) {  // first position >= j
-        const uint64_t mid = lo + ((hi - lo) >> 1);
-        if (__ldg(a.opt_pos + mid) < j)
-            lo = mid + 1;
-        else
-            hi = mid;
-    }
-    return lo < __ldg(a.opt_off + o + 1) && __ldg(a.opt_pos + lo) == j;
+    if (o >= o1) return;
+    *lo = __ldg(a.opt_off + o);
+    *hi = __ldg(a.opt_off + o + 1);
 }
 
-__global__ void __launch_bounds__(MC_THREADS) mc_cascade_kernel(McArgs a) {
-    __shared__ unsigned long long s_c;
+// Does v keep in-edge j in the world of sid?
+__device__ __forceinline__ bool edge_kept(const McArgs& a, uint32_t s0, uint32_t s1, uint32_t v,
+                                          uint32_t j) {
+    if (a.model == TIM_IC) {
+        const uint4 x = philox4x32_10(s0, s1, j >> 2, TIM_TAG_IC, a.K);
+        const uint32_t w = (j & 3) == 0 ? x.x : (j & 3) == 1 ? x.y : (j & 3) == 2 ? x.z : x.w;
+        const uint32_t t = __ldg(a.thr + j);
+        return t == 0xFFFFFFFFu || w < t;
+    }
+    if (a.model == TIM_TRIG) {
+        uint64_t lo, hi;
+        trig_pick(a, s0, s1, v, &lo, &hi);
+        const uint64_t stop = hi;
+        for (int it = 0; it < 40 && lo < hi; it++) {  // first position >= j (ascending)
+            const uint64_t mid = lo + ((hi - lo) >> 1);
+            if (__ldg(a.opt_pos + mid) < j)
+                lo = mid + 1;
+            else
+                hi = mid;
+        }
+        return lo < stop && __ldg(a.opt_pos + lo) == j;
+    }
+    uint64_t end;
+    const uint64_t p = lt_pick(a, s0, s1, v, &end);
+    return p < end && p == (uint64_t)j;
+}
+
+__device__ __forceinline__ void set_live(const McArgs& a, uint32_t* live, uint64_t j) {
+    const uint32_t e = __ldg(a.out_pos + j);
+    atomicOr(&live[e >> 5], 1u << (e & 31));
+}
+
+// A cascade walks at most 1 / MC_WALK as many out-edges as drawing its world takes draws: a
+// walked edge costs about three of them, and a cascade that has walked this much mostly
+// goes on (MC_WALK 2, 4, 12, 24: 50 seeds on R-MAT 18, IC, 16.0, 15.0, 11.1, 11.1 ms; one
+// seed on a 200,001-node Chung-Lu graph, 1000 cascades, 6.2, 4.9, 3.7, 3.6 ms).
+constexpr unsigned MC_WALK = 12;
+
+// Live in-CSR positions a warp collects (in shared memory) before it sets their bits, four
+// per lane in flight: setting each one as it is found would wait for its out-record index
+// every time.
+constexpr uint32_t MC_STAGE = 256;
+
+__device__ __forceinline__ void flush_live(const McArgs& a, uint32_t* live, const uint32_t* st,
+                                           uint32_t cnt, int lane) {
+    __syncwarp();
+    for (uint32_t i = lane; i < cnt; i += 128) {
+        uint32_t e[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) e[k] = i + 32 * k < cnt ? __ldg(a.out_pos + st[i + 32 * k]) : 0u;
+#pragma unroll
+        for (int k = 0; k < 4; k++)
+            if (i + 32 * k < cnt) atomicOr(&live[e[k] >> 5], 1u << (e[k] & 31));
+    }
+    __syncwarp();
+}
+
+// The world of sid as live bits over the out-records (all of the block's threads). Bound by
+// issue for IC (the Philox rounds of m / 4 blocks); nodes already visited need no pick.
+__device__ __forceinline__ void draw_world(const McArgs& a, uint32_t s0, uint32_t s1,
+                                           const uint32_t* bm, uint32_t* live,
+                                           uint32_t* stage) {
+    const int lane = threadIdx.x & 31;
+    uint4* l4 = reinterpret_cast<uint4*>(live);
+    for (uint64_t w = threadIdx.x; w < a.live_words >> 2; w += blockDim.x)
+        l4[w] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+    if (a.model == TIM_IC) {
+        const uint4* thr4 = reinterpret_cast<const uint4*>(a.thr);
+        const uint32_t groups = (uint32_t)((a.m + 3) >> 2);  // thr is zero past its end
+        // four groups per thread and step: their loads overlap, and the live in-edges of all
+        // four (about one in sixteen coins under weighted cascade) share one loop
+        uint32_t* st = stage + (threadIdx.x >> 5) * MC_STAGE;
+        uint32_t held = 0;
+        // four groups per thread and step, so that their loads overlap
+        for (uint32_t gw = threadIdx.x & ~31u; gw < groups; gw += 4 * blockDim.x) {
+            const uint32_t g0 = gw + lane;
+            uint32_t lm = 0;
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                const uint32_t g = g0 + i * blockDim.x;
+                const uint4 t = g < groups ? __ldg(thr4 + g) : make_uint4(0u, 0u, 0u, 0u);
+                const uint4 x = philox4x32_10(s0, s1, g, TIM_TAG_IC, a.K);
+                lm |= ((x.x < t.x || t.x == 0xFFFFFFFFu ? 1u : 0u) |
+                       (x.y < t.y || t.y == 0xFFFFFFFFu ? 2u : 0u) |
+                       (x.z < t.z || t.z == 0xFFFFFFFFu ? 4u : 0u) |
+                       (x.w < t.w || t.w == 0xFFFFFFFFu ? 8u : 0u)) << (4 * i);
+            }
+            const uint32_t cnt = __popc(lm);
+            uint32_t incl = cnt;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+            if (held + total > MC_STAGE) {
+                flush_live(a, live, st, held, lane);
+                held = 0;
+            }
+            uint32_t at = held + incl - cnt;
+            const bool fits = total <= MC_STAGE;
+            for (; lm; lm &= lm - 1) {
+                const uint32_t b = __ffs(lm) - 1;
+                const uint32_t j = ((g0 + (b >> 2) * blockDim.x) << 2) + (b & 3);
+                if (fits)
+                    st[at++] = j;
+                else
+                    set_live(a, live, j);
+            }
+            if (fits) held += total;
+        }
+        flush_live(a, live, st, held, lane);
+    } else if (a.model == TIM_TRIG) {
+        // the picked options' positions, flattened over the warp's lanes
+        for (uint64_t vw = threadIdx.x & ~31u; vw < a.n; vw += blockDim.x) {
+            const uint64_t v = vw + lane;
+            uint64_t lo = 0, hi = 0;
+            if (v < a.n && !((bm[v >> 5] >> (v & 31)) & 1u))
+                trig_pick(a, s0, s1, (uint32_t)v, &lo, &hi);
+            const uint32_t cnt = (uint32_t)(hi - lo);
+            uint32_t incl = cnt;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+            for (uint32_t base = 0; base < total; base += 32) {
+                const uint32_t t = base + lane;
+                int own = 0;  // number of lanes whose inclusive count is <= t
+#pragma unroll
+                for (int sft = 16; sft > 0; sft >>= 1) {
+                    const uint32_t ic = __shfl_sync(0xffffffffu, incl, own + sft - 1);
+                    if (ic <= t) own += sft;
+                }
+                const uint64_t ol = __shfl_sync(0xffffffffu, lo, own);
+                const uint32_t ox = __shfl_sync(0xffffffffu, incl - cnt, own);
+                if (t < total) set_live(a, live, __ldg(a.opt_pos + ol + (t - ox)));
+            }
+        }
+    } else {
+        // four picks per thread in flight
+        for (uint64_t v0 = threadIdx.x; v0 < a.n; v0 += 4 * blockDim.x) {
+            uint64_t p[4], end[4];
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                const uint64_t v = v0 + i * blockDim.x;
+                p[i] = end[i] = 0;
+                if (v < a.n && !((bm[v >> 5] >> (v & 31)) & 1u))
+                    p[i] = lt_pick(a, s0, s1, (uint32_t)v, &end[i]);
+            }
+            uint32_t e[4];
+#pragma unroll
+            for (int i = 0; i < 4; i++) e[i] = p[i] < end[i] ? __ldg(a.out_pos + p[i]) : 0u;
+#pragma unroll
+            for (int i = 0; i < 4; i++)
+                if (p[i] < end[i]) atomicOr(&live[e[i] >> 5], 1u << (e[i] & 31));
+        }
+    }
+    __syncthreads();
+}
+
+// SM: the visited bitmap in shared memory (n bits of dynamic shared memory).
+template <bool SM, int THREADS, int BLOCKS>
+__global__ void __launch_bounds__(THREADS, BLOCKS) mc_cascade_kernel(McArgs a) {
+    extern __shared__ uint32_t s_bm[];
+    __shared__ uint32_t s_stage[THREADS / 32 * MC_STAGE];
+    __shared__ unsigned long long s_c, s_edges;
     __shared__ uint32_t s_tail, s_next;
     const int lane = threadIdx.x & 31;
-    uint32_t* bm = a.bitmap + (uint64_t)blockIdx.x * a.words;
+    uint32_t* bm = SM ? s_bm : a.bitmap + (uint64_t)blockIdx.x * a.words;
     uint32_t* q = a.queue + (uint64_t)blockIdx.x * a.n;
+    uint32_t* live = a.live + (uint64_t)blockIdx.x * a.live_words;
+    uint32_t* st = s_stage + (threadIdx.x >> 5) * MC_STAGE;
+    if (SM)
+        for (uint32_t w = threadIdx.x; w < (uint32_t)a.words; w += blockDim.x) bm[w] = 0u;
+    // The round's nodes are q[cur .. ] and the next round's q[nxt .. ], step +1 or -1. With
+    // the bitmap in shared memory the rounds fill the queue from its two ends in turn (the
+    // nodes of two rounds are distinct, so they fit), which keeps its lines in L2; without,
+    // they follow one another, so that the bitmap can be cleared through the queue.
+    int64_t cur = 0, nxt = 0;
+    int dcur = 1, dnxt = 1;
+    auto add = [&](uint32_t v) {
+        const uint32_t b = 1u << (v & 31);
+        if (!(atomicOr(&bm[v >> 5], b) & b))
+            q[nxt + dnxt * (int64_t)atomicAdd(&s_tail, 1u)] = v;
+    };
+    // a plain read first: a stale zero only costs a draw or an atomic
+    auto seen = [&](uint32_t v) {
+        return ((SM ? ((volatile uint32_t*)bm)[v >> 5] : __ldcg(bm + (v >> 5))) >> (v & 31)) & 1u;
+    };
     for (;;) {
+        __syncthreads();
         if (threadIdx.x == 0) {
             s_c = atomicAdd(&a.scal[0], 1ull);
             s_tail = 0;
@@ -119,66 +332,200 @@ __global__ void __launch_bounds__(MC_THREADS) mc_cascade_kernel(McArgs a) {
         if (c >= a.count) break;
         const uint64_t sid = a.sid0 + c;
         const uint32_t s0 = (uint32_t)sid, s1 = (uint32_t)(sid >> 32);
-        for (int i = threadIdx.x; i < a.k; i += blockDim.x) {
-            const uint32_t v = (uint32_t)a.seeds[i];
-            const uint32_t b = 1u << (v & 31);
-            if (!(atomicOr(&bm[v >> 5], b) & b)) q[atomicAdd(&s_tail, 1u)] = v;
-        }
+        nxt = 0;
+        dnxt = 1;
+        for (int i = threadIdx.x; i < a.k; i += blockDim.x) add((uint32_t)a.seeds[i]);
         __syncthreads();
-        uint32_t head = 0;
+        uint32_t act = 0;  // nodes of the rounds before
+        bool drawn = false;
+        unsigned long long walked = 0;
         // every round either adds a node or ends the cascade: at most n + 1 rounds
         for (uint64_t round = 0; round <= a.n; round++) {
-            const uint32_t tail = s_tail;
-            if (head >= tail) break;
-            if (threadIdx.x == 0) s_next = head;
-            __syncthreads();
-            for (;;) {
-                uint32_t i = 0;
-                if (lane == 0) i = atomicAdd(&s_next, 1u);
-                i = __shfl_sync(0xffffffffu, i, 0);
-                if (i >= tail) break;
-                const uint32_t u = __ldcg(q + i);
-                const uint64_t e0 = __ldg(a.out_rowptr + u), e1 = __ldg(a.out_rowptr + u + 1);
-                for (uint64_t e = e0 + lane; e < e1; e += 32) {
-                    const uint2 r = __ldg(a.out_rec + e);
-                    const uint32_t j = r.x, v = r.y;
-                    const uint32_t b = 1u << (v & 31);
-                    // a plain (L2) read first: a stale zero only costs a draw
-                    if (__ldcg(bm + (v >> 5)) & b) continue;
-                    bool kept;
-                    if (a.model == TIM_IC) {
-                        const uint4 x = philox4x32_10(s0, s1, j >> 2, TIM_TAG_IC, a.K);
-                        const uint32_t w = (j & 3) == 0 ? x.x : (j & 3) == 1 ? x.y
-                                         : (j & 3) == 2 ? x.z : x.w;
-                        const uint32_t t = __ldg(a.thr + j);
-                        kept = t == 0xFFFFFFFFu || w < t;
-                    } else if (a.model == TIM_TRIG) {
-                        kept = trig_kept(a, s0, s1, v, j);
-                    } else {
-                        kept = lt_kept(a, s0, s1, v, j);
-                    }
-                    if (kept && !(atomicOr(&bm[v >> 5], b) & b)) q[atomicAdd(&s_tail, 1u)] = v;
-                }
+            const uint32_t f = s_tail;
+            if (f == 0) break;
+            cur = nxt;
+            dcur = dnxt;
+            if (SM) {
+                nxt = cur ? 0 : (int64_t)a.n - 1;
+                dnxt = -dcur;
+            } else {
+                nxt = cur + f;
+            }
+            act += f;
+            __syncthreads();  // every thread has read s_tail
+            if (threadIdx.x == 0) {
+                s_next = 0;
+                s_edges = 0;
+                s_tail = 0;
             }
             __syncthreads();
-            head = tail;
+            if (!drawn && a.draw_at != ~0ull) {
+                unsigned long long d = 0;
+                for (uint32_t i = threadIdx.x; i < f; i += blockDim.x) {
+                    const uint32_t u = __ldcg(q + cur + dcur * (int64_t)i);
+                    const uint2 row = __ldg(a.out_row + u);
+                    d += row.y - row.x;
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+                if (lane == 0 && d) atomicAdd(&s_edges, d);
+                __syncthreads();
+                walked += s_edges;
+                if (walked > a.draw_at) {
+                    draw_world(a, s0, s1, bm, live, s_stage);
+                    drawn = true;
+                }
+            }
+            // warps claim the round's nodes, up to 32 at a time (fewer when the round has
+            // few nodes for its warps), and flatten their rows over the lanes: one out-edge
+            // per lane, or one word of 32 live bits
+            const uint32_t per = min(32u, max(1u, f / (blockDim.x >> 5)));
+            uint32_t held = 0;  // live out-records staged by this warp
+            // destinations of the staged records, four per lane in flight; the new ones join
+            // the queue with one counter update per warp
+            auto take = [&]() {
+                __syncwarp();
+                for (uint32_t i = 0; i < held; i += 128) {
+                    uint32_t v[4];
+#pragma unroll
+                    for (int k = 0; k < 4; k++) {
+                        const uint32_t x = i + 32 * k + lane;
+                        v[k] = x < held ? __ldg(&a.out_rec[st[x]].y) : ~0u;
+                    }
+#pragma unroll
+                    for (int k = 0; k < 4; k++) {
+                        const uint32_t b = 1u << (v[k] & 31);
+                        const bool fresh = v[k] != ~0u && !seen(v[k]) &&
+                                           !(atomicOr(&bm[v[k] >> 5], b) & b);
+                        const uint32_t fm = __ballot_sync(0xffffffffu, fresh);
+                        if (!fm) continue;
+                        uint32_t base = 0;
+                        if (lane == 0) base = atomicAdd(&s_tail, (uint32_t)__popc(fm));
+                        base = __shfl_sync(0xffffffffu, base, 0) + __popc(fm & ((1u << lane) - 1u));
+                        if (fresh) q[nxt + dnxt * (int64_t)base] = v[k];
+                    }
+                }
+                __syncwarp();
+            };
+            for (;;) {
+                uint32_t i0 = 0;
+                if (lane == 0) i0 = atomicAdd(&s_next, per);
+                i0 = __shfl_sync(0xffffffffu, i0, 0);
+                if (i0 >= f) break;
+                uint2 row = make_uint2(0u, 0u);
+                if ((uint32_t)lane < per && i0 + lane < f)
+                    row = __ldg(a.out_row + __ldcg(q + cur + dcur * (int64_t)(i0 + lane)));
+                // m < 2^32: a warp's distinct rows have fewer than 2^32 edges together
+                const uint32_t n32 = row.y - row.x;
+                const uint32_t r0 = drawn ? row.x >> 5 : row.x;
+                const uint32_t cnt = n32 == 0 || !drawn ? n32 : ((row.y - 1) >> 5) - r0 + 1;
+                uint32_t incl = cnt;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += y;
+                }
+                const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+                const uint32_t excl = incl - cnt;
+                // the lane whose row holds unit t of the flattened rows
+                auto owner = [&](uint32_t t) {
+                    int own = 0;  // number of lanes whose inclusive count is <= t
+#pragma unroll
+                    for (int sft = 16; sft > 0; sft >>= 1) {
+                        const uint32_t ic = __shfl_sync(0xffffffffu, incl, own + sft - 1);
+                        if (ic <= t) own += sft;
+                    }
+                    return own;
+                };
+                if (!drawn) {
+                    for (uint32_t base = 0; base < total; base += 64) {
+                        uint2 r[2];
+#pragma unroll
+                        for (int i = 0; i < 2; i++) {
+                            const uint32_t t = base + 32 * i + lane;
+                            const int own = owner(t);
+                            const uint32_t at = __shfl_sync(0xffffffffu, r0, own) +
+                                                (t - __shfl_sync(0xffffffffu, excl, own));
+                            r[i] = t < total ? __ldg(a.out_rec + at) : make_uint2(0u, ~0u);
+                        }
+#pragma unroll
+                        for (int i = 0; i < 2; i++)
+                            if (r[i].y != ~0u && !seen(r[i].y) &&
+                                edge_kept(a, s0, s1, r[i].y, r[i].x))
+                                add(r[i].y);
+                    }
+                    continue;
+                }
+                for (uint32_t base = 0; base < total; base += 64) {
+                    uint32_t at[2], w[2];
+#pragma unroll
+                    for (int i = 0; i < 2; i++) {
+                        const uint32_t t = base + 32 * i + lane;
+                        const int own = owner(t);
+                        at[i] = __shfl_sync(0xffffffffu, r0, own) +
+                                (t - __shfl_sync(0xffffffffu, excl, own));
+                        const uint32_t ob = __shfl_sync(0xffffffffu, row.x, own);
+                        const uint32_t oe = __shfl_sync(0xffffffffu, row.y, own);
+                        w[i] = 0;
+                        if (t < total) {  // bits of word `at` of the out-records ob .. oe - 1
+                            w[i] = __ldcg(live + at[i]);
+                            if (at[i] == ob >> 5) w[i] &= 0xFFFFFFFFu << (ob & 31);
+                            if (at[i] == (oe - 1) >> 5) w[i] &= 0xFFFFFFFFu >> (31 - ((oe - 1) & 31));
+                        }
+                    }
+                    const uint32_t wc = __popc(w[0]) + __popc(w[1]);
+                    uint32_t wi = wc;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const uint32_t y = __shfl_up_sync(0xffffffffu, wi, o);
+                        if (lane >= o) wi += y;
+                    }
+                    const uint32_t wt = __shfl_sync(0xffffffffu, wi, 31);
+                    if (wt == 0) continue;
+                    if (held + wt > MC_STAGE) {
+                        take();
+                        held = 0;
+                    }
+                    uint32_t p = held + wi - wc;
+                    const bool fits = wt <= MC_STAGE;
+#pragma unroll
+                    for (int i = 0; i < 2; i++)
+                        for (uint32_t x = w[i]; x; x &= x - 1) {
+                            const uint32_t e = (at[i] << 5) + (__ffs(x) - 1);
+                            if (fits) {
+                                st[p++] = e;
+                            } else {
+                                const uint32_t v = __ldg(&a.out_rec[e].y);
+                                if (!seen(v)) add(v);
+                            }
+                        }
+                    if (fits) held += wt;
+                }
+            }
+            take();
+            held = 0;
+            __syncthreads();
         }
-        const uint32_t act = s_tail;
         if (threadIdx.x == 0) {
             a.counts[c] = act;
             atomicAdd(&a.scal[1], (unsigned long long)act);
         }
-        // leave the bitmap all-zero: every set bit belongs to a queued node
-        for (uint32_t i = threadIdx.x; i < act; i += blockDim.x) bm[__ldcg(q + i) >> 5] = 0u;
-        __syncthreads();
+        // leave the bitmap all-zero
+        if (SM)
+            for (uint32_t w = threadIdx.x; w < (uint32_t)a.words; w += blockDim.x) bm[w] = 0u;
+        else  // every set bit belongs to a queued node
+            for (uint32_t i = threadIdx.x; i < act; i += blockDim.x) bm[__ldcg(q + i) >> 5] = 0u;
     }
 }
 
-int build_out_records(tim_ctx* ctx) {
+// out_pos (4 B per edge) only when worlds are drawn (a function of the graph's size).
+int build_out_records(tim_ctx* ctx, bool draws) {
     if (ctx->have_out) return TIM_OK;
     const uint64_t n = (uint64_t)ctx->n, m = (uint64_t)ctx->m;
     TIM_TRY(tim_ensure(ctx, ctx->out_rowptr, (n + 1) * sizeof(uint64_t)));
     TIM_TRY(tim_ensure(ctx, ctx->out_rec, std::max<uint64_t>(m, 1) * sizeof(uint2)));
+    if (draws)
+        TIM_TRY(tim_ensure(ctx, ctx->out_pos, std::max<uint64_t>(m, 1) * sizeof(uint32_t)));
     TIM_TRY(tim_ensure(ctx, ctx->scratch_a, (n + 1) * sizeof(uint32_t)));
     auto* cnt = (uint32_t*)ctx->scratch_a.p;
     CUDA_TRY(ctx, cudaMemsetAsync(cnt, 0, (n + 1) * sizeof(uint32_t), ctx->stream));
@@ -188,11 +535,16 @@ int build_out_records(tim_ctx* ctx) {
         LAUNCH_CHECK(ctx, "out_count_kernel");
     }
     TIM_TRY(tim_scan_u32_to_u64(ctx, cnt, (uint64_t*)ctx->out_rowptr.p, n));
+    TIM_TRY(tim_ensure(ctx, ctx->out_row, n * sizeof(uint2)));
+    out_rows_kernel<<<G, 256, 0, ctx->stream>>>((const uint64_t*)ctx->out_rowptr.p, n,
+                                                (uint2*)ctx->out_row.p);
+    LAUNCH_CHECK(ctx, "out_rows_kernel");
     CUDA_TRY(ctx, cudaMemsetAsync(cnt, 0, (n + 1) * sizeof(uint32_t), ctx->stream));
     if (m) {
         out_scatter_kernel<<<G, 256, 0, ctx->stream>>>(
             (const uint64_t*)ctx->rowptr.p, (const uint32_t*)ctx->src.p, n,
-            (const uint64_t*)ctx->out_rowptr.p, cnt, (uint2*)ctx->out_rec.p);
+            (const uint64_t*)ctx->out_rowptr.p, cnt, (uint2*)ctx->out_rec.p,
+            draws ? (uint32_t*)ctx->out_pos.p : nullptr);
         LAUNCH_CHECK(ctx, "out_scatter_kernel");
     }
     ctx->have_out = true;
@@ -216,20 +568,44 @@ extern "C" int tim_spread_mc(tim_ctx* ctx, const int32_t* seeds, int k, uint64_t
     if (total) *total = 0;
     if (mean) *mean = 0.0;
     if (count == 0) return TIM_OK;
-    TIM_TRY(build_out_records(ctx));
-    // one bitmap + queue per resident block, within ~4 GiB
+    // visited bitmap in shared memory while one block of it fits on an SM; two blocks of 768
+    // threads per SM while two bitmaps fit, one of 1024 beyond that (50 seeds on R-MAT 18, 2000
+    // IC and 1000 LT cascades: 2 x 768 threads 10.9 and 7.4 ms, 1 x 1024 12.4 and 8.8, 3 x 512
+    // 10.9 and 8.2)
     const uint64_t words = n / 32 + 1;
-    const uint64_t per_slot = words * 4 + n * 4;
-    uint64_t slots = std::max<uint64_t>(1, (4ull << 30) / per_slot);
-    slots = std::min<uint64_t>(slots, (uint64_t)ctx->num_sms * 4);
+    const bool sm = words * 4 <= MC_SMEM_MAX, two = words * 4 <= MC_SMEM_TWO;
+    const size_t smem = sm ? (size_t)words * 4 : 0;
+    const int threads = sm && !two ? 1024 : 768;
+    const void* kernel = !sm ? (const void*)mc_cascade_kernel<false, 768, 2>
+                       : two ? (const void*)mc_cascade_kernel<true, 768, 2>
+                             : (const void*)mc_cascade_kernel<true, 1024, 1>;
+    if (sm)
+        CUDA_TRY(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)(two ? MC_SMEM_TWO : MC_SMEM_MAX)));
+    int nb = 0;
+    CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, threads, smem));
+    nb = std::max(nb, 1);
+    // queue, live bits and (outside shared memory) bitmap per resident block, within
+    // ~4 GiB; worlds are drawn when that leaves at least a block per SM
+    const uint64_t budget = 4ull << 30;
+    const uint64_t live_words = ((uint64_t)ctx->m + 127) / 128 * 4;
+    const uint64_t base = n * 4 + (sm ? 0 : words * 4);
+    const bool draws = budget / (base + live_words * 4) >= (uint64_t)ctx->num_sms;
+    TIM_TRY(build_out_records(ctx, draws));
+    const uint64_t per_slot = base + (draws ? live_words * 4 : 0);
+    uint64_t slots = std::max<uint64_t>(1, budget / per_slot);
+    slots = std::min<uint64_t>(slots, (uint64_t)ctx->num_sms * nb);
     slots = std::min<uint64_t>(slots, count);
-    void* prev = ctx->mc_bitmap.p;
-    TIM_TRY(tim_ensure(ctx, ctx->mc_bitmap, slots * words * 4));
-    if (ctx->mc_bitmap.p != prev || !ctx->mc_clean) {
-        CUDA_TRY(ctx, cudaMemsetAsync(ctx->mc_bitmap.p, 0, ctx->mc_bitmap.bytes, ctx->stream));
-        ctx->mc_clean = true;
+    if (!sm) {
+        void* prev = ctx->mc_bitmap.p;
+        TIM_TRY(tim_ensure(ctx, ctx->mc_bitmap, slots * words * 4));
+        if (ctx->mc_bitmap.p != prev || !ctx->mc_clean) {
+            CUDA_TRY(ctx, cudaMemsetAsync(ctx->mc_bitmap.p, 0, ctx->mc_bitmap.bytes, ctx->stream));
+            ctx->mc_clean = true;
+        }
     }
     TIM_TRY(tim_ensure(ctx, ctx->mc_queue, slots * n * 4));
+    TIM_TRY(tim_ensure(ctx, ctx->mc_live, draws ? slots * live_words * 4 : 16));
     TIM_TRY(tim_ensure(ctx, ctx->mc_counts, count * 4));
     TIM_TRY(tim_ensure(ctx, ctx->mc_seeds, std::max(k, 1) * sizeof(int32_t)));
     TIM_TRY(tim_ensure(ctx, ctx->mc_scal, 2 * sizeof(unsigned long long)));
@@ -241,10 +617,12 @@ extern "C" int tim_spread_mc(tim_ctx* ctx, const int32_t* seeds, int k, uint64_t
     a.rowptr = (const uint64_t*)ctx->rowptr.p;
     a.thr = (const uint32_t*)ctx->thr.p;
     a.node_thr = (const unsigned long long*)ctx->node_thr.p;
-    a.out_rowptr = (const uint64_t*)ctx->out_rowptr.p;
+    a.out_row = (const uint2*)ctx->out_row.p;
     a.out_rec = (const uint2*)ctx->out_rec.p;
+    a.out_pos = (const uint32_t*)ctx->out_pos.p;
     a.model = ctx->model;
     a.n = n;
+    a.m = (uint64_t)ctx->m;
     a.K = tim_philox_keys(seed);
     a.sid0 = first_set_id;
     a.count = count;
@@ -253,14 +631,19 @@ extern "C" int tim_spread_mc(tim_ctx* ctx, const int32_t* seeds, int k, uint64_t
     a.bitmap = (uint32_t*)ctx->mc_bitmap.p;
     a.queue = (uint32_t*)ctx->mc_queue.p;
     a.words = words;
+    a.live = (uint32_t*)ctx->mc_live.p;
+    a.live_words = draws ? live_words : 0;
+    a.draw_at = !draws ? ~0ull
+                       : (ctx->model == TIM_IC ? (unsigned long long)ctx->m / 4 : n) / MC_WALK;
     a.counts = (uint32_t*)ctx->mc_counts.p;
     a.scal = (unsigned long long*)ctx->mc_scal.p;
     a.node_opt = (const uint64_t*)ctx->node_opt.p;
     a.opt_cum = (const uint32_t*)ctx->opt_cum.p;
     a.opt_off = (const uint64_t*)ctx->opt_off.p;
     a.opt_pos = (const uint32_t*)ctx->opt_pos.p;
-    ctx->mc_clean = false;
-    mc_cascade_kernel<<<(unsigned)slots, MC_THREADS, 0, ctx->stream>>>(a);
+    if (!sm) ctx->mc_clean = false;
+    void* args[] = {&a};
+    CUDA_TRY(ctx, cudaLaunchKernel(kernel, dim3((unsigned)slots), dim3(threads), args, smem, ctx->stream));
     LAUNCH_CHECK(ctx, "mc_cascade_kernel");
     unsigned long long h[2] = {0, 0};
     CUDA_TRY(ctx, cudaMemcpyAsync(h, ctx->mc_scal.p, sizeof h, cudaMemcpyDeviceToHost,
@@ -269,7 +652,7 @@ extern "C" int tim_spread_mc(tim_ctx* ctx, const int32_t* seeds, int k, uint64_t
         CUDA_TRY(ctx, cudaMemcpyAsync(counts_out, ctx->mc_counts.p, count * 4,
                                       cudaMemcpyDeviceToHost, ctx->stream));
     TIM_TRY(tim_sync(ctx));
-    ctx->mc_clean = true;
+    if (!sm) ctx->mc_clean = true;
     if (total) *total = h[1];
     if (mean) *mean = (double)h[1] / (double)count;
     return TIM_OK;
