@@ -312,8 +312,10 @@ int tim_set_pass1_capacity(tim_ctx* ctx, int members);
 
 /* IC sampler tuning: pass 2 (a team of warps per RR set, queue of 8192 members) hands a
  * set to the heavy-set pass, whose warps spread each in-list over the whole GPU, once
- * the in-edges the team would examine exceed `budget` (default 2^64 - 1: only sets that
- * outgrow the queue go there). Results do not change. */
+ * the in-edges the team would examine exceed `budget` (default 2^64 - 1). Sets that outgrow
+ * the queue, or whose coins in long in-lists (512 in-edges or more, outside the
+ * geometric-skip rule) would pass a fixed number, go there whatever the budget. Results do
+ * not change. */
 int tim_set_pass2_budget(tim_ctx* ctx, uint64_t budget);
 
 /* Polls a block makes at a grid barrier of a persistent kernel (the heavy-set pass of

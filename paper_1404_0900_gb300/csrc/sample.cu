@@ -42,6 +42,14 @@ constexpr int ST_OVERFLOW = 1;
 constexpr int ST_COVERED = 2;
 constexpr int WARPS = 8;          // warps per CTA (tiers 1 and 2)
 constexpr int BIG_THREADS = 256;  // tier 3 LT CTA size
+// IC, tier 2 hands a set to the heavy-set pass once it would have drawn this many coins in
+// lists of TIM_SKIP_MIN_INDEG in-edges or more (lists under the skip rule draw none): one
+// team streams such a list while the rest of the GPU waits for it, the heavy-set pass
+// spreads it over every SM. TIM+ at 1024, 2048, 4096, 8192, 16384, 65536 and no limit:
+// trivalency on Chung-Lu graphs of 100,001 nodes 9.4 9.4 9.1 9.4 9.8 10.9 12.0 ms, 700,001
+// nodes 18.9 19.1 19.5 20.4 22.1 29.5 44.7, 4.16M nodes 38.1 38.5 38.8 40.2 42.4 59.4 83.5,
+// 41.6M nodes - 225.9 224.0 220.3 220.1 229.6 247.3.
+constexpr unsigned long long LONG_BUDGET2 = 6144;
 
 // Queue capacity Q and hash size 2^LOG2H (>= 2Q) of one warp's set.
 template <int QQ, int LG>
@@ -85,6 +93,7 @@ struct SampleArgs {
     uint64_t big_words;
     unsigned long long width_budget;  // tier 1 IC: in-edges one warp may examine per set
     unsigned long long width_budget2; // tier 2 IC: in-edges one team may examine per set
+    unsigned long long long_budget2;  // tier 2 IC: and in lists of 512 or more
     int chunk;                        // sets claimed per work-counter increment
     uint32_t* lt_col;                 // tier 1 LT: per-thread member columns
     // IC: the state pass 1 hands to pass 2 for the set at list1 position i < hcap, hw
@@ -247,7 +256,8 @@ struct Resume {
 template <int MODEL, class C, int T, class A>
 __device__ __forceinline__ int team_rr(const A& a, const PhiloxKeys& K, uint64_t sid, uint32_t* hash,
                                        uint32_t* queue, uint16_t* slot, int* ctl,
-                                       unsigned long long budget, int wt, int team,
+                                       unsigned long long budget,
+                                       unsigned long long long_budget, int wt, int team,
                                        unsigned long long* width_out,
                                        unsigned long long* live_out,
                                        unsigned long long* exam_out,
@@ -265,7 +275,7 @@ __device__ __forceinline__ int team_rr(const A& a, const PhiloxKeys& K, uint64_t
         ctl[1] = (cover && marked(a.seed_mark, root)) ? ST_COVERED : 0;
     }
     team_sync<T>(team);
-    unsigned long long width = in ? in->width : 0, live = 0, work = 0, exam = 0;
+    unsigned long long width = in ? in->width : 0, live = 0, work = 0, longs = 0, exam = 0;
     if constexpr (MODEL == TIM_IC) {
         const uint32_t s0 = (uint32_t)sid, s1 = (uint32_t)(sid >> 32);
         const uint4* thr4 = reinterpret_cast<const uint4*>(a.thr);
@@ -306,12 +316,17 @@ __device__ __forceinline__ int team_rr(const A& a, const PhiloxKeys& K, uint64_t
             // most 64
             const unsigned long long dx = __reduce_add_sync(
                 0xffffffffu, (unsigned)(skip_list ? min(end - beg, (uint64_t)64) : end - beg));
-            if (work + dx > budget) {
+            // in-edges of long lists that take a coin each, streamed by this team alone
+            const unsigned long long dl = __reduce_add_sync(
+                0xffffffffu,
+                (unsigned)(!skip_list && end - beg >= TIM_SKIP_MIN_INDEG ? end - beg : 0ull));
+            if (work + dx > budget || longs + dl > long_budget) {
                 // too heavy for this tier: list the set for the next one
                 if (wt == 0 && lane == 0) ctl[1] |= ST_OVERFLOW;
                 break;
             }
             work += dx;
+            longs += dl;
             width += dw;
             // examined in-edges: every in-edge of a list outside the skip rule (the live
             // ones the rule finds are added as they are found)
@@ -589,6 +604,7 @@ __global__ void __launch_bounds__(WARPS * 32, TIER == 1 ? 4 : 6) rr_team_kernel(
     int* ctl = TIER == 1 ? reinterpret_cast<int*>(queue + C::Q + C::Q / 2) : s_ctl[team];
     const unsigned long long budget =
         MODEL != TIM_IC ? ~0ull : TIER == 1 ? a.width_budget : a.width_budget2;
+    const unsigned long long long_budget = MODEL == TIM_IC && TIER == 2 ? a.long_budget2 : ~0ull;
     unsigned long long* counter = TIER == 1 ? &a.ds->next_set : &a.ds->next2;
     const uint64_t items =
         TIER == 1 ? a.count : (uint64_t)min(((volatile unsigned*)&a.ds->cnt1)[0], a.list_cap);
@@ -653,7 +669,7 @@ __global__ void __launch_bounds__(WARPS * 32, TIER == 1 ? 4 : 6) rr_team_kernel(
                 team_sync<T>(team);
             }
             const int st = team_rr<MODEL, C, T, SampleArgs>(
-                a, a.K, a.sid0 + j, hash, queue, slot, ctl, budget, wt, team, &width, &live,
+                a, a.K, a.sid0 + j, hash, queue, slot, ctl, budget, long_budget, wt, team, &width, &live,
                 &exam, resumed ? &rin : nullptr,
                 (HAND && ((TIER == 1 && a.hand) || (TIER == 2 && a.hand2))) ? &rout : nullptr);
             const int tail = min(T == 1 ? __shfl_sync(0xffffffffu, ((volatile int*)ctl)[0], 0)
@@ -1534,12 +1550,12 @@ __global__ void __launch_bounds__(WARPS * 32, 3) rr_multi_kernel(MultiArgs ma) {
             }
             if (model == TIM_IC)
                 st = team_rr<TIM_IC, C, T, QArgs>(qa, ma.K, d.sid0 + j, hash, queue, slot, ctl,
-                                                  budget, wt, team, &width, &acc.live,
+                                                  budget, ~0ull, wt, team, &width, &acc.live,
                                                   &acc.exam, resumed ? &rin : nullptr,
                                                   (TIER == 1 && ma.hand) ? &rout : nullptr);
             else
                 st = team_rr<TIM_LT, C, T, QArgs>(qa, ma.K, d.sid0 + j, hash, queue, slot, ctl,
-                                                  budget, wt, team, &width, &acc.live,
+                                                  budget, ~0ull, wt, team, &width, &acc.live,
                                                   &acc.exam);
             const int tail = min(T == 1 ? __shfl_sync(0xffffffffu, ((volatile int*)ctl)[0], 0)
                                         : ((volatile int*)ctl)[0],
@@ -1945,6 +1961,7 @@ int tim_sample(tim_ctx* ctx, const SampleRequest& req, SampleResult* res) {
     a.set_width = (uint64_t*)ctx->set_width.p;
     a.width_budget = ctx->width_budget;
     a.width_budget2 = ctx->width_budget2;
+    a.long_budget2 = LONG_BUDGET2;
     a.chunk = std::max(1, ctx->chunk);
     // IC: room for the pass-1 state of up to count / 8 + 4096 handed-over sets (at most
     // 1 GiB); sets listed beyond it start over in pass 2
