@@ -78,6 +78,8 @@ struct tim_ctx {
     DevBuf set_start;  // uint64[n_sets]
     DevBuf set_len;    // uint32[n_sets]
     DevBuf set_width;  // uint64[n_sets]
+    // second store: the rounds of Algorithm 2 sampled in one call, and their sums
+    DevBuf pool2, pool_sid2, set_start2, set_len2, set_width2, round_sums;
 
     // greedy / index
     DevBuf counts;     // int32[n]
@@ -252,9 +254,22 @@ int tim_trig_build(tim_ctx* ctx, const int32_t* d_out_dst, const uint64_t* d_nod
 
 // sample.cu
 enum : int { SAMPLE_EMIT = 1, SAMPLE_KAPPA = 2, SAMPLE_COVER = 4 };
+
+// Set ids of a sampling call: set j has id sid0 + j; with n > 0 the call holds the sets of n
+// consecutive rounds one after another, round r's at start[r] <= j < start[r + 1], with ids
+// sid0 + (r << 48) + (j - start[r]) (make_sid).
+constexpr int SID_ROUNDS = 16;
+struct SidMap {
+    uint64_t sid0;
+    uint32_t n;
+    uint32_t start[SID_ROUNDS];
+};
+
 struct SampleRequest {
     uint64_t seed = 0;
     uint64_t sid0 = 0;
+    int rounds = 0;                        // > 0: several rounds (SidMap)
+    uint32_t round_start[SID_ROUNDS] = {};
     uint64_t count = 0;
     int flags = 0;
     int k = 0;                         // kappa
@@ -269,6 +284,16 @@ struct SampleResult {
     uint64_t big_sets = 0;
 };
 int tim_sample(tim_ctx* ctx, const SampleRequest& req, SampleResult* res);
+// Algorithm 2's rounds first .. first + rounds - 1 in one sampling call, their sets kept apart
+// in the context's second store; per round the kappa sum (Eq. 6), the width sum and sum |R|.
+struct RoundSums {
+    unsigned long long lo, hi, width, members;
+};
+int tim_sample_rounds(tim_ctx* ctx, SampleRequest req, const uint64_t* counts, int rounds,
+                      RoundSums* sums);
+// Makes round r of the last tim_sample_rounds (the sets [start, start + count), `members` of
+// them in all) the RR-set store.
+int tim_keep_round(tim_ctx* ctx, uint64_t start, uint64_t count, uint64_t members);
 // Third tier for the heavy IC sets list[0 .. count) (sample_bulk.cu). With hand (may be
 // null), the set at list position i < hcap starts from the state pass 2 left at
 // hand + i hw: queue length, position of the batch to redo, then the queue.
@@ -331,6 +356,14 @@ struct PhiloxKeys {
     uint32_t k1[10];
 };
 
+static inline SidMap tim_sid_map(const SampleRequest& req) {
+    SidMap s{};
+    s.sid0 = req.sid0;
+    s.n = (uint32_t)req.rounds;
+    for (int r = 0; r < req.rounds; r++) s.start[r] = req.round_start[r];
+    return s;
+}
+
 static inline PhiloxKeys tim_philox_keys(uint64_t seed) {
     PhiloxKeys K;
     uint32_t a = (uint32_t)seed, b = (uint32_t)(seed >> 32);
@@ -344,6 +377,13 @@ static inline PhiloxKeys tim_philox_keys(uint64_t seed) {
 }
 
 #ifdef __CUDACC__
+__device__ __forceinline__ uint64_t sid_of(const SidMap& s, uint64_t j) {
+    uint64_t sid = s.sid0 + j;
+    for (uint32_t r = 1; r < s.n; r++)
+        if (j >= s.start[r]) sid = s.sid0 + ((uint64_t)r << 48) + (j - s.start[r]);
+    return sid;
+}
+
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11): ten rounds of two 32x32->64
 // multiplies and xors with the precomputed round keys.
 __device__ __forceinline__ uint4 philox4x32_10(uint32_t c0, uint32_t c1, uint32_t c2,

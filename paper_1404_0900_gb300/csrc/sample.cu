@@ -74,7 +74,8 @@ struct SampleArgs {
     const unsigned long long* qtab;      // IC: gap tables of skip-rule nodes
     uint64_t n, m;
     PhiloxKeys K;
-    uint64_t sid0, count;
+    SidMap ids;
+    uint64_t count;
     int flags, k;
     const uint32_t* seed_mark;
     uint32_t* pool;
@@ -669,7 +670,7 @@ __global__ void __launch_bounds__(WARPS * 32, TIER == 1 ? 4 : 6) rr_team_kernel(
                 team_sync<T>(team);
             }
             const int st = team_rr<MODEL, C, T, SampleArgs>(
-                a, a.K, a.sid0 + j, hash, queue, slot, ctl, budget, long_budget, wt, team, &width, &live,
+                a, a.K, sid_of(a.ids, j), hash, queue, slot, ctl, budget, long_budget, wt, team, &width, &live,
                 &exam, resumed ? &rin : nullptr,
                 (HAND && ((TIER == 1 && a.hand) || (TIER == 2 && a.hand2))) ? &rout : nullptr);
             const int tail = min(T == 1 ? __shfl_sync(0xffffffffu, ((volatile int*)ctl)[0], 0)
@@ -868,7 +869,7 @@ __global__ void __launch_bounds__(LT_THREADS) rr_lt_lane_kernel(SampleArgs a) {
                 const unsigned long long mine = base + __popc(nm & ((1u << lane) - 1u));
                 if (mine < a.count) {
                     j = mine;
-                    sid = a.sid0 + j;
+                    sid = sid_of(a.ids, j);
                     v = rr_root(sid, a.n, a.K);
                     col[0] = v;
                     len = 1;
@@ -1040,7 +1041,7 @@ __global__ void __launch_bounds__(BIG_THREADS) rr_lt_chain_kernel(SampleArgs a) 
         unsigned long long idx = s_j;
         if (idx >= nlist) break;
         uint64_t j = a.list2[idx];
-        uint64_t sid = a.sid0 + j;
+        uint64_t sid = sid_of(a.ids, j);
         uint32_t root = rr_root(sid, a.n, a.K);
         if (tid == 0) {
             atomicOr(&bitmap[root >> 5], 1u << (root & 31));
@@ -1162,7 +1163,7 @@ __global__ void __launch_bounds__(BIG_THREADS) rr_trig_big_kernel(SampleArgs a) 
         const unsigned long long idx = s_j;
         if (idx >= nlist) break;
         const uint64_t j = a.list2[idx];
-        const uint64_t sid = a.sid0 + j;
+        const uint64_t sid = sid_of(a.ids, j);
         const uint32_t root = rr_root(sid, a.n, a.K);
         if (tid == 0) {
             atomicOr(&bitmap[root >> 5], 1u << (root & 31));
@@ -1943,7 +1944,7 @@ int tim_sample(tim_ctx* ctx, const SampleRequest& req, SampleResult* res) {
     a.n = (uint64_t)ctx->n;
     a.m = (uint64_t)ctx->m;
     a.K = tim_philox_keys(req.seed);
-    a.sid0 = req.sid0;
+    a.ids = tim_sid_map(req);
     a.count = count;
     a.flags = req.flags;
     a.k = req.k;
@@ -1995,6 +1996,7 @@ int tim_sample(tim_ctx* ctx, const SampleRequest& req, SampleResult* res) {
         a.pool_cap = emit ? ctx->pool.bytes / sizeof(uint32_t) : 0;
         TIM_TRY(tim_zero_scalars(ctx));
         uint64_t live3 = 0;
+        bool read = false;
         if (count > 0) {
             cudaEventRecord(ctx->kev[0], ctx->stream);
             TIM_TRY(launch_tier1(ctx, a, grid1, smem1));
@@ -2017,6 +2019,7 @@ int tim_sample(tim_ctx* ctx, const SampleRequest& req, SampleResult* res) {
             if (ctx->model == TIM_IC) {
                 TIM_TRY(tim_read_scalars(ctx));
                 const unsigned n3 = std::min(ctx->h_scal->cnt2, list_cap);
+                read = n3 == 0;  // nothing runs after this read
                 TIM_TRY(tim_bulk_ic(ctx, req, a.list2, n3, a.pool, a.pool_sid, a.pool_cap, a.ds,
                                     &live3, a.hand2, a.h2cap, a.h2w));
             } else if (ctx->model == TIM_TRIG) {
@@ -2028,7 +2031,7 @@ int tim_sample(tim_ctx* ctx, const SampleRequest& req, SampleResult* res) {
             }
             cudaEventRecord(ctx->kev[3], ctx->stream);
         }
-        TIM_TRY(tim_read_scalars(ctx));
+        if (!read) TIM_TRY(tim_read_scalars(ctx));
         DevScalars& h = *ctx->h_scal;
         if (ctx->model == TIM_IC) h.live[2] = live3;
         if (h.err & TIM_DEV_ERR_POOL) {
@@ -2045,7 +2048,7 @@ int tim_sample(tim_ctx* ctx, const SampleRequest& req, SampleResult* res) {
         }
         if (count > 0) {
             float t[3] = {0.f, 0.f, 0.f};
-            for (int i = 0; i < 3; i++) cudaEventElapsedTime(&t[i], ctx->kev[i], ctx->kev[i + 1]);
+            for (int i = 0; i < (read ? 2 : 3); i++) cudaEventElapsedTime(&t[i], ctx->kev[i], ctx->kev[i + 1]);
             const uint64_t sets[3] = {count - h.cnt1, (uint64_t)h.cnt1 - h.cnt2, h.cnt2};
             tim_profile& P = ctx->prof;
             uint64_t* L[3] = {&P.pass1_launches, &P.pass2_launches, &P.pass3_launches};
@@ -2081,6 +2084,127 @@ int tim_sample(tim_ctx* ctx, const SampleRequest& req, SampleResult* res) {
         return TIM_OK;
     }
     return tim_fail(ctx, TIM_ERR_OOM, "RR-set store kept overflowing");
+}
+
+// --------------------------------------------- several rounds of Algorithm 2 at once
+
+namespace {
+
+// Round blockIdx.y: sum of kappa over its sets' widths, of the widths and of the sizes.
+__global__ void round_sums_kernel(SidMap ids, uint64_t count, const uint64_t* __restrict__ width,
+                                  const uint32_t* __restrict__ len, uint64_t m, int k,
+                                  RoundSums* __restrict__ out) {
+    const uint32_t r = blockIdx.y;
+    const uint64_t end = r + 1 < ids.n ? ids.start[r + 1] : count;
+    unsigned long long lo = 0, hi = 0, w = 0, memb = 0;
+    for (uint64_t j = ids.start[r] + blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; j < end;
+         j += (uint64_t)gridDim.x * blockDim.x) {
+        const unsigned long long kf = kappa_fixed(kappa_fp64(width[j], m, k));
+        lo += kf;
+        if (lo < kf) hi++;
+        w += width[j];
+        memb += len[j];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long l2 = __shfl_xor_sync(0xffffffffu, lo, o);
+        hi += __shfl_xor_sync(0xffffffffu, hi, o);
+        lo += l2;
+        if (lo < l2) hi++;
+    }
+    w = warp_sum_u64(w);
+    memb = warp_sum_u64(memb);
+    if ((threadIdx.x & 31) == 0 && memb) {
+        if (lo || hi) atomic_add_u128(&out[r].lo, &out[r].hi, lo, hi);
+        atomicAdd(&out[r].width, w);
+        atomicAdd(&out[r].members, memb);
+    }
+}
+
+// Sets [start, start + count) of one store into another, one warp per set.
+__global__ void keep_round_kernel(uint64_t start, uint64_t count,
+                                  const uint32_t* __restrict__ pool,
+                                  const uint64_t* __restrict__ set_start,
+                                  const uint32_t* __restrict__ set_len,
+                                  const uint64_t* __restrict__ set_width,
+                                  uint32_t* __restrict__ pool_out, uint32_t* __restrict__ sid_out,
+                                  uint64_t* __restrict__ start_out, uint32_t* __restrict__ len_out,
+                                  uint64_t* __restrict__ width_out, DevScalars* ds) {
+    const int lane = threadIdx.x & 31;
+    const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+    for (uint64_t j = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5; j < count; j += nw) {
+        const uint64_t from = set_start[start + j];
+        const uint32_t len = set_len[start + j];
+        unsigned long long to = 0;
+        if (lane == 0) {
+            to = atomicAdd(&ds->pool_used, (unsigned long long)len);
+            start_out[j] = to;
+            len_out[j] = len;
+            width_out[j] = set_width[start + j];
+        }
+        to = __shfl_sync(0xffffffffu, to, 0);
+        for (uint32_t i = lane; i < len; i += 32) {
+            pool_out[to + i] = pool[from + i];
+            sid_out[to + i] = (uint32_t)j;
+        }
+    }
+}
+
+void swap_stores(tim_ctx* ctx) {
+    std::swap(ctx->pool, ctx->pool2);
+    std::swap(ctx->pool_sid, ctx->pool_sid2);
+    std::swap(ctx->set_start, ctx->set_start2);
+    std::swap(ctx->set_len, ctx->set_len2);
+    std::swap(ctx->set_width, ctx->set_width2);
+}
+
+}  // namespace
+
+int tim_sample_rounds(tim_ctx* ctx, SampleRequest req, const uint64_t* counts, int rounds,
+                      RoundSums* sums) {
+    req.rounds = rounds;
+    req.count = 0;
+    for (int r = 0; r < rounds; r++) {
+        req.round_start[r] = (uint32_t)req.count;
+        req.count += counts[r];
+    }
+    req.flags = SAMPLE_EMIT;
+    swap_stores(ctx);
+    SampleResult res;
+    const int rc = tim_sample(ctx, req, &res);
+    swap_stores(ctx);
+    ctx->n_sets = ctx->members = 0;
+    TIM_TRY(rc);
+    TIM_TRY(tim_ensure(ctx, ctx->round_sums, SID_ROUNDS * sizeof(RoundSums)));
+    CUDA_TRY(ctx, cudaMemsetAsync(ctx->round_sums.p, 0, rounds * sizeof(RoundSums), ctx->stream));
+    round_sums_kernel<<<dim3(ctx->num_sms, rounds), 128, 0, ctx->stream>>>(
+        tim_sid_map(req), req.count, (const uint64_t*)ctx->set_width2.p,
+        (const uint32_t*)ctx->set_len2.p, (uint64_t)ctx->m, req.k, (RoundSums*)ctx->round_sums.p);
+    LAUNCH_CHECK(ctx, "round_sums_kernel");
+    CUDA_TRY(ctx, cudaMemcpyAsync(sums, ctx->round_sums.p, rounds * sizeof(RoundSums),
+                                  cudaMemcpyDeviceToHost, ctx->stream));
+    return tim_sync(ctx);
+}
+
+int tim_keep_round(tim_ctx* ctx, uint64_t start, uint64_t count, uint64_t members) {
+    TIM_TRY(tim_ensure(ctx, ctx->set_start, (count + 1) * sizeof(uint64_t)));
+    TIM_TRY(tim_ensure(ctx, ctx->set_len, (count + 1) * sizeof(uint32_t)));
+    TIM_TRY(tim_ensure(ctx, ctx->set_width, (count + 1) * sizeof(uint64_t)));
+    if (ctx->pool.bytes < members * sizeof(uint32_t) ||
+        ctx->pool_sid.bytes < members * sizeof(uint32_t)) {
+        TIM_TRY(tim_ensure(ctx, ctx->pool, members * sizeof(uint32_t)));
+        TIM_TRY(tim_ensure(ctx, ctx->pool_sid, members * sizeof(uint32_t)));
+    }
+    TIM_TRY(tim_zero_scalars(ctx));
+    keep_round_kernel<<<(unsigned)(ctx->num_sms * 4), 256, 0, ctx->stream>>>(
+        start, count, (const uint32_t*)ctx->pool2.p, (const uint64_t*)ctx->set_start2.p,
+        (const uint32_t*)ctx->set_len2.p, (const uint64_t*)ctx->set_width2.p,
+        (uint32_t*)ctx->pool.p, (uint32_t*)ctx->pool_sid.p, (uint64_t*)ctx->set_start.p,
+        (uint32_t*)ctx->set_len.p, (uint64_t*)ctx->set_width.p, tim_dscal(ctx));
+    LAUNCH_CHECK(ctx, "keep_round_kernel");
+    ctx->n_sets = count;
+    ctx->members = members;
+    return TIM_OK;
 }
 
 // ----------------------------------------------------- multi-query host driver
@@ -2129,7 +2253,7 @@ int run_tier3(tim_ctx* ctx, cudaStream_t stream, const SampleRequest& req, DevSc
             a.n = (uint64_t)ctx->n;
             a.m = (uint64_t)ctx->m;
             a.K = tim_philox_keys(req.seed);
-            a.sid0 = req.sid0;
+            a.ids = tim_sid_map(req);
             a.count = req.count;
             a.flags = req.flags;
             a.k = req.k;

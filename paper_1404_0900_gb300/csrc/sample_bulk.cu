@@ -56,7 +56,7 @@ struct BulkArgs {
     const unsigned long long* qtab;      // gap tables of skip-rule nodes
     uint64_t n, m;
     PhiloxKeys K;
-    uint64_t sid0;
+    SidMap ids;
     int flags, k;
     const uint32_t* seed_mark;
     const uint32_t* list;  // heavy set indices (relative to sid0)
@@ -66,6 +66,7 @@ struct BulkArgs {
     uint32_t* bitmap;
     uint64_t words;
     unsigned long long* slot_width;
+    uint64_t* slot_sid;  // set id of each slot
     uint32_t* slot_cnt;
     uint32_t* slot_flag;
     unsigned long long* slot_start;
@@ -158,6 +159,8 @@ __global__ void bulk_init_kernel(BulkArgs a) {
         const uint64_t li = (uint64_t)a.base + s;
         const uint32_t* hs = bulk_hand(a, li);
         a.slot_cursor[s] = 0;
+        const uint64_t sid = sid_of(a.ids, a.list[li]);
+        a.slot_sid[s] = sid;
         if (hs) {
             // the width pass 2 counted for the members before the batch it stopped at;
             // bulk_hand_kernel adds the in-degrees of the rest
@@ -166,8 +169,6 @@ __global__ void bulk_init_kernel(BulkArgs a) {
             a.slot_flag[s] = 0u;
             continue;
         }
-        const uint32_t j = a.list[li];
-        const uint64_t sid = a.sid0 + j;
         const uint32_t root = rr_root(sid, a.n, a.K);
         atomicOr(&a.bitmap[(uint64_t)s * a.words + (root >> 5)], 1u << (root & 31));
         const uint64_t beg = a.rowptr[root], end = a.rowptr[root + 1];
@@ -496,7 +497,7 @@ __device__ __forceinline__ void expand_level(const BulkArgs& a, uint64_t lo, uin
                 }
                 uint4 tv[4];
                 uint64_t g[4];
-                uint32_t jj[4];
+                uint64_t sid[4];
                 bool wk[4];
 #pragma unroll
                 for (int k = 0; k < 4; k++) {
@@ -506,14 +507,13 @@ __device__ __forceinline__ void expand_level(const BulkArgs& a, uint64_t lo, uin
                             !(cover && *(volatile uint32_t*)&a.slot_flag[sl]);
                     tv[k] = wk[k] ? __ldg(reinterpret_cast<const uint4*>(a.thr) + g[k])
                                   : make_uint4(0u, 0u, 0u, 0u);
-                    jj[k] = wk[k] ? __ldg(a.list + a.base + sl) : 0u;
+                    sid[k] = wk[k] ? __ldg(a.slot_sid + sl) : 0u;
                 }
                 uint32_t lm = 0;  // bit 4k + cc: position 4 g[k] + cc is live
 #pragma unroll
                 for (int k = 0; k < 4; k++) {
                     if (!wk[k]) continue;
-                    const uint64_t sid = a.sid0 + jj[k];
-                    const uint4 x = philox4x32_10((uint32_t)sid, (uint32_t)(sid >> 32),
+                    const uint4 x = philox4x32_10((uint32_t)sid[k], (uint32_t)(sid[k] >> 32),
                                                   (uint32_t)g[k], TIM_TAG_IC, a.K);
 #pragma unroll
                     for (int cc = 0; cc < 4; cc++) {
@@ -600,7 +600,7 @@ __device__ __forceinline__ void skip_level(const BulkArgs& a, uint64_t lo, uint6
         const uint64_t beg = it.x, end = it.y;
         const unsigned long long nt = __ldg(a.node_thr + v);
         if (cover && *(volatile uint32_t*)&a.slot_flag[s]) continue;
-        const uint64_t sid = a.sid0 + __ldg(a.list + a.base + s);
+        const uint64_t sid = __ldg(a.slot_sid + s);
         skip_live_warp((uint32_t)sid, (uint32_t)(sid >> 32), a.K, (uint32_t)beg,
                        (uint32_t)(end - beg), skip_table(a.qtab, nt), lane, [&](uint32_t p) {
                            bool fresh = false;
@@ -914,7 +914,7 @@ int tim_bulk_ic(tim_ctx* ctx, const SampleRequest& req, const uint32_t* list, ui
     a.n = n;
     a.m = (uint64_t)ctx->m;
     a.K = tim_philox_keys(req.seed);
-    a.sid0 = req.sid0;
+    a.ids = tim_sid_map(req);
     a.flags = req.flags;
     a.k = req.k;
     a.seed_mark = req.seed_mark;
@@ -930,6 +930,7 @@ int tim_bulk_ic(tim_ctx* ctx, const SampleRequest& req, const uint32_t* list, ui
     a.slot_cnt = (uint32_t*)(sl + smax * 16);
     a.slot_flag = (uint32_t*)(sl + smax * 20);
     a.slot_cursor = (uint32_t*)(sl + smax * 24);
+    a.slot_sid = (uint64_t*)(sl + smax * 32);
     a.bs = (BulkScalars*)ctx->bulk_scal.p;
     a.ds = ds;
     a.pool = pool;
