@@ -180,7 +180,7 @@ int tim_destroy(tim_ctx* ctx) {
     DeviceGuard g(ctx->device);
     if (ctx->stream) cudaStreamSynchronize(ctx->stream);
     DevBuf* bufs[] = {&ctx->rowptr,   &ctx->src,        &ctx->thr,       &ctx->pool,
-                      &ctx->node_thr,  &ctx->qtab,      &ctx->ld_keys,   &ctx->ld_vals,
+                      &ctx->node,  &ctx->qtab,      &ctx->ld_keys,   &ctx->ld_vals,
                       &ctx->ld_lt_t,   &ctx->ld_lt_e,   &ctx->ld_nonuni,
                       &ctx->ld_srcof,
                       &ctx->pool2, &ctx->pool_sid2, &ctx->set_start2, &ctx->set_len2, &ctx->set_width2,

@@ -66,9 +66,10 @@ struct tim_ctx {
     // per option its inclusive cumulative threshold (u32) and its in-edges at opt_off[o]
     // .. opt_off[o+1] (u64) as in-CSR positions opt_pos (u32)
     DevBuf node_opt, opt_cum, opt_off, opt_pos, opt_node;
-    DevBuf node_thr;  // IC: uint64[n], low word = threshold shared by all in-edges of v,
-                      // bit 32 set when they do share one (empty in-lists included),
-                      // bits 33..63 = 1 + index of the node's qtab entry (skip rule)
+    DevBuf node;  // uint4[n]: all that a visit of node v reads about its in-list, one 16-byte
+                  // load: {begin, end, t, bit 0: all in-edges share threshold (IC; empty
+                  // in-lists included) or weight (LT) t | (1 + index of v's qtab entry) << 1,
+                  // the latter only under IC's skip rule}
 
     // RR-set store
     uint64_t n_sets = 0;
@@ -377,6 +378,15 @@ static inline PhiloxKeys tim_philox_keys(uint64_t seed) {
 }
 
 #ifdef __CUDACC__
+// The shared-threshold word of a node record: low word t, bit 32 "shared", bits 33..63 the
+// qtab index + 1.
+__device__ __forceinline__ unsigned long long node_nt(uint4 r) {
+    return ((unsigned long long)r.w << 32) | r.z;
+}
+
+// The node's in-list is under IC's geometric-skip rule (tim_skip_rule, decided at load).
+__device__ __forceinline__ bool node_skips(uint4 r) { return (r.w >> 1) != 0u; }
+
 __device__ __forceinline__ uint64_t sid_of(const SidMap& s, uint64_t j) {
     uint64_t sid = s.sid0 + j;
     for (uint32_t r = 1; r < s.n; r++)

@@ -145,49 +145,47 @@ __global__ void lt_thr_kernel(const uint64_t* __restrict__ rowptr, const uint32_
     }
 }
 
-// Per-node threshold word: IC: low word = the first in-edge's threshold, bit 32 set when
-// all in-edges share it (empty in-lists included); LT: bit 32 set, low word = t, when
-// all in-edges share t < 2^32 (empty in-lists get 0).
-__global__ void node_thr_kernel(const uint64_t* __restrict__ rowptr, int64_t n, int model,
-                                const uint32_t* __restrict__ thr,
-                                const unsigned long long* __restrict__ lt_t,
-                                const uint8_t* __restrict__ nonuni,
-                                unsigned long long* __restrict__ node_thr) {
+// Node records (tim_ctx::node): begin, end, and the threshold word: IC: the first in-edge's
+// threshold, "shared" when all in-edges have it (empty in-lists included); LT: t, shared,
+// when all in-edges share t < 2^32 (0, not shared, otherwise and for empty in-lists).
+__global__ void node_kernel(const uint64_t* __restrict__ rowptr, int64_t n, int model,
+                            const uint32_t* __restrict__ thr,
+                            const unsigned long long* __restrict__ lt_t,
+                            const uint8_t* __restrict__ nonuni, uint4* __restrict__ node) {
     for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
          v += (int64_t)gridDim.x * blockDim.x) {
-        const uint64_t a = rowptr[v], b = rowptr[v + 1];
+        const uint64_t a = rowptr[v], b = rowptr[v + 1];  // b <= m < 2^32
+        uint32_t t = 0u, shared = 0u;
         if (model == TIM_IC) {
-            const uint32_t t0 = b > a ? thr[a] : 0u;
-            node_thr[v] = (unsigned long long)t0 | (nonuni[v] ? 0ull : (1ull << 32));
-        } else if (model == TIM_TRIG) {
-            node_thr[v] = 0ull;
-        } else {
+            t = b > a ? thr[a] : 0u;
+            shared = nonuni[v] ? 0u : 1u;
+        } else if (model == TIM_LT) {
             const unsigned long long t0 = b > a ? lt_t[a] : 0ull;
-            const bool same = b > a && !nonuni[v] && t0 <= 0xFFFFFFFFull;
-            node_thr[v] = same ? ((1ull << 32) | t0) : 0ull;
+            shared = b > a && !nonuni[v] && t0 <= 0xFFFFFFFFull ? 1u : 0u;
+            if (shared) t = (uint32_t)t0;
         }
+        node[v] = make_uint4((uint32_t)a, (uint32_t)b, t, shared);
     }
 }
 
 // IC: nodes under the geometric-skip rule get a gap table Q_0..Q_31 (Q_0 = (2^32 - t)
-// 2^32, Q_(b+1) = floor(Q_b^2 / 2^64)) and 1 + its index in bits 33..63 of node_thr.
+// 2^32, Q_(b+1) = floor(Q_b^2 / 2^64)) and 1 + its index in their record.
 // With tab == nullptr only counts them.
-__global__ void skip_tables_kernel(const uint64_t* __restrict__ rowptr, int64_t n,
-                                   unsigned long long* __restrict__ node_thr,
+__global__ void skip_tables_kernel(int64_t n, uint4* __restrict__ node,
                                    unsigned long long* __restrict__ tab, unsigned long long cap,
                                    unsigned long long* __restrict__ counter) {
     for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
          v += (int64_t)gridDim.x * blockDim.x) {
-        const unsigned long long nt = node_thr[v];
-        if (!tim_skip_rule(nt, rowptr[v + 1] - rowptr[v])) continue;
+        const uint4 r = node[v];
+        if (!tim_skip_rule(node_nt(r), r.y - r.x)) continue;
         const unsigned long long idx = atomicAdd(counter, 1ull);
         if (!tab || idx >= cap) continue;
-        unsigned long long q = (0x100000000ull - (unsigned long long)(uint32_t)nt) << 32;
+        unsigned long long q = (0x100000000ull - (unsigned long long)r.z) << 32;
         for (int b = 0; b < 32; b++) {
             tab[idx * 32 + b] = q;
             q = __umul64hi(q, q);
         }
-        node_thr[v] = (nt & 0x1FFFFFFFFull) | ((idx + 1ull) << 33);
+        node[v].w = (r.w & 1u) | ((uint32_t)(idx + 1ull) << 1);
     }
 }
 
@@ -394,11 +392,10 @@ int tim_graph_build(tim_ctx* ctx, int64_t n, int64_t m, const int64_t* d_rowptr,
                 (uint8_t*)nonuni.p, &ds->err);
             ctx->launches++;
         }
-        if ((rc = tim_ensure(ctx, ctx->node_thr, (size_t)(n + 1) * 8))) break;
-        node_thr_kernel<<<G, T, 0, ctx->stream>>>(
+        if ((rc = tim_ensure(ctx, ctx->node, (size_t)n * sizeof(uint4)))) break;
+        node_kernel<<<G, T, 0, ctx->stream>>>(
             (const uint64_t*)ctx->rowptr.p, n, model, (const uint32_t*)ctx->thr.p,
-            (const unsigned long long*)lt_t.p, (const uint8_t*)nonuni.p,
-            (unsigned long long*)ctx->node_thr.p);
+            (const unsigned long long*)lt_t.p, (const uint8_t*)nonuni.p, (uint4*)ctx->node.p);
         ctx->launches++;
         if (model == TIM_IC) {
             // count the skip-rule nodes, then give each its gap table
@@ -406,9 +403,7 @@ int tim_graph_build(tim_ctx* ctx, int64_t n, int64_t m, const int64_t* d_rowptr,
             auto* ctr = (unsigned long long*)lt_e.p;
             if ((rc = tim_cuda_check(ctx, cudaMemsetAsync(ctr, 0, 16, ctx->stream), "memset")))
                 break;
-            skip_tables_kernel<<<G, T, 0, ctx->stream>>>((const uint64_t*)ctx->rowptr.p, n,
-                                                          (unsigned long long*)ctx->node_thr.p,
-                                                          nullptr, 0, ctr);
+            skip_tables_kernel<<<G, T, 0, ctx->stream>>>(n, (uint4*)ctx->node.p, nullptr, 0, ctr);
             ctx->launches++;
             unsigned long long nskip = 0;
             if ((rc = tim_cuda_check(ctx, cudaMemcpyAsync(&nskip, ctr, 8, cudaMemcpyDeviceToHost,
@@ -417,8 +412,7 @@ int tim_graph_build(tim_ctx* ctx, int64_t n, int64_t m, const int64_t* d_rowptr,
             if ((rc = tim_sync(ctx))) break;
             if ((rc = tim_ensure(ctx, ctx->qtab, (size_t)(nskip + 1) * 32 * 8))) break;
             skip_tables_kernel<<<G, T, 0, ctx->stream>>>(
-                (const uint64_t*)ctx->rowptr.p, n, (unsigned long long*)ctx->node_thr.p,
-                (unsigned long long*)ctx->qtab.p, nskip, ctr + 1);
+                n, (uint4*)ctx->node.p, (unsigned long long*)ctx->qtab.p, nskip, ctr + 1);
             ctx->launches++;
         }
         if ((rc = tim_cuda_check(ctx, cudaGetLastError(), "graph kernels"))) break;

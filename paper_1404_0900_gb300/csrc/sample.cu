@@ -67,10 +67,9 @@ using Tier1L = Cap<512, 10>;
 using Tier2 = Cap<8192, 14>;
 
 struct SampleArgs {
-    const uint64_t* rowptr;
+    const uint4* node;  // node records
     const uint32_t* src;
     const uint32_t* thr;
-    const unsigned long long* node_thr;  // IC: per-node shared threshold (bit 32: shared)
     const unsigned long long* qtab;      // IC: gap tables of skip-rule nodes
     uint64_t n, m;
     PhiloxKeys K;
@@ -306,11 +305,12 @@ __device__ __forceinline__ int team_rr(const A& a, const PhiloxKeys& K, uint64_t
             unsigned long long nt = 0;
             if (lane < nb) {
                 const uint32_t v = queue[head + lane];
-                beg = __ldg(a.rowptr + v);
-                end = __ldg(a.rowptr + v + 1);
-                nt = __ldg(a.node_thr + v);
+                const uint4 r = __ldg(a.node + v);
+                beg = r.x;
+                end = r.y;
+                nt = node_nt(r);
             }
-            const bool skip_list = lane < nb && tim_skip_rule(nt, end - beg);
+            const bool skip_list = (nt >> 33) != 0ull;  // under the skip rule
             // the frontier's nodes are distinct, so these sums stay below m < 2^32
             const unsigned long long dw = __reduce_add_sync(0xffffffffu, (unsigned)(end - beg));
             // the budget counts in-edges that take a coin; a skipped list counts as at
@@ -352,7 +352,7 @@ __device__ __forceinline__ int team_rr(const A& a, const PhiloxKeys& K, uint64_t
                 const bool shared = (bt >> 32) != 0;
                 const uint32_t t = (uint32_t)bt;
                 if (shared && t == 0u) continue;
-                if (tim_skip_rule(bt, be - bb)) {
+                if (bt >> 33) {
                     // geometric skipping: one step per live in-edge, by one warp of the team
                     if (hubi++ % T == wt) {
                         int f = 0;
@@ -479,8 +479,9 @@ __device__ __forceinline__ int team_rr(const A& a, const PhiloxKeys& K, uint64_t
             uint64_t beg = 0, end = 0, ob = 0, oe = 0;
             if (lane < nb) {
                 const uint32_t v = queue[head + lane];
-                beg = __ldg(a.rowptr + v);
-                end = __ldg(a.rowptr + v + 1);
+                const uint4 r = __ldg(a.node + v);
+                beg = r.x;
+                end = r.y;
                 const uint64_t o0 = __ldg(a.node_opt + v), o1 = __ldg(a.node_opt + v + 1);
                 if (o1 > o0) {
                     const uint32_t x = philox4x32_10(s0, s1, v, TIM_TAG_LT, K).x;
@@ -534,12 +535,13 @@ __device__ __forceinline__ int team_rr(const A& a, const PhiloxKeys& K, uint64_t
         uint32_t v = root;
         for (int guard = 0; guard < C::Q + 1; guard++) {
             if (__shfl_sync(0xffffffffu, vctl[1], 0)) break;
-            const uint64_t beg = __ldg(a.rowptr + v), end = __ldg(a.rowptr + v + 1);
+            const uint4 rec = __ldg(a.node + v);
+            const uint64_t beg = rec.x, end = rec.y;
             width += end - beg;
             if (beg == end) break;
             const uint32_t x =
                 philox4x32_10((uint32_t)sid, (uint32_t)(sid >> 32), v, TIM_TAG_LT, K).x;
-            const unsigned long long nt = __ldg(a.node_thr + v);
+            const unsigned long long nt = node_nt(rec);
             const uint64_t j = (nt >> 32) ? lt_uniform_pick(nt, beg, end, x)
                                           : warp_lt_search(a.thr, beg, end, x, lane);
             if (j >= end) break;
@@ -893,8 +895,9 @@ __global__ void __launch_bounds__(LT_THREADS) rr_lt_lane_kernel(SampleArgs a) {
             if (status) {
                 fin = true;
             } else {
-                const uint64_t beg = __ldg(a.rowptr + v), end = __ldg(a.rowptr + v + 1);
-                const unsigned long long nt = __ldg(a.node_thr + v);
+                const uint4 rec = __ldg(a.node + v);
+                const uint64_t beg = rec.x, end = rec.y;
+                const unsigned long long nt = node_nt(rec);
                 width += end - beg;
                 uint64_t jj = end;
                 if (beg < end) {
@@ -1057,11 +1060,12 @@ __global__ void __launch_bounds__(BIG_THREADS) rr_lt_chain_kernel(SampleArgs a) 
             int tail = 1;
             int status = s_status;
             for (uint64_t guard = 0; guard <= a.n && !status; guard++) {
-                uint64_t beg = __ldg(a.rowptr + v), end = __ldg(a.rowptr + v + 1);
+                const uint4 rec = __ldg(a.node + v);
+                const uint64_t beg = rec.x, end = rec.y;
                 width += end - beg;
                 if (beg == end) break;
                 uint32_t x = draw(a, sid, v, TIM_TAG_LT).x;
-                const unsigned long long nt = __ldg(a.node_thr + v);
+                const unsigned long long nt = node_nt(rec);
                 uint64_t jj = (nt >> 32) ? lt_uniform_pick(nt, beg, end, x)
                                          : warp_lt_search(a.thr, beg, end, x, lane);
                 if (jj >= end) break;
@@ -1186,8 +1190,9 @@ __global__ void __launch_bounds__(BIG_THREADS) rr_trig_big_kernel(SampleArgs a) 
                 uint64_t beg = 0, end = 0, ob = 0, oe = 0;
                 if (lane < nb) {
                     const uint32_t v = queue[h0 + lane];
-                    beg = __ldg(a.rowptr + v);
-                    end = __ldg(a.rowptr + v + 1);
+                    const uint4 r = __ldg(a.node + v);
+                    beg = r.x;
+                    end = r.y;
                     const uint64_t o0 = __ldg(a.node_opt + v), o1 = __ldg(a.node_opt + v + 1);
                     if (o1 > o0) {
                         const uint32_t x = draw(a, sid, v, TIM_TAG_LT).x;
@@ -1356,10 +1361,9 @@ int launch_tier2(tim_ctx* ctx, const SampleArgs& a, unsigned grid, int T) {
 
 // One query of a multi-query launch (device memory).
 struct QueryDesc {
-    const uint64_t* rowptr;
+    const uint4* node;
     const uint32_t* src;
     const uint32_t* thr;
-    const unsigned long long* node_thr;
     const unsigned long long* qtab;
     uint64_t n, m;
     uint64_t sid0, count;
@@ -1395,10 +1399,9 @@ struct MultiArgs {
 
 // What team_rr reads of one query: its graph and flags, plus the launch's keys.
 struct QArgs {
-    const uint64_t* rowptr;
+    const uint4* node;
     const uint32_t* src;
     const uint32_t* thr;
-    const unsigned long long* node_thr;
     const unsigned long long* qtab;
     uint64_t n, m;
     int flags, k;
@@ -1512,8 +1515,7 @@ __global__ void __launch_bounds__(WARPS * 32, 3) rr_multi_kernel(MultiArgs ma) {
                 cur_q = qi;
             }
             const QueryDesc& d = ma.q[qi];
-            const QArgs qa{d.rowptr, d.src, d.thr, d.node_thr, d.qtab,
-                           d.n,      d.m,   d.flags, d.k,     d.seed_mark};
+            const QArgs qa{d.node, d.src, d.thr, d.qtab, d.n, d.m, d.flags, d.k, d.seed_mark};
             const int model = d.model;
             const unsigned long long budget =
                 model != TIM_IC ? ~0ull : TIER == 1 ? d.width_budget : d.width_budget2;
@@ -1658,10 +1660,9 @@ rr_lt_lane_multi_kernel(MultiArgs ma, const unsigned long long* lt_prefix,
     bool has = false, exhausted = false;
     int qi = -1, flags = 0, kk = 0, len = 0, status = 0;
     uint64_t j = 0, sid = 0, n = 0, m = 0;
-    const uint64_t* rowptr = nullptr;
+    const uint4* node = nullptr;
     const uint32_t* src = nullptr;
     const uint32_t* thr = nullptr;
-    const unsigned long long* node_thr = nullptr;
     const uint32_t* seed_mark = nullptr;
     uint32_t v = 0;
     unsigned long long width = 0;
@@ -1701,10 +1702,9 @@ rr_lt_lane_multi_kernel(MultiArgs ma, const unsigned long long* lt_prefix,
                         acc = QAcc{0, 0, 0, 0, 0, 0, 0};
                         cur_q = lo;
                         const QueryDesc& d = ma.q[lo];
-                        rowptr = d.rowptr;
+                        node = d.node;
                         src = d.src;
                         thr = d.thr;
-                        node_thr = d.node_thr;
                         seed_mark = d.seed_mark;
                         n = d.n;
                         m = d.m;
@@ -1733,8 +1733,9 @@ rr_lt_lane_multi_kernel(MultiArgs ma, const unsigned long long* lt_prefix,
             if (status) {
                 fin = true;
             } else {
-                const uint64_t beg = __ldg(rowptr + v), end = __ldg(rowptr + v + 1);
-                const unsigned long long nt = __ldg(node_thr + v);
+                const uint4 rec = __ldg(node + v);
+                const uint64_t beg = rec.x, end = rec.y;
+                const unsigned long long nt = node_nt(rec);
                 width += end - beg;
                 uint64_t jj = end;
                 if (beg < end) {
@@ -1936,10 +1937,9 @@ int tim_sample(tim_ctx* ctx, const SampleRequest& req, SampleResult* res) {
         }
     }
     SampleArgs a;
-    a.rowptr = (const uint64_t*)ctx->rowptr.p;
+    a.node = (const uint4*)ctx->node.p;
     a.src = (const uint32_t*)ctx->src.p;
     a.thr = (const uint32_t*)ctx->thr.p;
-    a.node_thr = (const unsigned long long*)ctx->node_thr.p;
     a.qtab = (const unsigned long long*)ctx->qtab.p;
     a.n = (uint64_t)ctx->n;
     a.m = (uint64_t)ctx->m;
@@ -2247,7 +2247,7 @@ int run_tier3(tim_ctx* ctx, cudaStream_t stream, const SampleRequest& req, DevSc
         rc = ensure_lt_slots(ctx, &slots, &words);
         if (rc == TIM_OK) {
             SampleArgs a{};
-            a.rowptr = (const uint64_t*)ctx->rowptr.p;
+            a.node = (const uint4*)ctx->node.p;
             a.src = (const uint32_t*)ctx->src.p;
             a.thr = (const uint32_t*)ctx->thr.p;
             a.n = (uint64_t)ctx->n;
@@ -2405,10 +2405,9 @@ int tim_sample_multi(tim_ctx* owner, MultiQuery* qs, int nq, uint64_t seed) {
             tim_ctx* c = qs[i].ctx;
             const SampleRequest& r = qs[i].req;
             QueryDesc& d = h_desc[i];
-            d.rowptr = (const uint64_t*)c->rowptr.p;
+            d.node = (const uint4*)c->node.p;
             d.src = (const uint32_t*)c->src.p;
             d.thr = (const uint32_t*)c->thr.p;
-            d.node_thr = (const unsigned long long*)c->node_thr.p;
             d.qtab = (const unsigned long long*)c->qtab.p;
             d.n = (uint64_t)c->n;
             d.m = (uint64_t)c->m;

@@ -49,10 +49,9 @@ struct BulkScalars {
 };
 
 struct BulkArgs {
-    const uint64_t* rowptr;
+    const uint4* node;  // node records
     const uint32_t* src;
     const uint32_t* thr;
-    const unsigned long long* node_thr;  // per-node shared threshold (bit 32: shared)
     const unsigned long long* qtab;      // gap tables of skip-rule nodes
     uint64_t n, m;
     PhiloxKeys K;
@@ -171,7 +170,8 @@ __global__ void bulk_init_kernel(BulkArgs a) {
         }
         const uint32_t root = rr_root(sid, a.n, a.K);
         atomicOr(&a.bitmap[(uint64_t)s * a.words + (root >> 5)], 1u << (root & 31));
-        const uint64_t beg = a.rowptr[root], end = a.rowptr[root + 1];
+        const uint4 rec = a.node[root];
+        const uint64_t beg = rec.x, end = rec.y;
         a.slot_width[s] = end - beg;
         a.slot_cnt[s] = 1;
         const bool cov = cover && marked(a.seed_mark, root);
@@ -183,7 +183,7 @@ __global__ void bulk_init_kernel(BulkArgs a) {
             atomicOr(&a.bs->err, 2);
         if (end > beg && !cov) {
             unsigned long long pf = atomicAdd(&a.bs->f_count, 1ull);
-            const bool sk = tim_skip_rule(a.node_thr[root], end - beg);
+            const bool sk = node_skips(rec);
             if (pf < a.fcap)
                 a.F[pf] = make_uint4((uint32_t)beg, (uint32_t)end, s | (sk ? 0x80000000u : 0u),
                                      root);
@@ -216,12 +216,14 @@ __global__ void bulk_hand_kernel(BulkArgs a, uint32_t chunks_per_slot) {
         const bool h = i < t0;
         const uint32_t u = h ? hs[4 + i] : 0u;
         uint64_t beg = 0, end = 0;
-        bool cov = false;
+        bool cov = false, sk = false;
         if (h) {
             atomicOr(&a.bitmap[(uint64_t)s * a.words + (u >> 5)], 1u << (u & 31));
             if (i >= h0) {  // not yet expanded: its in-degree is not in the width yet
-                beg = a.rowptr[u];
-                end = a.rowptr[u + 1];
+                const uint4 rec = a.node[u];
+                beg = rec.x;
+                end = rec.y;
+                sk = node_skips(rec);
             }
             cov = cover && marked(a.seed_mark, u);
         }
@@ -231,8 +233,7 @@ __global__ void bulk_hand_kernel(BulkArgs a, uint32_t chunks_per_slot) {
         if (__any_sync(0xffffffffu, cov) && lane == 0) a.slot_flag[s] = 1u;
         const bool push = h && i >= h0 && end > beg;
         const uint4 item = make_uint4((uint32_t)beg, (uint32_t)end,
-                                      s | (push && tim_skip_rule(a.node_thr[u], end - beg)
-                                               ? 0x80000000u : 0u), u);
+                                      s | (sk ? 0x80000000u : 0u), u);
         warp_append_f(push, item, &a.bs->f_count, a.F, a.fcap, &a.bs->err, lane);
     }
 }
@@ -406,13 +407,11 @@ __device__ __forceinline__ void expand_level(const BulkArgs& a, uint64_t lo, uin
             for (int q = 0; q < 4; q++) {
                 mi[q] = make_uint2(sv[q], u[q]);
                 if ((fr >> q) & 1u) {
-                    const uint64_t ub = __ldg(a.rowptr + u[q]), ue = __ldg(a.rowptr + u[q] + 1);
-                    const unsigned long long nt = __ldg(a.node_thr + u[q]);
-                    d[q] = ue - ub;
+                    const uint4 rec = __ldg(a.node + u[q]);
+                    d[q] = rec.y - rec.x;
                     if (d[q]) push |= 1u << q;
-                    fi[q] = make_uint4((uint32_t)ub, (uint32_t)ue,
-                                       sv[q] | (tim_skip_rule(nt, ue - ub) ? 0x80000000u : 0u),
-                                       u[q]);
+                    fi[q] = make_uint4(rec.x, rec.y,
+                                       sv[q] | (node_skips(rec) ? 0x80000000u : 0u), u[q]);
                     if (cover && marked(a.seed_mark, u[q])) a.slot_flag[sv[q]] = 1u;
                 }
             }
@@ -598,7 +597,7 @@ __device__ __forceinline__ void skip_level(const BulkArgs& a, uint64_t lo, uint6
         const uint4 it = __ldcg(&a.F[lo + i]);
         const uint32_t s = it.z & 0x7FFFFFFFu, v = it.w;
         const uint64_t beg = it.x, end = it.y;
-        const unsigned long long nt = __ldg(a.node_thr + v);
+        const unsigned long long nt = node_nt(__ldg(a.node + v));
         if (cover && *(volatile uint32_t*)&a.slot_flag[s]) continue;
         const uint64_t sid = __ldg(a.slot_sid + s);
         skip_live_warp((uint32_t)sid, (uint32_t)(sid >> 32), a.K, (uint32_t)beg,
@@ -615,9 +614,10 @@ __device__ __forceinline__ void skip_level(const BulkArgs& a, uint64_t lo, uint6
                                    atomicOr(&a.bitmap[(uint64_t)s * a.words + (u >> 5)], b);
                                fresh = !(old & b);
                                if (fresh) {
-                                   ub = __ldg(a.rowptr + u);
-                                   ue = __ldg(a.rowptr + u + 1);
-                                   unt = __ldg(a.node_thr + u);
+                                   const uint4 rec = __ldg(a.node + u);
+                                   ub = rec.x;
+                                   ue = rec.y;
+                                   unt = node_nt(rec);
                                    atomicAdd(&a.slot_width[s], ue - ub);
                                    atomicAdd(&a.slot_cnt[s], 1u);
                                    if (cover && marked(a.seed_mark, u)) a.slot_flag[s] = 1u;
@@ -628,7 +628,7 @@ __device__ __forceinline__ void skip_level(const BulkArgs& a, uint64_t lo, uint6
                            const bool push = fresh && ue > ub && !(cover && a.slot_flag[s]);
                            const uint4 item = make_uint4(
                                (uint32_t)ub, (uint32_t)ue,
-                               s | (tim_skip_rule(unt, ue - ub) ? 0x80000000u : 0u), u);
+                               s | ((unt >> 33) ? 0x80000000u : 0u), u);
                            warp_append_f(push, item, &a.bs->f_count, a.F, a.fcap, &a.bs->err,
                                          lane);
                            return false;
@@ -906,10 +906,9 @@ int tim_bulk_ic(tim_ctx* ctx, const SampleRequest& req, const uint32_t* list, ui
     }
 
     BulkArgs a;
-    a.rowptr = (const uint64_t*)ctx->rowptr.p;
+    a.node = (const uint4*)ctx->node.p;
     a.src = (const uint32_t*)ctx->src.p;
     a.thr = (const uint32_t*)ctx->thr.p;
-    a.node_thr = (const unsigned long long*)ctx->node_thr.p;
     a.qtab = (const unsigned long long*)ctx->qtab.p;
     a.n = n;
     a.m = (uint64_t)ctx->m;

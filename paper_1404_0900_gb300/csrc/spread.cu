@@ -78,9 +78,8 @@ __global__ void out_scatter_kernel(const uint64_t* __restrict__ rowptr,
 }
 
 struct McArgs {
-    const uint64_t* rowptr;
+    const uint4* node;  // node records
     const uint32_t* thr;
-    const unsigned long long* node_thr;
     const uint2* out_row;
     const uint2* out_rec;
     const uint32_t* out_pos;
@@ -108,9 +107,10 @@ struct McArgs {
 // The in-edge node v keeps in the world of sid (LT), or the end of its in-list for none.
 __device__ __forceinline__ uint64_t lt_pick(const McArgs& a, uint32_t s0, uint32_t s1, uint32_t v,
                                             uint64_t* end_out) {
-    const uint64_t beg = __ldg(a.rowptr + v), end = __ldg(a.rowptr + v + 1);
+    const uint4 rec = __ldg(a.node + v);
+    const uint64_t beg = rec.x, end = rec.y;
     const uint32_t x = philox4x32_10(s0, s1, v, TIM_TAG_LT, a.K).x;
-    const unsigned long long nt = __ldg(a.node_thr + v);
+    const unsigned long long nt = node_nt(rec);
     *end_out = end;
     return (nt >> 32) ? lt_uniform_pick(nt, beg, end, x) : lane_lt_search(a.thr, beg, end, x);
 }
@@ -614,9 +614,8 @@ extern "C" int tim_spread_mc(tim_ctx* ctx, const int32_t* seeds, int k, uint64_t
                                       cudaMemcpyHostToDevice, ctx->stream));
     CUDA_TRY(ctx, cudaMemsetAsync(ctx->mc_scal.p, 0, 2 * sizeof(unsigned long long), ctx->stream));
     McArgs a;
-    a.rowptr = (const uint64_t*)ctx->rowptr.p;
+    a.node = (const uint4*)ctx->node.p;
     a.thr = (const uint32_t*)ctx->thr.p;
-    a.node_thr = (const unsigned long long*)ctx->node_thr.p;
     a.out_row = (const uint2*)ctx->out_row.p;
     a.out_rec = (const uint2*)ctx->out_rec.p;
     a.out_pos = (const uint32_t*)ctx->out_pos.p;
