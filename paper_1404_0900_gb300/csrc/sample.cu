@@ -215,31 +215,18 @@ __device__ __forceinline__ uint32_t live_mask(uint4 x, uint4 t) {
            ((x.w < t.w) | (t.w == 0xFFFFFFFFu) ? 8u : 0u);
 }
 
-// Follow the live in-edges of group g given their mask: insert each source. Returns
-// bit 0 if the set overflowed, bit 1 if it met the seed set.
-template <class C, class A>
-__device__ __forceinline__ int follow_live(const A& a, uint32_t g, uint32_t mask,
-                                        uint32_t* hash, uint32_t* queue, uint16_t* slot,
-                                        int* ctl) {
-    int f = 0;
-    while (mask) {
-        const int c = __ffs(mask) - 1;
-        mask &= mask - 1;
-        const uint32_t u = __ldg(a.src + ((g << 2) + c));
-        const int r = set_insert<C>(hash, queue, slot, ctl, u);
-        if (r == INS_FULL) {
-            f |= 1;
-        } else if (r == INS_NEW && (a.flags & SAMPLE_COVER) && marked(a.seed_mark, u)) {
-            atomicOr(&ctl[1], ST_COVERED);
-            f |= 2;
-        }
-    }
-    return f;
-}
+// Shared memory of one warp of the IC passes: the in-lists of a frontier batch that the warp
+// flattens over its lanes ({begin, end, first group | own thresholds << 31, threshold}), and
+// the live in-CSR positions it has found and not inserted yet (fewer than 32, plus one step's
+// 32 x 4).
+struct alignas(16) WarpScratch {
+    uint4 info[32];
+    uint32_t stage[160];
+};
 
-// In-lists with at least this many 4-edge groups are expanded one at a time by the
-// whole team (no ownership search, two groups in flight per lane).
-constexpr uint32_t BIG_GROUPS = 32;
+// In-lists with at least this many 4-edge groups (512 in-edges, the skip rule's length) that
+// take their own coins are streamed one at a time, two groups in flight per lane.
+constexpr uint32_t BIG_GROUPS = TIM_SKIP_MIN_INDEG / 4;
 
 // Where an IC expansion stopped: the queue position of the frontier batch to process
 // next and the width of the members before it.
@@ -251,8 +238,20 @@ struct Resume {
 // Expand one RR set with a team of T warps (wt = warp index in the team, team = team
 // index in the block). IC only: with `in` the queue, hash and ctl already hold a set
 // that an earlier pass stopped (queue[0 .. ctl[0])), and the expansion goes on from
-// in->head with width in->width; with `out`, an expansion that stops records where. Returns the status bits; *width_out = w(R) (Eq. 1); *live_out
-// counts live in-edges followed (per lane).
+// in->head with width in->width; with `out`, an expansion that stops records where; wsp is
+// the warp's scratch and tot the team's (T > 1). Returns the status bits; *width_out = w(R)
+// (Eq. 1); *live_out counts live in-edges followed (per lane).
+//
+// An IC batch holds up to 32 T frontier nodes, dealt to the warps of the team. A warp lays
+// the groups of its nodes' in-lists out over its lanes: the lanes whose list starts within
+// the next 32 groups set a bit each (one OR-reduction), popcounts give every lane its list,
+// one 16-byte shared load its bounds. Live positions are staged in shared memory and
+// inserted 32 at a time, so that the loads of their sources and the hash probes run with
+// full lanes and overlap, instead of one by one as each group or gap finds them. Against a
+// shuffle search per group, five shuffles for the list's bounds, insertion by the finding
+// lane and one batch of 32 nodes per team: R-MAT 20, weighted cascade, pass 1 19.6 -> 16.9 ms
+// and pass 2 17.5 -> 12.6 ms per TIM+ run, Algorithm 2 3.3 -> 1.6 ms. Both passes are now
+// bound by issue (67 to 73 % active).
 template <int MODEL, class C, int T, class A>
 __device__ __forceinline__ int team_rr(const A& a, const PhiloxKeys& K, uint64_t sid, uint32_t* hash,
                                        uint32_t* queue, uint16_t* slot, int* ctl,
@@ -261,6 +260,7 @@ __device__ __forceinline__ int team_rr(const A& a, const PhiloxKeys& K, uint64_t
                                        unsigned long long* width_out,
                                        unsigned long long* live_out,
                                        unsigned long long* exam_out,
+                                       WarpScratch* wsp, uint32_t* tot,
                                        const Resume* in = nullptr, Resume* out = nullptr) {
     const int lane = threadIdx.x & 31;
     volatile int* vctl = ctl;
@@ -274,14 +274,18 @@ __device__ __forceinline__ int team_rr(const A& a, const PhiloxKeys& K, uint64_t
         ctl[0] = 1;
         ctl[1] = (cover && marked(a.seed_mark, root)) ? ST_COVERED : 0;
     }
+    if (MODEL == TIM_IC && T > 1 && wt == 0 && lane < 4) tot[lane] = 0u;
     team_sync<T>(team);
-    unsigned long long width = in ? in->width : 0, live = 0, work = 0, longs = 0, exam = 0;
+    // a set's members are distinct nodes, so every sum of in-degrees stays below m < 2^32
+    uint32_t width = in ? (uint32_t)in->width : 0u, live = 0, work = 0, longs = 0, exam = 0;
     if constexpr (MODEL == TIM_IC) {
         const uint32_t s0 = (uint32_t)sid, s1 = (uint32_t)(sid >> 32);
         const uint4* thr4 = reinterpret_cast<const uint4*>(a.thr);
         int head = in ? in->head : 0;
         int bh = head;                // the batch being processed and the width before it
-        unsigned long long bw = width;
+        uint32_t bw = width;
+        const uint32_t cap1 = (uint32_t)min(budget, 0xFFFFFFFFull);
+        const uint32_t cap2 = (uint32_t)min(long_budget, 0xFFFFFFFFull);
         for (int guard = 0; guard < C::Q + 1; guard++) {
             // a consistent snapshot of (tail, status) for the whole team
             int tail, stat;
@@ -296,32 +300,45 @@ __device__ __forceinline__ int team_rr(const A& a, const PhiloxKeys& K, uint64_t
             if (stat || head >= tail) break;
             bh = head;
             bw = width;
-            const int nb = min(32, tail - head);
-            uint64_t beg = 0, end = 0;
+            const int nb = min(32 * T, tail - head);
+            uint32_t beg = 0, end = 0, t = 0, word = 0;
             // a node's in-edges often share one threshold (weighted cascade: p = 1/indeg);
             // then no threshold is loaded, t = 0 needs no coins, t = 2^32-1 (p >= 1)
             // makes every in-edge live without a draw, and a long list is sampled by
             // geometric skipping
-            unsigned long long nt = 0;
-            if (lane < nb) {
-                const uint32_t v = queue[head + lane];
-                const uint4 r = __ldg(a.node + v);
+            if (wt + T * lane < nb) {
+                const uint4 r = __ldg(a.node + queue[head + wt + T * lane]);
                 beg = r.x;
                 end = r.y;
-                nt = node_nt(r);
+                t = r.z;
+                word = r.w;
             }
-            const bool skip_list = (nt >> 33) != 0ull;  // under the skip rule
-            // the frontier's nodes are distinct, so these sums stay below m < 2^32
-            const unsigned long long dw = __reduce_add_sync(0xffffffffu, (unsigned)(end - beg));
-            // the budget counts in-edges that take a coin; a skipped list counts as at
-            // most 64
-            const unsigned long long dx = __reduce_add_sync(
-                0xffffffffu, (unsigned)(skip_list ? min(end - beg, (uint64_t)64) : end - beg));
-            // in-edges of long lists that take a coin each, streamed by this team alone
-            const unsigned long long dl = __reduce_add_sync(
-                0xffffffffu,
-                (unsigned)(!skip_list && end - beg >= TIM_SKIP_MIN_INDEG ? end - beg : 0ull));
-            if (work + dx > budget || longs + dl > long_budget) {
+            const bool shared = word & 1u, skip_list = (word >> 1) != 0u;
+            const uint32_t deg = end - beg;
+            const uint32_t ng = deg ? ((end - 1) >> 2) - (beg >> 2) + 1 : 0u;
+            const bool big = !skip_list && deg >= TIM_SKIP_MIN_INDEG;
+            const uint32_t skips = __ballot_sync(0xffffffffu, skip_list);
+            uint32_t bigs = __ballot_sync(0xffffffffu, big);
+            // width of the batch; in-edges that take a coin each (a list under the skip rule
+            // counts as 64 against the budget and as the live ones it finds among the
+            // examined); those of them in long lists. The frontier's nodes are distinct, so
+            // these sums stay below m < 2^32
+            const uint32_t dt = __reduce_add_sync(0xffffffffu, skip_list ? 0u : deg);
+            uint32_t dw = dt, dx = dt + 64u * __popc(skips), dl = 0;
+            if (skips) dw += __reduce_add_sync(0xffffffffu, skip_list ? deg : 0u);
+            if (bigs) dl = __reduce_add_sync(0xffffffffu, big ? deg : 0u);
+            if (T > 1) {
+                if (lane == 0) {
+                    if (dw) atomicAdd(&tot[0], dw);
+                    if (dx) atomicAdd(&tot[1], dx);
+                    if (dl) atomicAdd(&tot[2], dl);
+                }
+                team_sync<T>(team);
+                dw = ((volatile uint32_t*)tot)[0] + (in ? (uint32_t)in->width : 0u) - width;
+                dx = ((volatile uint32_t*)tot)[1] - work;
+                dl = ((volatile uint32_t*)tot)[2] - longs;
+            }
+            if (work + dx > cap1 || longs + dl > cap2) {
                 // too heavy for this tier: list the set for the next one
                 if (wt == 0 && lane == 0) ctl[1] |= ST_OVERFLOW;
                 break;
@@ -329,128 +346,133 @@ __device__ __forceinline__ int team_rr(const A& a, const PhiloxKeys& K, uint64_t
             work += dx;
             longs += dl;
             width += dw;
-            // examined in-edges: every in-edge of a list outside the skip rule (the live
-            // ones the rule finds are added as they are found)
-            const unsigned long long dt =
-                __reduce_add_sync(0xffffffffu, (unsigned)(skip_list ? 0ull : end - beg));
-            if (wt == 0 && lane == 0) exam += dt;
-            // 32-bit in-CSR positions (m < 2^32)
-            const uint32_t b32 = (uint32_t)beg, e32 = (uint32_t)end;
-            const uint32_t ng = e32 > b32 ? ((e32 - 1) >> 2) - (b32 >> 2) + 1 : 0u;
-            const bool big = ng >= BIG_GROUPS;
-            int flags = 0;
-            // hubs first: the whole team strides over one in-list at a time, two groups in
-            // flight per lane; only the in-list's first and last group need a range mask
-            uint32_t bigmask = __ballot_sync(0xffffffffu, big);
-            int hubi = 0;  // hubs under the skip rule go to the team's warps in turn
-            while (bigmask && !(flags & 3)) {
-                const int b = __ffs(bigmask) - 1;
-                bigmask &= bigmask - 1;
-                const uint32_t bb = __shfl_sync(0xffffffffu, b32, b);
-                const uint32_t be = __shfl_sync(0xffffffffu, e32, b);
-                const unsigned long long bt = __shfl_sync(0xffffffffu, nt, b);
-                const bool shared = (bt >> 32) != 0;
-                const uint32_t t = (uint32_t)bt;
-                if (shared && t == 0u) continue;
-                if (bt >> 33) {
-                    // geometric skipping: one step per live in-edge, by one warp of the team
-                    if (hubi++ % T == wt) {
-                        int f = 0;
-                        skip_live_warp(s0, s1, K, bb, be - bb, skip_table(a.qtab, bt), lane,
-                                       [&](uint32_t j) {
-                            if (lane == 0) {
-                                live++;
-                                exam++;
-                                const uint32_t u = __ldg(a.src + j);
-                                const int r = set_insert<C>(hash, queue, slot, ctl, u);
-                                if (r == INS_FULL) {
-                                    f |= 1;
-                                } else if (r == INS_NEW && cover && marked(a.seed_mark, u)) {
-                                    atomicOr(&ctl[1], ST_COVERED);
-                                    f |= 2;
-                                }
-                            }
-                            f = __shfl_sync(0xffffffffu, f, 0);
-                            return (f & 3) != 0;
-                        });
-                        flags |= f;
-                    }
-                    continue;
-                }
-                const uint32_t gfirst = bb >> 2, glast = (be - 1) >> 2;
-                for (uint32_t gb = gfirst + (uint32_t)(wt * 32); gb <= glast; gb += 64u * T) {
-                    const uint32_t g0 = gb + lane, g1 = gb + 32u * T + lane;
-                    const bool v0 = g0 <= glast, v1 = g1 <= glast;
-                    uint32_t m0 = 0, m1 = 0;
-                    if (shared) {
-                        if (t == 0xFFFFFFFFu) {
-                            m0 = v0 ? 0xFu : 0u;
-                            m1 = v1 ? 0xFu : 0u;
-                        } else {
-                            if (v0) m0 = live_mask_shared(philox4x32_10(s0, s1, g0, TIM_TAG_IC, K), t);
-                            if (v1) m1 = live_mask_shared(philox4x32_10(s0, s1, g1, TIM_TAG_IC, K), t);
-                        }
-                    } else {
-                        if (v0) {
-                            const uint4 x = philox4x32_10(s0, s1, g0, TIM_TAG_IC, K);
-                            m0 = live_mask(x, __ldg(thr4 + g0));
-                        }
-                        if (v1) {
-                            const uint4 x = philox4x32_10(s0, s1, g1, TIM_TAG_IC, K);
-                            m1 = live_mask(x, __ldg(thr4 + g1));
-                        }
-                    }
-                    if (__any_sync(0xffffffffu, (m0 | m1) != 0u)) {
-                        if (m0 && (g0 == gfirst || g0 == glast)) m0 &= range_mask(g0, bb, be);
-                        if (m1 && (g1 == gfirst || g1 == glast)) m1 &= range_mask(g1, bb, be);
-                        live += __popc(m0) + __popc(m1);
-                        if (m0) flags |= follow_live<C, A>(a, g0, m0, hash, queue, slot, ctl);
-                        if (m1) flags |= follow_live<C, A>(a, g1, m1, hash, queue, slot, ctl);
-                        if (__any_sync(0xffffffffu, flags & 3)) break;
+            if (lane == 0) exam += dt;
+            uint32_t held = 0;  // staged positions
+            // insert the sources of stage[from .. from + cnt); true: the set stops
+            auto take = [&](uint32_t from, uint32_t cnt) {
+                __syncwarp();
+                bool stop = false;
+                if ((uint32_t)lane < cnt) {
+                    const uint32_t u = __ldg(a.src + wsp->stage[from + lane]);
+                    const int r = set_insert<C>(hash, queue, slot, ctl, u);
+                    stop = r == INS_FULL;
+                    if (r == INS_NEW && cover && marked(a.seed_mark, u)) {
+                        atomicOr(&ctl[1], ST_COVERED);
+                        stop = true;
                     }
                 }
-                flags = __reduce_or_sync(0xffffffffu, flags);
+                return __any_sync(0xffffffffu, stop) != 0;
+            };
+            // stage the live positions 4 g + c of each lane's mask; true: the set stops
+            auto append = [&](uint32_t m, uint32_t g) {
+                const uint32_t b0 = __ballot_sync(0xffffffffu, m & 1u);
+                const uint32_t b1 = __ballot_sync(0xffffffffu, m & 2u);
+                const uint32_t b2 = __ballot_sync(0xffffffffu, m & 4u);
+                const uint32_t b3 = __ballot_sync(0xffffffffu, m & 8u);
+                if (!(b0 | b1 | b2 | b3)) return false;
+                const uint32_t below = (1u << lane) - 1u;
+                const uint32_t at = held;
+                if (m & 1u) wsp->stage[held + __popc(b0 & below)] = g << 2;
+                held += __popc(b0);
+                if (m & 2u) wsp->stage[held + __popc(b1 & below)] = (g << 2) + 1;
+                held += __popc(b1);
+                if (m & 4u) wsp->stage[held + __popc(b2 & below)] = (g << 2) + 2;
+                held += __popc(b2);
+                if (m & 8u) wsp->stage[held + __popc(b3 & below)] = (g << 2) + 3;
+                held += __popc(b3);
+                if (lane == 0) live += held - at;
+                while (held >= 32) {
+                    held -= 32;
+                    if (take(held, 32)) return true;
+                }
+                __syncwarp();
+                return false;
+            };
+            bool stop = false;
+            // lists under the skip rule: one step per live in-edge
+            for (uint32_t todo = skips; todo && !stop; todo &= todo - 1) {
+                const int b = __ffs(todo) - 1;
+                const uint32_t bb = __shfl_sync(0xffffffffu, beg, b);
+                const uint32_t be = __shfl_sync(0xffffffffu, end, b);
+                const uint32_t bw2 = __shfl_sync(0xffffffffu, word, b);
+                skip_live_warp(s0, s1, K, bb, be - bb, a.qtab + (uint64_t)((bw2 >> 1) - 1) * 32,
+                               lane, [&](uint32_t j) {
+                    if (lane == 0) {
+                        live++;
+                        exam++;
+                        wsp->stage[held] = j;
+                    }
+                    if (++held < 32) return false;
+                    held = 0;
+                    stop = take(0, 32);
+                    __syncwarp();
+                    return stop;
+                });
             }
-            // the rest, flattened over the lanes: lane -> (owner node, group)
-            const uint32_t ngs = big ? 0u : ng;  // lists under the skip rule are big
+            // long lists with their own coins; only a list's first and last group need a
+            // range mask
+            for (; bigs && !stop; bigs &= bigs - 1) {
+                const int b = __ffs(bigs) - 1;
+                const uint32_t bb = __shfl_sync(0xffffffffu, beg, b);
+                const uint32_t be = __shfl_sync(0xffffffffu, end, b);
+                const uint32_t bt = __shfl_sync(0xffffffffu, t, b);
+                const bool bs = __shfl_sync(0xffffffffu, word, b) & 1u;
+                if (bs && bt == 0u) continue;
+                const uint32_t gfirst = bb >> 2, glast = (be - 1) >> 2;
+                for (uint32_t gb = gfirst; gb <= glast && !stop; gb += 64u) {
+                    uint32_t m[2], g[2] = {gb + lane, gb + 32u + lane};
+#pragma unroll
+                    for (int i = 0; i < 2; i++) {
+                        m[i] = 0;
+                        if (g[i] > glast) continue;
+                        if (bs && bt == 0xFFFFFFFFu) {
+                            m[i] = 0xFu;
+                        } else {
+                            const uint4 th = bs ? make_uint4(bt, bt, bt, bt) : __ldg(thr4 + g[i]);
+                            m[i] = live_mask(philox4x32_10(s0, s1, g[i], TIM_TAG_IC, K), th);
+                        }
+                        if (m[i] && (g[i] == gfirst || g[i] == glast)) m[i] &= range_mask(g[i], bb, be);
+                    }
+                    stop = append(m[0], g[0]) || append(m[1], g[1]);
+                }
+            }
+            // the rest, flattened over the lanes
+            const uint32_t ngs = skip_list || big || (shared && t == 0u) ? 0u : ng;
             uint32_t incl = ngs;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
                 const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
                 if (lane >= o) incl += y;
             }
-            const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
-            const uint32_t excl = incl - ngs;
-            for (uint32_t base = wt * 32; base < total && !(flags & 3); base += 32 * T) {
-                const uint32_t t = base + lane;
-                int own = 0;  // number of lanes whose inclusive count is <= t
-#pragma unroll
-                for (int sft = 16; sft > 0; sft >>= 1) {
-                    const uint32_t ic = __shfl_sync(0xffffffffu, incl, own + sft - 1);
-                    if (ic <= t) own += sft;
-                }
-                const uint32_t o_beg = __shfl_sync(0xffffffffu, b32, own);
-                const uint32_t o_end = __shfl_sync(0xffffffffu, e32, own);
-                const uint32_t o_excl = __shfl_sync(0xffffffffu, excl, own);
-                const unsigned long long o_nt = __shfl_sync(0xffffffffu, nt, own);
+            const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);  // < 32 BIG_GROUPS
+            const uint32_t excl = ngs ? incl - ngs : ~0u;
+            const uint32_t lists = __ballot_sync(0xffffffffu, ngs != 0u);
+            if (ngs)
+                wsp->info[__popc(lists & ((1u << lane) - 1u))] =
+                    make_uint4(beg, end, excl | (shared ? 0u : 0x80000000u), t);
+            __syncwarp();
+            for (uint32_t base = 0; base < total && !stop; base += 32) {
+                // lists that start before these 32 groups, and at which of them others do
+                const uint32_t before = base ? __popc(__ballot_sync(0xffffffffu, excl < base)) : 0u;
+                const uint32_t starts = __reduce_or_sync(
+                    0xffffffffu, excl - base < 32u ? 1u << (excl - base) : 0u);
+                const uint32_t own =
+                    before + __popc(starts & (0xFFFFFFFFu >> (31 - lane))) - 1u;
                 uint32_t m = 0, g = 0;
-                if (t < total) {
-                    g = (o_beg >> 2) + (t - o_excl);
-                    const uint32_t ot = (uint32_t)o_nt;
-                    if (!(o_nt >> 32))
+                if (base + lane < total) {
+                    const uint4 f = wsp->info[own];
+                    g = (f.x >> 2) + (base + lane - (f.z & 0x7FFFFFFFu));
+                    if (f.z >> 31)
                         m = live_mask(philox4x32_10(s0, s1, g, TIM_TAG_IC, K), __ldg(thr4 + g));
-                    else if (ot == 0xFFFFFFFFu)
+                    else if (f.w == 0xFFFFFFFFu)
                         m = 0xFu;
-                    else if (ot != 0u)
-                        m = live_mask_shared(philox4x32_10(s0, s1, g, TIM_TAG_IC, K), ot);
-                    if (m) m &= range_mask(g, o_beg, o_end);
+                    else
+                        m = live_mask_shared(philox4x32_10(s0, s1, g, TIM_TAG_IC, K), f.w);
+                    if (m) m &= range_mask(g, f.x, f.y);
                 }
-                if (__any_sync(0xffffffffu, m != 0u)) {
-                    live += __popc(m);
-                    if (m) flags |= follow_live<C, A>(a, g, m, hash, queue, slot, ctl);
-                    flags = __reduce_or_sync(0xffffffffu, flags);
-                }
+                stop = append(m, g);
             }
+            if (held && !stop) take(0, held);
             team_sync<T>(team);
             head += nb;
         }
@@ -582,13 +604,15 @@ __device__ __forceinline__ void kappa_lanes(unsigned long long w, unsigned cnt, 
 // TIER 1: teams of one warp, storage in shared memory, every set index of [0, count),
 // in-edge budget (IC); listed sets go to list1. TIER 2: teams of T warps, storage in
 // the global arena, the sets of list1, no budget; listed sets go to list2.
-// Tier 1 is bound by integer arithmetic (coins), tier 2 by latency: tier 2 trades
-// registers for resident warps.
+// Four blocks of 64 registers per SM: both IC tiers are bound by issue (tier 2 with six blocks
+// of 40 registers spills and is no faster; tier 1 with five blocks 17.3 ms instead of 16.9).
 template <int MODEL, class C, int TIER, int T>
-__global__ void __launch_bounds__(WARPS * 32, TIER == 1 ? 4 : 6) rr_team_kernel(SampleArgs a) {
+__global__ void __launch_bounds__(WARPS * 32, TIER == 1 || MODEL == TIM_IC ? 4 : 6) rr_team_kernel(SampleArgs a) {
     extern __shared__ uint32_t smem[];
     __shared__ unsigned long long s_claim[WARPS];
     __shared__ int s_ctl[WARPS][4];  // tier 2: a team's tail and status (shared atomics)
+    __shared__ WarpScratch s_scratch[MODEL == TIM_IC ? WARPS : 1];
+    __shared__ uint32_t s_tot[WARPS][4];  // a team's batch sums
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int wt = wid % T, team = wid / T;
     const int tl = wt * 32 + lane;  // thread index inside the team
@@ -673,7 +697,8 @@ __global__ void __launch_bounds__(WARPS * 32, TIER == 1 ? 4 : 6) rr_team_kernel(
             }
             const int st = team_rr<MODEL, C, T, SampleArgs>(
                 a, a.K, sid_of(a.ids, j), hash, queue, slot, ctl, budget, long_budget, wt, team, &width, &live,
-                &exam, resumed ? &rin : nullptr,
+                &exam, &s_scratch[MODEL == TIM_IC ? wid : 0], s_tot[team],
+                resumed ? &rin : nullptr,
                 (HAND && ((TIER == 1 && a.hand) || (TIER == 2 && a.hand2))) ? &rout : nullptr);
             const int tail = min(T == 1 ? __shfl_sync(0xffffffffu, ((volatile int*)ctl)[0], 0)
                                         : ((volatile int*)ctl)[0],
@@ -1435,11 +1460,13 @@ __device__ __forceinline__ void flush_acc(const QueryDesc* qd, int qi, QAcc& acc
 // TIER 1: shared-memory sets of every query (global set index across queries); TIER 2:
 // the listed (query, set) pairs with a global arena and teams of T warps.
 template <class C, int TIER, int T>
-__global__ void __launch_bounds__(WARPS * 32, 3) rr_multi_kernel(MultiArgs ma) {
+__global__ void __launch_bounds__(WARPS * 32, 4) rr_multi_kernel(MultiArgs ma) {
     extern __shared__ uint32_t smem[];
     __shared__ unsigned long long s_claim[WARPS];
     __shared__ unsigned long long s_prefix[MAXQ + 1];
     __shared__ int s_ctl[WARPS][4];  // tier 2: a team's tail and status (shared atomics)
+    __shared__ WarpScratch s_scratch[WARPS];
+    __shared__ uint32_t s_tot[WARPS][4];  // a team's batch sums
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int wt = wid % T, team = wid / T;
     const int tl = wt * 32 + lane;
@@ -1554,12 +1581,13 @@ __global__ void __launch_bounds__(WARPS * 32, 3) rr_multi_kernel(MultiArgs ma) {
             if (model == TIM_IC)
                 st = team_rr<TIM_IC, C, T, QArgs>(qa, ma.K, d.sid0 + j, hash, queue, slot, ctl,
                                                   budget, ~0ull, wt, team, &width, &acc.live,
-                                                  &acc.exam, resumed ? &rin : nullptr,
+                                                  &acc.exam, &s_scratch[wid], s_tot[team],
+                                                  resumed ? &rin : nullptr,
                                                   (TIER == 1 && ma.hand) ? &rout : nullptr);
             else
                 st = team_rr<TIM_LT, C, T, QArgs>(qa, ma.K, d.sid0 + j, hash, queue, slot, ctl,
                                                   budget, ~0ull, wt, team, &width, &acc.live,
-                                                  &acc.exam);
+                                                  &acc.exam, nullptr, nullptr);
             const int tail = min(T == 1 ? __shfl_sync(0xffffffffu, ((volatile int*)ctl)[0], 0)
                                         : ((volatile int*)ctl)[0],
                                  C::Q);
