@@ -61,7 +61,7 @@ struct tim_ctx {
     DevBuf rowptr;  // uint64[n+1]
     DevBuf src;     // uint32[m + 4]
     DevBuf thr;     // uint32[m + 4] IC thresholds or LT inclusive cumulative thresholds
-    DevBuf qtab;      // IC: per skip-rule node, Q_0..Q_31 of its geometric gaps (u64[32])
+    DevBuf qtab;      // IC: per skip-rule node, the table of its geometric gaps (u64[SKIP_TABLE])
     // triggering model: options of node v at node_opt[v] .. node_opt[v+1] (u64[n+1]);
     // per option its inclusive cumulative threshold (u32) and its in-edges at opt_off[o]
     // .. opt_off[o+1] (u64) as in-CSR positions opt_pos (u32)
@@ -428,6 +428,10 @@ __device__ __forceinline__ uint4 philox4x32_10(uint32_t c0, uint32_t c1, uint32_
 // sid hi, beg + (r >> 1), TIM_TAG_SKIP + b); beg = in-CSR position of the list's first
 // in-edge (r <= pos < d keeps beg + (r >> 1) inside the list). G >= R or G >= 2^B ends
 // the list; otherwise position pos + G is live and the next gap starts after it.
+//   skip_digit is monotone in U, so a node's table holds beside Q_b the threshold T_b = the
+// number of U that decide 1 (SKIP_TABLE words per node: Q_0..Q_31, then T_0..T_31): a digit
+// is one comparison instead of a 64 x 64-bit product.
+constexpr int SKIP_TABLE = 64;
 __device__ __forceinline__ bool tim_skip_rule(unsigned long long nt, unsigned long long d) {
     const uint32_t t = (uint32_t)nt;
     if (!(nt >> 32) || t == 0u || d < TIM_SKIP_MIN_INDEG) return false;
@@ -439,15 +443,28 @@ __device__ __forceinline__ bool skip_digit(unsigned long long U, unsigned long l
     return U < Q && __umul64hi(U, Q) < Q - U;
 }
 
-// The gap table of a node under the rule: Q_b for b = 0..31, computed at load.
+// T_b of Q_b: the smallest U that does not decide 1.
+__device__ __forceinline__ unsigned long long skip_threshold(unsigned long long Q) {
+    unsigned long long lo = 0, hi = Q;  // U >= Q never decides 1
+    while (lo < hi) {
+        const unsigned long long mid = lo + ((hi - lo) >> 1);
+        if (skip_digit(mid, Q))
+            lo = mid + 1;
+        else
+            hi = mid;
+    }
+    return lo;
+}
+
+// The gap table of a node under the rule, computed at load.
 __device__ __forceinline__ const unsigned long long* skip_table(const unsigned long long* qtab,
                                                                 unsigned long long nt) {
-    return qtab + ((nt >> 33) - 1ull) * 32ull;
+    return qtab + ((nt >> 33) - 1ull) * (unsigned long long)SKIP_TABLE;
 }
 
 // Live in-edges of a list under the rule, warp-cooperatively: lane b decides digit b
-// of each gap (Q_b from the node's table), one ballot gives G; a lane's draw for gap 2i
-// also serves gap 2i + 1. visit(j) runs on every lane with the same in-CSR position j
+// of each gap (T_b from the node's table) and lane B whether the gap is 2^B or more (Q_B), one
+// ballot gives G; a lane's draw for gap 2i also serves gap 2i + 1. visit(j) runs on every lane with the same in-CSR position j
 // of each live in-edge, in increasing order, and returns true to stop early. All 32
 // lanes must call it with the same arguments.
 template <class Visit>
@@ -455,8 +472,7 @@ __device__ __forceinline__ void skip_live_warp(uint32_t s0, uint32_t s1, const P
                                                uint32_t beg, uint32_t d,
                                                const unsigned long long* qtab_node, int lane,
                                                Visit&& visit) {
-    const int bmax = 32 - __clz((int)d);
-    const unsigned long long Q = lane <= bmax && lane < 32 ? __ldg(qtab_node + lane) : 0ull;
+    const unsigned long long Q = __ldg(qtab_node + lane), Tb = __ldg(qtab_node + 32 + lane);
     uint4 x = make_uint4(0u, 0u, 0u, 0u);
     uint32_t pos = 0;
     for (uint32_t r = 0; pos < d; r++) {
@@ -467,10 +483,11 @@ __device__ __forceinline__ void skip_live_warp(uint32_t s0, uint32_t s1, const P
             x = philox4x32_10(s0, s1, beg + (r >> 1), TIM_TAG_SKIP + (uint32_t)lane, K);
         const unsigned long long U = (r & 1u) ? (((unsigned long long)x.w << 32) | x.z)
                                              : (((unsigned long long)x.y << 32) | x.x);
-        const bool digit = lane < B && skip_digit(U, Q);
-        const bool over = lane == B && U < Q;
-        const uint32_t G = __ballot_sync(0xffffffffu, digit);
-        if (__any_sync(0xffffffffu, over) || G >= rem) break;
+        // d < n <= 2^31 - 1, so B <= 31
+        const uint32_t bits =
+            __ballot_sync(0xffffffffu, U < (lane < B ? Tb : lane == B ? Q : 0ull));
+        const uint32_t G = bits & ((1u << B) - 1u);
+        if ((bits >> B) || G >= rem) break;
         if (visit(beg + pos + G)) break;
         pos += G + 1u;
     }

@@ -169,23 +169,35 @@ __global__ void node_kernel(const uint64_t* __restrict__ rowptr, int64_t n, int 
 }
 
 // IC: nodes under the geometric-skip rule get a gap table Q_0..Q_31 (Q_0 = (2^32 - t)
-// 2^32, Q_(b+1) = floor(Q_b^2 / 2^64)) and 1 + its index in their record.
+// 2^32, Q_(b+1) = floor(Q_b^2 / 2^64)), T_0..T_31 and 1 + its index in their record.
 // With tab == nullptr only counts them.
 __global__ void skip_tables_kernel(int64_t n, uint4* __restrict__ node,
                                    unsigned long long* __restrict__ tab, unsigned long long cap,
                                    unsigned long long* __restrict__ counter) {
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
-         v += (int64_t)gridDim.x * blockDim.x) {
-        const uint4 r = node[v];
-        if (!tim_skip_rule(node_nt(r), r.y - r.x)) continue;
-        const unsigned long long idx = atomicAdd(counter, 1ull);
-        if (!tab || idx >= cap) continue;
-        unsigned long long q = (0x100000000ull - (unsigned long long)r.z) << 32;
-        for (int b = 0; b < 32; b++) {
-            tab[idx * 32 + b] = q;
-            q = __umul64hi(q, q);
+    const int lane = threadIdx.x & 31;
+    for (int64_t v0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31u); v0 < n;
+         v0 += (int64_t)gridDim.x * blockDim.x) {
+        uint4 r = make_uint4(0u, 0u, 0u, 0u);
+        if (v0 + lane < n) r = node[v0 + lane];
+        const bool rule = tim_skip_rule(node_nt(r), r.y - r.x);
+        const uint32_t todo = __ballot_sync(0xffffffffu, rule);
+        if (!todo) continue;
+        unsigned long long first = 0;
+        if (lane == 0) first = atomicAdd(counter, (unsigned long long)__popc(todo));
+        first = __shfl_sync(0xffffffffu, first, 0);
+        if (!tab) continue;
+        // the warp fills each node's table together: lane b squares its way to Q_b
+        for (uint32_t m = todo; m; m &= m - 1) {
+            const int l = __ffs(m) - 1;
+            const unsigned long long idx = first + __popc(todo & ((1u << l) - 1u));
+            if (idx >= cap) break;
+            const uint32_t t = __shfl_sync(0xffffffffu, r.z, l);
+            unsigned long long q = (0x100000000ull - (unsigned long long)t) << 32;
+            for (int b = 0; b < lane; b++) q = __umul64hi(q, q);
+            tab[idx * SKIP_TABLE + lane] = q;
+            tab[idx * SKIP_TABLE + 32 + lane] = skip_threshold(q);
+            if (lane == l) node[v0 + lane].w = (r.w & 1u) | ((uint32_t)(idx + 1ull) << 1);
         }
-        node[v].w = (r.w & 1u) | ((uint32_t)(idx + 1ull) << 1);
     }
 }
 
@@ -410,7 +422,7 @@ int tim_graph_build(tim_ctx* ctx, int64_t n, int64_t m, const int64_t* d_rowptr,
                                                           ctx->stream), "copy")))
                 break;
             if ((rc = tim_sync(ctx))) break;
-            if ((rc = tim_ensure(ctx, ctx->qtab, (size_t)(nskip + 1) * 32 * 8))) break;
+            if ((rc = tim_ensure(ctx, ctx->qtab, (size_t)(nskip + 1) * SKIP_TABLE * 8))) break;
             skip_tables_kernel<<<G, T, 0, ctx->stream>>>(
                 n, (uint4*)ctx->node.p, (unsigned long long*)ctx->qtab.p, nskip, ctr + 1);
             ctx->launches++;

@@ -395,7 +395,7 @@ __device__ __forceinline__ int team_rr(const A& a, const PhiloxKeys& K, uint64_t
                 const uint32_t bb = __shfl_sync(0xffffffffu, beg, b);
                 const uint32_t be = __shfl_sync(0xffffffffu, end, b);
                 const uint32_t bw2 = __shfl_sync(0xffffffffu, word, b);
-                skip_live_warp(s0, s1, K, bb, be - bb, a.qtab + (uint64_t)((bw2 >> 1) - 1) * 32,
+                skip_live_warp(s0, s1, K, bb, be - bb, a.qtab + (uint64_t)((bw2 >> 1) - 1) * SKIP_TABLE,
                                lane, [&](uint32_t j) {
                     if (lane == 0) {
                         live++;
