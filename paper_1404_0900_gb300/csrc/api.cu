@@ -190,7 +190,7 @@ int tim_destroy(tim_ctx* ctx) {
                       &ctx->covered,  &ctx->chosen,     &ctx->best,      &ctx->seed_mark,
                       &ctx->seeds_dev, &ctx->ovf_list,  &ctx->big_bitmap, &ctx->big_queue,
                       &ctx->ovf_list2, &ctx->hand, &ctx->hand2, &ctx->arena,    &ctx->lt_col,    &ctx->greedy_bar,
-                      &ctx->greedy_chunks, &ctx->greedy_nchunk,
+                      &ctx->cand, &ctx->set_rec, &ctx->greedy_chunks, &ctx->greedy_nchunk,
                       &ctx->scratch_a, &ctx->scratch_b, &ctx->scratch_c, &ctx->scratch_d,
                       &ctx->scratch_e, &ctx->scratch_f, &ctx->scal,     &ctx->bulk_bitmap,
                       &ctx->bulk_slot, &ctx->bulk_bsum, &ctx->bulk_bar,
@@ -882,7 +882,6 @@ int tim_refine_kpt(tim_ctx* ctx, int k, double ell, double eps, uint64_t seed, d
         return tim_fail(ctx, TIM_ERR_ARG, "need 1 <= k <= n, eps > 0, l > 0");
     DeviceGuard g(ctx->device);
     // greedy on R' (the store holds the last round of Algorithm 2)
-    TIM_TRY(tim_build_index(ctx));
     TIM_TRY(tim_greedy(ctx, k, nullptr, nullptr));
     TIM_TRY(tim_mark_seeds(ctx, (const int32_t*)ctx->seeds_dev.p, k));
     // eps' and theta'
@@ -917,7 +916,6 @@ int tim_node_select(tim_ctx* ctx, int k, int32_t* seeds, double* covered_fractio
     if (!ctx || !seeds) return TIM_ERR_ARG;
     if (!ctx->have_graph) return tim_fail(ctx, TIM_ERR_STATE, "no graph loaded");
     DeviceGuard g(ctx->device);
-    TIM_TRY(tim_build_index(ctx));
     uint64_t cov = 0;
     TIM_TRY(tim_greedy(ctx, k, seeds, &cov));
     if (covered_fraction) *covered_fraction = ctx->n_sets ? (double)cov / (double)ctx->n_sets : 0.0;
@@ -929,7 +927,7 @@ int tim_coverage_counts(tim_ctx* ctx, int32_t* counts) {
     if (!ctx || !counts) return TIM_ERR_ARG;
     if (!ctx->have_graph) return tim_fail(ctx, TIM_ERR_STATE, "no graph loaded");
     DeviceGuard g(ctx->device);
-    TIM_TRY(tim_build_index(ctx));
+    TIM_TRY(tim_count_members(ctx));
     CUDA_TRY(ctx, cudaMemcpyAsync(counts, ctx->counts.p, (size_t)ctx->n * sizeof(int32_t),
                                   cudaMemcpyDeviceToHost, ctx->stream));
     return tim_sync(ctx);
@@ -994,7 +992,6 @@ static int run_common(tim_ctx* ctx, bool plus, int k, double eps, double ell, ui
     TIM_TRY(tim_sample(ctx, req, &res));
     cudaEventRecord(ctx->ev[3], ctx->stream);
     uint64_t cov = 0;
-    TIM_TRY(tim_build_index(ctx));
     TIM_TRY(tim_greedy(ctx, k, seeds, &cov));
     cudaEventRecord(ctx->ev[4], ctx->stream);
     TIM_TRY(tim_sync(ctx));

@@ -30,7 +30,7 @@ struct DevScalars {
     unsigned int cnt1;             // sets tier 1 listed for tier 2
     unsigned int cnt2;             // sets tier 2 listed for tier 3
     int err;                       // device-side error bits (TIM_DEV_ERR_*)
-    int pad0;
+    unsigned int done;             // greedy over candidates: rounds done
     unsigned long long width[3];   // sum of widths per tier
     unsigned long long live[3];    // live in-edges followed per tier
     unsigned long long memb[3];    // members per tier
@@ -93,6 +93,8 @@ struct tim_ctx {
     DevBuf seed_mark;  // uint32 bitmap[n/32 + 1]
     DevBuf seeds_dev;  // int32[n]
     DevBuf greedy_bar; // grid barrier of the cooperative greedy launch
+    DevBuf set_rec;    // greedy over candidates: a 16-byte record per set
+    DevBuf cand;       // greedy over candidates: their state and table
     DevBuf greedy_chunks;  // cooperative greedy: member chunks of the round's large sets
     DevBuf greedy_nchunk;  // and their count per round
 
@@ -314,7 +316,8 @@ struct MultiQuery {
 int tim_sample_multi(tim_ctx* owner, MultiQuery* qs, int nq, uint64_t seed);
 
 // select.cu
-int tim_build_index(tim_ctx* ctx);
+int tim_count_members(tim_ctx* ctx);  // coverage counts of the store
+int tim_build_index(tim_ctx* ctx);    // counts and the full node -> sets index
 int tim_greedy(tim_ctx* ctx, int k, int32_t* host_seeds, uint64_t* covered);
 int tim_mark_seeds(tim_ctx* ctx, const int32_t* d_seeds, int k);
 // Stepwise greedy on the store: index and reset, then one caller-chosen node at a time.
@@ -575,7 +578,7 @@ __device__ __forceinline__ bool grid_barrier(GridBarrier* bar, int* err, unsigne
         } else {
             unsigned it = 0;
             while (((volatile unsigned*)&bar->gen)[0] == g && it < limit) {
-                __nanosleep(64);
+                if (it > 16) __nanosleep(32);
                 it++;
             }
             if (((volatile unsigned*)&bar->gen)[0] == g) {

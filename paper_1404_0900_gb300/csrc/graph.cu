@@ -11,6 +11,8 @@
 //   LT (Section 6):   thr = inclusive prefix over the in-list of floor(b * 2^32),
 //                     saturated at 2^32 - 1; the triggering in-edge of a node is the
 //                     first whose prefix exceeds the node's draw.
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace {
@@ -168,12 +170,12 @@ __global__ void node_kernel(const uint64_t* __restrict__ rowptr, int64_t n, int 
     }
 }
 
-// IC: nodes under the geometric-skip rule get a gap table Q_0..Q_31 (Q_0 = (2^32 - t)
-// 2^32, Q_(b+1) = floor(Q_b^2 / 2^64)), T_0..T_31 and 1 + its index in their record.
-// With tab == nullptr only counts them.
-__global__ void skip_tables_kernel(int64_t n, uint4* __restrict__ node,
-                                   unsigned long long* __restrict__ tab, unsigned long long cap,
-                                   unsigned long long* __restrict__ counter) {
+// IC: nodes under the geometric-skip rule get an index (in their record and in list), then
+// a gap table Q_0..Q_31 (Q_0 = (2^32 - t) 2^32, Q_(b+1) = floor(Q_b^2 / 2^64)), T_0..T_31,
+// one warp per table (hubs have neighbouring ids in many graphs, so the nodes are listed
+// before their tables are shared out).
+__global__ void skip_list_kernel(int64_t n, uint4* __restrict__ node, uint32_t* __restrict__ list,
+                                 unsigned long long cap, unsigned long long* __restrict__ counter) {
     const int lane = threadIdx.x & 31;
     for (int64_t v0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31u); v0 < n;
          v0 += (int64_t)gridDim.x * blockDim.x) {
@@ -185,19 +187,26 @@ __global__ void skip_tables_kernel(int64_t n, uint4* __restrict__ node,
         unsigned long long first = 0;
         if (lane == 0) first = atomicAdd(counter, (unsigned long long)__popc(todo));
         first = __shfl_sync(0xffffffffu, first, 0);
-        if (!tab) continue;
-        // the warp fills each node's table together: lane b squares its way to Q_b
-        for (uint32_t m = todo; m; m &= m - 1) {
-            const int l = __ffs(m) - 1;
-            const unsigned long long idx = first + __popc(todo & ((1u << l) - 1u));
-            if (idx >= cap) break;
-            const uint32_t t = __shfl_sync(0xffffffffu, r.z, l);
-            unsigned long long q = (0x100000000ull - (unsigned long long)t) << 32;
-            for (int b = 0; b < lane; b++) q = __umul64hi(q, q);
-            tab[idx * SKIP_TABLE + lane] = q;
-            tab[idx * SKIP_TABLE + 32 + lane] = skip_threshold(q);
-            if (lane == l) node[v0 + lane].w = (r.w & 1u) | ((uint32_t)(idx + 1ull) << 1);
+        const unsigned long long idx = first + __popc(todo & ((1u << lane) - 1u));
+        if (rule && idx < cap) {
+            list[idx] = (uint32_t)(v0 + lane);
+            node[v0 + lane].w = (r.w & 1u) | ((uint32_t)(idx + 1ull) << 1);
         }
+    }
+}
+
+__global__ void skip_tables_kernel(const uint4* __restrict__ node,
+                                   const uint32_t* __restrict__ list, unsigned long long count,
+                                   unsigned long long* __restrict__ tab) {
+    const int lane = threadIdx.x & 31;
+    const unsigned long long nw = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
+    for (unsigned long long i = (blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x) >> 5;
+         i < count; i += nw) {
+        // lane b squares its way to Q_b
+        unsigned long long q = (0x100000000ull - (unsigned long long)node[list[i]].z) << 32;
+        for (int b = 0; b < lane; b++) q = __umul64hi(q, q);
+        tab[i * SKIP_TABLE + lane] = q;
+        tab[i * SKIP_TABLE + 32 + lane] = skip_threshold(q);
     }
 }
 
@@ -410,12 +419,15 @@ int tim_graph_build(tim_ctx* ctx, int64_t n, int64_t m, const int64_t* d_rowptr,
             (const unsigned long long*)lt_t.p, (const uint8_t*)nonuni.p, (uint4*)ctx->node.p);
         ctx->launches++;
         if (model == TIM_IC) {
-            // count the skip-rule nodes, then give each its gap table
-            if ((rc = tim_ensure(ctx, lt_e, 2 * sizeof(unsigned long long)))) break;
+            // list the skip-rule nodes (at least TIM_SKIP_MIN_INDEG in-edges each), then give
+            // each its gap table
+            const uint64_t cap = (uint64_t)m / TIM_SKIP_MIN_INDEG + 1;
+            if ((rc = tim_ensure(ctx, lt_e, 16 + cap * sizeof(uint32_t)))) break;
             auto* ctr = (unsigned long long*)lt_e.p;
+            auto* list = (uint32_t*)(ctr + 2);
             if ((rc = tim_cuda_check(ctx, cudaMemsetAsync(ctr, 0, 16, ctx->stream), "memset")))
                 break;
-            skip_tables_kernel<<<G, T, 0, ctx->stream>>>(n, (uint4*)ctx->node.p, nullptr, 0, ctr);
+            skip_list_kernel<<<G, T, 0, ctx->stream>>>(n, (uint4*)ctx->node.p, list, cap, ctr);
             ctx->launches++;
             unsigned long long nskip = 0;
             if ((rc = tim_cuda_check(ctx, cudaMemcpyAsync(&nskip, ctr, 8, cudaMemcpyDeviceToHost,
@@ -423,9 +435,12 @@ int tim_graph_build(tim_ctx* ctx, int64_t n, int64_t m, const int64_t* d_rowptr,
                 break;
             if ((rc = tim_sync(ctx))) break;
             if ((rc = tim_ensure(ctx, ctx->qtab, (size_t)(nskip + 1) * SKIP_TABLE * 8))) break;
-            skip_tables_kernel<<<G, T, 0, ctx->stream>>>(
-                n, (uint4*)ctx->node.p, (unsigned long long*)ctx->qtab.p, nskip, ctr + 1);
-            ctx->launches++;
+            if (nskip) {
+                skip_tables_kernel<<<G, T, 0, ctx->stream>>>(
+                    (const uint4*)ctx->node.p, list, std::min<unsigned long long>(nskip, cap),
+                    (unsigned long long*)ctx->qtab.p);
+                ctx->launches++;
+            }
         }
         if ((rc = tim_cuda_check(ctx, cudaGetLastError(), "graph kernels"))) break;
         if ((rc = tim_read_scalars(ctx))) break;
