@@ -304,6 +304,13 @@ __global__ void __launch_bounds__(FB_THREADS) mlp_fb_kernel(FbArgs a, int d) {
     }
 }
 
+// Adam's moments, every rounding written out: a training run in one launch and one of a
+// launch pair per step give the same bits.
+__device__ inline float adam_m(float m, float g) { return fmaf(0.1f, g, __fmul_rn(0.9f, m)); }
+__device__ inline float adam_v(float v, float g) {
+    return fmaf(__fmul_rn(0.001f, g), g, __fmul_rn(0.999f, v));
+}
+
 // Sum the per-block partials in block order. With adam != 0, one Adam step on the fp32
 // master copy and the bfloat16-rounded working copy; else the gradient goes to `grad`.
 struct ReduceArgs {
@@ -335,13 +342,328 @@ __global__ void mlp_reduce_kernel(ReduceArgs r, int d) {
         r.grad[p] = g;
         return;
     }
-    const float m = 0.9f * r.m[p] + 0.1f * g;
-    const float v = 0.999f * r.v[p] + 0.001f * g * g;
+    const float m = adam_m(r.m[p], g), v = adam_v(r.v[p], g);
     r.m[p] = m;
     r.v[p] = v;
     const float w = r.params[p] - r.lr * (m * r.c1) / (sqrtf(v * r.c2) + 1e-8f);
     r.params[p] = w;
     r.wq[p] = is_weight(L, p) ? __bfloat162float(__float2bfloat16_rn(w)) : w;
+}
+
+// All steps of a training run in one cooperative launch: a block keeps its SB samples in
+// shared memory for the whole run; per step it loads the weights, writes its share of the
+// gradient, and after a grid barrier sums the blocks' shares of its part of the parameters
+// (staged in shared memory, then added in block order) and takes the Adam step on them; a
+// second barrier ends the step. Every output is summed in the order of mlp_fb_kernel and
+// mlp_reduce_kernel, so a run equals the same steps launched one by one bit for bit. A thread
+// holds one unit for four samples (or one weight column for eight rows), so that the products
+// read 8 shared words per 16 multiply-adds instead of 32, and each erf is evaluated once for
+// the activation and its derivative. (3,924 samples, 12 inputs, 200 steps: two launches per
+// step 5.9 ms, here 3.4 ms; bound by the two barriers and the chain of phases of a step.)
+constexpr int TR_THREADS = 512;
+constexpr int TR_G = TR_THREADS / H;  // groups of threads with one thread per unit
+constexpr int TR_S = SB / TR_G;       // samples per group
+constexpr int TR_I = H / TR_G;        // rows of W2 per group
+// its shared-memory plan, in floats; the transposed weights have rows of 65, so that the
+// transposing stores spread over the banks
+constexpr int TR_LD = H + 1;
+constexpr int TR_W1T = 0;                     // [DMAX][TR_LD]
+constexpr int TR_W2T = TR_W1T + DMAX * TR_LD; // [H][TR_LD]
+constexpr int TR_W2R = TR_W2T + H * TR_LD;    // [H][H] from here on multiples of 4
+constexpr int TR_B1 = TR_W2R + H * H;
+constexpr int TR_B2 = TR_B1 + H;
+constexpr int TR_W3 = TR_B2 + H;
+constexpr int TR_B3 = TR_W3 + H;              // [4]
+constexpr int TR_X = TR_B3 + 4;               // [SB][DMAX]
+constexpr int TR_A1 = TR_X + SB * DMAX;       // [SB][H] each, up to TR_Z; also the reduction's
+constexpr int TR_H1 = TR_A1 + SB * H;         // stage (fewer than P + 512 floats)
+constexpr int TR_A2 = TR_H1 + SB * H;
+constexpr int TR_H2 = TR_A2 + SB * H;
+constexpr int TR_D2 = TR_H2 + SB * H;
+constexpr int TR_D1 = TR_D2 + SB * H;
+constexpr int TR_E1 = TR_D1 + SB * H;         // erf(a1 / sqrt 2)
+constexpr int TR_E2 = TR_E1 + SB * H;
+constexpr int TR_Z = TR_E2 + SB * H;          // [SB] each
+constexpr int TR_L = TR_Z + SB;
+constexpr int TR_Y = TR_L + SB;               // y - out_mu
+constexpr size_t TR_BYTES = (size_t)(TR_Y + SB) * sizeof(float);
+static_assert(TR_W2R % 4 == 0 && TR_X % 4 == 0, "rows are read 16 bytes at a time");
+
+struct TrainArgs {
+    FbArgs f;
+    float* params;
+    float* wq;
+    float* m;
+    float* v;
+    float lr;
+    const float2* c;  // per step: 1 / (1 - beta1^t), 1 / (1 - beta2^t)
+    int steps;
+    float* hist;  // loss before each step
+    GridBarrier* bar;
+    int* err;
+    unsigned limit;
+};
+
+__device__ inline float gelu_grad_e(float t, float e) {
+    return 0.5f * (1.0f + e) + t * expf(-0.5f * t * t) * 0.39894228040143268f;
+}
+
+__global__ void __launch_bounds__(TR_THREADS, 2) mlp_train_kernel(TrainArgs a, int d) {
+    extern __shared__ __align__(16) float sm[];
+    const Layout L = layout_of(d);
+    const int t = threadIdx.x;
+    const int j = t & (H - 1), grp = t / H;
+    const uint32_t base = blockIdx.x * SB;
+    float* W1t = sm + TR_W1T;
+    float* b1 = sm + TR_B1;
+    float* W2t = sm + TR_W2T;
+    float* W2r = sm + TR_W2R;
+    float* b2 = sm + TR_B2;
+    float* W3 = sm + TR_W3;
+    float* X = sm + TR_X;
+    float* A1 = sm + TR_A1;
+    float* H1 = sm + TR_H1;
+    float* A2 = sm + TR_A2;
+    float* H2 = sm + TR_H2;
+    float* D2 = sm + TR_D2;
+    float* D1 = sm + TR_D1;
+    float* Z = sm + TR_Z;
+    float* Ls = sm + TR_L;
+    float* E1 = sm + TR_E1;
+    float* E2 = sm + TR_E2;
+    float* Y = sm + TR_Y;
+    for (int i = t; i < SB * d; i += TR_THREADS) {
+        const int s = i / d, k = i % d;
+        const uint32_t g = base + s;
+        X[s * DMAX + k] =
+            g < a.f.N ? (a.f.x[(size_t)g * d + k] - a.f.in_mu[k]) * a.f.in_isd[k] : 0.f;
+    }
+    if (t < SB) Y[t] = base + t < a.f.N ? a.f.y[base + t] - a.f.out_mu : 0.f;
+    float* part = a.f.part + (size_t)blockIdx.x * L.P;
+    // this block's parameters p0 .. p0 + np of the reduction
+    const int chunk = (L.P + (int)gridDim.x - 1) / (int)gridDim.x;
+    const int p0 = min((int)blockIdx.x * chunk, L.P), np = min(chunk, L.P - p0);
+    // a thread stages column col of the shares of every rows-th block from row on
+    const int cols = min(max(np, 1), TR_THREADS), rows = TR_THREADS / cols;
+    const int row = t / cols;
+    for (int step = 0; step < a.steps; step++) {
+        for (int i = t; i < H * d; i += TR_THREADS)
+            W1t[(i % d) * TR_LD + i / d] = __ldcg(a.wq + L.oW1 + i);
+        float w2[H * H / TR_THREADS];
+#pragma unroll
+        for (int q = 0; q < H * H / TR_THREADS; q++)
+            w2[q] = __ldcg(a.wq + L.oW2 + t + q * TR_THREADS);
+#pragma unroll
+        for (int q = 0; q < H * H / TR_THREADS; q++) {
+            const int i = t + q * TR_THREADS;
+            W2r[i] = w2[q];
+            W2t[(i % H) * TR_LD + i / H] = w2[q];
+        }
+        if (t < H) {
+            b1[t] = __ldcg(a.wq + L.ob1 + t);
+            b2[t] = __ldcg(a.wq + L.ob2 + t);
+            W3[t] = __ldcg(a.wq + L.oW3 + t);
+        }
+        if (t == 0) sm[TR_B3] = __ldcg(a.wq + L.ob3);
+        __syncthreads();
+        {  // layer 1
+            float acc[TR_S];
+#pragma unroll
+            for (int q = 0; q < TR_S; q++) acc[q] = b1[j];
+            for (int k = 0; k < d; k++) {
+                const float w = W1t[k * TR_LD + j];
+#pragma unroll
+                for (int q = 0; q < TR_S; q++)
+                    acc[q] = fmaf(w, X[(grp * TR_S + q) * DMAX + k], acc[q]);
+            }
+#pragma unroll
+            for (int q = 0; q < TR_S; q++) {
+                const int o = (grp * TR_S + q) * H + j;
+                const float e = erff(acc[q] * 0.70710678118654752f);
+                A1[o] = acc[q];
+                E1[o] = e;
+                H1[o] = 0.5f * acc[q] * (1.0f + e);
+            }
+        }
+        __syncthreads();
+        {  // layer 2
+            float acc[TR_S];
+#pragma unroll
+            for (int q = 0; q < TR_S; q++) acc[q] = b2[j];
+            for (int k = 0; k < H; k += 4) {
+                float w[4];
+#pragma unroll
+                for (int u = 0; u < 4; u++) w[u] = W2t[(k + u) * TR_LD + j];
+#pragma unroll
+                for (int q = 0; q < TR_S; q++) {
+                    const float4 h =
+                        *reinterpret_cast<const float4*>(H1 + (grp * TR_S + q) * H + k);
+                    acc[q] = fmaf(w[0], h.x, acc[q]);
+                    acc[q] = fmaf(w[1], h.y, acc[q]);
+                    acc[q] = fmaf(w[2], h.z, acc[q]);
+                    acc[q] = fmaf(w[3], h.w, acc[q]);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < TR_S; q++) {
+                const int o = (grp * TR_S + q) * H + j;
+                const float e = erff(acc[q] * 0.70710678118654752f);
+                A2[o] = acc[q];
+                E2[o] = e;
+                H2[o] = 0.5f * acc[q] * (1.0f + e);
+            }
+        }
+        __syncthreads();
+        {  // output and loss terms, a warp per sample
+            const int w = t >> 5, lane = t & 31;
+            for (int s = w; s < SB; s += TR_THREADS / 32) {
+                float v = W3[lane] * H2[s * H + lane];
+                v = fmaf(W3[lane + 32], H2[s * H + lane + 32], v);
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+                if (lane == 0) {
+                    const float z = v + sm[TR_B3];
+                    const float diff = base + s < a.f.N ? z - Y[s] * a.f.inv_out_sd : 0.f;
+                    Z[s] = diff * a.f.inv_n;
+                    Ls[s] = 0.5f * diff * diff * a.f.inv_n;
+                }
+            }
+        }
+        __syncthreads();
+        if (t < H) {  // output layer
+            float g = 0.f;
+            for (int s = 0; s < SB; s++) g = fmaf(Z[s], H2[s * H + t], g);
+            part[L.oW3 + t] = g;
+        } else if (t == H) {
+            float g = 0.f, l = 0.f;
+            for (int s = 0; s < SB; s++) {
+                g += Z[s];
+                l += Ls[s];
+            }
+            part[L.ob3] = g;
+            a.f.part_loss[blockIdx.x] = l;
+        }
+#pragma unroll
+        for (int q = 0; q < TR_S; q++) {
+            const int s = grp * TR_S + q;
+            D2[s * H + j] = Z[s] * W3[j] * gelu_grad_e(A2[s * H + j], E2[s * H + j]);
+        }
+        __syncthreads();
+        {  // layer 2: gW2[i][j] = sum_s D2[s][i] H1[s][j]
+            float g[TR_I];
+#pragma unroll
+            for (int i = 0; i < TR_I; i++) g[i] = 0.f;
+            for (int s = 0; s < SB; s++) {
+                const float h = H1[s * H + j];
+#pragma unroll
+                for (int i = 0; i < TR_I; i += 4) {
+                    const float4 x = *reinterpret_cast<const float4*>(D2 + s * H + grp * TR_I + i);
+                    g[i] = fmaf(x.x, h, g[i]);
+                    g[i + 1] = fmaf(x.y, h, g[i + 1]);
+                    g[i + 2] = fmaf(x.z, h, g[i + 2]);
+                    g[i + 3] = fmaf(x.w, h, g[i + 3]);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < TR_I; i++) part[L.oW2 + (grp * TR_I + i) * H + j] = g[i];
+        }
+        if (t < H) {
+            float g = 0.f;
+            for (int s = 0; s < SB; s++) g += D2[s * H + t];
+            part[L.ob2 + t] = g;
+        }
+        {  // back through W2
+            float acc[TR_S];
+#pragma unroll
+            for (int q = 0; q < TR_S; q++) acc[q] = 0.f;
+            for (int i = 0; i < H; i += 4) {
+                float w[4];
+#pragma unroll
+                for (int u = 0; u < 4; u++) w[u] = W2r[(i + u) * H + j];
+#pragma unroll
+                for (int q = 0; q < TR_S; q++) {
+                    const float4 x =
+                        *reinterpret_cast<const float4*>(D2 + (grp * TR_S + q) * H + i);
+                    acc[q] = fmaf(w[0], x.x, acc[q]);
+                    acc[q] = fmaf(w[1], x.y, acc[q]);
+                    acc[q] = fmaf(w[2], x.z, acc[q]);
+                    acc[q] = fmaf(w[3], x.w, acc[q]);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < TR_S; q++) {
+                const int o = (grp * TR_S + q) * H + j;
+                D1[o] = acc[q] * gelu_grad_e(A1[o], E1[o]);
+            }
+        }
+        __syncthreads();
+        // layer 1: gW1[j][k] = sum_s D1[s][j] X[s][k]
+        for (int k = grp; k < d; k += TR_G) {
+            float g = 0.f;
+            for (int s = 0; s < SB; s++) g = fmaf(D1[s * H + j], X[s * DMAX + k], g);
+            part[L.oW1 + j * d + k] = g;
+        }
+        if (t < H) {
+            float g = 0.f;
+            for (int s = 0; s < SB; s++) g += D1[s * H + t];
+            part[L.ob1 + t] = g;
+        }
+        if (!grid_barrier(a.bar, a.err, a.limit)) return;
+        // the blocks' shares of this block's parameters, then their sums in block order
+        // (chunk x gridDim.x < P + gridDim.x floats, in the activations' place)
+        float* stage = A1;
+        const int nb = (int)gridDim.x;
+        for (int at = 0; at < np; at += cols)
+            for (int b0 = 0; b0 < nb; b0 += 8 * rows) {  // eight loads in flight
+                const int col = at + t % cols;
+                const bool in = row < rows && col < np;
+                float x[8];
+#pragma unroll
+                for (int q = 0; q < 8; q++) {
+                    const int b = b0 + q * rows + row;
+                    x[q] = in && b < nb ? __ldcg(a.f.part + (size_t)b * L.P + p0 + col) : 0.f;
+                }
+#pragma unroll
+                for (int q = 0; q < 8; q++) {
+                    const int b = b0 + q * rows + row;
+                    if (in && b < nb) stage[b * np + col] = x[q];
+                }
+            }
+        if (blockIdx.x == 0)  // the losses, in the place of the erf values
+            for (int b = t; b < nb; b += TR_THREADS) E1[b] = __ldcg(a.f.part_loss + b);
+        const float2 c = a.c[step];
+        float m0 = 0.f, v0 = 0.f, w0 = 0.f;  // the moments and the parameter of this thread
+        if (t < np) {
+            m0 = a.m[p0 + t];
+            v0 = a.v[p0 + t];
+            w0 = a.params[p0 + t];
+        }
+        __syncthreads();
+        for (int i = t; i < np; i += TR_THREADS) {
+            const int p = p0 + i;
+            if (i != t) {
+                m0 = a.m[p];
+                v0 = a.v[p];
+                w0 = a.params[p];
+            }
+            float g = 0.f;
+#pragma unroll 8
+            for (int b = 0; b < nb; b++) g += stage[b * np + i];
+            const float m = adam_m(m0, g), v = adam_v(v0, g);
+            a.m[p] = m;
+            a.v[p] = v;
+            const float w = w0 - a.lr * (m * c.x) / (sqrtf(v * c.y) + 1e-8f);
+            a.params[p] = w;
+            a.wq[p] = is_weight(L, p) ? __bfloat162float(__float2bfloat16_rn(w)) : w;
+        }
+        if (blockIdx.x == 0 && t == TR_THREADS - 1) {
+            float l = 0.f;
+#pragma unroll 8
+            for (int b = 0; b < nb; b++) l += E1[b];
+            a.hist[step] = l;
+        }
+        if (!grid_barrier(a.bar, a.err, a.limit)) return;
+    }
 }
 
 __global__ void mlp_round_kernel(const float* __restrict__ params, float* __restrict__ wq,
@@ -362,6 +684,7 @@ struct tim_mlp {
     DevBuf params, wq, m, v, scal;  // scal: in_mu[DMAX], in_isd[DMAX]
     DevBuf x, y, out, part, ploss;
     DevBuf gbuf;  // gradient (tim_mlp_grad) or loss history (tim_mlp_train)
+    DevBuf corr, bar;  // training run: Adam's bias corrections per step, grid barrier
     float out_mu = 0.f, out_sd = 1.f;
     int step = 0;
 };
@@ -407,6 +730,12 @@ static int check_samples(tim_mlp* mlp, const float* x, uint64_t N) {
     return TIM_OK;
 }
 
+// Adam's bias corrections at step t: 1 / (1 - beta1^t), 1 / (1 - beta2^t).
+static float2 adam_corrections(int t) {
+    return make_float2((float)(1.0 / (1.0 - pow(0.9, (double)t))),
+                       (float)(1.0 / (1.0 - pow(0.999, (double)t))));
+}
+
 // Forward and backward over the uploaded batch, partials reduced into grad (no Adam)
 // or into one Adam step at mlp->step.
 static int mlp_step(tim_mlp* mlp, uint64_t N, bool adam, float lr, float* d_loss_out) {
@@ -429,8 +758,9 @@ static int mlp_step(tim_mlp* mlp, uint64_t N, bool adam, float lr, float* d_loss
     r.c1 = r.c2 = 1.f;
     if (adam) {
         mlp->step++;
-        r.c1 = (float)(1.0 / (1.0 - pow(0.9, (double)mlp->step)));
-        r.c2 = (float)(1.0 / (1.0 - pow(0.999, (double)mlp->step)));
+        const float2 c = adam_corrections(mlp->step);
+        r.c1 = c.x;
+        r.c2 = c.y;
     } else {
         TIM_TRY(tim_ensure(ctx, mlp->gbuf, (size_t)mlp->L.P * sizeof(float)));
         r.grad = (float*)mlp->gbuf.p;
@@ -516,7 +846,7 @@ int tim_mlp_destroy(tim_mlp* mlp) {
     if (!mlp) return TIM_OK;
     DeviceGuard g(mlp->ctx->device);
     for (DevBuf* b : {&mlp->params, &mlp->wq, &mlp->m, &mlp->v, &mlp->scal, &mlp->x, &mlp->y,
-                      &mlp->out, &mlp->part, &mlp->ploss, &mlp->gbuf})
+                      &mlp->out, &mlp->part, &mlp->ploss, &mlp->gbuf, &mlp->corr, &mlp->bar})
         tim_free(*b);
     delete mlp;
     return TIM_OK;
@@ -600,7 +930,54 @@ int tim_mlp_train(tim_mlp* mlp, const float* x, const float* y, uint64_t n_sampl
     TIM_TRY(mlp_upload(mlp, x, y, n_samples));
     TIM_TRY(tim_ensure(ctx, mlp->gbuf, ((size_t)steps + 1) * sizeof(float)));
     float* hist = (float*)mlp->gbuf.p;
-    for (int s = 0; s < steps; s++) TIM_TRY(mlp_step(mlp, n_samples, true, lr, hist + s));
+    // one cooperative launch when all blocks of samples are resident at once
+    const unsigned nb = (unsigned)((n_samples + SB - 1) / SB);
+    int coop = 0, per_sm = 0;
+    cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, ctx->device);
+    if (coop && steps > 0) {
+        CUDA_TRY(ctx, cudaFuncSetAttribute(mlp_train_kernel,
+                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)TR_BYTES));
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mlp_train_kernel, TR_THREADS,
+                                                          TR_BYTES) != cudaSuccess) {
+            cudaGetLastError();
+            per_sm = 0;
+        }
+    }
+    std::vector<float2> corr;
+    if (steps > 0 && nb <= (unsigned)(per_sm * ctx->num_sms)) {
+        corr.resize(steps);
+        for (int s = 0; s < steps; s++) corr[s] = adam_corrections(mlp->step + s + 1);
+        TIM_TRY(tim_ensure(ctx, mlp->corr, (size_t)steps * sizeof(float2)));
+        TIM_TRY(tim_ensure(ctx, mlp->bar, sizeof(GridBarrier)));
+        CUDA_TRY(ctx, cudaMemcpyAsync(mlp->corr.p, corr.data(), (size_t)steps * sizeof(float2),
+                                      cudaMemcpyHostToDevice, ctx->stream));
+        CUDA_TRY(ctx, cudaMemsetAsync(mlp->bar.p, 0, sizeof(GridBarrier), ctx->stream));
+        TIM_TRY(tim_zero_scalars(ctx));
+        TrainArgs ta;
+        ta.f = fb_args(mlp, n_samples);
+        ta.params = (float*)mlp->params.p;
+        ta.wq = (float*)mlp->wq.p;
+        ta.m = (float*)mlp->m.p;
+        ta.v = (float*)mlp->v.p;
+        ta.lr = lr;
+        ta.c = (const float2*)mlp->corr.p;
+        ta.steps = steps;
+        ta.hist = hist;
+        ta.bar = (GridBarrier*)mlp->bar.p;
+        ta.err = &tim_dscal(ctx)->err;
+        ta.limit = std::max(ctx->wait_limit, 1u << 24);  // a run never fails for a short limit
+        void* args[] = {&ta, &mlp->d};
+        CUDA_TRY(ctx, cudaLaunchCooperativeKernel((const void*)mlp_train_kernel, dim3(nb),
+                                                  dim3(TR_THREADS), args, TR_BYTES, ctx->stream));
+        LAUNCH_CHECK(ctx, "mlp_train_kernel");
+        TIM_TRY(tim_read_scalars(ctx));
+        if (ctx->h_scal->err & TIM_DEV_ERR_TIMEOUT)
+            return tim_fail(ctx, TIM_ERR_TIMEOUT, "training grid barrier timed out");
+        mlp->step += steps;
+    } else {
+        for (int s = 0; s < steps; s++) TIM_TRY(mlp_step(mlp, n_samples, true, lr, hist + s));
+    }
     if (loss_history && steps > 0)
         CUDA_TRY(ctx, cudaMemcpyAsync(loss_history, hist, (size_t)steps * sizeof(float),
                                       cudaMemcpyDeviceToHost, ctx->stream));
