@@ -554,7 +554,7 @@ __device__ __forceinline__ unsigned long long kappa_fixed(double kappa) {
     return __double2ull_rz(__dmul_rn(kappa, 9223372036854775808.0));
 }
 
-// Barrier over all blocks of a co-resident (cooperative) launch: sense reversal on a
+// Barrier over all blocks (or the first `blocks`) of a co-resident (cooperative) launch: sense reversal on a
 // generation counter, which the host zeroes before each launch. The wait is bounded:
 // after `limit` polls a block sets TIM_DEV_ERR_TIMEOUT in *err and the barrier returns
 // false; it also returns false once any block has set that bit, so every block of the
@@ -564,14 +564,15 @@ struct GridBarrier {
     unsigned gen;
 };
 
-__device__ __forceinline__ bool grid_barrier(GridBarrier* bar, int* err, unsigned limit) {
+__device__ __forceinline__ bool grid_barrier(GridBarrier* bar, int* err, unsigned limit,
+                                             unsigned blocks) {
     __shared__ int s_ok;
     __syncthreads();
     if (threadIdx.x == 0) {
         int ok = 1;
         __threadfence();
         const unsigned g = ((volatile unsigned*)&bar->gen)[0];
-        if (atomicAdd(&bar->count, 1u) == gridDim.x - 1) {
+        if (atomicAdd(&bar->count, 1u) == blocks - 1) {
             atomicExch(&bar->count, 0u);
             __threadfence();
             atomicAdd(&bar->gen, 1u);
@@ -591,6 +592,55 @@ __device__ __forceinline__ bool grid_barrier(GridBarrier* bar, int* err, unsigne
     }
     __syncthreads();
     return s_ok != 0;
+}
+
+__device__ __forceinline__ bool grid_barrier(GridBarrier* bar, int* err, unsigned limit) {
+    return grid_barrier(bar, err, limit, gridDim.x);
+}
+
+// Greedy key of a node: larger counts first, then smaller ids.
+__device__ __forceinline__ unsigned long long greedy_key(int cnt, uint32_t v) {
+    return ((unsigned long long)(uint32_t)max(cnt, 0) << 32) | (unsigned long long)(~v);
+}
+
+// Best key of nodes 4q .. 4q+3 (0 for chosen nodes): counts as one 16-byte load, the
+// chosen flags as one 32-bit word.
+__device__ __forceinline__ unsigned long long quad_key(int4 c, uint32_t ch, uint64_t q) {
+    const uint32_t v = (uint32_t)(q << 2);
+    unsigned long long b = (ch & 0xFFu) ? 0ull : greedy_key(c.x, v);
+    b = max(b, (ch & 0xFF00u) ? 0ull : greedy_key(c.y, v + 1));
+    b = max(b, (ch & 0xFF0000u) ? 0ull : greedy_key(c.z, v + 2));
+    b = max(b, (ch & 0xFF000000u) ? 0ull : greedy_key(c.w, v + 3));
+    return b;
+}
+
+// Best key over the thread's share of the nodes (thread t of `stride` takes quads t,
+// t + stride, ...; four quads in flight; the last n mod 4 nodes one by one). Counts
+// and flags are read from L2 (__ldcg): other blocks change them between rounds. Both
+// arrays start 16-byte aligned (cudaMalloc).
+__device__ __forceinline__ unsigned long long slice_argmax(const int* counts,
+                                                           const uint8_t* chosen, uint64_t n,
+                                                           uint64_t t, uint64_t stride) {
+    const int4* c4 = reinterpret_cast<const int4*>(counts);
+    const uint32_t* h4 = reinterpret_cast<const uint32_t*>(chosen);
+    const uint64_t nq = n >> 2;
+    unsigned long long b = 0;
+    uint64_t q = t;
+    for (; q + 3 * stride < nq; q += 4 * stride) {
+        int4 c[4];
+        uint32_t h[4];
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            c[i] = __ldcg(c4 + q + i * stride);
+            h[i] = __ldcg(h4 + q + i * stride);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; i++) b = max(b, quad_key(c[i], h[i], q + i * stride));
+    }
+    for (; q < nq; q += stride) b = max(b, quad_key(__ldcg(c4 + q), __ldcg(h4 + q), q));
+    for (uint64_t v = (nq << 2) + t; v < n; v += stride)
+        if (!__ldcg(chosen + v)) b = max(b, greedy_key(__ldcg(counts + v), (uint32_t)v));
+    return b;
 }
 
 // Add a 128-bit (hi, lo) into a global 128-bit accumulator.

@@ -25,8 +25,7 @@ constexpr int64_t NA_MAX_NODES = 1 << 18;        // n
 constexpr uint64_t NA_MAX_SETS = 1 << 20;        // number of RR sets
 constexpr uint64_t NA_MAX_MEMBERS = 1 << 21;     // sum of |R|
 constexpr int NA_MAX_K = 1024;                   // seeds
-constexpr int NA_SCAN_TILE = 4096;
-constexpr uint64_t NA_SCAN_BLOCKS = (NA_MAX_NODES + NA_SCAN_TILE - 1) / NA_SCAN_TILE + 1;
+constexpr uint64_t NA_MAX_BLOCKS = 1024;         // blocks of the launch (one per SM)
 
 // Layout of the scratch array (byte offsets, each a multiple of 256).
 constexpr uint64_t al(uint64_t x) { return (x + 255) & ~uint64_t(255); }
@@ -38,8 +37,8 @@ constexpr uint64_t OFF_COVERED = al(OFF_NODE_SETS + 4 * NA_MAX_MEMBERS);     // 
 constexpr uint64_t OFF_CHOSEN = al(OFF_COVERED + NA_MAX_SETS);               // u8[n]
 constexpr uint64_t OFF_BEST = al(OFF_CHOSEN + NA_MAX_NODES);                 // u64[k]
 constexpr uint64_t OFF_SUMS = al(OFF_BEST + 8 * NA_MAX_K);                   // u64[blocks]
-constexpr uint64_t OFF_FLAGS = al(OFF_SUMS + 8 * NA_SCAN_BLOCKS);            // u64[4]
-constexpr uint64_t NA_SCRATCH_BYTES = al(OFF_FLAGS + 32);
+constexpr uint64_t OFF_FLAGS = al(OFF_SUMS + 8 * NA_MAX_BLOCKS);            // u64[8]
+constexpr uint64_t NA_SCRATCH_BYTES = al(OFF_FLAGS + 64);
 
 static __device__ __align__(256) unsigned char na_scratch[NA_SCRATCH_BYTES];
 
@@ -52,7 +51,7 @@ struct NaView {
     uint8_t* chosen;
     unsigned long long* best;
     unsigned long long* sums;
-    unsigned long long* flags;  // [0] covered count, [1] error bits
+    unsigned long long* flags;  // [0] covered count, [1] error bits, [2] barrier, [3] barrier error, [4] the rounds' barrier
 };
 
 NaView view_of(unsigned char* base) {
@@ -69,167 +68,196 @@ NaView view_of(unsigned char* base) {
     return v;
 }
 
-// Histogram of members; members outside [0, n) are skipped and flagged.
-__global__ void na_count_kernel(const int64_t* __restrict__ off, const int32_t* __restrict__ mem,
-                                uint64_t n_sets, int64_t n, NaView v) {
-    const uint64_t members = (uint64_t)off[n_sets];
-    for (uint64_t p = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p < members;
-         p += (uint64_t)gridDim.x * blockDim.x) {
-        const int32_t u = mem[p];
-        if (u < 0 || u >= n) {
-            atomicOr(&v.flags[1], 1ull);
-            continue;
-        }
-        atomicAdd(&v.counts[u], 1);
-    }
-}
+constexpr int NA_THREADS = 512;
+// blocks that run the greedy rounds (8, 16, 32, 64, 152 blocks: 951, 762, 700, 672, 673 us at
+// the size below)
+constexpr unsigned NA_ROUNDS_GRID = 64;
+constexpr uint32_t NA_SLOTS = 4096;  // hot-node table of the histogram
+constexpr uint32_t NA_EMPTY = 0xFFFFFFFFu;
 
-// Exclusive scan of the counts into node_off (one block per 4096 entries, then one
-// block over the block sums, then the fix-up), as in the library's own scan.
-__device__ unsigned long long na_block_scan(unsigned long long x, unsigned long long* total) {
-    __shared__ unsigned long long wsum[33];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+// Exclusive scan of one value per thread over the block.
+__device__ unsigned long long na_block_scan(unsigned long long x, unsigned long long* wsum,
+                                            unsigned long long* total) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     unsigned long long inc = x;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        unsigned long long y = __shfl_up_sync(0xffffffffu, inc, o);
+        const unsigned long long y = __shfl_up_sync(0xffffffffu, inc, o);
         if (lane >= o) inc += y;
     }
+    __syncthreads();
     if (lane == 31) wsum[w] = inc;
     __syncthreads();
-    if (w == 0) {
-        unsigned long long t = lane < nw ? wsum[lane] : 0ull, ti = t;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            unsigned long long y = __shfl_up_sync(0xffffffffu, ti, o);
-            if (lane >= o) ti += y;
-        }
-        if (lane < nw) wsum[lane] = ti - t;
-        if (lane == nw - 1) wsum[32] = ti;
+    unsigned long long before = 0, all = 0;
+    for (int i = 0; i < NA_THREADS / 32; i++) {
+        if (i < w) before += wsum[i];
+        all += wsum[i];
     }
-    __syncthreads();
-    const unsigned long long r = wsum[w] + inc - x;
-    *total = wsum[32];
-    __syncthreads();
-    return r;
+    *total = all;
+    return before + inc - x;
 }
 
-__global__ void na_scan_sums_kernel(int64_t n, NaView v) {
-    const uint64_t base = (uint64_t)blockIdx.x * NA_SCAN_TILE;
-    unsigned long long s = 0;
-    for (int i = threadIdx.x; i < NA_SCAN_TILE; i += blockDim.x)
-        if (base + i < (uint64_t)n) s += (uint32_t)v.counts[base + i];
-    unsigned long long tot;
-    na_block_scan(s, &tot);
-    if (threadIdx.x == 0) v.sums[blockIdx.x] = tot;
-}
+struct NaArgs {
+    const int64_t* off;
+    const int32_t* mem;
+    uint64_t n_sets;
+    int64_t n;
+    uint64_t members;
+    int k;
+    int32_t* seeds;
+    uint64_t* covered_out;
+    unsigned rounds_grid;
+    NaView v;
+    unsigned limit;
+};
 
-__global__ void na_scan_top_kernel(uint64_t nblocks, int64_t n, NaView v) {
-    unsigned long long carry = 0;
-    for (uint64_t b = 0; b < nblocks; b += blockDim.x) {
-        const uint64_t i = b + threadIdx.x;
-        const unsigned long long x = i < nblocks ? v.sums[i] : 0ull;
-        unsigned long long tot;
-        const unsigned long long ex = na_block_scan(x, &tot);
-        if (i < nblocks) v.sums[i] = carry + ex;
-        carry += tot;
+// The whole selection in one cooperative launch; a grid barrier separates its phases:
+// clearing, the histogram of members (hub nodes counted in a shared-memory table first, since
+// atomics on one address take turns), the scan into node offsets, node -> sets, and per round
+// an argmax over the counts and the cover of the chosen node's sets (eight lanes per set).
+// One launch per phase and two per round: 150,001 nodes, 250,007 sets of six members, k = 50,
+// 870 us, this 672 us; bound by a round's chain of about fourteen dependent L2 accesses, two
+// barriers among them.
+__global__ void __launch_bounds__(NA_THREADS) na_select_kernel(NaArgs a) {
+    __shared__ uint32_t tag[NA_SLOTS], num[NA_SLOTS];
+    __shared__ unsigned long long wsum[NA_THREADS / 32];
+    const NaView v = a.v;
+    GridBarrier* bar = reinterpret_cast<GridBarrier*>(v.flags + 2);
+    int* err = reinterpret_cast<int*>(v.flags + 3);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const uint64_t tid = blockIdx.x * (uint64_t)NA_THREADS + threadIdx.x;
+    const uint64_t nt = (uint64_t)gridDim.x * NA_THREADS;
+    const uint64_t n = (uint64_t)a.n;
+    for (uint64_t i = tid; i < n; i += nt) {
+        v.counts[i] = 0;
+        v.chosen[i] = 0;
     }
-    if (threadIdx.x == 0) v.node_off[n] = carry;
-}
-
-__global__ void na_scan_apply_kernel(int64_t n, NaView v) {
-    // each thread scans 16 consecutive counts of the block's 4096
-    const uint64_t base = (uint64_t)blockIdx.x * NA_SCAN_TILE + (uint64_t)threadIdx.x * 16;
-    unsigned long long loc = 0;
-    for (int i = 0; i < 16; i++)
-        if (base + i < (uint64_t)n) loc += (uint32_t)v.counts[base + i];
-    unsigned long long tot;
-    unsigned long long ex = na_block_scan(loc, &tot) + v.sums[blockIdx.x];
-    for (int i = 0; i < 16; i++)
-        if (base + i < (uint64_t)n) {
-            v.node_off[base + i] = ex;
-            ex += (uint32_t)v.counts[base + i];
-        }
-}
-
-// node -> sets: one warp per set writes the set id into each member's list.
-__global__ void na_scatter_kernel(const int64_t* __restrict__ off, const int32_t* __restrict__ mem,
-                                  uint64_t n_sets, int64_t n, NaView v) {
-    const int lane = threadIdx.x & 31;
-    const uint64_t w0 = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
-    const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t members = off[n_sets];
-    for (uint64_t s = w0; s < n_sets; s += nw) {
-        const int64_t a = off[s], b = off[s + 1];
-        if (a < 0 || b < a || b > members) {  // malformed offsets: flag, skip the set
-            if (lane == 0) atomicOr(&v.flags[1], 2ull);
+    for (uint64_t i = tid; i < a.n_sets; i += nt) v.covered[i] = 0;
+    for (uint64_t i = tid; i < (uint64_t)a.k; i += nt) v.best[i] = 0;
+    for (uint32_t i = threadIdx.x; i < NA_SLOTS; i += NA_THREADS) {
+        tag[i] = NA_EMPTY;
+        num[i] = 0u;
+    }
+    if (!grid_barrier(bar, err, a.limit)) return;
+    // histogram; members outside [0, n) are skipped and flagged
+    for (uint64_t p = tid; p < a.members; p += nt) {
+        const int32_t u = a.mem[p];
+        if (u < 0 || u >= a.n) {
+            atomicOr(&v.flags[1], 1ull);
             continue;
         }
-        for (int64_t p = a + lane; p < b; p += 32) {
-            const int32_t u = mem[p];
-            if (u < 0 || u >= n) continue;
-            const uint32_t slot = atomicAdd(&v.cursor[u], 1u);
-            if (v.node_off[u] + slot < v.node_off[u + 1])
-                v.node_sets[v.node_off[u] + slot] = (uint32_t)s;
+        const uint32_t h = ((uint32_t)u * 0x9E3779B1u) >> 20;  // 12 bits
+        uint32_t t = ((volatile uint32_t*)tag)[h];
+        if (t == NA_EMPTY) {
+            t = atomicCAS(&tag[h], NA_EMPTY, (uint32_t)u);
+            if (t == NA_EMPTY) t = (uint32_t)u;
+        }
+        if (t == (uint32_t)u)
+            atomicAdd(&num[h], 1u);
+        else
+            atomicAdd(&v.counts[u], 1);
+    }
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < NA_SLOTS; i += NA_THREADS)
+        if (num[i]) atomicAdd(&v.counts[tag[i]], (int)num[i]);
+    if (!grid_barrier(bar, err, a.limit)) return;
+    // node offsets: every block scans a contiguous range of nodes
+    const uint64_t per = (n + gridDim.x - 1) / gridDim.x;
+    const uint64_t ib = min(blockIdx.x * per, n), ie = min(ib + per, n);
+    unsigned long long sum = 0, tot = 0;
+    for (uint64_t i = ib + threadIdx.x; i < ie; i += NA_THREADS) sum += (uint32_t)__ldcg(v.counts + i);
+    na_block_scan(sum, wsum, &tot);
+    if (threadIdx.x == 0) v.sums[blockIdx.x] = tot;
+    if (!grid_barrier(bar, err, a.limit)) return;
+    unsigned long long before = 0;
+    for (uint32_t b = threadIdx.x; b < blockIdx.x; b += NA_THREADS) before += __ldcg(v.sums + b);
+    na_block_scan(before, wsum, &before);  // the blocks' totals below this one
+    for (uint64_t c = ib; c < ie; c += NA_THREADS) {
+        const uint64_t i = c + threadIdx.x;
+        const unsigned long long x = i < ie ? (uint32_t)__ldcg(v.counts + i) : 0ull;
+        const unsigned long long ex = na_block_scan(x, wsum, &tot);
+        if (i < ie) {
+            v.node_off[i] = before + ex;
+            v.cursor[i] = (uint32_t)(before + ex);  // at most NA_MAX_MEMBERS
+        }
+        before += tot;
+    }
+    if (ie == n && ib < n && threadIdx.x == 0) v.node_off[n] = before;
+    if (!grid_barrier(bar, err, a.limit)) return;
+    // node -> sets, eight lanes per set
+    const int sub = lane & 7;
+    for (uint64_t s = tid >> 3; s < a.n_sets; s += nt >> 3) {
+        const int64_t pa = a.off[s], pb = a.off[s + 1];
+        if (pa < 0 || pb < pa || (uint64_t)pb > a.members) {  // malformed offsets: skip the set
+            if (sub == 0) atomicOr(&v.flags[1], 2ull);
+            continue;
+        }
+        for (int64_t p = pa + sub; p < pb; p += 8) {
+            const int32_t u = a.mem[p];
+            if (u < 0 || u >= a.n) continue;
+            const uint32_t at = atomicAdd(&v.cursor[u], 1u);
+            if (at < __ldcg(v.node_off + u + 1))
+                v.node_sets[at] = (uint32_t)s;
             else
                 atomicOr(&v.flags[1], 2ull);
         }
     }
-}
-
-__global__ void na_argmax_kernel(int64_t n, NaView v, int r) {
-    unsigned long long b = 0;
-    for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < n;
-         u += (int64_t)gridDim.x * blockDim.x) {
-        if (!v.chosen[u]) {
-            const unsigned long long key =
-                ((unsigned long long)(uint32_t)max(v.counts[u], 0) << 32) |
-                (unsigned long long)(~(uint32_t)u);
-            b = key > b ? key : b;
+    if (!grid_barrier(bar, err, a.limit)) return;
+    // the rounds are short: the first few blocks run them, with barriers of their own
+    if (blockIdx.x >= a.rounds_grid) return;
+    bar = reinterpret_cast<GridBarrier*>(v.flags + 4);
+    const uint64_t nr = (uint64_t)a.rounds_grid * NA_THREADS;
+    unsigned long long fresh = 0;
+    for (int r = 0; r < a.k; r++) {
+        unsigned long long b = slice_argmax(v.counts, v.chosen, n, tid, nr);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long y = __shfl_xor_sync(0xffffffffu, b, o);
+            b = y > b ? y : b;
         }
+        __syncthreads();
+        if (lane == 0) wsum[wid] = b;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int i = 1; i < NA_THREADS / 32; i++) b = wsum[i] > b ? wsum[i] : b;
+            if (b) atomicMax(&v.best[r], b);
+        }
+        if (!grid_barrier(bar, err, a.limit, a.rounds_grid)) return;
+        const unsigned long long key = __ldcg(v.best + r);
+        if (key != 0) {
+            const uint32_t u = ~(uint32_t)(key & 0xFFFFFFFFull);
+            if (tid == 0) {
+                v.chosen[u] = 1;
+                a.seeds[r] = (int32_t)u;
+            }
+            const uint64_t e0 = __ldcg(v.node_off + u), e1 = __ldcg(v.node_off + u + 1);
+            for (uint64_t i = e0 + (tid >> 3); i < e1; i += nr >> 3) {
+                const uint32_t s = __ldcg(v.node_sets + i);
+                const int64_t pa = a.off[s], pb = a.off[s + 1];
+                // the eight lanes read the flag before one of them sets it
+                const unsigned group = 0xFFu << (lane & 24);
+                const bool done = __ldcg(v.covered + s) != 0;
+                __syncwarp(group);
+                if (done) continue;
+                if (sub == 0) {
+                    v.covered[s] = 1;
+                    fresh++;
+                }
+                if (pa < 0 || pb < pa || (uint64_t)pb > a.members) continue;
+                for (int64_t p = pa + sub; p < pb; p += 8) {
+                    const int32_t x = a.mem[p];
+                    if (x >= 0 && x < a.n) atomicSub(&v.counts[x], 1);
+                }
+            }
+        }
+        if (!grid_barrier(bar, err, a.limit, a.rounds_grid)) return;
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long y = __shfl_xor_sync(0xffffffffu, b, o);
-        b = y > b ? y : b;
-    }
-    if ((threadIdx.x & 31) == 0 && b) atomicMax(&v.best[r], b);
-}
-
-__global__ void na_cover_kernel(const int64_t* __restrict__ off, const int32_t* __restrict__ mem,
-                                uint64_t n_sets, int64_t n, NaView v, int r,
-                                int32_t* __restrict__ seeds) {
-    const unsigned long long key = v.best[r];
-    if (key == 0) return;
-    const uint32_t u = ~(uint32_t)(key & 0xFFFFFFFFull);
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        v.chosen[u] = 1;
-        seeds[r] = (int32_t)u;
-    }
-    const int lane = threadIdx.x & 31;
-    const uint64_t w0 = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
-    const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-    const uint64_t a = v.node_off[u], b = v.node_off[u + 1];
-    unsigned long long fresh = 0;
-    for (uint64_t i = a + w0; i < b; i += nw) {
-        const uint32_t s = v.node_sets[i];
-        if (v.covered[s]) continue;
-        __syncwarp();
-        if (lane == 0) {
-            v.covered[s] = 1;
-            fresh++;
-        }
-        const int64_t pa = off[s], pb = off[s + 1];
-        if (pa < 0 || pb < pa || pb > off[n_sets]) continue;
-        for (int64_t p = pa + lane; p < pb; p += 32) {
-            const int32_t x = mem[p];
-            if (x >= 0 && x < n) atomicSub(&v.counts[x], 1);
-        }
-    }
+    for (int o = 16; o > 0; o >>= 1) fresh += __shfl_xor_sync(0xffffffffu, fresh, o);
     if (lane == 0 && fresh) atomicAdd(&v.flags[0], fresh);
+    if (!grid_barrier(bar, err, a.limit, a.rounds_grid)) return;
+    if (tid == 0) *a.covered_out = __ldcg(v.flags);
 }
-
-__global__ void na_finish_kernel(NaView v, uint64_t* covered_out) { *covered_out = v.flags[0]; }
 
 std::mutex na_mutex;
 unsigned char* na_base[64] = {};
@@ -277,41 +305,54 @@ extern "C" int tim_node_select_noalloc(int device, void* cuda_stream, int64_t n,
             break;
         }
         const NaView v = view_of(base);
-        // clear what must start at zero
-        if (cudaMemsetAsync(v.counts, 0, 4 * (size_t)n, st) != cudaSuccess ||
-            cudaMemsetAsync(v.cursor, 0, 4 * (size_t)n, st) != cudaSuccess ||
-            cudaMemsetAsync(v.chosen, 0, (size_t)n, st) != cudaSuccess ||
-            cudaMemsetAsync(v.covered, 0, (size_t)n_sets + 1, st) != cudaSuccess ||
-            cudaMemsetAsync(v.best, 0, 8 * (size_t)k, st) != cudaSuccess ||
-            cudaMemsetAsync(v.flags, 0, 32, st) != cudaSuccess) {
+        // counters, error bits and the grid barrier
+        if (cudaMemsetAsync(v.flags, 0, 64, st) != cudaSuccess) {
             rc = TIM_ERR_CUDA;
             break;
         }
-        const uint64_t nblocks = ((uint64_t)n + NA_SCAN_TILE - 1) / NA_SCAN_TILE;
-        int sms = 0;
+        int sms = 0, nb = 0;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-        const unsigned G = (unsigned)(sms > 0 ? sms * 4 : 128);
-        if (n_sets > 0) na_count_kernel<<<G, 256, 0, st>>>(d_off, d_mem, n_sets, n, v);
-        na_scan_sums_kernel<<<(unsigned)nblocks, 256, 0, st>>>(n, v);
-        na_scan_top_kernel<<<1, 256, 0, st>>>(nblocks, n, v);
-        na_scan_apply_kernel<<<(unsigned)nblocks, 256, 0, st>>>(n, v);
-        if (n_sets > 0) na_scatter_kernel<<<G, 256, 0, st>>>(d_off, d_mem, n_sets, n, v);
-        for (int r = 0; r < k; r++) {
-            na_argmax_kernel<<<G, 256, 0, st>>>(n, v, r);
-            na_cover_kernel<<<G, 256, 0, st>>>(d_off, d_mem, n_sets, n, v, r, d_seeds);
-        }
-        na_finish_kernel<<<1, 1, 0, st>>>(v, d_covered);
-        if (cudaGetLastError() != cudaSuccess) {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, na_select_kernel, NA_THREADS, 0) !=
+                cudaSuccess ||
+            nb < 1 || sms < 1) {
+            cudaGetLastError();
             rc = TIM_ERR_CUDA;
             break;
         }
-        unsigned long long err = 0;
-        if (cudaMemcpyAsync(&err, v.flags + 1, 8, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        NaArgs na;
+        na.off = d_off;
+        na.mem = d_mem;
+        na.n_sets = n_sets;
+        na.n = n;
+        na.members = (uint64_t)ends[1];
+        na.k = k;
+        na.seeds = d_seeds;
+        na.covered_out = d_covered;
+        na.v = v;
+        na.limit = 1u << 24;
+        // one block per SM, fewer for a small problem (a barrier of few blocks is shorter)
+        uint64_t work = (uint64_t)n;
+        if (work < na.members) work = na.members;
+        if (work < n_sets) work = n_sets;
+        const uint64_t want = work / (2 * NA_THREADS) + 1;
+        uint64_t G64 = want < (uint64_t)sms ? want : (uint64_t)sms;
+        const unsigned G = (unsigned)(G64 < NA_MAX_BLOCKS ? G64 : NA_MAX_BLOCKS);
+        na.rounds_grid = G < NA_ROUNDS_GRID ? G : NA_ROUNDS_GRID;
+        void* args[] = {&na};
+        if (cudaLaunchCooperativeKernel((const void*)na_select_kernel, dim3(G), dim3(NA_THREADS),
+                                        args, 0, st) != cudaSuccess ||
+            cudaGetLastError() != cudaSuccess) {
+            rc = TIM_ERR_CUDA;
+            break;
+        }
+        unsigned long long err[3] = {0, 0, 0};  // error bits, barrier, barrier's error
+        if (cudaMemcpyAsync(err, v.flags + 1, 24, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
             cudaStreamSynchronize(st) != cudaSuccess) {
             rc = TIM_ERR_CUDA;
             break;
         }
-        if (err) rc = TIM_ERR_ARG;
+        if (err[2]) rc = TIM_ERR_TIMEOUT;
+        else if (err[0]) rc = TIM_ERR_ARG;
     } while (0);
     if (prev >= 0 && prev != device) cudaSetDevice(prev);
     return rc;

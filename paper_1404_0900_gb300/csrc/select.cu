@@ -110,50 +110,6 @@ __global__ void scatter_sets_kernel(const uint32_t* __restrict__ pool,
         node_sets[atomicAdd(&next[pool[p]], 1ull)] = pool_sid[p];
 }
 
-__device__ __forceinline__ unsigned long long greedy_key(int cnt, uint32_t v) {
-    return ((unsigned long long)(uint32_t)max(cnt, 0) << 32) | (unsigned long long)(~v);
-}
-
-// Best key of nodes 4q .. 4q+3 (0 for chosen nodes): counts as one 16-byte load, the
-// chosen flags as one 32-bit word.
-__device__ __forceinline__ unsigned long long quad_key(int4 c, uint32_t ch, uint64_t q) {
-    const uint32_t v = (uint32_t)(q << 2);
-    unsigned long long b = (ch & 0xFFu) ? 0ull : greedy_key(c.x, v);
-    b = max(b, (ch & 0xFF00u) ? 0ull : greedy_key(c.y, v + 1));
-    b = max(b, (ch & 0xFF0000u) ? 0ull : greedy_key(c.z, v + 2));
-    b = max(b, (ch & 0xFF000000u) ? 0ull : greedy_key(c.w, v + 3));
-    return b;
-}
-
-// Best key over the thread's share of the nodes (thread t of `stride` takes quads t,
-// t + stride, ...; four quads in flight; the last n mod 4 nodes one by one). Counts
-// and flags are read from L2 (__ldcg): other blocks change them between rounds. Both
-// arrays start 16-byte aligned (cudaMalloc).
-__device__ __forceinline__ unsigned long long slice_argmax(const int* counts,
-                                                           const uint8_t* chosen, uint64_t n,
-                                                           uint64_t t, uint64_t stride) {
-    const int4* c4 = reinterpret_cast<const int4*>(counts);
-    const uint32_t* h4 = reinterpret_cast<const uint32_t*>(chosen);
-    const uint64_t nq = n >> 2;
-    unsigned long long b = 0;
-    uint64_t q = t;
-    for (; q + 3 * stride < nq; q += 4 * stride) {
-        int4 c[4];
-        uint32_t h[4];
-#pragma unroll
-        for (int i = 0; i < 4; i++) {
-            c[i] = __ldcg(c4 + q + i * stride);
-            h[i] = __ldcg(h4 + q + i * stride);
-        }
-#pragma unroll
-        for (int i = 0; i < 4; i++) b = max(b, quad_key(c[i], h[i], q + i * stride));
-    }
-    for (; q < nq; q += stride) b = max(b, quad_key(__ldcg(c4 + q), __ldcg(h4 + q), q));
-    for (uint64_t v = (nq << 2) + t; v < n; v += stride)
-        if (!__ldcg(chosen + v)) b = max(b, greedy_key(__ldcg(counts + v), (uint32_t)v));
-    return b;
-}
-
 __global__ void argmax_kernel(const int* __restrict__ counts, const uint8_t* __restrict__ chosen,
                               uint64_t n, unsigned long long* __restrict__ best) {
     unsigned long long b = slice_argmax(counts, chosen, n,
@@ -339,6 +295,8 @@ constexpr int CG_THREADS = 1024;
 constexpr uint32_t TILE_ITEMS = 16;     // members per thread of an index tile
 constexpr uint32_t CAND_BITS = 1u << 17;  // bits of the filter in front of the table
 constexpr uint32_t CAND_PREFIX = 512;   // candidates in play at the start
+// stores up to this many members are selected from by one block, without grid barriers
+constexpr uint64_t CAND_SOLO = 100'000;
 constexpr uint32_t CG_BLOCK = 32768;    // members of a set that one block lowers
 constexpr uint32_t CG_CHUNK = 512;      // members per chunk of a larger one
 // shared memory of a table and its filter; then the rounds' counts, decrements, list offsets
@@ -662,10 +620,15 @@ cand_rounds_kernel(CandState* st, const uint32_t* __restrict__ sets,
     }
     __syncthreads();
     unsigned long long fresh = 0;
+    const bool solo = gridDim.x == 1;  // no other block: counts are lowered in place
     auto lower = [&](uint32_t u) {
         if (u == NONE || !maybe_cand(tab, u)) return;
         const uint32_t c = find_cand(tab, u);
-        if (c != NONE) atomicAdd(&dec[c], 1u);
+        if (c == NONE) return;
+        if (solo)
+            atomicSub(&cnt[c], 1);
+        else
+            atomicAdd(&dec[c], 1u);
     };
     // add the block's decrements of candidates lo .. hi - 1 to the global ones
     auto flush = [&](uint32_t* delta, uint32_t lo, uint32_t hi) {
@@ -709,13 +672,15 @@ cand_rounds_kernel(CandState* st, const uint32_t* __restrict__ sets,
         }
         // the same in every block. No candidate out of play exceeds the largest count of the
         // next one's bin; when the best does not, bring more into play
-        if (np < nc && (uint32_t)(b >> 32) < bin_floor(count_bin((uint32_t)cnt[np]) + 1u)) {
+        if (np < nc && (uint32_t)(b >> 32) < bin_floor(count_bin(__ldg(&st->cnt[np])) + 1u)) {
             const uint32_t more = min(nc, 2 * np);
             uint32_t* late = st->late;
-            flush(late, np, more);
-            if (!grid_barrier(bar, err, limit)) return;
-            for (uint32_t i = np + threadIdx.x; i < more; i += CG_THREADS)
-                cnt[i] -= (int)__ldcg(late + i);
+            if (!solo) {
+                flush(late, np, more);
+                if (!grid_barrier(bar, err, limit)) return;
+                for (uint32_t i = np + threadIdx.x; i < more; i += CG_THREADS)
+                    cnt[i] -= (int)__ldcg(late + i);
+            }
             np = more;
             __syncthreads();
             continue;
@@ -742,7 +707,7 @@ cand_rounds_kernel(CandState* st, const uint32_t* __restrict__ sets,
                     reinterpret_cast<uint32_t*>(rec + s)[3] = 1u;
                     covered[s] = 1;
                     fresh++;
-                    if (len > CG_BLOCK) {
+                    if (len > CG_BLOCK && !solo) {
                         const uint32_t n = (len + CG_CHUNK - 1) / CG_CHUNK;
                         const unsigned long long base =
                             atomicAdd(nchunk + r, (unsigned long long)n);
@@ -757,7 +722,7 @@ cand_rounds_kernel(CandState* st, const uint32_t* __restrict__ sets,
                     }
                 }
             }
-            // at most CG_THREADS x CG_BLOCK = 2^25 members
+            // at most CG_THREADS x CG_BLOCK = 2^25 members (solo: CAND_SOLO)
             const unsigned long long v = len ? (1ull << 32) | len : 0ull;
             unsigned long long inc = v;
 #pragma unroll
@@ -817,6 +782,13 @@ cand_rounds_kernel(CandState* st, const uint32_t* __restrict__ sets,
                 for (uint32_t q = 0; q < 4; q++) lower(u[q]);
             }
             __syncthreads();
+        }
+        if (solo) {  // the tiles end with a barrier of the block
+            __syncthreads();
+            if (threadIdx.x == 0) cnt[bc] = -1;
+            __syncthreads();
+            r++;
+            continue;
         }
         flush(delta, 0, np);
         if (!grid_barrier(bar, err, limit)) return;
@@ -1058,7 +1030,10 @@ int tim_greedy(tim_ctx* ctx, int k, int32_t* host_seeds, uint64_t* covered) {
     const uint64_t tiles = members / ((uint64_t)CG_THREADS * TILE_ITEMS) + 1;
     const unsigned GN = (unsigned)std::min<uint64_t>(n / 1024 + 1, (uint64_t)ctx->num_sms * 4);
     const unsigned GT = (unsigned)std::min<uint64_t>(tiles, (uint64_t)ctx->num_sms);
-    const unsigned GR = (unsigned)std::min<uint64_t>(members / 8192 + 1, (uint64_t)ctx->num_sms);
+    const unsigned GR =
+        members <= CAND_SOLO
+            ? 1u
+            : (unsigned)std::min<uint64_t>(members / 8192 + 1, (uint64_t)ctx->num_sms);
     TIM_TRY(tim_ensure(ctx, ctx->set_rec, (ctx->n_sets + 1) * sizeof(uint4)));
     if (ctx->n_sets) {
         set_rec_kernel<<<(unsigned)std::min<uint64_t>(ctx->n_sets / 256 + 1,
