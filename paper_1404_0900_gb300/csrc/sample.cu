@@ -811,15 +811,21 @@ __global__ void __launch_bounds__(WARPS * 32, TIER == 1 || MODEL == TIM_IC ? 4 :
 //
 // An LT RR set is a chain (Section 4.2: each node keeps at most one live in-edge), so
 // its walk has no parallelism of its own: every thread walks one chain. The members go
-// to the thread's column of a global array (member k at k * lanes + thread, so a warp's
-// stores are contiguous); a 1024-bit Bloom filter per thread in shared memory screens
-// the revisit test, which scans the column only on a filter hit. Chains longer than
-// LT_CAP go to tier 2 (list1). Idle lanes claim sets together (one atomic per warp) at
-// the top of every step, and finished lanes reserve store space together, so a warp
-// keeps all 32 chains moving.
+// to the thread's column of a global array (contiguous per thread: a warp that reads one
+// column, to test a revisit or to store the set, reads whole sectors); a 1024-bit Bloom
+// filter per thread in shared memory screens the revisit test, which scans the column only
+// on a filter hit. Chains longer than LT_CAP go to tier 2 (list1). Finished lanes wait until
+// LT_BATCH of them (or the whole warp) are idle; then they store their sets and claim new
+// ones together: in chains of some forty steps nearly every step of a warp ends one, and the
+// claim, the store and the filter's clearing took several times the step's own work.
+// (58.8M members of R-MAT 20, 1/indeg weights: handled as each chain ended, columns
+// interleaved by lane, 4.4 ms with the reads that follow; here 1.9 ms; LT_BATCH 1, 4, 8, 12, 16:
+// 2.4, 1.9, 1.9, 2.0, 2.1.)
 constexpr int LT_THREADS = 128;
 constexpr int LT_CAP = 1024;                 // members per chain in this pass
 constexpr int LT_BLOOM_WORDS = 32;           // 1024 bits per thread
+constexpr int LT_BATCH = 8;                  // idle lanes of a warp handled together
+enum : int { LT_IDLE = 0, LT_WALK = 1, LT_DONE = 2, LT_NONE = 3 };  // a lane's chain
 constexpr size_t LT_SMEM = (size_t)LT_BLOOM_WORDS * LT_THREADS * sizeof(uint32_t);
 
 __device__ __forceinline__ void lt_bloom_bits(uint32_t u, uint32_t& w1, uint32_t& m1, uint32_t& w2,
@@ -845,18 +851,19 @@ __device__ __forceinline__ bool lane_bloom_test(const uint32_t* bloom, uint32_t 
     return (bloom[w1 * LT_THREADS] & m1) && (bloom[w2 * LT_THREADS] & m2);
 }
 
-// Revisit test of the lanes with hit set: does lane l's column (the warp's columns
-// start at wcol; member k of lane l at wcol[k * lanes + l]) hold u among its first len
-// members? All lanes scan each such column together. Warp-collective.
-__device__ __forceinline__ bool lane_cols_contain(const uint32_t* wcol, uint64_t lanes, int lane,
-                                                  bool hit, uint32_t u, int len) {
+// Revisit test of the lanes with hit set: does lane l's column (wcol + l LT_CAP) hold u among
+// its first len members? All lanes scan each such column together. Warp-collective.
+__device__ __forceinline__ bool lane_cols_contain(const uint32_t* wcol, int lane, bool hit,
+                                                  uint32_t u, int len) {
     bool seen = false;
-    for (unsigned hm = __ballot_sync(0xffffffffu, hit); hm; hm &= hm - 1) {
+    const unsigned hits = __ballot_sync(0xffffffffu, hit);
+    if (hits) __syncwarp();
+    for (unsigned hm = hits; hm; hm &= hm - 1) {
         const int l = __ffs(hm) - 1;
         const uint32_t ul = __shfl_sync(0xffffffffu, u, l);
         const int ll = __shfl_sync(0xffffffffu, len, l);
         bool f = false;
-        for (int k = lane; k < ll; k += 32) f |= wcol[(uint64_t)k * lanes + l] == ul;
+        for (int k = lane; k < ll; k += 32) f |= wcol[l * LT_CAP + k] == ul;
         f = __any_sync(0xffffffffu, f);
         if (lane == l) seen = f;
     }
@@ -868,32 +875,91 @@ __global__ void __launch_bounds__(LT_THREADS) rr_lt_lane_kernel(SampleArgs a) {
     const int tid = threadIdx.x, lane = tid & 31;
     uint32_t* bloom = bloom_all + tid;  // word w at bloom[w * LT_THREADS]
     for (int w = 0; w < LT_BLOOM_WORDS; w++) bloom[w * LT_THREADS] = 0u;
-    const uint64_t lanes = (uint64_t)gridDim.x * LT_THREADS;
-    // member k of lane l of this warp's columns: wcol[k * lanes + l]
-    uint32_t* wcol = a.lt_col + (uint64_t)blockIdx.x * LT_THREADS + (tid & ~31);
-    uint32_t* col = wcol + lane;
+    // member k of lane l of this warp's columns: wcol[l * LT_CAP + k]
+    uint32_t* wcol = a.lt_col + ((uint64_t)blockIdx.x * LT_THREADS + (tid & ~31)) * LT_CAP;
+    uint32_t* col = wcol + lane * LT_CAP;
     const bool emit = a.flags & SAMPLE_EMIT, kap = a.flags & SAMPLE_KAPPA,
                cover = a.flags & SAMPLE_COVER;
     unsigned long long k_lo = 0, k_hi = 0, wsum = 0, cov = 0, live = 0, memb = 0;
-    bool has = false, exhausted = false;
+    int state = LT_IDLE;
     uint64_t j = 0, sid = 0;
     uint32_t v = 0;
-    int len = 0, status = 0;
-    unsigned long long width = 0;
+    int len = 0;
+    bool covered = false, ovf = false;
+    uint32_t width = 0;  // a chain's nodes are distinct: below m < 2^32
     // bounded: every step either advances a chain (at most LT_CAP steps each) or
     // finishes it, and the lanes take at most count sets between them
     const uint64_t steps = (a.count + 1) * (uint64_t)(LT_CAP + 2) + 64;
     for (uint64_t guard = 0; guard < steps; guard++) {
-        // idle lanes claim the next sets, one atomic for the warp
-        const bool need = !has && !exhausted;
-        const unsigned nm = __ballot_sync(0xffffffffu, need);
-        if (nm) {
-            const int leader = __ffs(nm) - 1;
+        const unsigned idle = __ballot_sync(0xffffffffu, state == LT_IDLE || state == LT_DONE);
+        const unsigned walk = __ballot_sync(0xffffffffu, state == LT_WALK);
+        if (__popc(idle) >= LT_BATCH || (idle && !walk)) {
+            const bool fin = state == LT_DONE;
+            if (fin && ovf) {
+                const unsigned idx = atomicAdd(&a.ds->cnt1, 1u);
+                if (idx < a.list_cap)
+                    a.list1[idx] = (uint32_t)j;
+                else
+                    atomicOr(&a.ds->err, TIM_DEV_ERR_OVF_LIST);
+            } else if (fin) {
+                wsum += width;
+                memb += len;
+                if (covered) cov++;
+                if (kap) {
+                    const unsigned long long kf = kappa_fixed(kappa_fp64(width, a.m, a.k));
+                    k_lo += kf;
+                    if (k_lo < kf) k_hi++;
+                }
+            }
+            // finished chains reserve their store space together and the warp copies each
+            // one's column with all its lanes
+            const bool put = emit && fin && !ovf;
+            const unsigned pm = __ballot_sync(0xffffffffu, put);
+            if (pm) {
+                unsigned incl = put ? (unsigned)len : 0u;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const unsigned y = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += y;
+                }
+                const unsigned total = __shfl_sync(0xffffffffu, incl, 31);
+                unsigned long long base = 0;
+                if (lane == 0) base = atomicAdd(&a.ds->pool_used, (unsigned long long)total);
+                base = __shfl_sync(0xffffffffu, base, 0);
+                const unsigned first = incl - (put ? (unsigned)len : 0u);
+                const bool fits = base + total <= a.pool_cap;
+                if (put) {
+                    if (fits) {
+                        a.set_start[j] = base + first;
+                        a.set_len[j] = (uint32_t)len;
+                        a.set_width[j] = width;
+                    } else {
+                        atomicOr(&a.ds->err, TIM_DEV_ERR_POOL);
+                    }
+                }
+                __syncwarp();
+                for (unsigned m = fits ? pm : 0u; m; m &= m - 1) {
+                    const int l = __ffs(m) - 1;
+                    const unsigned long long sl = base + __shfl_sync(0xffffffffu, first, l);
+                    const int ll = __shfl_sync(0xffffffffu, len, l);
+                    const uint32_t jl = (uint32_t)__shfl_sync(0xffffffffu, j, l);
+                    for (int k = lane; k < ll; k += 32) {
+                        a.pool[sl + k] = wcol[l * LT_CAP + k];
+                        a.pool_sid[sl + k] = jl;
+                    }
+                }
+                __syncwarp();
+            }
+            if (fin)
+                for (int w = 0; w < LT_BLOOM_WORDS; w++) bloom[w * LT_THREADS] = 0u;
+            // the idle lanes claim the next sets, one atomic for the warp
+            const int leader = __ffs(idle) - 1;
             unsigned long long base = 0;
-            if (lane == leader) base = atomicAdd(&a.ds->next_set, (unsigned long long)__popc(nm));
+            if (lane == leader) base = atomicAdd(&a.ds->next_set, (unsigned long long)__popc(idle));
             base = __shfl_sync(0xffffffffu, base, leader);
-            if (need) {
-                const unsigned long long mine = base + __popc(nm & ((1u << lane) - 1u));
+            if ((idle >> lane) & 1u) {
+                const unsigned long long mine = base + __popc(idle & ((1u << lane) - 1u));
+                state = LT_NONE;
                 if (mine < a.count) {
                     j = mine;
                     sid = sid_of(a.ids, j);
@@ -901,29 +967,28 @@ __global__ void __launch_bounds__(LT_THREADS) rr_lt_lane_kernel(SampleArgs a) {
                     col[0] = v;
                     len = 1;
                     width = 0;
-                    uint32_t w1, m1, w2, m2;
-                    lt_bloom_bits(v, w1, m1, w2, m2);
-                    bloom[w1 * LT_THREADS] |= m1;
-                    bloom[w2 * LT_THREADS] |= m2;
-                    status = (cover && marked(a.seed_mark, v)) ? ST_COVERED : 0;
-                    has = true;
-                } else {
-                    exhausted = true;
+                    ovf = false;
+                    lane_bloom_add(bloom, v);
+                    covered = cover && marked(a.seed_mark, v);
+                    state = LT_WALK;
                 }
             }
         }
-        if (!__any_sync(0xffffffffu, has)) break;
+        if (!__any_sync(0xffffffffu, state == LT_WALK)) {
+            if (__any_sync(0xffffffffu, state == LT_DONE)) continue;
+            break;
+        }
         // one step of every lane's chain: the next member u, if any
-        bool fin = false, cand = false;
+        bool cand = false;
         uint32_t u = 0;
-        if (has) {
-            if (status) {
-                fin = true;
+        if (state == LT_WALK) {
+            if (covered) {
+                state = LT_DONE;
             } else {
                 const uint4 rec = __ldg(a.node + v);
                 const uint64_t beg = rec.x, end = rec.y;
                 const unsigned long long nt = node_nt(rec);
-                width += end - beg;
+                width += rec.y - rec.x;
                 uint64_t jj = end;
                 if (beg < end) {
                     const uint32_t x =
@@ -932,7 +997,7 @@ __global__ void __launch_bounds__(LT_THREADS) rr_lt_lane_kernel(SampleArgs a) {
                                     : lane_lt_search(a.thr, beg, end, x);
                 }
                 if (jj >= end) {
-                    fin = true;
+                    state = LT_DONE;
                 } else {
                     u = __ldg(a.src + jj);
                     live++;
@@ -941,95 +1006,21 @@ __global__ void __launch_bounds__(LT_THREADS) rr_lt_lane_kernel(SampleArgs a) {
             }
         }
         // revisit test: the filter first; on a hit the whole warp scans that column
-        uint32_t w1 = 0, m1 = 0, w2 = 0, m2 = 0;
-        bool hit = false;
-        if (cand) {
-            lt_bloom_bits(u, w1, m1, w2, m2);
-            hit = (bloom[w1 * LT_THREADS] & m1) && (bloom[w2 * LT_THREADS] & m2);
-        }
-        bool seen = false;
-        for (unsigned hm = __ballot_sync(0xffffffffu, hit); hm; hm &= hm - 1) {
-            const int l = __ffs(hm) - 1;
-            const uint32_t ul = __shfl_sync(0xffffffffu, u, l);
-            const int ll = __shfl_sync(0xffffffffu, len, l);
-            bool f = false;
-            for (int k = lane; k < ll; k += 32) f |= wcol[(uint64_t)k * lanes + l] == ul;
-            f = __any_sync(0xffffffffu, f);
-            if (lane == l) seen = f;
-        }
-        bool ovf = false;
+        const bool seen =
+            lane_cols_contain(wcol, lane, cand && lane_bloom_test(bloom, u), u, len);
         if (cand) {
             if (seen) {
-                fin = true;
+                state = LT_DONE;
             } else if (len == LT_CAP) {
-                fin = ovf = true;
+                state = LT_DONE;
+                ovf = true;
             } else {
-                col[(uint64_t)len * lanes] = u;
+                col[len] = u;
                 len++;
-                bloom[w1 * LT_THREADS] |= m1;
-                bloom[w2 * LT_THREADS] |= m2;
-                if (cover && marked(a.seed_mark, u)) status |= ST_COVERED;
+                lane_bloom_add(bloom, u);
+                covered = cover && marked(a.seed_mark, u);
                 v = u;
             }
-        }
-        if (fin && ovf) {
-            const unsigned idx = atomicAdd(&a.ds->cnt1, 1u);
-            if (idx < a.list_cap)
-                a.list1[idx] = (uint32_t)j;
-            else
-                atomicOr(&a.ds->err, TIM_DEV_ERR_OVF_LIST);
-        } else if (fin) {
-            wsum += width;
-            memb += len;
-            if (status & ST_COVERED) cov++;
-            if (kap) {
-                const unsigned long long kf = kappa_fixed(kappa_fp64(width, a.m, a.k));
-                k_lo += kf;
-                if (k_lo < kf) k_hi++;
-            }
-        }
-        // finished chains reserve their store space together and the warp copies each
-        // one's column with all its lanes
-        const bool put = emit && fin && !ovf;
-        const unsigned pm = __ballot_sync(0xffffffffu, put);
-        if (pm) {
-            unsigned incl = put ? (unsigned)len : 0u;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned y = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += y;
-            }
-            const unsigned total = __shfl_sync(0xffffffffu, incl, 31);
-            unsigned long long base = 0;
-            if (lane == 0) base = atomicAdd(&a.ds->pool_used, (unsigned long long)total);
-            base = __shfl_sync(0xffffffffu, base, 0);
-            const unsigned long long st = base + incl - (put ? (unsigned)len : 0u);
-            const bool fits = base + total <= a.pool_cap;
-            if (put) {
-                if (fits) {
-                    a.set_start[j] = st;
-                    a.set_len[j] = (uint32_t)len;
-                    a.set_width[j] = width;
-                } else {
-                    atomicOr(&a.ds->err, TIM_DEV_ERR_POOL);
-                }
-            }
-            if (fits) {
-                for (unsigned m = pm; m; m &= m - 1) {
-                    const int l = __ffs(m) - 1;
-                    const unsigned long long sl = __shfl_sync(0xffffffffu, st, l);
-                    const int ll = __shfl_sync(0xffffffffu, len, l);
-                    const uint32_t jl = (uint32_t)__shfl_sync(0xffffffffu, j, l);
-                    for (int k = lane; k < ll; k += 32) {
-                        a.pool[sl + k] = wcol[(uint64_t)k * lanes + l];
-                        a.pool_sid[sl + k] = jl;
-                    }
-                }
-            }
-        }
-        if (fin) {
-            for (int w = 0; w < LT_BLOOM_WORDS; w++) bloom[w * LT_THREADS] = 0u;
-            has = false;
         }
     }
     live = warp_sum_u64(live);
@@ -1680,31 +1671,97 @@ rr_lt_lane_multi_kernel(MultiArgs ma, const unsigned long long* lt_prefix,
     for (int w = 0; w < LT_BLOOM_WORDS; w++) bloom[w * LT_THREADS] = 0u;
     __syncthreads();
     const uint64_t total = s_prefix[ma.nq];
-    const uint64_t lanes = (uint64_t)gridDim.x * LT_THREADS;
-    uint32_t* wcol = lt_col + (uint64_t)blockIdx.x * LT_THREADS + (tid & ~31);
-    uint32_t* col = wcol + lane;
+    uint32_t* wcol = lt_col + ((uint64_t)blockIdx.x * LT_THREADS + (tid & ~31)) * LT_CAP;
+    uint32_t* col = wcol + lane * LT_CAP;
     QAcc acc{0, 0, 0, 0, 0, 0, 0};
     int cur_q = -1;
-    bool has = false, exhausted = false;
-    int qi = -1, flags = 0, kk = 0, len = 0, status = 0;
+    auto flush = [&]() {
+        if (cur_q < 0) return;
+        DevScalars* ds = ma.q[cur_q].ds;
+        if (acc.k_lo || acc.k_hi)
+            atomic_add_u128(&ds->ksum_lo, &ds->ksum_hi, acc.k_lo, acc.k_hi);
+        if (acc.wsum) {
+            atomicAdd(&ds->wsum, acc.wsum);
+            atomicAdd(&ds->width[0], acc.wsum);
+        }
+        if (acc.cov) atomicAdd(&ds->covered, acc.cov);
+        if (acc.live) atomicAdd(&ds->live[0], acc.live);
+        if (acc.memb) atomicAdd(&ds->memb[0], acc.memb);
+        acc = QAcc{0, 0, 0, 0, 0, 0, 0};
+    };
+    int state = LT_IDLE;
+    int flags = 0, kk = 0, len = 0;
+    bool covered = false, ovf = false;
     uint64_t j = 0, sid = 0, n = 0, m = 0;
     const uint4* node = nullptr;
     const uint32_t* src = nullptr;
     const uint32_t* thr = nullptr;
     const uint32_t* seed_mark = nullptr;
-    uint32_t v = 0;
-    unsigned long long width = 0;
+    uint32_t v = 0, width = 0;
     const uint64_t steps = (total + 1) * (uint64_t)(LT_CAP + 2) + 64;
     for (uint64_t guard = 0; guard < steps; guard++) {
-        const bool need = !has && !exhausted;
-        const unsigned nm = __ballot_sync(0xffffffffu, need);
-        if (nm) {
-            const int leader = __ffs(nm) - 1;
+        const unsigned idle = __ballot_sync(0xffffffffu, state == LT_IDLE || state == LT_DONE);
+        const unsigned walk = __ballot_sync(0xffffffffu, state == LT_WALK);
+        if (__popc(idle) >= LT_BATCH || (idle && !walk)) {
+            bool put = false;
+            unsigned long long st = 0;
+            uint32_t* pool = nullptr;
+            uint32_t* pool_sid = nullptr;
+            if (state == LT_DONE && ovf) {
+                const unsigned idx = atomicAdd(&ma.cnt[0], 1u);
+                if (idx < ma.list_cap)
+                    ma.list1[idx] = make_uint2((uint32_t)cur_q, (uint32_t)j);
+                else
+                    atomicOr(ma.err, TIM_DEV_ERR_OVF_LIST);
+            } else if (state == LT_DONE) {
+                acc.wsum += width;
+                acc.memb += len;
+                if (covered) acc.cov++;
+                if (flags & SAMPLE_KAPPA) {
+                    const unsigned long long kf = kappa_fixed(kappa_fp64(width, m, kk));
+                    acc.k_lo += kf;
+                    if (acc.k_lo < kf) acc.k_hi++;
+                }
+                if (flags & SAMPLE_EMIT) {
+                    const QueryDesc& d = ma.q[cur_q];
+                    st = atomicAdd(&d.ds->pool_used, (unsigned long long)len);
+                    if (st + (unsigned)len <= d.pool_cap) {
+                        put = true;
+                        pool = d.pool;
+                        pool_sid = d.pool_sid;
+                        d.set_start[j] = st;
+                        d.set_len[j] = (uint32_t)len;
+                        d.set_width[j] = width;
+                    } else {
+                        atomicOr(&d.ds->err, TIM_DEV_ERR_POOL);
+                    }
+                }
+            }
+            // the warp copies each stored chain's column with all its lanes
+            __syncwarp();
+            for (unsigned pm = __ballot_sync(0xffffffffu, put); pm; pm &= pm - 1) {
+                const int l = __ffs(pm) - 1;
+                const unsigned long long sl = __shfl_sync(0xffffffffu, st, l);
+                const int ll = __shfl_sync(0xffffffffu, len, l);
+                const uint32_t jl = (uint32_t)__shfl_sync(0xffffffffu, (unsigned long long)j, l);
+                uint32_t* pl = (uint32_t*)__shfl_sync(0xffffffffu, (unsigned long long)pool, l);
+                uint32_t* psl = (uint32_t*)__shfl_sync(0xffffffffu, (unsigned long long)pool_sid, l);
+                for (int k = lane; k < ll; k += 32) {
+                    pl[sl + k] = wcol[l * LT_CAP + k];
+                    psl[sl + k] = jl;
+                }
+            }
+            __syncwarp();
+            if (state == LT_DONE)
+                for (int w = 0; w < LT_BLOOM_WORDS; w++) bloom[w * LT_THREADS] = 0u;
+            // the idle lanes claim the next sets, one atomic for the warp
+            const int leader = __ffs(idle) - 1;
             unsigned long long base = 0;
-            if (lane == leader) base = atomicAdd(lt_next, (unsigned long long)__popc(nm));
+            if (lane == leader) base = atomicAdd(lt_next, (unsigned long long)__popc(idle));
             base = __shfl_sync(0xffffffffu, base, leader);
-            if (need) {
-                const unsigned long long mine = base + __popc(nm & ((1u << lane) - 1u));
+            if ((idle >> lane) & 1u) {
+                const unsigned long long mine = base + __popc(idle & ((1u << lane) - 1u));
+                state = LT_NONE;
                 if (mine < total) {
                     int lo = 0, hi = ma.nq;  // s_prefix[lo] <= mine < s_prefix[hi]
                     while (hi - lo > 1) {
@@ -1715,19 +1772,7 @@ rr_lt_lane_multi_kernel(MultiArgs ma, const unsigned long long* lt_prefix,
                             hi = mid;
                     }
                     if (lo != cur_q) {
-                        if (cur_q >= 0) {
-                            DevScalars* ds = ma.q[cur_q].ds;
-                            if (acc.k_lo || acc.k_hi)
-                                atomic_add_u128(&ds->ksum_lo, &ds->ksum_hi, acc.k_lo, acc.k_hi);
-                            if (acc.wsum) {
-                                atomicAdd(&ds->wsum, acc.wsum);
-                                atomicAdd(&ds->width[0], acc.wsum);
-                            }
-                            if (acc.cov) atomicAdd(&ds->covered, acc.cov);
-                            if (acc.live) atomicAdd(&ds->live[0], acc.live);
-                            if (acc.memb) atomicAdd(&ds->memb[0], acc.memb);
-                        }
-                        acc = QAcc{0, 0, 0, 0, 0, 0, 0};
+                        flush();
                         cur_q = lo;
                         const QueryDesc& d = ma.q[lo];
                         node = d.node;
@@ -1739,32 +1784,33 @@ rr_lt_lane_multi_kernel(MultiArgs ma, const unsigned long long* lt_prefix,
                         flags = d.flags;
                         kk = d.k;
                     }
-                    qi = lo;
                     j = mine - s_prefix[lo];
                     sid = ma.q[lo].sid0 + j;
                     v = rr_root(sid, n, ma.K);
                     col[0] = v;
                     len = 1;
                     width = 0;
+                    ovf = false;
                     lane_bloom_add(bloom, v);
-                    status = ((flags & SAMPLE_COVER) && marked(seed_mark, v)) ? ST_COVERED : 0;
-                    has = true;
-                } else {
-                    exhausted = true;
+                    covered = (flags & SAMPLE_COVER) && marked(seed_mark, v);
+                    state = LT_WALK;
                 }
             }
         }
-        if (!__any_sync(0xffffffffu, has)) break;
-        bool fin = false, cand = false;
+        if (!__any_sync(0xffffffffu, state == LT_WALK)) {
+            if (__any_sync(0xffffffffu, state == LT_DONE)) continue;
+            break;
+        }
+        bool cand = false;
         uint32_t u = 0;
-        if (has) {
-            if (status) {
-                fin = true;
+        if (state == LT_WALK) {
+            if (covered) {
+                state = LT_DONE;
             } else {
                 const uint4 rec = __ldg(node + v);
                 const uint64_t beg = rec.x, end = rec.y;
                 const unsigned long long nt = node_nt(rec);
-                width += end - beg;
+                width += rec.y - rec.x;
                 uint64_t jj = end;
                 if (beg < end) {
                     const uint32_t x =
@@ -1773,7 +1819,7 @@ rr_lt_lane_multi_kernel(MultiArgs ma, const unsigned long long* lt_prefix,
                                     : lane_lt_search(thr, beg, end, x);
                 }
                 if (jj >= end) {
-                    fin = true;
+                    state = LT_DONE;
                 } else {
                     u = __ldg(src + jj);
                     acc.live++;
@@ -1782,84 +1828,23 @@ rr_lt_lane_multi_kernel(MultiArgs ma, const unsigned long long* lt_prefix,
             }
         }
         const bool seen =
-            lane_cols_contain(wcol, lanes, lane, cand && lane_bloom_test(bloom, u), u, len);
-        bool ovf = false;
+            lane_cols_contain(wcol, lane, cand && lane_bloom_test(bloom, u), u, len);
         if (cand) {
             if (seen) {
-                fin = true;
+                state = LT_DONE;
             } else if (len == LT_CAP) {
-                fin = ovf = true;
+                state = LT_DONE;
+                ovf = true;
             } else {
-                col[(uint64_t)len * lanes] = u;
+                col[len] = u;
                 len++;
                 lane_bloom_add(bloom, u);
-                if ((flags & SAMPLE_COVER) && marked(seed_mark, u)) status |= ST_COVERED;
+                covered = (flags & SAMPLE_COVER) && marked(seed_mark, u);
                 v = u;
             }
         }
-        bool put = false;
-        unsigned long long st = 0;
-        uint32_t* pool = nullptr;
-        uint32_t* pool_sid = nullptr;
-        if (fin && ovf) {
-            const unsigned idx = atomicAdd(&ma.cnt[0], 1u);
-            if (idx < ma.list_cap)
-                ma.list1[idx] = make_uint2((uint32_t)qi, (uint32_t)j);
-            else
-                atomicOr(ma.err, TIM_DEV_ERR_OVF_LIST);
-        } else if (fin) {
-            acc.wsum += width;
-            acc.memb += len;
-            if (status & ST_COVERED) acc.cov++;
-            if (flags & SAMPLE_KAPPA) {
-                const unsigned long long kf = kappa_fixed(kappa_fp64(width, m, kk));
-                acc.k_lo += kf;
-                if (acc.k_lo < kf) acc.k_hi++;
-            }
-            if (flags & SAMPLE_EMIT) {
-                const QueryDesc& d = ma.q[qi];
-                st = atomicAdd(&d.ds->pool_used, (unsigned long long)len);
-                if (st + (unsigned)len <= d.pool_cap) {
-                    put = true;
-                    pool = d.pool;
-                    pool_sid = d.pool_sid;
-                    d.set_start[j] = st;
-                    d.set_len[j] = (uint32_t)len;
-                    d.set_width[j] = width;
-                } else {
-                    atomicOr(&d.ds->err, TIM_DEV_ERR_POOL);
-                }
-            }
-        }
-        // the warp copies each stored chain's column with all its lanes
-        for (unsigned pm = __ballot_sync(0xffffffffu, put); pm; pm &= pm - 1) {
-            const int l = __ffs(pm) - 1;
-            const unsigned long long sl = __shfl_sync(0xffffffffu, st, l);
-            const int ll = __shfl_sync(0xffffffffu, len, l);
-            const uint32_t jl = (uint32_t)__shfl_sync(0xffffffffu, (unsigned long long)j, l);
-            uint32_t* pl = (uint32_t*)__shfl_sync(0xffffffffu, (unsigned long long)pool, l);
-            uint32_t* psl = (uint32_t*)__shfl_sync(0xffffffffu, (unsigned long long)pool_sid, l);
-            for (int k = lane; k < ll; k += 32) {
-                pl[sl + k] = wcol[(uint64_t)k * lanes + l];
-                psl[sl + k] = jl;
-            }
-        }
-        if (fin) {
-            for (int w = 0; w < LT_BLOOM_WORDS; w++) bloom[w * LT_THREADS] = 0u;
-            has = false;
-        }
     }
-    if (cur_q >= 0) {
-        DevScalars* ds = ma.q[cur_q].ds;
-        if (acc.k_lo || acc.k_hi) atomic_add_u128(&ds->ksum_lo, &ds->ksum_hi, acc.k_lo, acc.k_hi);
-        if (acc.wsum) {
-            atomicAdd(&ds->wsum, acc.wsum);
-            atomicAdd(&ds->width[0], acc.wsum);
-        }
-        if (acc.cov) atomicAdd(&ds->covered, acc.cov);
-        if (acc.live) atomicAdd(&ds->live[0], acc.live);
-        if (acc.memb) atomicAdd(&ds->memb[0], acc.memb);
-    }
+    flush();
 }
 
 int launch_multi(tim_ctx* owner, const MultiArgs& ma, int tier, int T, unsigned grid,
