@@ -21,7 +21,7 @@
 //   member takes a tail atomic) and no edge budget, run by teams of T warps per set: T = 1 when the
 //   listed sets are many (parallelism across sets fills the GPU), up to 8 when they are
 //   few (the team splits each in-list, so one heavy set does not leave the GPU idle).
-// In-lists of at least BIG_GROUPS groups (hubs) are streamed by the whole team one at
+// In-lists of at least 512 edges (hubs) that take their own coins are streamed by the whole team one at
 // a time with two groups in flight per lane; the rest of a frontier is flattened.
 // Tier 3: sets beyond tier 2's queue: IC goes to the batched level-synchronous pass of
 //   sample_bulk.cu; LT (a chain) is walked by one warp per set with a visited bitmap; a
@@ -51,9 +51,12 @@ constexpr int BIG_THREADS = 256;  // tier 3 LT CTA size
 // 41.6M nodes - 225.9 224.0 220.3 220.1 229.6 247.3.
 constexpr unsigned long long LONG_BUDGET2 = 6144;
 
-// Queue capacity Q and hash size 2^LOG2H (>= 2Q) of one warp's set.
-template <int QQ, int LG>
+// Queue capacity Q and hash size 2^LOG2H (>= 2Q) of one warp's set. With BM the visited set is
+// a bitmap (bit 0: a member) instead of the hash, in the hash's place or in shared memory; like
+// the hash it holds only EMPTY words between sets.
+template <int QQ, int LG, bool BM = false>
 struct Cap {
+    static constexpr bool BITMAP = BM;
     static constexpr int Q = QQ;
     static constexpr int LOG2H = LG;
     static constexpr int H = 1 << LG;
@@ -65,6 +68,19 @@ using Tier1 = Cap<256, 9>;
 using Tier1S = Cap<128, 8>;
 using Tier1L = Cap<512, 10>;
 using Tier2 = Cap<8192, 14>;
+// Second pass of IC, triggering and batched queries on graphs whose bitmap is no larger than the
+// hash: one atomic tells whether a node is new, nothing is probed, and a bitmap of n / 8 bytes per
+// team stays in L2 where 64 KB per team do not. (Triggering sets of R-MAT 13, 15, 16, 17, 60,001 of
+// them: 5.6, 15.9, 28.6, 91.6 ms with the hash, 2.5, 7.1, 13.0, 79.5 ms with the bitmap; weighted
+// cascade queries on R-MAT 14 to 18 2-3 % faster.)
+using Tier2B = Cap<8192, 14, true>;
+constexpr uint32_t BITMAP_GLOBAL = Tier2::H;  // words
+// The bitmaps go to shared memory where they leave the blocks resident (the first figure), and
+// with teams of a whole block, that is for few sets, up to what a block may have: there also on
+// graphs past the line above. (Queries: R-MAT 14 1.63 -> 1.57 ms, R-MAT 20 weighted cascade
+// 12.88 -> 12.65 ms. Triggering with 36 KB a block, R-MAT 15, loses: 7.1 -> 11.7 ms, four blocks
+// per SM instead of six.)
+constexpr size_t BITMAP_SMEM = 16 * 1024, BITMAP_SMEM_FEW = 200 * 1024;
 
 struct SampleArgs {
     const uint4* node;  // node records
@@ -88,6 +104,8 @@ struct SampleArgs {
     uint32_t* list2;   // tier 2 -> tier 3
     uint32_t list_cap;
     uint32_t* arena;   // tier 2 per-warp storage
+    uint32_t bm_words;   // tier 2 with bitmaps: words of each
+    uint32_t bm_shared;  // they are in shared memory (otherwise in the hash regions)
     uint32_t* big_bitmap;  // tier 3 LT
     uint32_t* big_queue;
     uint64_t big_words;
@@ -134,6 +152,17 @@ constexpr int INS_OLD = 0, INS_NEW = 1, INS_FULL = 2;
 template <class C>
 __device__ __forceinline__ int set_insert(uint32_t* hash, uint32_t* queue, uint16_t* slot,
                                           int* ctl, uint32_t u) {
+    if constexpr (C::BITMAP) {
+        const uint32_t bit = 1u << (u & 31);
+        if (!(atomicAnd(&hash[u >> 5], ~bit) & bit)) return INS_OLD;
+        const int pos = atomicAdd(&ctl[0], 1);
+        if (pos < C::Q) {
+            queue[pos] = u;
+            return INS_NEW;
+        }
+        atomicOr(&ctl[1], ST_OVERFLOW);
+        return INS_FULL;
+    }
     uint32_t h = (u * 0x9E3779B1u) >> (32 - C::LOG2H);
     for (int probe = 0; probe < C::H; probe++) {
         uint32_t old = atomicCAS(&hash[h], EMPTY, u);
@@ -152,6 +181,42 @@ __device__ __forceinline__ int set_insert(uint32_t* hash, uint32_t* queue, uint1
     }
     atomicOr(&ctl[1], ST_OVERFLOW);
     return INS_FULL;
+}
+
+// Member queue[i] = u of a handed-over set (members are distinct): into the visited set.
+template <class C>
+__device__ __forceinline__ void set_restore(uint32_t* hash, uint16_t* slot, uint32_t i,
+                                            uint32_t u) {
+    if constexpr (C::BITMAP) {
+        atomicAnd(&hash[u >> 5], ~(1u << (u & 31)));
+    } else {
+        uint32_t h = (u * 0x9E3779B1u) >> (32 - C::LOG2H);  // the first empty slot it finds
+        for (int probe = 0; probe < C::H; probe++) {
+            if (atomicCAS(&hash[h], EMPTY, u) == EMPTY) break;
+            h = (h + 1) & (C::H - 1);
+        }
+        slot[i] = (uint16_t)h;
+    }
+}
+
+// The visited set empty again: of its members, or of everything (words: the bitmap's).
+template <class C>
+__device__ __forceinline__ void set_clear(uint32_t* hash, const uint32_t* queue,
+                                          const uint16_t* slot, int tail, int tl, int step) {
+    for (int i = tl; i < tail; i += step) {
+        if constexpr (C::BITMAP)
+            hash[queue[i] >> 5] = EMPTY;
+        else
+            hash[slot[i]] = EMPTY;
+    }
+}
+
+template <class C>
+__device__ __forceinline__ void set_clear_all(uint32_t* hash, uint32_t words, int tl, int step) {
+    if constexpr (C::BITMAP)
+        for (uint32_t i = tl; i < words; i += step) hash[i] = EMPTY;
+    else
+        for (int i = tl; i < C::H; i += step) hash[i] = EMPTY;
 }
 
 // First position j in [lo, hi) with thr[j] > x (thr non-decreasing), or hi.
@@ -224,10 +289,6 @@ struct alignas(16) WarpScratch {
     uint32_t stage[160];
 };
 
-// In-lists with at least this many 4-edge groups (512 in-edges, the skip rule's length) that
-// take their own coins are streamed one at a time, two groups in flight per lane.
-constexpr uint32_t BIG_GROUPS = TIM_SKIP_MIN_INDEG / 4;
-
 // Where an IC expansion stopped: the queue position of the frontier batch to process
 // next and the width of the members before it.
 struct Resume {
@@ -267,10 +328,14 @@ __device__ __forceinline__ int team_rr(const A& a, const PhiloxKeys& K, uint64_t
     const bool cover = a.flags & SAMPLE_COVER;
     const uint32_t root = rr_root(sid, a.n, K);
     if (!in && wt == 0 && lane == 0) {
-        uint32_t h = (root * 0x9E3779B1u) >> (32 - C::LOG2H);
-        hash[h] = root;
+        if constexpr (C::BITMAP) {
+            hash[root >> 5] = ~(1u << (root & 31));
+        } else {
+            const uint32_t h = (root * 0x9E3779B1u) >> (32 - C::LOG2H);
+            hash[h] = root;
+            slot[0] = (uint16_t)h;
+        }
         queue[0] = root;
-        slot[0] = (uint16_t)h;
         ctl[0] = 1;
         ctl[1] = (cover && marked(a.seed_mark, root)) ? ST_COVERED : 0;
     }
@@ -444,7 +509,7 @@ __device__ __forceinline__ int team_rr(const A& a, const PhiloxKeys& K, uint64_t
                 const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
                 if (lane >= o) incl += y;
             }
-            const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);  // < 32 BIG_GROUPS
+            const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);  
             const uint32_t excl = ngs ? incl - ngs : ~0u;
             const uint32_t lists = __ballot_sync(0xffffffffu, ngs != 0u);
             if (ngs)
@@ -617,16 +682,22 @@ __global__ void __launch_bounds__(WARPS * 32, TIER == 1 || MODEL == TIM_IC ? 4 :
     const int wt = wid % T, team = wid / T;
     const int tl = wt * 32 + lane;  // thread index inside the team
     uint32_t* hash;
+    uint32_t* queue;
     if (TIER == 1) {
         hash = smem + team * C::WORDS;
+        queue = hash + C::H;
         for (int i = tl; i < C::H; i += 32 * T) hash[i] = EMPTY;
     } else {
         // the arena's hash regions are all EMPTY between sets
         const uint64_t slot_id = (uint64_t)blockIdx.x * (WARPS / T) + team;
         hash = a.arena + slot_id * C::WORDS;
+        queue = hash + C::H;
+        if (C::BITMAP && a.bm_shared) {
+            hash = smem + team * a.bm_words;
+            set_clear_all<C>(hash, a.bm_words, tl, 32 * T);
+        }
     }
     team_sync<T>(team);
-    uint32_t* queue = hash + C::H;
     uint16_t* slot = reinterpret_cast<uint16_t*>(queue + C::Q);
     int* ctl = TIER == 1 ? reinterpret_cast<int*>(queue + C::Q + C::Q / 2) : s_ctl[team];
     const unsigned long long budget =
@@ -677,13 +748,7 @@ __global__ void __launch_bounds__(WARPS * 32, TIER == 1 || MODEL == TIM_IC ? 4 :
                     for (uint32_t i = tl; i < t0; i += 32 * T) {
                         const uint32_t u = hs[4 + i];
                         queue[i] = u;
-                        // the members are distinct: each takes the first empty slot it finds
-                        uint32_t h = (u * 0x9E3779B1u) >> (32 - C::LOG2H);
-                        for (int probe = 0; probe < C::H; probe++) {
-                            if (atomicCAS(&hash[h], EMPTY, u) == EMPTY) break;
-                            h = (h + 1) & (C::H - 1);
-                        }
-                        slot[i] = (uint16_t)h;
+                        set_restore<C>(hash, slot, i, u);
                         // a member in the seed set found in the batch that overflowed pass
                         // 1's queue: the set is covered (as a fresh expansion would find)
                         if ((a.flags & SAMPLE_COVER) && marked(a.seed_mark, u))
@@ -746,7 +811,7 @@ __global__ void __launch_bounds__(WARPS * 32, TIER == 1 || MODEL == TIM_IC ? 4 :
                     }
                     team_sync<T>(team);
                 }
-                for (int i = tl; i < C::H; i += 32 * T) hash[i] = EMPTY;
+                set_clear_all<C>(hash, a.bm_words, tl, 32 * T);
                 team_sync<T>(team);
                 continue;
             }
@@ -786,7 +851,7 @@ __global__ void __launch_bounds__(WARPS * 32, TIER == 1 || MODEL == TIM_IC ? 4 :
                     atomicOr(&a.ds->err, TIM_DEV_ERR_POOL);
                 }
             }
-            for (int i = tl; i < tail; i += 32 * T) hash[slot[i]] = EMPTY;
+            set_clear<C>(hash, queue, slot, tail, tl, 32 * T);
             team_sync<T>(team);
         }
     }
@@ -1353,8 +1418,46 @@ int launch_tier1(tim_ctx* ctx, const SampleArgs& a, unsigned grid, size_t smem) 
     return TIM_OK;
 }
 
-int launch_tier2(tim_ctx* ctx, const SampleArgs& a, unsigned grid, int T) {
-    if (ctx->model != TIM_IC || T == 1) {
+// Bytes of shared memory for the bitmaps of tier 2's teams of T warps (`words` words each), or 0:
+// they don't go there.
+size_t bitmap_smem(uint64_t words, int T) {
+    const size_t bytes = (size_t)(WARPS / T) * words * sizeof(uint32_t);
+    return bytes <= (T == 8 ? BITMAP_SMEM_FEW : BITMAP_SMEM) ? bytes : 0;
+}
+
+// Blocks of a tier-2 launch with bitmaps in shared memory: at most `grid` (the arena's slots).
+template <class K>
+int bitmap_grid(tim_ctx* ctx, K kernel, size_t smem, unsigned grid, unsigned* out) {
+    CUDA_TRY(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)BITMAP_SMEM_FEW));
+    int nb = 0;
+    CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, WARPS * 32, smem));
+    *out = std::min(grid, (unsigned)(ctx->num_sms * std::max(nb, 1)));
+    return TIM_OK;
+}
+
+template <class K>
+int launch_bitmap(tim_ctx* ctx, K kernel, const SampleArgs& a, unsigned grid, size_t smem) {
+    if (smem) TIM_TRY(bitmap_grid(ctx, kernel, smem, grid, &grid));
+    kernel<<<grid, WARPS * 32, smem, ctx->stream>>>(a);
+    return TIM_OK;
+}
+
+int launch_tier2(tim_ctx* ctx, SampleArgs& a, unsigned grid, int T) {
+    const size_t smem = bitmap_smem(a.bm_words, T);
+    a.bm_shared = smem > 0;
+    if (ctx->model != TIM_LT && (smem || a.bm_words <= BITMAP_GLOBAL)) {
+        if (ctx->model == TIM_TRIG)
+            TIM_TRY(launch_bitmap(ctx, rr_team_kernel<TIM_TRIG, Tier2B, 2, 1>, a, grid, smem));
+        else if (T == 1)
+            TIM_TRY(launch_bitmap(ctx, rr_team_kernel<TIM_IC, Tier2B, 2, 1>, a, grid, smem));
+        else if (T == 2)
+            TIM_TRY(launch_bitmap(ctx, rr_team_kernel<TIM_IC, Tier2B, 2, 2>, a, grid, smem));
+        else if (T == 4)
+            TIM_TRY(launch_bitmap(ctx, rr_team_kernel<TIM_IC, Tier2B, 2, 4>, a, grid, smem));
+        else
+            TIM_TRY(launch_bitmap(ctx, rr_team_kernel<TIM_IC, Tier2B, 2, 8>, a, grid, smem));
+    } else if (ctx->model != TIM_IC || T == 1) {
         if (ctx->model == TIM_IC)
             rr_team_kernel<TIM_IC, Tier2, 2, 1><<<grid, WARPS * 32, 0, ctx->stream>>>(a);
         else if (ctx->model == TIM_TRIG)
@@ -1408,6 +1511,8 @@ struct MultiArgs {
     uint2* list2;
     uint32_t list_cap;
     uint32_t* arena;
+    uint32_t bm_words;   // tier 2 with bitmaps: words of each
+    uint32_t bm_shared;  // they are in shared memory (otherwise in the hash regions)
     // IC: pass-1 state handed to pass 2 for list1 position i < hcap (as in SampleArgs)
     uint32_t* hand;
     uint32_t hcap, hw;
@@ -1464,15 +1569,21 @@ __global__ void __launch_bounds__(WARPS * 32, 4) rr_multi_kernel(MultiArgs ma) {
     for (int i = threadIdx.x; i <= ma.nq; i += blockDim.x) s_prefix[i] = ma.prefix[i];
     __syncthreads();
     uint32_t* hash;
+    uint32_t* queue;
     if (TIER == 1) {
         hash = smem + team * C::WORDS;
+        queue = hash + C::H;
         for (int i = tl; i < C::H; i += 32 * T) hash[i] = EMPTY;
     } else {
         const uint64_t slot_id = (uint64_t)blockIdx.x * (WARPS / T) + team;
         hash = ma.arena + slot_id * C::WORDS;
+        queue = hash + C::H;
+        if (C::BITMAP && ma.bm_shared) {
+            hash = smem + team * ma.bm_words;
+            set_clear_all<C>(hash, ma.bm_words, tl, 32 * T);
+        }
     }
     team_sync<T>(team);
-    uint32_t* queue = hash + C::H;
     uint16_t* slot = reinterpret_cast<uint16_t*>(queue + C::Q);
     int* ctl = TIER == 1 ? reinterpret_cast<int*>(queue + C::Q + C::Q / 2) : s_ctl[team];
     unsigned long long* counter = &ma.next[TIER - 1];
@@ -1554,12 +1665,7 @@ __global__ void __launch_bounds__(WARPS * 32, 4) rr_multi_kernel(MultiArgs ma) {
                     for (uint32_t i = tl; i < t0; i += 32 * T) {
                         const uint32_t u = hs[4 + i];
                         queue[i] = u;
-                        uint32_t h = (u * 0x9E3779B1u) >> (32 - C::LOG2H);
-                        for (int probe = 0; probe < C::H; probe++) {
-                            if (atomicCAS(&hash[h], EMPTY, u) == EMPTY) break;
-                            h = (h + 1) & (C::H - 1);
-                        }
-                        slot[i] = (uint16_t)h;
+                        set_restore<C>(hash, slot, i, u);
                         if ((d.flags & SAMPLE_COVER) && marked(d.seed_mark, u))
                             atomicOr(&ctl[1], ST_COVERED);
                     }
@@ -1605,7 +1711,7 @@ __global__ void __launch_bounds__(WARPS * 32, 4) rr_multi_kernel(MultiArgs ma) {
                         }
                     }
                 }
-                for (int i = tl; i < C::H; i += 32 * T) hash[i] = EMPTY;
+                set_clear_all<C>(hash, ma.bm_words, tl, 32 * T);
                 team_sync<T>(team);
                 continue;
             }
@@ -1647,7 +1753,7 @@ __global__ void __launch_bounds__(WARPS * 32, 4) rr_multi_kernel(MultiArgs ma) {
                     atomicOr(&d.ds->err, TIM_DEV_ERR_POOL);
                 }
             }
-            for (int i = tl; i < tail; i += 32 * T) hash[slot[i]] = EMPTY;
+            set_clear<C>(hash, queue, slot, tail, tl, 32 * T);
             team_sync<T>(team);
         }
     }
@@ -1856,6 +1962,14 @@ int launch_multi(tim_ctx* owner, const MultiArgs& ma, int tier, int T, unsigned 
             rr_multi_kernel<Tier1L, 1, 1><<<grid, WARPS * 32, smem, owner->stream>>>(ma);
         else
             rr_multi_kernel<Tier1, 1, 1><<<grid, WARPS * 32, smem, owner->stream>>>(ma);
+    } else if (ma.bm_shared || ma.bm_words <= BITMAP_GLOBAL) {
+        const size_t bytes = bitmap_smem(ma.bm_words, T);
+        auto* kernel = T == 1   ? rr_multi_kernel<Tier2B, 2, 1>
+                       : T == 2 ? rr_multi_kernel<Tier2B, 2, 2>
+                       : T == 4 ? rr_multi_kernel<Tier2B, 2, 4>
+                                : rr_multi_kernel<Tier2B, 2, 8>;
+        if (bytes) TIM_TRY(bitmap_grid(owner, kernel, bytes, grid, &grid));
+        kernel<<<grid, WARPS * 32, bytes, owner->stream>>>(ma);
     } else if (T == 1) {
         rr_multi_kernel<Tier2, 2, 1><<<grid, WARPS * 32, 0, owner->stream>>>(ma);
     } else if (T == 2) {
@@ -1967,6 +2081,7 @@ int tim_sample(tim_ctx* ctx, const SampleRequest& req, SampleResult* res) {
     a.list2 = (uint32_t*)ctx->ovf_list2.p;
     a.list_cap = list_cap;
     a.arena = (uint32_t*)ctx->arena.p;
+    a.bm_words = (uint32_t)((uint64_t)ctx->n / 32 + 1);
     a.big_bitmap = (uint32_t*)ctx->big_bitmap.p;
     a.big_queue = (uint32_t*)ctx->big_queue.p;
     a.big_words = words;
@@ -2401,6 +2516,9 @@ int tim_sample_multi(tim_ctx* owner, MultiQuery* qs, int nq, uint64_t seed) {
     ma.list2 = (uint2*)owner->ovf_list2.p;
     ma.list_cap = (uint32_t)(total + 1);
     ma.arena = (uint32_t*)owner->arena.p;
+    ma.bm_words = 1;
+    for (int i = 0; i < nq; i++)
+        ma.bm_words = std::max(ma.bm_words, (uint32_t)((uint64_t)qs[i].ctx->n / 32 + 1));
     // pass-1 state handed to pass 2 (IC queries), in the owner's scratch
     ma.hw = 4u + (uint32_t)cap1;
     {
@@ -2470,6 +2588,7 @@ int tim_sample_multi(tim_ctx* owner, MultiQuery* qs, int nq, uint64_t seed) {
                 while (T < 8 && (uint64_t)h_cnt[0] * (uint64_t)owner->team_factor < slots1 / T)
                     T *= 2;
             }
+            ma.bm_shared = bitmap_smem(ma.bm_words, T) > 0;
             TIM_TRY(launch_multi(owner, ma, 2, T, grid2, 0));
             CUDA_TRY(owner, cudaMemcpyAsync(h_cnt, d_cnt, sizeof h_cnt, cudaMemcpyDeviceToHost,
                                             owner->stream));
