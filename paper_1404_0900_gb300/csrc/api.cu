@@ -55,6 +55,7 @@ int tim_ensure(tim_ctx* ctx, DevBuf& b, size_t bytes) {
     }
     b.p = p;
     b.bytes = bytes;
+    b.made++;
     return TIM_OK;
 }
 

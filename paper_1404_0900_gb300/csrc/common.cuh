@@ -14,6 +14,7 @@
 struct DevBuf {
     void* p = nullptr;
     size_t bytes = 0;
+    uint64_t made = 0;  // allocations so far: a new one may be larger at the same address
 };
 
 // Scalars the kernels update; one block of device memory per context, mirrored in

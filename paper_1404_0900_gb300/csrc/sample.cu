@@ -2038,9 +2038,9 @@ int tim_sample(tim_ctx* ctx, const SampleRequest& req, SampleResult* res) {
     const unsigned grid1 = (unsigned)(ctx->num_sms * nb1);
     const unsigned grid2 = (unsigned)(ctx->num_sms * nb2);
     const size_t arena_bytes = (size_t)grid2 * WARPS * Tier2::WORDS * sizeof(uint32_t);
-    void* prev_arena = ctx->arena.p;
+    const uint64_t made_arena = ctx->arena.made;
     TIM_TRY(tim_ensure(ctx, ctx->arena, arena_bytes));
-    if (ctx->arena.p != prev_arena || !ctx->arena_clean) {
+    if (ctx->arena.made != made_arena || !ctx->arena_clean) {
         CUDA_TRY(ctx, cudaMemsetAsync(ctx->arena.p, 0xFF, ctx->arena.bytes, ctx->stream));
         ctx->arena_clean = true;
     }
@@ -2054,11 +2054,11 @@ int tim_sample(tim_ctx* ctx, const SampleRequest& req, SampleResult* res) {
         const uint64_t budget = 2ull << 30;
         if ((uint64_t)slots * per_slot > budget)
             slots = (int)std::max<uint64_t>(1, budget / per_slot);
-        void* prev_bm = ctx->big_bitmap.p;
+        const uint64_t made_bm = ctx->big_bitmap.made;
         TIM_TRY(tim_ensure(ctx, ctx->big_bitmap, (size_t)slots * words * sizeof(uint32_t)));
         TIM_TRY(tim_ensure(ctx, ctx->big_queue,
                            (size_t)slots * (uint64_t)ctx->n * sizeof(uint32_t)));
-        if (ctx->big_bitmap.p != prev_bm || !ctx->big_bitmap_clean) {
+        if (ctx->big_bitmap.made != made_bm || !ctx->big_bitmap_clean) {
             CUDA_TRY(ctx, cudaMemsetAsync(ctx->big_bitmap.p, 0, ctx->big_bitmap.bytes, ctx->stream));
             ctx->big_bitmap_clean = true;
         }
@@ -2347,10 +2347,10 @@ int ensure_lt_slots(tim_ctx* ctx, int* slots_out, uint64_t* words_out) {
     int slots = ctx->num_sms;
     const uint64_t budget = 2ull << 30;
     if ((uint64_t)slots * per_slot > budget) slots = (int)std::max<uint64_t>(1, budget / per_slot);
-    void* prev_bm = ctx->big_bitmap.p;
+    const uint64_t made_bm = ctx->big_bitmap.made;
     TIM_TRY(tim_ensure(ctx, ctx->big_bitmap, (size_t)slots * words * sizeof(uint32_t)));
     TIM_TRY(tim_ensure(ctx, ctx->big_queue, (size_t)slots * (uint64_t)ctx->n * sizeof(uint32_t)));
-    if (ctx->big_bitmap.p != prev_bm || !ctx->big_bitmap_clean) {
+    if (ctx->big_bitmap.made != made_bm || !ctx->big_bitmap_clean) {
         CUDA_TRY(ctx, cudaMemsetAsync(ctx->big_bitmap.p, 0, ctx->big_bitmap.bytes, ctx->stream));
         ctx->big_bitmap_clean = true;
     }
@@ -2497,9 +2497,9 @@ int tim_sample_multi(tim_ctx* owner, MultiQuery* qs, int nq, uint64_t seed) {
     const unsigned grid1 = (unsigned)(owner->num_sms * nb1);
     const unsigned grid2 = (unsigned)(owner->num_sms * nb2);
     const size_t arena_bytes = (size_t)grid2 * WARPS * Tier2::WORDS * sizeof(uint32_t);
-    void* prev_arena = owner->arena.p;
+    const uint64_t made_arena = owner->arena.made;
     TIM_TRY(tim_ensure(owner, owner->arena, arena_bytes));
-    if (owner->arena.p != prev_arena || !owner->arena_clean) {
+    if (owner->arena.made != made_arena || !owner->arena_clean) {
         CUDA_TRY(owner, cudaMemsetAsync(owner->arena.p, 0xFF, owner->arena.bytes, owner->stream));
         owner->arena_clean = true;
     }

@@ -868,9 +868,9 @@ int tim_bulk_ic(tim_ctx* ctx, const SampleRequest& req, const uint32_t* list, ui
     while (slots < count && slots < smax) slots <<= 1;
     smax = std::min<uint64_t>(slots, smax);
     uint32_t S = (uint32_t)std::min<uint64_t>(smax, count);
-    void* prev_bitmap = ctx->bulk_bitmap.p;
+    const uint64_t made = ctx->bulk_bitmap.made;
     TIM_TRY(tim_ensure(ctx, ctx->bulk_bitmap, (size_t)smax * words * 4));
-    if (ctx->bulk_bitmap.p != prev_bitmap) ctx->bulk_bitmap_clean = false;
+    if (ctx->bulk_bitmap.made != made) ctx->bulk_bitmap_clean = false;
     if (!ctx->bulk_bitmap_clean) {
         CUDA_TRY(ctx, cudaMemsetAsync(ctx->bulk_bitmap.p, 0, ctx->bulk_bitmap.bytes, ctx->stream));
         ctx->bulk_bitmap_clean = true;
