@@ -497,6 +497,43 @@ __device__ __forceinline__ void skip_live_warp(uint32_t s0, uint32_t s1, const P
     }
 }
 
+// The same for two lists at once, of fewer than SKIP_HALF in-edges each: lanes 0 .. 15 take one
+// (s0, s1, beg, d, qtab_node are theirs), lanes 16 .. 31 the other; d = 0: no list there. Such a
+// list needs at most 16 digits a gap, so a warp of its own would leave half the lanes idle.
+// visit(live, j) runs on every lane, with each half's position j if it found one (live), and
+// returns true on the lanes of a half that stops early. (Queries, weighted cascade, R-MAT 20
+// 29.0 -> 28.3 ms, in both passes together.)
+constexpr uint32_t SKIP_HALF = 1u << 15;
+template <class Visit>
+__device__ __forceinline__ void skip_live_half(uint32_t s0, uint32_t s1, const PhiloxKeys& K,
+                                               uint32_t beg, uint32_t d,
+                                               const unsigned long long* qtab_node, int lane,
+                                               Visit&& visit) {
+    const int h = lane & 15;
+    unsigned long long Q = 0, Tb = 0;
+    if (d) {
+        Q = __ldg(qtab_node + h);
+        Tb = __ldg(qtab_node + 32 + h);
+    }
+    uint4 x = make_uint4(0u, 0u, 0u, 0u);
+    uint32_t pos = 0;
+    for (uint32_t r = 0; __any_sync(0xffffffffu, pos < d); r++) {
+        const uint32_t rem = d - pos;  // 0: this half is through
+        const int B = 32 - __clz((int)rem);
+        if ((r & 1u) == 0u && rem && h <= B)
+            x = philox4x32_10(s0, s1, beg + (r >> 1), TIM_TAG_SKIP + (uint32_t)h, K);
+        const unsigned long long U = (r & 1u) ? (((unsigned long long)x.w << 32) | x.z)
+                                              : (((unsigned long long)x.y << 32) | x.x);
+        const uint32_t bits =
+            (__ballot_sync(0xffffffffu, U < (h < B ? Tb : h == B ? Q : 0ull)) >> (lane & 16)) &
+            0xFFFFu;
+        const uint32_t G = bits & ((1u << B) - 1u);
+        const bool live = rem && !(bits >> B) && G < rem;
+        const bool stop = visit(live, beg + pos + G);
+        pos = live && !stop ? pos + G + 1u : d;
+    }
+}
+
 // Uniform root: floor(x * n / 2^64) with x the first two words of the ROOT draw.
 // LT triggering pick when all in-edges of v carry the same t = floor(b 2^32) (per-node
 // word nt: bit 32 set, low word t): the cumulative thresholds are C_j = min((j + 1) t,

@@ -6,23 +6,24 @@
 // set id, node), so a set does not depend on which kernel expands it, in what order,
 // or on how many threads: the three tiers below give identical sets.
 //
-// Tier 1: a persistent kernel with one warp per RR set; the set's BFS queue (which is
-//   also its member list) and a visited hash live in shared memory. A frontier of up
-//   to 32 nodes is expanded at once: their in-lists are cut into 4-aligned groups of
+// Tier 1: a persistent kernel. IC: a warp keeps eight RR sets in flight (rr_pack_kernel),
+//   triggering: one (rr_team_kernel), LT: each thread one (rr_lt_lane_kernel). A set's BFS
+//   queue (which is also its member list) and a visited hash live in shared memory. Up to 32
+//   frontier nodes are expanded at once: their in-lists are cut into 4-aligned groups of
 //   in-CSR positions, spread over the lanes, and each lane draws one Philox block (4
-//   coin words) and loads 4 thresholds with one 16-byte load. A set whose members
-//   outgrow the queue, or (IC) whose examined in-edges would pass a budget, is listed
-//   for tier 2. This keeps the kernel's tail short: light sets are most sets.
-// An IC set that tier 1 gives up on is handed over with its state (the queue so far,
+//   coin words) and, where the list's thresholds differ, loads 4 of them with one 16-byte
+//   load. A set whose members outgrow the queue, or (IC) whose examined in-edges would pass
+//   a budget, is listed for tier 2. This keeps the kernel's tail short: light sets are most
+//   sets. An IC set that tier 1 gives up on is handed over with its state (the queue so far,
 //   the frontier batch to redo, the width before it), and tier 2 goes on from there
 //   instead of starting again from the root (the coins are keyed, so the set is the same).
-// Tier 2: the same code with a 32x larger queue and hash in global memory (one arena
-//   slot per team; the queue tail and status stay in shared memory, since every new
-//   member takes a tail atomic) and no edge budget, run by teams of T warps per set: T = 1 when the
-//   listed sets are many (parallelism across sets fills the GPU), up to 8 when they are
-//   few (the team splits each in-list, so one heavy set does not leave the GPU idle).
-// In-lists of at least 512 edges (hubs) that take their own coins are streamed by the whole team one at
-// a time with two groups in flight per lane; the rest of a frontier is flattened.
+// Tier 2: a queue of 8192 members and a visited hash or bitmap per team of T warps (rr_team_kernel;
+//   one arena slot per team in global memory; the queue tail and status stay in shared memory,
+//   since every new member takes a tail atomic): T = 1 when the listed sets are many
+//   (parallelism across sets fills the GPU), up to 8 when they are few (the team splits each
+//   batch, so one heavy set does not leave the GPU idle).
+// In all of them in-lists of at least 512 edges (hubs) go by the skip rule, or, with thresholds of
+// their own, are streamed one at a time; the rest of a frontier is flattened.
 // Tier 3: sets beyond tier 2's queue: IC goes to the batched level-synchronous pass of
 //   sample_bulk.cu; LT (a chain) is walked by one warp per set with a visited bitmap; a
 //   general triggering model's set is expanded level by level by one block per set.
@@ -64,9 +65,11 @@ struct Cap {
     static constexpr int WORDS = (1 << LG) + QQ + QQ / 2 + 4;
 };
 using Tier1 = Cap<256, 9>;
-// the other first-pass capacities the autotuner may choose for IC
-using Tier1S = Cap<128, 8>;
-using Tier1L = Cap<512, 10>;
+// IC: a warp's eight sets in flight take an eighth of the first-pass capacity (128, 256 or 512
+// members) each
+using PackS = Cap<16, 5>;
+using PackM = Cap<32, 6>;
+using PackL = Cap<64, 7>;
 using Tier2 = Cap<8192, 14>;
 // Second pass of IC, triggering and batched queries on graphs whose bitmap is no larger than the
 // hash: one atomic tells whether a node is new, nothing is probed, and a bitmap of n / 8 bytes per
@@ -113,6 +116,7 @@ struct SampleArgs {
     unsigned long long width_budget2; // tier 2 IC: in-edges one team may examine per set
     unsigned long long long_budget2;  // tier 2 IC: and in lists of 512 or more
     int chunk;                        // sets claimed per work-counter increment
+    int inflight;                     // tier 1 IC: sets in flight per warp
     uint32_t* lt_col;                 // tier 1 LT: per-thread member columns
     // IC: the state pass 1 hands to pass 2 for the set at list1 position i < hcap, hw
     // words at hand + i hw: queue length, resume position, width so far (2 words), queue
@@ -282,11 +286,10 @@ __device__ __forceinline__ uint32_t live_mask(uint4 x, uint4 t) {
 
 // Shared memory of one warp of the IC passes: the in-lists of a frontier batch that the warp
 // flattens over its lanes ({begin, end, first group | own thresholds << 31, threshold}), and
-// the live in-CSR positions it has found and not inserted yet (fewer than 32, plus one step's
-// 32 x 4).
+// the live in-CSR positions it has found and not inserted yet (fewer than 32, plus a step's 32).
 struct alignas(16) WarpScratch {
     uint4 info[32];
-    uint32_t stage[160];
+    uint32_t stage[64];
 };
 
 // Where an IC expansion stopped: the queue position of the frontier batch to process
@@ -428,34 +431,57 @@ __device__ __forceinline__ int team_rr(const A& a, const PhiloxKeys& K, uint64_t
                 }
                 return __any_sync(0xffffffffu, stop) != 0;
             };
-            // stage the live positions 4 g + c of each lane's mask; true: the set stops
+            // stage the live positions 4 g + c of each lane's mask, one of every lane per turn
+            // (few groups have more than one); true: the set stops
             auto append = [&](uint32_t m, uint32_t g) {
-                const uint32_t b0 = __ballot_sync(0xffffffffu, m & 1u);
-                const uint32_t b1 = __ballot_sync(0xffffffffu, m & 2u);
-                const uint32_t b2 = __ballot_sync(0xffffffffu, m & 4u);
-                const uint32_t b3 = __ballot_sync(0xffffffffu, m & 8u);
-                if (!(b0 | b1 | b2 | b3)) return false;
-                const uint32_t below = (1u << lane) - 1u;
-                const uint32_t at = held;
-                if (m & 1u) wsp->stage[held + __popc(b0 & below)] = g << 2;
-                held += __popc(b0);
-                if (m & 2u) wsp->stage[held + __popc(b1 & below)] = (g << 2) + 1;
-                held += __popc(b1);
-                if (m & 4u) wsp->stage[held + __popc(b2 & below)] = (g << 2) + 2;
-                held += __popc(b2);
-                if (m & 8u) wsp->stage[held + __popc(b3 & below)] = (g << 2) + 3;
-                held += __popc(b3);
-                if (lane == 0) live += held - at;
-                while (held >= 32) {
-                    held -= 32;
-                    if (take(held, 32)) return true;
+                for (uint32_t b; (b = __ballot_sync(0xffffffffu, m != 0u)) != 0u;) {
+                    if (m) {
+                        wsp->stage[held + __popc(b & ((1u << lane) - 1u))] = (g << 2) + (__ffs(m) - 1);
+                        m &= m - 1;
+                    }
+                    const uint32_t cnt = __popc(b);
+                    held += cnt;
+                    if (lane == 0) live += cnt;
+                    if (held >= 32) {
+                        held -= 32;
+                        if (take(held, 32)) return true;
+                        __syncwarp();
+                    }
                 }
-                __syncwarp();
                 return false;
             };
             bool stop = false;
-            // lists under the skip rule: one step per live in-edge
-            for (uint32_t todo = skips; todo && !stop; todo &= todo - 1) {
+            // lists under the skip rule: one step per live in-edge, two lists at a time but for
+            // the longest
+            const uint32_t halves = __ballot_sync(0xffffffffu, skip_list && deg < SKIP_HALF);
+            for (uint32_t todo = halves; todo && !stop;) {
+                const int b0 = __ffs(todo) - 1;
+                todo &= todo - 1;
+                const int b1 = todo ? __ffs(todo) - 1 : -1;
+                todo &= todo - 1;
+                const int b = lane < 16 ? b0 : b1;
+                const uint32_t bb = __shfl_sync(0xffffffffu, beg, b & 31);
+                uint32_t bd = __shfl_sync(0xffffffffu, deg, b & 31);
+                const uint32_t bw2 = __shfl_sync(0xffffffffu, word, b & 31);
+                if (b < 0) bd = 0u;
+                skip_live_half(s0, s1, K, bb, bd, a.qtab + (uint64_t)((bw2 >> 1) - 1) * SKIP_TABLE,
+                               lane, [&](bool found, uint32_t j) {
+                    const uint32_t f = __ballot_sync(0xffffffffu, found && (lane & 15) == 0);
+                    if (found && (lane & 15) == 0)
+                        wsp->stage[held + __popc(f & ((1u << lane) - 1u))] = j;
+                    if (lane == 0) {
+                        live += __popc(f);
+                        exam += __popc(f);
+                    }
+                    held += __popc(f);
+                    if (held < 32) return false;
+                    held -= 32;
+                    stop = take(held, 32);
+                    __syncwarp();
+                    return stop;
+                });
+            }
+            for (uint32_t todo = skips & ~halves; todo && !stop; todo &= todo - 1) {
                 const int b = __ffs(todo) - 1;
                 const uint32_t bb = __shfl_sync(0xffffffffu, beg, b);
                 const uint32_t be = __shfl_sync(0xffffffffu, end, b);
@@ -666,11 +692,11 @@ __device__ __forceinline__ void kappa_lanes(unsigned long long w, unsigned cnt, 
     }
 }
 
-// TIER 1: teams of one warp, storage in shared memory, every set index of [0, count),
-// in-edge budget (IC); listed sets go to list1. TIER 2: teams of T warps, storage in
-// the global arena, the sets of list1, no budget; listed sets go to list2.
-// Four blocks of 64 registers per SM: both IC tiers are bound by issue (tier 2 with six blocks
-// of 40 registers spills and is no faster; tier 1 with five blocks 17.3 ms instead of 16.9).
+// TIER 1 (triggering): teams of one warp, storage in shared memory, every set index of
+// [0, count); listed sets go to list1. TIER 2: teams of T warps, storage in
+// the global arena, the sets of list1; listed sets go to list2.
+// Four blocks of 64 registers per SM for IC: it is bound by issue (six blocks of 40 registers
+// spill and are no faster).
 template <int MODEL, class C, int TIER, int T>
 __global__ void __launch_bounds__(WARPS * 32, TIER == 1 || MODEL == TIM_IC ? 4 : 6) rr_team_kernel(SampleArgs a) {
     extern __shared__ uint32_t smem[];
@@ -700,9 +726,8 @@ __global__ void __launch_bounds__(WARPS * 32, TIER == 1 || MODEL == TIM_IC ? 4 :
     team_sync<T>(team);
     uint16_t* slot = reinterpret_cast<uint16_t*>(queue + C::Q);
     int* ctl = TIER == 1 ? reinterpret_cast<int*>(queue + C::Q + C::Q / 2) : s_ctl[team];
-    const unsigned long long budget =
-        MODEL != TIM_IC ? ~0ull : TIER == 1 ? a.width_budget : a.width_budget2;
-    const unsigned long long long_budget = MODEL == TIM_IC && TIER == 2 ? a.long_budget2 : ~0ull;
+    const unsigned long long budget = MODEL == TIM_IC ? a.width_budget2 : ~0ull;
+    const unsigned long long long_budget = MODEL == TIM_IC ? a.long_budget2 : ~0ull;
     unsigned long long* counter = TIER == 1 ? &a.ds->next_set : &a.ds->next2;
     const uint64_t items =
         TIER == 1 ? a.count : (uint64_t)min(((volatile unsigned*)&a.ds->cnt1)[0], a.list_cap);
@@ -736,7 +761,7 @@ __global__ void __launch_bounds__(WARPS * 32, TIER == 1 || MODEL == TIM_IC ? 4 :
             constexpr bool HAND = MODEL == TIM_IC;
             Resume rin{0, 0ull}, rout{0, 0ull};
             bool resumed = false;
-            if (HAND && TIER == 2 && a.hand && it < a.hcap) {
+            if (HAND && a.hand && it < a.hcap) {
                 const uint32_t* hs = a.hand + it * (uint64_t)a.hw;
                 const uint32_t t0 = hs[0];
                 if (t0 > 0 && t0 <= (uint32_t)C::Q) {
@@ -764,7 +789,7 @@ __global__ void __launch_bounds__(WARPS * 32, TIER == 1 || MODEL == TIM_IC ? 4 :
                 a, a.K, sid_of(a.ids, j), hash, queue, slot, ctl, budget, long_budget, wt, team, &width, &live,
                 &exam, &s_scratch[MODEL == TIM_IC ? wid : 0], s_tot[team],
                 resumed ? &rin : nullptr,
-                (HAND && ((TIER == 1 && a.hand) || (TIER == 2 && a.hand2))) ? &rout : nullptr);
+                (HAND && a.hand2) ? &rout : nullptr);
             const int tail = min(T == 1 ? __shfl_sync(0xffffffffu, ((volatile int*)ctl)[0], 0)
                                         : ((volatile int*)ctl)[0],
                                  C::Q);
@@ -778,20 +803,7 @@ __global__ void __launch_bounds__(WARPS * 32, TIER == 1 || MODEL == TIM_IC ? 4 :
                     else
                         atomicOr(&a.ds->err, TIM_DEV_ERR_OVF_LIST);
                 }
-                if (HAND && TIER == 1 && T == 1 && a.hand) {  // hand the state to pass 2
-                    idx = __shfl_sync(0xffffffffu, idx, 0);
-                    if (idx < a.hcap) {
-                        uint32_t* hs = a.hand + idx * (uint64_t)a.hw;
-                        for (int i = lane; i < tail; i += 32) hs[4 + i] = queue[i];
-                        if (lane == 0) {
-                            hs[0] = (uint32_t)tail;
-                            hs[1] = (uint32_t)rout.head;
-                            hs[2] = (uint32_t)rout.width;
-                            hs[3] = (uint32_t)(rout.width >> 32);
-                        }
-                    }
-                }
-                if (HAND && TIER == 2 && a.hand2) {  // hand the state to the heavy pass
+                if (HAND && a.hand2) {  // hand the state to the heavy pass
                     if (T == 1) {
                         idx = __shfl_sync(0xffffffffu, idx, 0);
                     } else {
@@ -870,6 +882,495 @@ __global__ void __launch_bounds__(WARPS * 32, TIER == 1 || MODEL == TIM_IC ? 4 :
         if (cov) atomicAdd(&a.ds->covered, cov);
         if (memb) atomicAdd(&a.ds->memb[TIER - 1], memb);
     }
+}
+
+// What team_rr and pack_run read of one query: its graph and flags, plus the launch's keys.
+struct QArgs {
+    const uint4* node;
+    const uint32_t* src;
+    const uint32_t* thr;
+    const unsigned long long* qtab;
+    uint64_t n, m;
+    int flags, k;
+    const uint32_t* seed_mark;
+};
+
+// ------------------------------------------- tier 1 for IC: several sets per warp
+//
+// Most RR sets are small (R-MAT 20, weighted cascade: 93 % of 4.9M have at most 32 members), and
+// a batch of their frontier is a node or two: a warp that expands one set at a time spends its
+// instructions on the batch's bookkeeping with most lanes idle. Here a warp holds eight sets. A
+// batch takes up to 32 frontier nodes from all of them, the groups of all their lists are laid
+// out over the lanes together (each group draws with its own set's id), and live positions are
+// staged with their set and inserted 32 at a time. Lane s keeps set s's queue position; tails,
+// widths and work are shared-memory atomics. Finished sets are stored, and new ones claimed,
+// two or more at a time.
+// A set has room for an eighth of the first-pass capacity, 32 members of 256: small enough for
+// four blocks per SM, and a larger set fills a warp's lanes by itself, which is what the second
+// pass gives it (rr_team_kernel, from the state that it had here). Bound by issue, as the second
+// pass. Queries, weighted cascade, one set per warp with room for 256 -> this:
+// R-MAT 20 (eps 0.1) 33.9 -> 28.3 ms, R-MAT 18 8.1 -> 7.3, R-MAT 16 5.6 -> 5.0 (eps 0.2),
+// 24 mixed queries 33.1 -> 28.4, 4.16M nodes trivalency 32.5 -> 29.2 ms; R-MAT 14 1.57 -> 1.56.
+// With room for 256 / 4 sets: 34.0 ms on R-MAT 20; 128 / 4: 30.7; 64 / 8: 29.2 (before lists under
+// the skip rule were taken in pairs); 16 or 64 members in place of 32: within 2 %.
+constexpr int PACK_SETS = 8;  // in flight per warp
+template <class C>
+struct Pack {
+    static constexpr int WORDS = PACK_SETS * (C::H + C::Q);  // of a warp: its hashes, then its queues
+};
+// finished sets wait until 1 / PACK_WAIT of the warp's sets have finished
+constexpr int PACK_WAIT = 4;
+
+// Shared memory of one warp: as in WarpScratch, with the set of each list (info.z bits 24 ..) and
+// of each staged position, and every set's state.
+struct alignas(16) PackScratch {
+    uint4 info[32];
+    uint32_t stage[64];
+    uint8_t stage_set[64];
+    int tail[PACK_SETS], stat[PACK_SETS];
+    uint32_t width[PACK_SETS], work[PACK_SETS];
+    uint32_t s0[PACK_SETS], s1[PACK_SETS];  // the set id
+    uint32_t kw[32];                      // widths that wait for their kappa
+};
+
+template <class C>
+__device__ __forceinline__ int pack_insert(uint32_t* hash, uint32_t* queue, int* tail,
+                                           uint32_t u) {
+    uint32_t h = (u * 0x9E3779B1u) >> (32 - C::LOG2H);
+    for (int probe = 0; probe < C::H; probe++) {
+        const uint32_t old = atomicCAS(&hash[h], EMPTY, u);
+        if (old == u) return INS_OLD;
+        if (old == EMPTY) {
+            const int pos = atomicAdd(tail, 1);
+            if (pos >= C::Q) return INS_FULL;
+            queue[pos] = u;
+            return INS_NEW;
+        }
+        h = (h + 1) & (C::H - 1);
+    }
+    return INS_FULL;
+}
+
+// The sets that next(want, &first) hands to this warp (indexes first .. first + returned, 0 when
+// there are no more), up to `inflight` of them at a time. d: where the results go; list(j) puts
+// set j on the list for pass 2 and returns its position there.
+template <class C, class D, class SidOf, class Next, class List>
+__device__ __forceinline__ void pack_run(const QArgs& a, const D& d, const PhiloxKeys& K,
+                                         unsigned long long budget, int inflight, uint32_t* mem,
+                                         PackScratch* w, uint32_t* hand, uint32_t hcap,
+                                         uint32_t hw, SidOf&& sid_at, Next&& next, List&& list) {
+    constexpr int S = PACK_SETS, Q = C::Q, H = C::H;
+    const int lane = threadIdx.x & 31;
+    const uint32_t below = (1u << lane) - 1u;
+    uint32_t* hash = mem;
+    uint32_t* queue = mem + S * H;
+    const bool cover = a.flags & SAMPLE_COVER, emit = a.flags & SAMPLE_EMIT,
+               kap = a.flags & SAMPLE_KAPPA;
+    const uint4* thr4 = reinterpret_cast<const uint4*>(a.thr);
+    const uint32_t cap1 = (uint32_t)min(budget, 0xFFFFFFFFull);
+    const int wait = max(1, inflight / PACK_WAIT);
+    // lane s: the state of set s; the frontier batch being processed starts at bh, its width
+    // before it is bw
+    int head = 0, bh = 0;
+    uint32_t bw = 0, item = 0;
+    bool alive = false;
+    unsigned long long wsum = 0, memb = 0, cov = 0, live = 0, exam = 0, k_lo = 0, k_hi = 0;
+    unsigned kcnt = 0;
+    auto kflush = [&]() {
+        __syncwarp();
+        kappa_lanes(w->kw[lane], kcnt, lane, a.m, a.k, k_lo, k_hi);
+        kcnt = 0;
+        __syncwarp();
+    };
+    for (;;) {
+        __syncwarp();
+        int tail = 0, stat = 0;
+        if (alive) {
+            tail = ((volatile int*)w->tail)[lane];
+            stat = ((volatile int*)w->stat)[lane];
+        }
+        const bool done = alive && (stat || head >= tail);
+        const uint32_t fin = __ballot_sync(0xffffffffu, done);
+        const bool running = __any_sync(0xffffffffu, alive && !done);
+        if (__popc(fin) >= wait || !running) {
+            if (fin) {
+                tail = min(tail, Q);
+                const bool over = done && (stat & ST_OVERFLOW), good = done && !over;
+                const uint32_t overs = __ballot_sync(0xffffffffu, over);
+                const uint32_t goods = __ballot_sync(0xffffffffu, good);
+                uint32_t idx = 0;
+                if (over) idx = list(item);
+                for (uint32_t o = overs; o && hand; o &= o - 1) {
+                    const int s = __ffs(o) - 1;
+                    const uint32_t at = __shfl_sync(0xffffffffu, idx, s);
+                    const int cnt = __shfl_sync(0xffffffffu, tail, s);
+                    if (at >= hcap) continue;
+                    uint32_t* hs = hand + at * (uint64_t)hw;
+                    for (int i = lane; i < cnt; i += 32) hs[4 + i] = queue[s * Q + i];
+                    if (lane == s) {
+                        hs[0] = (uint32_t)tail;
+                        hs[1] = (uint32_t)bh;
+                        hs[2] = bw;
+                        hs[3] = 0u;
+                    }
+                }
+                const uint32_t width = good ? ((volatile uint32_t*)w->width)[lane] : 0u;
+                if (good) {
+                    wsum += width;
+                    memb += tail;
+                    if (stat & ST_COVERED) cov++;
+                }
+                if (kap) {
+                    if (kcnt + __popc(goods) > 32) kflush();
+                    if (good) w->kw[kcnt + __popc(goods & below)] = width;
+                    kcnt += __popc(goods);
+                }
+                if (emit && goods) {
+                    const uint32_t mine = good ? (uint32_t)tail : 0u;
+                    uint32_t incl = mine;
+#pragma unroll
+                    for (int o = 1; o < S; o <<= 1) {
+                        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+                        if (lane >= o) incl += y;
+                    }
+                    unsigned long long base = 0;
+                    if (lane == S - 1) base = atomicAdd(&d.ds->pool_used, (unsigned long long)incl);
+                    base = __shfl_sync(0xffffffffu, base, S - 1) + (incl - mine);
+                    const bool fits = base + mine <= d.pool_cap;
+                    if (good && fits) {
+                        d.set_start[item] = base;
+                        d.set_len[item] = mine;
+                        d.set_width[item] = width;
+                    } else if (good) {
+                        atomicOr(&d.ds->err, TIM_DEV_ERR_POOL);
+                    }
+                    for (uint32_t o = __ballot_sync(0xffffffffu, good && fits); o; o &= o - 1) {
+                        const int s = __ffs(o) - 1;
+                        const int cnt = __shfl_sync(0xffffffffu, tail, s);
+                        const unsigned long long to = __shfl_sync(0xffffffffu, base, s);
+                        const uint32_t j = __shfl_sync(0xffffffffu, item, s);
+                        for (int i = lane; i < cnt; i += 32) {
+                            d.pool[to + i] = queue[s * Q + i];
+                            d.pool_sid[to + i] = j;
+                        }
+                    }
+                }
+                // the hashes empty again: member by member, or all of it
+                for (uint32_t o = fin; o; o &= o - 1) {
+                    const int s = __ffs(o) - 1;
+                    const int cnt = __shfl_sync(0xffffffffu, tail, s);
+                    uint32_t* hs = hash + s * H;
+                    if (cnt <= 32 && !((overs >> s) & 1u)) {
+                        if (lane < cnt) {
+                            const uint32_t u = queue[s * Q + lane];
+                            uint32_t h = (u * 0x9E3779B1u) >> (32 - C::LOG2H);
+                            for (int probe = 0; probe < H; probe++) {
+                                if (((volatile uint32_t*)hs)[h] == u) break;
+                                h = (h + 1) & (H - 1);
+                            }
+                            hs[h] = EMPTY;
+                        }
+                    } else {
+                        for (int i = lane; i < H / 4; i += 32)
+                            reinterpret_cast<uint4*>(hs)[i] = make_uint4(EMPTY, EMPTY, EMPTY, EMPTY);
+                    }
+                }
+                if (done) alive = false;
+                __syncwarp();
+            }
+            const uint32_t idle = __ballot_sync(0xffffffffu, lane < inflight && !alive);
+            if (idle) {
+                unsigned long long first = 0;
+                const unsigned got = next(__popc(idle), &first);
+                const unsigned rank = __popc(idle & below);
+                if (((idle >> lane) & 1u) && rank < got) {
+                    item = (uint32_t)(first + rank);
+                    const uint64_t sid = sid_at(item);
+                    const uint32_t root = rr_root(sid, a.n, K);
+                    hash[lane * H + ((root * 0x9E3779B1u) >> (32 - C::LOG2H))] = root;
+                    queue[lane * Q] = root;
+                    tail = 1;
+                    stat = (cover && marked(a.seed_mark, root)) ? ST_COVERED : 0;
+                    w->tail[lane] = tail;
+                    w->stat[lane] = stat;
+                    w->width[lane] = 0u;
+                    w->work[lane] = 0u;
+                    w->s0[lane] = (uint32_t)sid;
+                    w->s1[lane] = (uint32_t)(sid >> 32);
+                    head = bh = 0;
+                    bw = 0;
+                    alive = true;
+                }
+                if (!__any_sync(0xffffffffu, alive)) break;
+                __syncwarp();
+            }
+        }
+        // the batch: up to 32 frontier nodes, set by set
+        const int av = alive && !stat ? min(tail - head, 32) : 0;
+        int incl_n = av;
+#pragma unroll
+        for (int o = 1; o < S; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl_n, o);
+            if (lane >= o) incl_n += y;
+        }
+        const int nb = min(__shfl_sync(0xffffffffu, incl_n, S - 1), 32);
+        int set = 0;  // this lane's node's
+#pragma unroll
+        for (int s = 0; s + 1 < S; s++)
+            if (lane >= __shfl_sync(0xffffffffu, incl_n, s)) set++;
+        const int at = __shfl_sync(0xffffffffu, head - (incl_n - av), set) + lane;
+        const int mine = min(av, 32 - (incl_n - av));  // nodes that the batch takes from set `lane`
+        uint32_t beg = 0, end = 0, t = 0, word = 0;
+        if (lane < nb) {
+            const uint4 r = __ldg(a.node + queue[set * Q + at]);
+            beg = r.x;
+            end = r.y;
+            t = r.z;
+            word = r.w;
+        }
+        if (mine > 0) {
+            bh = head;
+            bw = w->width[lane];
+        }
+        __syncwarp();
+        const bool shared = word & 1u;
+        bool skip_list = (word >> 1) != 0u;
+        uint32_t deg = end - beg;
+        // widths; in-edges that take a coin each (a list under the skip rule counts as 64 against
+        // the budget and as the live ones it finds among the examined). A set's members are
+        // distinct, so its sums stay below m < 2^32
+        if (deg) {
+            atomicAdd(&w->width[set], deg);
+            atomicAdd(&w->work[set], skip_list ? 64u : deg);
+        }
+        __syncwarp();
+        const bool heavy = mine > 0 && w->work[lane] > cap1;
+        if (heavy) w->stat[lane] |= ST_OVERFLOW;  // too heavy for this tier: on to the next
+        const uint32_t heavies = __ballot_sync(0xffffffffu, heavy);
+        if ((heavies >> set) & 1u) {
+            deg = 0;
+            skip_list = false;
+        }
+        if (!skip_list) exam += deg;
+        const bool big = !skip_list && deg >= TIM_SKIP_MIN_INDEG;
+        uint32_t held = 0;  // staged positions
+        // insert the sources of stage[from .. from + cnt) into their sets
+        auto take = [&](uint32_t from, uint32_t cnt) {
+            __syncwarp();
+            if ((uint32_t)lane < cnt) {
+                const int s = w->stage_set[from + lane];
+                const uint32_t u = __ldg(a.src + w->stage[from + lane]);
+                if (!((volatile int*)w->stat)[s]) {
+                    const int r = pack_insert<C>(hash + s * H, queue + s * Q, &w->tail[s], u);
+                    if (r == INS_FULL)
+                        atomicOr(&w->stat[s], ST_OVERFLOW);
+                    else if (r == INS_NEW && cover && marked(a.seed_mark, u))
+                        atomicOr(&w->stat[s], ST_COVERED);
+                }
+            }
+            __syncwarp();
+        };
+        // stage the live positions 4 g + c of each lane's mask, of set s: one of every lane per
+        // turn (few groups have more than one)
+        auto append = [&](uint32_t m, uint32_t g, int s) {
+            for (uint32_t b; (b = __ballot_sync(0xffffffffu, m != 0u)) != 0u;) {
+                if (m) {
+                    const uint32_t i = held + __popc(b & below);
+                    w->stage[i] = (g << 2) + (__ffs(m) - 1);
+                    w->stage_set[i] = (uint8_t)s;
+                    m &= m - 1;
+                }
+                const uint32_t cnt = __popc(b);
+                held += cnt;
+                if (lane == 0) live += cnt;
+                if (held >= 32) {
+                    held -= 32;
+                    take(held, 32);
+                }
+            }
+        };
+        // lists under the skip rule: one step per live in-edge, two lists at a time but for the
+        // longest
+        const uint32_t skips = __ballot_sync(0xffffffffu, skip_list);
+        const uint32_t halves = __ballot_sync(0xffffffffu, skip_list && deg < SKIP_HALF);
+        for (uint32_t todo = halves; todo;) {
+            const int b0 = __ffs(todo) - 1;
+            todo &= todo - 1;
+            const int b1 = todo ? __ffs(todo) - 1 : -1;
+            todo &= todo - 1;
+            const int b = lane < 16 ? b0 : b1;
+            const uint32_t bb = __shfl_sync(0xffffffffu, beg, b & 31);
+            uint32_t bd = __shfl_sync(0xffffffffu, deg, b & 31);
+            if (b < 0) bd = 0u;
+            const uint32_t wd = __shfl_sync(0xffffffffu, word, b & 31);
+            const int s = __shfl_sync(0xffffffffu, set, b & 31);
+            skip_live_half(w->s0[s], w->s1[s], K, bb, bd,
+                           a.qtab + (uint64_t)((wd >> 1) - 1) * SKIP_TABLE, lane,
+                           [&](bool found, uint32_t j) {
+                const uint32_t f = __ballot_sync(0xffffffffu, found && (lane & 15) == 0);
+                if (found && (lane & 15) == 0) {
+                    live++;
+                    exam++;
+                    const uint32_t i = held + __popc(f & below);
+                    w->stage[i] = j;
+                    w->stage_set[i] = (uint8_t)s;
+                }
+                held += __popc(f);
+                if (held < 32) return false;
+                held -= 32;
+                take(held, 32);
+                return ((volatile int*)w->stat)[s] != 0;
+            });
+        }
+        for (uint32_t todo = skips & ~halves; todo; todo &= todo - 1) {
+            const int b = __ffs(todo) - 1;
+            const uint32_t bb = __shfl_sync(0xffffffffu, beg, b);
+            const uint32_t bd = __shfl_sync(0xffffffffu, deg, b);
+            const uint32_t wd = __shfl_sync(0xffffffffu, word, b);
+            const int s = __shfl_sync(0xffffffffu, set, b);
+            skip_live_warp(w->s0[s], w->s1[s], K, bb, bd,
+                           a.qtab + (uint64_t)((wd >> 1) - 1) * SKIP_TABLE, lane, [&](uint32_t j) {
+                if (lane == 0) {
+                    live++;
+                    exam++;
+                    w->stage[held] = j;
+                    w->stage_set[held] = (uint8_t)s;
+                }
+                if (++held < 32) return false;
+                held = 0;
+                take(0, 32);
+                return __shfl_sync(0xffffffffu, ((volatile int*)w->stat)[s], 0) != 0;
+            });
+        }
+        // long lists with their own coins; only a list's first and last group need a range mask
+        for (uint32_t todo = __ballot_sync(0xffffffffu, big); todo; todo &= todo - 1) {
+            const int b = __ffs(todo) - 1;
+            const uint32_t bb = __shfl_sync(0xffffffffu, beg, b);
+            const uint32_t be = __shfl_sync(0xffffffffu, end, b);
+            const uint32_t bt = __shfl_sync(0xffffffffu, t, b);
+            const bool bs = __shfl_sync(0xffffffffu, word, b) & 1u;
+            const int s = __shfl_sync(0xffffffffu, set, b);
+            if (bs && bt == 0u) continue;
+            const uint32_t z0 = w->s0[s], z1 = w->s1[s];
+            const uint32_t gfirst = bb >> 2, glast = (be - 1) >> 2;
+            for (uint32_t gb = gfirst; gb <= glast; gb += 64u) {
+                uint32_t m[2], g[2] = {gb + lane, gb + 32u + lane};
+#pragma unroll
+                for (int i = 0; i < 2; i++) {
+                    m[i] = 0;
+                    if (g[i] > glast) continue;
+                    if (bs && bt == 0xFFFFFFFFu) {
+                        m[i] = 0xFu;
+                    } else {
+                        const uint4 th = bs ? make_uint4(bt, bt, bt, bt) : __ldg(thr4 + g[i]);
+                        m[i] = live_mask(philox4x32_10(z0, z1, g[i], TIM_TAG_IC, K), th);
+                    }
+                    if (m[i] && (g[i] == gfirst || g[i] == glast)) m[i] &= range_mask(g[i], bb, be);
+                }
+                append(m[0], g[0], s);
+                append(m[1], g[1], s);
+                if (__shfl_sync(0xffffffffu, ((volatile int*)w->stat)[s], 0)) break;
+            }
+        }
+        // the rest, flattened over the lanes
+        const uint32_t ngs = skip_list || big || deg == 0u || (shared && t == 0u)
+                                 ? 0u
+                                 : ((end - 1) >> 2) - (beg >> 2) + 1;
+        uint32_t incl = ngs;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);  // at most 32 x 129
+        const uint32_t excl = ngs ? incl - ngs : ~0u;
+        const uint32_t lists = __ballot_sync(0xffffffffu, ngs != 0u);
+        if (ngs)
+            w->info[__popc(lists & below)] =
+                make_uint4(beg, end, excl | ((uint32_t)set << 24) | (shared ? 0u : 0x80000000u), t);
+        __syncwarp();
+        for (uint32_t base = 0; base < total; base += 32) {
+            // lists that start before these 32 groups, and at which of them others do
+            const uint32_t before = base ? __popc(__ballot_sync(0xffffffffu, excl < base)) : 0u;
+            const uint32_t starts = __reduce_or_sync(
+                0xffffffffu, excl - base < 32u ? 1u << (excl - base) : 0u);
+            const uint32_t own = before + __popc(starts & (0xFFFFFFFFu >> (31 - lane))) - 1u;
+            uint32_t m = 0, g = 0;
+            int s = 0;
+            if (base + lane < total) {
+                const uint4 f = w->info[own];
+                s = (f.z >> 24) & (PACK_SETS - 1);
+                g = (f.x >> 2) + (base + lane - (f.z & 0xFFFFFFu));
+                if (!(f.z >> 31) && f.w == 0xFFFFFFFFu) {
+                    m = 0xFu;
+                } else {
+                    const uint4 x = philox4x32_10(w->s0[s], w->s1[s], g, TIM_TAG_IC, K);
+                    m = f.z >> 31 ? live_mask(x, __ldg(thr4 + g)) : live_mask_shared(x, f.w);
+                }
+                if (m) m &= range_mask(g, f.x, f.y);
+            }
+            append(m, g, s);
+        }
+        if (held) take(0, held);
+        if (mine > 0) head += mine;
+    }
+    if (kap) {
+        kflush();
+        if (k_lo || k_hi) atomic_add_u128(&d.ds->ksum_lo, &d.ds->ksum_hi, k_lo, k_hi);
+    }
+    wsum = warp_sum_u64(wsum);
+    memb = warp_sum_u64(memb);
+    cov = warp_sum_u64(cov);
+    live = warp_sum_u64(live);
+    exam = warp_sum_u64(exam);
+    if (lane == 0) {
+        if (wsum) {
+            atomicAdd(&d.ds->wsum, wsum);
+            atomicAdd(&d.ds->width[0], wsum);
+        }
+        if (cov) atomicAdd(&d.ds->covered, cov);
+        if (memb) atomicAdd(&d.ds->memb[0], memb);
+        if (live) atomicAdd(&d.ds->live[0], live);
+        if (exam) atomicAdd(&d.ds->exam[0], exam);
+    }
+}
+
+template <class C>
+__global__ void __launch_bounds__(WARPS * 32, 4) rr_pack_kernel(SampleArgs a) {
+    extern __shared__ uint4 smem4[];
+    __shared__ PackScratch s_scratch[WARPS];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint32_t* mem = reinterpret_cast<uint32_t*>(smem4) + wid * Pack<C>::WORDS;
+    for (int i = lane; i < PACK_SETS * C::H; i += 32) mem[i] = EMPTY;
+    __syncwarp();
+    const QArgs qa{a.node, a.src, a.thr, a.qtab, a.n, a.m, a.flags, a.k, a.seed_mark};
+    unsigned long long ci = 0, ce = 0;  // claimed
+    bool more = true;
+    pack_run<C>(
+        qa, a, a.K, a.width_budget, a.inflight, mem, &s_scratch[wid], a.hand, a.hcap, a.hw,
+        [&](uint32_t j) { return sid_of(a.ids, j); },
+        [&](int want, unsigned long long* first) -> unsigned {
+            if (ci == ce && more) {
+                const int step = max(a.chunk, want);
+                if (lane == 0) ci = atomicAdd(&a.ds->next_set, (unsigned long long)step);
+                ci = __shfl_sync(0xffffffffu, ci, 0);
+                more = ci < a.count;
+                if (!more) ci = a.count;
+                ce = min(ci + step, (unsigned long long)a.count);
+            }
+            *first = ci;
+            const unsigned got = (unsigned)min((unsigned long long)want, ce - ci);
+            ci += got;
+            return got;
+        },
+        [&](uint32_t j) {
+            const uint32_t at = atomicAdd(&a.ds->cnt1, 1u);
+            if (at < a.list_cap)
+                a.list1[at] = j;
+            else
+                atomicOr(&a.ds->err, TIM_DEV_ERR_OVF_LIST);
+            return at;
+        });
 }
 
 // ------------------------------------------------- tier 1 for LT: a chain per lane
@@ -1377,13 +1878,12 @@ __global__ void __launch_bounds__(BIG_THREADS) rr_trig_big_kernel(SampleArgs a) 
     }
 }
 
-template <int MODEL, class C, int TIER, int T>
-int occupancy(size_t smem) {
+// Resident blocks per SM of a kernel of WARPS warps with smem bytes of dynamic shared memory.
+template <class K>
+int occupancy(K kernel, size_t smem) {
     int nb = 0;
-    auto k = rr_team_kernel<MODEL, C, TIER, T>;
-    if (smem > 48 * 1024)
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, WARPS * 32, smem) != cudaSuccess ||
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, WARPS * 32, smem) != cudaSuccess ||
         nb < 1) {
         cudaGetLastError();
         nb = 1;
@@ -1391,15 +1891,41 @@ int occupancy(size_t smem) {
     return nb;
 }
 
-int launch_tier1(tim_ctx* ctx, const SampleArgs& a, unsigned grid, size_t smem) {
+// First pass of IC over `sets` sets: sets in flight per warp, members per set, kernel. With no more
+// sets than warps a warp has one set, and hands it over at 16 members whatever the capacity: what
+// counts then is the largest set, and the teams of pass 2 expand it faster than one warp (R-MAT 14
+// query: 16, 32, 64 members 1.56, 1.61, 1.63 ms; a kernel for one set of 256 per warp 1.68).
+template <class Args>
+struct PackPlan {
+    int inflight, members;
+    size_t smem;
+    unsigned grid;
+    void (*kernel)(Args);
+};
+
+template <class C, class Args>
+PackPlan<Args> pack_plan_of(const tim_ctx* ctx, void (*kernel)(Args)) {
+    const size_t smem = (size_t)WARPS * sizeof(uint32_t) * Pack<C>::WORDS;
+    return {PACK_SETS, C::Q, smem, (unsigned)(ctx->num_sms * occupancy(kernel, smem)), kernel};
+}
+
+// small, middle, large: the kernel for PackS, PackM and PackL.
+template <class Args>
+PackPlan<Args> pack_plan(const tim_ctx* ctx, uint64_t sets, void (*small)(Args),
+                         void (*middle)(Args), void (*large)(Args)) {
+    PackPlan<Args> p = pack_plan_of<PackS>(ctx, small);
+    if (sets > (uint64_t)p.grid * WARPS && ctx->cap1 != 128)
+        p = ctx->cap1 == 512 ? pack_plan_of<PackL>(ctx, large) : pack_plan_of<PackM>(ctx, middle);
+    const uint64_t warps = (uint64_t)p.grid * WARPS;
+    p.inflight = (int)std::min<uint64_t>(p.inflight, std::max<uint64_t>(1, (sets + warps - 1) / warps));
+    return p;
+}
+
+int launch_tier1(tim_ctx* ctx, const SampleArgs& a, const PackPlan<SampleArgs>& plan, unsigned grid,
+                 size_t smem) {
     if (ctx->model == TIM_IC) {
-        if (ctx->cap1 == 128)
-            rr_team_kernel<TIM_IC, Tier1S, 1, 1><<<grid, WARPS * 32, smem, ctx->stream>>>(a);
-        else if (ctx->cap1 == 512)
-            rr_team_kernel<TIM_IC, Tier1L, 1, 1><<<grid, WARPS * 32, smem, ctx->stream>>>(a);
-        else
-            rr_team_kernel<TIM_IC, Tier1, 1, 1><<<grid, WARPS * 32, smem, ctx->stream>>>(a);
-        LAUNCH_CHECK(ctx, "rr_team_kernel (tier 1)");
+        plan.kernel<<<plan.grid, WARPS * 32, plan.smem, ctx->stream>>>(a);
+        LAUNCH_CHECK(ctx, "rr_pack_kernel (tier 1)");
     } else if (ctx->model == TIM_TRIG) {
         rr_team_kernel<TIM_TRIG, Tier1, 1, 1><<<grid, WARPS * 32, smem, ctx->stream>>>(a);
         LAUNCH_CHECK(ctx, "rr_team_kernel (tier 1, triggering)");
@@ -1504,6 +2030,7 @@ struct MultiArgs {
     const unsigned long long* prefix;  // prefix[i] = sets of queries before i; [nq] = total
     int nq;
     int chunk;
+    int inflight;                      // tier 1 IC: sets in flight per warp
     unsigned long long* next;  // [0] tier-1, [1] tier-2 work counters
     unsigned* cnt;             // [0] sets listed for tier 2, [1] for tier 3
     int* err;
@@ -1516,17 +2043,6 @@ struct MultiArgs {
     // IC: pass-1 state handed to pass 2 for list1 position i < hcap (as in SampleArgs)
     uint32_t* hand;
     uint32_t hcap, hw;
-};
-
-// What team_rr reads of one query: its graph and flags, plus the launch's keys.
-struct QArgs {
-    const uint4* node;
-    const uint32_t* src;
-    const uint32_t* thr;
-    const unsigned long long* qtab;
-    uint64_t n, m;
-    int flags, k;
-    const uint32_t* seed_mark;
 };
 
 constexpr int MAXQ = 256;  // queries per multi-query launch
@@ -1553,44 +2069,29 @@ __device__ __forceinline__ void flush_acc(const QueryDesc* qd, int qi, QAcc& acc
     acc = QAcc{0, 0, 0, 0, 0, 0, 0};
 }
 
-// TIER 1: shared-memory sets of every query (global set index across queries); TIER 2:
-// the listed (query, set) pairs with a global arena and teams of T warps.
-template <class C, int TIER, int T>
+// Tier 2: the listed (query, set) pairs with a global arena and teams of T warps.
+template <class C, int T>
 __global__ void __launch_bounds__(WARPS * 32, 4) rr_multi_kernel(MultiArgs ma) {
     extern __shared__ uint32_t smem[];
     __shared__ unsigned long long s_claim[WARPS];
-    __shared__ unsigned long long s_prefix[MAXQ + 1];
     __shared__ int s_ctl[WARPS][4];  // tier 2: a team's tail and status (shared atomics)
     __shared__ WarpScratch s_scratch[WARPS];
     __shared__ uint32_t s_tot[WARPS][4];  // a team's batch sums
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int wt = wid % T, team = wid / T;
     const int tl = wt * 32 + lane;
-    for (int i = threadIdx.x; i <= ma.nq; i += blockDim.x) s_prefix[i] = ma.prefix[i];
-    __syncthreads();
-    uint32_t* hash;
-    uint32_t* queue;
-    if (TIER == 1) {
-        hash = smem + team * C::WORDS;
-        queue = hash + C::H;
-        for (int i = tl; i < C::H; i += 32 * T) hash[i] = EMPTY;
-    } else {
-        const uint64_t slot_id = (uint64_t)blockIdx.x * (WARPS / T) + team;
-        hash = ma.arena + slot_id * C::WORDS;
-        queue = hash + C::H;
-        if (C::BITMAP && ma.bm_shared) {
-            hash = smem + team * ma.bm_words;
-            set_clear_all<C>(hash, ma.bm_words, tl, 32 * T);
-        }
+    const uint64_t slot_id = (uint64_t)blockIdx.x * (WARPS / T) + team;
+    uint32_t* hash = ma.arena + slot_id * C::WORDS;
+    uint32_t* queue = hash + C::H;
+    if (C::BITMAP && ma.bm_shared) {
+        hash = smem + team * ma.bm_words;
+        set_clear_all<C>(hash, ma.bm_words, tl, 32 * T);
     }
     team_sync<T>(team);
     uint16_t* slot = reinterpret_cast<uint16_t*>(queue + C::Q);
-    int* ctl = TIER == 1 ? reinterpret_cast<int*>(queue + C::Q + C::Q / 2) : s_ctl[team];
-    unsigned long long* counter = &ma.next[TIER - 1];
-    const uint64_t items = TIER == 1 ? s_prefix[ma.nq]
-                                     : (uint64_t)min(((volatile unsigned*)ma.cnt)[0], ma.list_cap);
-    uint2* out_list = TIER == 1 ? ma.list1 : ma.list2;
-    unsigned* out_cnt = TIER == 1 ? &ma.cnt[0] : &ma.cnt[1];
+    int* ctl = s_ctl[team];
+    unsigned long long* counter = &ma.next[1];
+    const uint64_t items = min(((volatile unsigned*)ma.cnt)[0], ma.list_cap);
     const bool leader = wt == 0 && lane == 0;
     QAcc acc{0, 0, 0, 0, 0, 0, 0};
     int cur_q = -1;
@@ -1620,40 +2121,25 @@ __global__ void __launch_bounds__(WARPS * 32, 4) rr_multi_kernel(MultiArgs ma) {
         if (i0 >= items) break;
         const unsigned long long i1 = min(i0 + (unsigned long long)ma.chunk, (unsigned long long)items);
         for (unsigned long long it = i0; it < i1; it++) {
-            int qi;
-            uint64_t j;
-            if (TIER == 1) {
-                int lo = 0, hi = ma.nq;  // s_prefix[lo] <= it < s_prefix[hi]
-                while (hi - lo > 1) {
-                    const int mid = (lo + hi) >> 1;
-                    if (s_prefix[mid] <= it)
-                        lo = mid;
-                    else
-                        hi = mid;
-                }
-                qi = lo;
-                j = it - s_prefix[lo];
-            } else {
-                const uint2 e = ma.list1[it];
-                qi = (int)e.x;
-                j = e.y;
-            }
+            const uint2 e = ma.list1[it];
+            const int qi = (int)e.x;
+            const uint64_t j = e.y;
             if (qi != cur_q) {
                 if (wt == 0) kflush(cur_q);
-                flush_acc<TIER>(ma.q, cur_q, acc, lane);
+                flush_acc<2>(ma.q, cur_q, acc, lane);
                 cur_q = qi;
             }
             const QueryDesc& d = ma.q[qi];
             const QArgs qa{d.node, d.src, d.thr, d.qtab, d.n, d.m, d.flags, d.k, d.seed_mark};
             const int model = d.model;
             const unsigned long long budget =
-                model != TIM_IC ? ~0ull : TIER == 1 ? d.width_budget : d.width_budget2;
+                model != TIM_IC ? ~0ull : d.width_budget2;
             unsigned long long width;
             int st;
             // IC: pass 2 goes on from the state pass 1 handed over (see rr_team_kernel)
-            Resume rin{0, 0ull}, rout{0, 0ull};
+            Resume rin{0, 0ull};
             bool resumed = false;
-            if (TIER == 2 && model == TIM_IC && ma.hand && it < ma.hcap) {
+            if (model == TIM_IC && ma.hand && it < ma.hcap) {
                 const uint32_t* hs = ma.hand + it * (uint64_t)ma.hw;
                 const uint32_t t0 = hs[0];
                 if (t0 > 0 && t0 <= (uint32_t)C::Q) {
@@ -1679,8 +2165,7 @@ __global__ void __launch_bounds__(WARPS * 32, 4) rr_multi_kernel(MultiArgs ma) {
                 st = team_rr<TIM_IC, C, T, QArgs>(qa, ma.K, d.sid0 + j, hash, queue, slot, ctl,
                                                   budget, ~0ull, wt, team, &width, &acc.live,
                                                   &acc.exam, &s_scratch[wid], s_tot[team],
-                                                  resumed ? &rin : nullptr,
-                                                  (TIER == 1 && ma.hand) ? &rout : nullptr);
+                                                  resumed ? &rin : nullptr);
             else
                 st = team_rr<TIM_LT, C, T, QArgs>(qa, ma.K, d.sid0 + j, hash, queue, slot, ctl,
                                                   budget, ~0ull, wt, team, &width, &acc.live,
@@ -1690,26 +2175,12 @@ __global__ void __launch_bounds__(WARPS * 32, 4) rr_multi_kernel(MultiArgs ma) {
                                  C::Q);
             team_sync<T>(team);
             if (st & ST_OVERFLOW) {
-                unsigned idx = 0;
                 if (leader) {
-                    idx = atomicAdd(out_cnt, 1u);
+                    const unsigned idx = atomicAdd(&ma.cnt[1], 1u);
                     if (idx < ma.list_cap)
-                        out_list[idx] = make_uint2((uint32_t)qi, (uint32_t)j);
+                        ma.list2[idx] = make_uint2((uint32_t)qi, (uint32_t)j);
                     else
                         atomicOr(ma.err, TIM_DEV_ERR_OVF_LIST);
-                }
-                if (TIER == 1 && T == 1 && model == TIM_IC && ma.hand) {
-                    idx = __shfl_sync(0xffffffffu, idx, 0);
-                    if (idx < ma.hcap) {
-                        uint32_t* hs = ma.hand + idx * (uint64_t)ma.hw;
-                        for (int i = lane; i < tail; i += 32) hs[4 + i] = queue[i];
-                        if (lane == 0) {
-                            hs[0] = (uint32_t)tail;
-                            hs[1] = (uint32_t)rout.head;
-                            hs[2] = (uint32_t)rout.width;
-                            hs[3] = (uint32_t)(rout.width >> 32);
-                        }
-                    }
                 }
                 set_clear_all<C>(hash, ma.bm_words, tl, 32 * T);
                 team_sync<T>(team);
@@ -1758,7 +2229,68 @@ __global__ void __launch_bounds__(WARPS * 32, 4) rr_multi_kernel(MultiArgs ma) {
         }
     }
     if (wt == 0) kflush(cur_q);
-    flush_acc<TIER>(ma.q, cur_q, acc, lane);
+    flush_acc<2>(ma.q, cur_q, acc, lane);
+}
+
+// Tier 1 of the IC queries of a multi-query launch (several sets of one query per warp); a warp
+// drains a query's sets before it goes on to the next query's.
+template <class C>
+__global__ void __launch_bounds__(WARPS * 32, 3) rr_pack_multi_kernel(MultiArgs ma) {
+    extern __shared__ uint4 smem4[];
+    __shared__ PackScratch s_scratch[WARPS];
+    __shared__ unsigned long long s_prefix[MAXQ + 1];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint32_t* mem = reinterpret_cast<uint32_t*>(smem4) + wid * Pack<C>::WORDS;
+    for (int i = lane; i < PACK_SETS * C::H; i += 32) mem[i] = EMPTY;
+    for (int i = threadIdx.x; i <= ma.nq; i += blockDim.x) s_prefix[i] = ma.prefix[i];
+    __syncthreads();
+    const unsigned long long items = s_prefix[ma.nq];
+    unsigned long long ci = 0, ce = 0;  // claimed
+    bool more = true;
+    auto claim = [&](int want) {
+        if (ci != ce || !more) return;
+        const int step = max(ma.chunk, want);
+        if (lane == 0) ci = atomicAdd(&ma.next[0], (unsigned long long)step);
+        ci = __shfl_sync(0xffffffffu, ci, 0);
+        more = ci < items;
+        if (!more) ci = items;
+        ce = min(ci + step, items);
+    };
+    for (;;) {
+        claim(ma.inflight);
+        if (ci == ce) break;
+        int lo = 0, hi = ma.nq;  // s_prefix[lo] <= ci < s_prefix[hi]
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (s_prefix[mid] <= ci)
+                lo = mid;
+            else
+                hi = mid;
+        }
+        const unsigned long long q0 = s_prefix[lo], q1 = s_prefix[lo + 1];
+        const QueryDesc& d = ma.q[lo];
+        const QArgs qa{d.node, d.src, d.thr, d.qtab, d.n, d.m, d.flags, d.k, d.seed_mark};
+        const uint64_t sid0 = d.sid0;
+        pack_run<C>(
+            qa, d, ma.K, d.width_budget, ma.inflight, mem, &s_scratch[wid], ma.hand, ma.hcap,
+            ma.hw, [&](uint32_t j) { return sid0 + j; },
+            [&](int want, unsigned long long* first) -> unsigned {
+                claim(want);
+                if (ci >= q1) return 0u;
+                *first = ci - q0;
+                const unsigned got = (unsigned)min((unsigned long long)want, min(ce, q1) - ci);
+                ci += got;
+                return got;
+            },
+            [&](uint32_t j) {
+                const uint32_t at = atomicAdd(&ma.cnt[0], 1u);
+                if (at < ma.list_cap)
+                    ma.list1[at] = make_uint2((uint32_t)lo, j);
+                else
+                    atomicOr(ma.err, TIM_DEV_ERR_OVF_LIST);
+                return at;
+            });
+    }
 }
 
 // Tier 1 of the LT queries of a multi-query launch: one chain per thread as in
@@ -1953,48 +2485,27 @@ rr_lt_lane_multi_kernel(MultiArgs ma, const unsigned long long* lt_prefix,
     flush();
 }
 
-int launch_multi(tim_ctx* owner, const MultiArgs& ma, int tier, int T, unsigned grid,
-                 size_t smem) {
-    if (tier == 1) {
-        if (owner->cap1 == 128)
-            rr_multi_kernel<Tier1S, 1, 1><<<grid, WARPS * 32, smem, owner->stream>>>(ma);
-        else if (owner->cap1 == 512)
-            rr_multi_kernel<Tier1L, 1, 1><<<grid, WARPS * 32, smem, owner->stream>>>(ma);
-        else
-            rr_multi_kernel<Tier1, 1, 1><<<grid, WARPS * 32, smem, owner->stream>>>(ma);
-    } else if (ma.bm_shared || ma.bm_words <= BITMAP_GLOBAL) {
+// Tier 2 of a multi-query launch with teams of T warps.
+int launch_multi(tim_ctx* owner, const MultiArgs& ma, int T, unsigned grid) {
+    if (ma.bm_shared || ma.bm_words <= BITMAP_GLOBAL) {
         const size_t bytes = bitmap_smem(ma.bm_words, T);
-        auto* kernel = T == 1   ? rr_multi_kernel<Tier2B, 2, 1>
-                       : T == 2 ? rr_multi_kernel<Tier2B, 2, 2>
-                       : T == 4 ? rr_multi_kernel<Tier2B, 2, 4>
-                                : rr_multi_kernel<Tier2B, 2, 8>;
+        auto* kernel = T == 1   ? rr_multi_kernel<Tier2B, 1>
+                       : T == 2 ? rr_multi_kernel<Tier2B, 2>
+                       : T == 4 ? rr_multi_kernel<Tier2B, 4>
+                                : rr_multi_kernel<Tier2B, 8>;
         if (bytes) TIM_TRY(bitmap_grid(owner, kernel, bytes, grid, &grid));
         kernel<<<grid, WARPS * 32, bytes, owner->stream>>>(ma);
     } else if (T == 1) {
-        rr_multi_kernel<Tier2, 2, 1><<<grid, WARPS * 32, 0, owner->stream>>>(ma);
+        rr_multi_kernel<Tier2, 1><<<grid, WARPS * 32, 0, owner->stream>>>(ma);
     } else if (T == 2) {
-        rr_multi_kernel<Tier2, 2, 2><<<grid, WARPS * 32, 0, owner->stream>>>(ma);
+        rr_multi_kernel<Tier2, 2><<<grid, WARPS * 32, 0, owner->stream>>>(ma);
     } else if (T == 4) {
-        rr_multi_kernel<Tier2, 2, 4><<<grid, WARPS * 32, 0, owner->stream>>>(ma);
+        rr_multi_kernel<Tier2, 4><<<grid, WARPS * 32, 0, owner->stream>>>(ma);
     } else {
-        rr_multi_kernel<Tier2, 2, 8><<<grid, WARPS * 32, 0, owner->stream>>>(ma);
+        rr_multi_kernel<Tier2, 8><<<grid, WARPS * 32, 0, owner->stream>>>(ma);
     }
-    LAUNCH_CHECK(owner, tier == 1 ? "rr_multi_kernel (tier 1)" : "rr_multi_kernel (tier 2)");
+    LAUNCH_CHECK(owner, "rr_multi_kernel (tier 2)");
     return TIM_OK;
-}
-
-template <class C, int TIER, int T>
-int multi_occupancy(size_t smem) {
-    int nb = 0;
-    auto k = rr_multi_kernel<C, TIER, T>;
-    if (smem > 48 * 1024)
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, WARPS * 32, smem) != cudaSuccess ||
-        nb < 1) {
-        cudaGetLastError();
-        nb = 1;
-    }
-    return nb;
 }
 
 }  // namespace
@@ -2023,19 +2534,19 @@ int tim_sample(tim_ctx* ctx, const SampleRequest& req, SampleResult* res) {
     TIM_TRY(tim_ensure(ctx, ctx->ovf_list2, (size_t)cap_sets * sizeof(uint32_t)));
 
     // tier 2 arena: one slot per resident warp, hash regions kept EMPTY between sets
-    const int cap1 = ctx->model == TIM_IC ? ctx->cap1 : 256;
-    const size_t smem1 = (size_t)WARPS * sizeof(uint32_t) *
-                         (cap1 == 128 ? Tier1S::WORDS : cap1 == 512 ? Tier1L::WORDS : Tier1::WORDS);
-    const int nb1 = ctx->model == TIM_IC
-                        ? (cap1 == 128   ? occupancy<TIM_IC, Tier1S, 1, 1>(smem1)
-                           : cap1 == 512 ? occupancy<TIM_IC, Tier1L, 1, 1>(smem1)
-                                         : occupancy<TIM_IC, Tier1, 1, 1>(smem1))
-                    : ctx->model == TIM_TRIG ? occupancy<TIM_TRIG, Tier1, 1, 1>(smem1)
-                                             : occupancy<TIM_LT, Tier1, 1, 1>(smem1);
-    const int nb2 = ctx->model == TIM_IC     ? occupancy<TIM_IC, Tier2, 2, 1>(0)
-                    : ctx->model == TIM_TRIG ? occupancy<TIM_TRIG, Tier2, 2, 1>(0)
-                                             : occupancy<TIM_LT, Tier2, 2, 1>(0);
-    const unsigned grid1 = (unsigned)(ctx->num_sms * nb1);
+    PackPlan<SampleArgs> plan{};
+    size_t smem1 = 0;
+    unsigned grid1 = 0;  // triggering
+    if (ctx->model == TIM_IC) {
+        plan = pack_plan(ctx, count, rr_pack_kernel<PackS>,
+                         rr_pack_kernel<PackM>, rr_pack_kernel<PackL>);
+    } else if (ctx->model == TIM_TRIG) {
+        smem1 = (size_t)WARPS * sizeof(uint32_t) * Tier1::WORDS;
+        grid1 = (unsigned)(ctx->num_sms * occupancy(rr_team_kernel<TIM_TRIG, Tier1, 1, 1>, smem1));
+    }
+    const int nb2 = ctx->model == TIM_IC     ? occupancy(rr_team_kernel<TIM_IC, Tier2, 2, 1>, 0)
+                    : ctx->model == TIM_TRIG ? occupancy(rr_team_kernel<TIM_TRIG, Tier2, 2, 1>, 0)
+                                             : occupancy(rr_team_kernel<TIM_LT, Tier2, 2, 1>, 0);
     const unsigned grid2 = (unsigned)(ctx->num_sms * nb2);
     const size_t arena_bytes = (size_t)grid2 * WARPS * Tier2::WORDS * sizeof(uint32_t);
     const uint64_t made_arena = ctx->arena.made;
@@ -2092,14 +2603,15 @@ int tim_sample(tim_ctx* ctx, const SampleRequest& req, SampleResult* res) {
     a.width_budget2 = ctx->width_budget2;
     a.long_budget2 = LONG_BUDGET2;
     a.chunk = std::max(1, ctx->chunk);
-    // IC: room for the pass-1 state of up to count / 8 + 4096 handed-over sets (at most
+    a.inflight = plan.inflight;
+    // IC: room for the pass-1 state of up to count / 2 + 4096 handed-over sets (at most
     // 1 GiB); sets listed beyond it start over in pass 2
     a.hand = nullptr;
     a.hcap = 0;
-    a.hw = 4u + (uint32_t)cap1;
+    a.hw = 4u + (uint32_t)plan.members;
     if (ctx->model == TIM_IC && count > 0) {
         const uint64_t maxslots = (1ull << 30) / ((uint64_t)a.hw * sizeof(uint32_t));
-        const uint64_t hcap = std::min<uint64_t>(std::min<uint64_t>(count / 8 + 4096, maxslots),
+        const uint64_t hcap = std::min<uint64_t>(std::min<uint64_t>(count / 2 + 4096, maxslots),
                                                  list_cap);
         TIM_TRY(tim_ensure(ctx, ctx->hand, (size_t)hcap * a.hw * sizeof(uint32_t)));
         a.hand = (uint32_t*)ctx->hand.p;
@@ -2127,7 +2639,7 @@ int tim_sample(tim_ctx* ctx, const SampleRequest& req, SampleResult* res) {
         bool read = false;
         if (count > 0) {
             cudaEventRecord(ctx->kev[0], ctx->stream);
-            TIM_TRY(launch_tier1(ctx, a, grid1, smem1));
+            TIM_TRY(launch_tier1(ctx, a, plan, grid1, smem1));
             cudaEventRecord(ctx->kev[1], ctx->stream);
             // team size of tier 2: intra-set parallelism when the listed sets are few
             int T = 1;
@@ -2487,14 +2999,10 @@ int tim_sample_multi(tim_ctx* owner, MultiQuery* qs, int nq, uint64_t seed) {
     TIM_TRY(tim_ensure(owner, owner->ovf_list, (size_t)(total + 1) * sizeof(uint2)));
     TIM_TRY(tim_ensure(owner, owner->ovf_list2, (size_t)(total + 1) * sizeof(uint2)));
     // arena and occupancy as in the single-query path
-    const int cap1 = owner->cap1;
-    const size_t smem1 = (size_t)WARPS * sizeof(uint32_t) *
-                         (cap1 == 128 ? Tier1S::WORDS : cap1 == 512 ? Tier1L::WORDS : Tier1::WORDS);
-    const int nb1 = cap1 == 128   ? multi_occupancy<Tier1S, 1, 1>(smem1)
-                    : cap1 == 512 ? multi_occupancy<Tier1L, 1, 1>(smem1)
-                                  : multi_occupancy<Tier1, 1, 1>(smem1);
-    const int nb2 = multi_occupancy<Tier2, 2, 1>(0);
-    const unsigned grid1 = (unsigned)(owner->num_sms * nb1);
+    const PackPlan<MultiArgs> plan =
+        pack_plan(owner, total_ic, rr_pack_multi_kernel<PackS>,
+                  rr_pack_multi_kernel<PackM>, rr_pack_multi_kernel<PackL>);
+    const int nb2 = occupancy(rr_multi_kernel<Tier2, 1>, 0);
     const unsigned grid2 = (unsigned)(owner->num_sms * nb2);
     const size_t arena_bytes = (size_t)grid2 * WARPS * Tier2::WORDS * sizeof(uint32_t);
     const uint64_t made_arena = owner->arena.made;
@@ -2509,6 +3017,7 @@ int tim_sample_multi(tim_ctx* owner, MultiQuery* qs, int nq, uint64_t seed) {
     ma.prefix = d_prefix;
     ma.nq = nq;
     ma.chunk = std::max(1, owner->chunk);
+    ma.inflight = plan.inflight;
     ma.next = d_next;
     ma.cnt = d_cnt;
     ma.err = d_err;
@@ -2520,11 +3029,11 @@ int tim_sample_multi(tim_ctx* owner, MultiQuery* qs, int nq, uint64_t seed) {
     for (int i = 0; i < nq; i++)
         ma.bm_words = std::max(ma.bm_words, (uint32_t)((uint64_t)qs[i].ctx->n / 32 + 1));
     // pass-1 state handed to pass 2 (IC queries), in the owner's scratch
-    ma.hw = 4u + (uint32_t)cap1;
+    ma.hw = 4u + (uint32_t)plan.members;
     {
         const uint64_t maxslots = (1ull << 30) / ((uint64_t)ma.hw * sizeof(uint32_t));
         const uint64_t hcap =
-            std::min<uint64_t>(std::min<uint64_t>(total_ic / 8 + 4096, maxslots), total + 1);
+            std::min<uint64_t>(std::min<uint64_t>(total_ic / 2 + 4096, maxslots), total + 1);
         TIM_TRY(tim_ensure(owner, owner->hand, (size_t)hcap * ma.hw * sizeof(uint32_t)));
         ma.hand = (uint32_t*)owner->hand.p;
         ma.hcap = (uint32_t)hcap;
@@ -2571,7 +3080,10 @@ int tim_sample_multi(tim_ctx* owner, MultiQuery* qs, int nq, uint64_t seed) {
         uint64_t live3_total = 0;
         std::vector<uint64_t> live3(nq, 0);
         if (total > 0) {
-            if (total_ic > 0) TIM_TRY(launch_multi(owner, ma, 1, 1, grid1, smem1));
+            if (total_ic > 0) {
+                plan.kernel<<<plan.grid, WARPS * 32, plan.smem, owner->stream>>>(ma);
+                LAUNCH_CHECK(owner, "rr_pack_multi_kernel (tier 1)");
+            }
             if (total_lt > 0) {
                 rr_lt_lane_multi_kernel<<<grid_lt, LT_THREADS, LT_SMEM, owner->stream>>>(
                     ma, d_prefix_lt, d_lt_next, (uint32_t*)owner->lt_col.p);
@@ -2589,7 +3101,7 @@ int tim_sample_multi(tim_ctx* owner, MultiQuery* qs, int nq, uint64_t seed) {
                     T *= 2;
             }
             ma.bm_shared = bitmap_smem(ma.bm_words, T) > 0;
-            TIM_TRY(launch_multi(owner, ma, 2, T, grid2, 0));
+            TIM_TRY(launch_multi(owner, ma, T, grid2));
             CUDA_TRY(owner, cudaMemcpyAsync(h_cnt, d_cnt, sizeof h_cnt, cudaMemcpyDeviceToHost,
                                             owner->stream));
             TIM_TRY(tim_sync(owner));
