@@ -305,9 +305,9 @@ int tim_set_team_size(tim_ctx* ctx, int warps);
 int tim_set_team_factor(tim_ctx* ctx, int factor);
 
 /* IC sampler tuning: pass 1's queue capacity per RR set, 128, 256 (default) or 512
- * members (the visited hash has twice as many slots; both sit in shared memory, so a
- * larger capacity leaves fewer warps per SM). Larger sets move on to pass 2. Results do
- * not change. */
+ * members per warp, of which each of its eight sets has an eighth (the visited hash has
+ * twice as many slots; both sit in shared memory). Larger sets move on to pass 2. Results
+ * do not change. */
 int tim_set_pass1_capacity(tim_ctx* ctx, int members);
 
 /* IC sampler tuning: pass 2 (a team of warps per RR set, queue of 8192 members) hands a
@@ -319,7 +319,7 @@ int tim_set_pass1_capacity(tim_ctx* ctx, int members);
 int tim_set_pass2_budget(tim_ctx* ctx, uint64_t budget);
 
 /* Polls a block makes at a grid barrier of a persistent kernel (the heavy-set pass of
- * the IC sampler, the greedy of Algorithm 1) before it gives up; default 2^24 (about a
+ * the IC sampler, the greedy of Algorithm 1; a training run waits at least the default) before it gives up; default 2^24 (about a
  * second). When one block gives up, every block of the launch stops and the call
  * returns TIM_ERR_TIMEOUT; the context stays usable. Results do not change. */
 int tim_set_wait_limit(tim_ctx* ctx, uint32_t polls);
@@ -372,7 +372,8 @@ int tim_get_profile(tim_ctx* ctx, tim_profile* out, int reset);
  *   d_seeds     device int32[k] (output)
  *   d_covered   device uint64[1] (output): number of sets the seeds cover
  * Returns TIM_ERR_ARG, without running anything, for sizes beyond these limits, and
- * after the run if a member or an offset was out of range. Every call copies d_off[0]
+ * after the run if a member or an offset was out of range; TIM_ERR_TIMEOUT if the blocks
+ * of its one cooperative launch waited too long for each other. Every call copies d_off[0]
  * and d_off[n_sets] to the host and waits for the stream before its kernels, and
  * waits again before it returns. Scratch is one __device__ array of about 13.3 MiB
  * that every GPU holds once the library is loaded; the first call on a device also
@@ -518,8 +519,9 @@ uint64_t tim_launch_count(tim_ctx* ctx);
  * its root in that world, so root in cascade(S) <=> RR set meets S, world by world.
  * Outputs (each may be NULL): *total = sum over cascades of the activated nodes
  * (seeds included; exact), *mean = total / count in FP64, counts_out = host
- * uint32[count] of per-cascade counts. G as out-records (8 B per edge) is built from
- * G^T on the first call after a load and kept. Errors: TIM_ERR_STATE without a graph,
+ * uint32[count] of per-cascade counts. G as out-records (8 B per node and per edge,
+ * and 4 B per edge more once whole worlds are drawn) is built from G^T on the first call
+ * after a load and kept. Errors: TIM_ERR_STATE without a graph,
  * TIM_ERR_ARG for a seed out of range or count >= 2^32, TIM_ERR_OOM. */
 int tim_spread_mc(tim_ctx* ctx, const int32_t* seeds, int k, uint64_t count, uint64_t seed,
                   uint64_t first_set_id, uint64_t* total, double* mean, uint32_t* counts_out);

@@ -9,6 +9,8 @@
 // are kept in) and every sum accumulated in fp32. Reductions over samples run in a
 // fixed order (per-block partials, then a block-ordered sum), so gradients and
 // training runs are reproducible bit for bit.
+// A training run is one cooperative launch (mlp_train_kernel), or launches per step where its
+// blocks would not be resident together; both give the same bits.
 #include <cuda_bf16.h>
 #include <math.h>
 #include <string.h>

@@ -1,10 +1,12 @@
 // select.cu -- greedy maximum coverage over the RR-set store (the selection of
 // Algorithm 1; also the greedy on R' of Algorithm 3).
 //
-// Index: coverage counts (how many stored sets contain each node) by a histogram over
-// the store, an exclusive scan into node offsets, and a scatter of set ids into
-// per-node lists (node -> sets).
-// Greedy round r: an argmax over the counts with a warp-shuffle reduction of the key
+// Only nodes with large counts are ever chosen: the counts (a histogram over the store) pick at
+// most CAND candidate nodes, only their lists are built, and the rounds run over them in one
+// cooperative launch, in epochs (see CandState).
+// Where that does not pay, the full index: an exclusive scan of the counts into node offsets,
+// and a scatter of set ids into per-node lists (node -> sets).
+// Its greedy round r: an argmax over the counts with a warp-shuffle reduction of the key
 // (count << 32 | ~node) so ties go to the smallest id and chosen nodes are skipped
 // (counts read four at a time, several loads in flight per thread: the scan runs at
 // DRAM speed when the counts outgrow L2); then every not-yet-covered set in the chosen
