@@ -597,9 +597,9 @@ extern "C" int tim_spread_mc(tim_ctx* ctx, const int32_t* seeds, int k, uint64_t
     slots = std::min<uint64_t>(slots, (uint64_t)ctx->num_sms * nb);
     slots = std::min<uint64_t>(slots, count);
     if (!sm) {
-        void* prev = ctx->mc_bitmap.p;
+        const uint64_t made = ctx->mc_bitmap.made;
         TIM_TRY(tim_ensure(ctx, ctx->mc_bitmap, slots * words * 4));
-        if (ctx->mc_bitmap.p != prev || !ctx->mc_clean) {
+        if (ctx->mc_bitmap.made != made || !ctx->mc_clean) {
             CUDA_TRY(ctx, cudaMemsetAsync(ctx->mc_bitmap.p, 0, ctx->mc_bitmap.bytes, ctx->stream));
             ctx->mc_clean = true;
         }

@@ -1,6 +1,8 @@
 """Workspaces that grow between calls start out clean even when the allocator returns the address
 of the one they replace: few heavy sets first, many later, on one engine, with neighbouring buffers
 of several sizes. RR set sizes and widths equal the oracle's."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -33,3 +35,48 @@ def test_growing_calls(case, capacity, counts):
             off, _, wid = tim.tim_get_rr(eng.ctx)
             assert np.array_equal(np.diff(off), sizes[:count])
             assert np.array_equal(wid, widths[:count])
+
+
+@pytest.mark.parametrize("counts", [(1, 4), (1, 2, 4), (2, 1, 3, 4)])
+def test_growing_cascades(counts):
+    """Cascades whose visited bitmaps (200,004 bytes each) sit in global memory, when the only
+    hole that the allocator has for them holds other data: one bitmap and four start at the same
+    address. Without live edges every cascade activates its seeds and nothing else."""
+    n, k = 1_600_001, 1000
+    seeds = np.random.default_rng(7).choice(n, k, replace=False).astype(np.int32)
+    rowptr = np.ones(n + 1, dtype=np.int64)
+    rowptr[0] = 0
+    import torch
+    torch.zeros(1, device="cuda")
+    rt = ctypes.CDLL("libcudart.so.13")
+    held = []
+
+    def malloc(size):
+        p = ctypes.c_void_p()
+        assert rt.cudaMalloc(ctypes.byref(p), ctypes.c_size_t(size)) == 0
+        held.append(p.value)
+        return p.value
+
+    try:
+        with tim.Engine(0) as eng:
+            tim.tim_load_graph(eng.ctx, n, rowptr, np.array([1], np.int32),
+                               np.zeros(1, np.float32), tim.TIM_IC)
+            # no hole of 200 KB left in the 2 MiB blocks that small allocations share, then one
+            # of 1000 KB
+            for _ in range(1000):
+                if malloc(200 << 10) % (2 << 20) == 0:
+                    break
+            for _ in range(9):
+                malloc(200 << 10)
+            malloc(1000 << 10)
+            hole = malloc(1000 << 10)
+            assert rt.cudaMemset(ctypes.c_void_p(hole), 0xFF, ctypes.c_size_t(1000 << 10)) == 0
+            torch.cuda.synchronize()
+            held.remove(hole)
+            assert rt.cudaFree(ctypes.c_void_p(hole)) == 0
+            for count in counts:
+                _, total, each = tim.tim_spread_mc(eng.ctx, seeds, count, 3, 0, want_counts=True)
+                assert np.array_equal(each, np.full(count, k)) and total == count * k
+    finally:
+        for p in held:
+            rt.cudaFree(ctypes.c_void_p(p))
