@@ -324,6 +324,13 @@ int tim_set_pass2_budget(tim_ctx* ctx, uint64_t budget);
  * returns TIM_ERR_TIMEOUT; the context stays usable. Results do not change. */
 int tim_set_wait_limit(tim_ctx* ctx, uint32_t polls);
 
+/* Device memory that the context's buffers may take in all (default: no limit); an
+ * allocation beyond it fails as one that the device has no room for: TIM_ERR_OOM, after
+ * which the context stays usable (a call that was storing RR sets leaves an empty store).
+ * tim_memory_held: the bytes they take now. */
+int tim_set_memory_limit(tim_ctx* ctx, uint64_t bytes);
+uint64_t tim_memory_held(tim_ctx* ctx);
+
 /* IC sampler: stepped = 0 (default) runs the levels of the heavy-set pass (sets beyond
  * pass 2's capacity) in one persistent launch per batch; stepped = 1 steps them from the
  * host, a launch sequence per level. Results do not change. */

@@ -34,7 +34,10 @@ int tim_cuda_check(tim_ctx* ctx, cudaError_t e, const char* what) {
 }
 
 void tim_free(DevBuf& b) {
-    if (b.p) cudaFree(b.p);
+    if (b.p) {
+        cudaFree(b.p);
+        *b.held -= b.bytes;
+    }
     b.p = nullptr;
     b.bytes = 0;
 }
@@ -46,8 +49,8 @@ int tim_ensure(tim_ctx* ctx, DevBuf& b, size_t bytes) {
     // Allocation is stream-ordered with respect to previous work only through the
     // device-wide synchronisation of cudaMalloc/cudaFree.
     void* p = nullptr;
-    cudaError_t e = cudaMalloc(&p, bytes);
-    if (e != cudaSuccess) {
+    const bool room = bytes <= ctx->mem_limit && ctx->mem_held <= ctx->mem_limit - bytes;
+    if (!room || cudaMalloc(&p, bytes) != cudaSuccess) {
         cudaGetLastError();
         char buf[128];
         snprintf(buf, sizeof buf, "cudaMalloc of %zu bytes failed", bytes);
@@ -56,6 +59,8 @@ int tim_ensure(tim_ctx* ctx, DevBuf& b, size_t bytes) {
     b.p = p;
     b.bytes = bytes;
     b.made++;
+    b.held = &ctx->mem_held;
+    ctx->mem_held += bytes;
     return TIM_OK;
 }
 
@@ -249,6 +254,14 @@ int tim_set_wait_limit(tim_ctx* ctx, uint32_t polls) {
     ctx->wait_limit = polls;
     return TIM_OK;
 }
+
+int tim_set_memory_limit(tim_ctx* ctx, uint64_t bytes) {
+    if (!ctx) return TIM_ERR_ARG;
+    ctx->mem_limit = bytes;
+    return TIM_OK;
+}
+
+uint64_t tim_memory_held(tim_ctx* ctx) { return ctx ? ctx->mem_held : 0; }
 
 int tim_set_heavy_pass(tim_ctx* ctx, int stepped) {
     if (!ctx) return TIM_ERR_ARG;

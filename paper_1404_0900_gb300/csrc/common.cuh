@@ -15,6 +15,7 @@ struct DevBuf {
     void* p = nullptr;
     size_t bytes = 0;
     uint64_t made = 0;  // allocations so far: a new one may be larger at the same address
+    uint64_t* held = nullptr;  // the owning context's count of bytes
 };
 
 // Scalars the kernels update; one block of device memory per context, mirrored in
@@ -139,6 +140,8 @@ struct tim_ctx {
     // polls a block makes at a grid barrier of a persistent kernel before it gives up
     // (the call then fails with TIM_ERR_TIMEOUT)
     unsigned wait_limit = 1u << 24;
+    // bytes of device memory held, and the most that tim_ensure may hold
+    uint64_t mem_held = 0, mem_limit = ~0ull;
     // batch scratch (owner of a multi-query launch / batched greedy)
     DevBuf batch, greedy_batch;
     int last_team = 1;

@@ -2510,6 +2510,31 @@ int launch_multi(tim_ctx* owner, const MultiArgs& ma, int T, unsigned grid) {
 
 }  // namespace
 
+// Room for `entries` members in the store: both arrays, whatever an earlier call that ran out of
+// memory left of them.
+static int ensure_pool(tim_ctx* ctx, uint64_t entries) {
+    TIM_TRY(tim_ensure(ctx, ctx->pool, entries * sizeof(uint32_t)));
+    return tim_ensure(ctx, ctx->pool_sid, entries * sizeof(uint32_t));
+}
+
+static uint64_t pool_entries(const tim_ctx* ctx) {
+    return std::min(ctx->pool.bytes, ctx->pool_sid.bytes) / sizeof(uint32_t);
+}
+
+static int regrow_pool(tim_ctx* ctx, uint64_t used) {
+    tim_free(ctx->pool);
+    tim_free(ctx->pool_sid);
+    return ensure_pool(ctx, used + used / 16 + 4096);
+}
+
+// The store and what refers to it while a call writes into it: empty until the call succeeds, since
+// a failed one may have given its arrays back.
+static void open_store(tim_ctx* ctx) {
+    ctx->n_sets = ctx->members = 0;
+    ctx->select_open = false;
+    ctx->have_kpt = false;
+}
+
 int tim_sample(tim_ctx* ctx, const SampleRequest& req, SampleResult* res) {
     if (!ctx->have_graph) return tim_fail(ctx, TIM_ERR_STATE, "no graph loaded");
     const uint64_t count = req.count;
@@ -2519,15 +2544,13 @@ int tim_sample(tim_ctx* ctx, const SampleRequest& req, SampleResult* res) {
     // Algorithm 2 do not reallocate every round
     uint64_t cap_sets = 1024;
     while (cap_sets < count + 1) cap_sets <<= 1;
+    const bool have_kpt = ctx->have_kpt;
     if (emit) {
+        open_store(ctx);
         TIM_TRY(tim_ensure(ctx, ctx->set_start, cap_sets * sizeof(uint64_t)));
         TIM_TRY(tim_ensure(ctx, ctx->set_len, cap_sets * sizeof(uint32_t)));
         TIM_TRY(tim_ensure(ctx, ctx->set_width, cap_sets * sizeof(uint64_t)));
-        uint64_t want = cap_sets * 8 + 4096;
-        if (ctx->pool.bytes < want * sizeof(uint32_t)) {
-            TIM_TRY(tim_ensure(ctx, ctx->pool, want * sizeof(uint32_t)));
-            TIM_TRY(tim_ensure(ctx, ctx->pool_sid, want * sizeof(uint32_t)));
-        }
+        TIM_TRY(ensure_pool(ctx, cap_sets * 8 + 4096));
     }
     const uint32_t list_cap = (uint32_t)(count + 1);
     TIM_TRY(tim_ensure(ctx, ctx->ovf_list, (size_t)cap_sets * sizeof(uint32_t)));
@@ -2633,7 +2656,7 @@ int tim_sample(tim_ctx* ctx, const SampleRequest& req, SampleResult* res) {
     for (int attempt = 0; attempt < 4; attempt++) {
         a.pool = (uint32_t*)ctx->pool.p;
         a.pool_sid = (uint32_t*)ctx->pool_sid.p;
-        a.pool_cap = emit ? ctx->pool.bytes / sizeof(uint32_t) : 0;
+        a.pool_cap = emit ? pool_entries(ctx) : 0;
         TIM_TRY(tim_zero_scalars(ctx));
         uint64_t live3 = 0;
         bool read = false;
@@ -2675,11 +2698,7 @@ int tim_sample(tim_ctx* ctx, const SampleRequest& req, SampleResult* res) {
         DevScalars& h = *ctx->h_scal;
         if (ctx->model == TIM_IC) h.live[2] = live3;
         if (h.err & TIM_DEV_ERR_POOL) {
-            uint64_t need = h.pool_used + h.pool_used / 16 + 4096;
-            tim_free(ctx->pool);
-            tim_free(ctx->pool_sid);
-            TIM_TRY(tim_ensure(ctx, ctx->pool, need * sizeof(uint32_t)));
-            TIM_TRY(tim_ensure(ctx, ctx->pool_sid, need * sizeof(uint32_t)));
+            TIM_TRY(regrow_pool(ctx, h.pool_used));
             continue;
         }
         if (h.err) {
@@ -2719,7 +2738,7 @@ int tim_sample(tim_ctx* ctx, const SampleRequest& req, SampleResult* res) {
         if (emit) {
             ctx->n_sets = count;
             ctx->members = h.pool_used;
-            ctx->select_open = false;
+            ctx->have_kpt = have_kpt;
         }
         return TIM_OK;
     }
@@ -2830,11 +2849,7 @@ int tim_keep_round(tim_ctx* ctx, uint64_t start, uint64_t count, uint64_t member
     TIM_TRY(tim_ensure(ctx, ctx->set_start, (count + 1) * sizeof(uint64_t)));
     TIM_TRY(tim_ensure(ctx, ctx->set_len, (count + 1) * sizeof(uint32_t)));
     TIM_TRY(tim_ensure(ctx, ctx->set_width, (count + 1) * sizeof(uint64_t)));
-    if (ctx->pool.bytes < members * sizeof(uint32_t) ||
-        ctx->pool_sid.bytes < members * sizeof(uint32_t)) {
-        TIM_TRY(tim_ensure(ctx, ctx->pool, members * sizeof(uint32_t)));
-        TIM_TRY(tim_ensure(ctx, ctx->pool_sid, members * sizeof(uint32_t)));
-    }
+    TIM_TRY(ensure_pool(ctx, members));
     TIM_TRY(tim_zero_scalars(ctx));
     keep_round_kernel<<<(unsigned)(ctx->num_sms * 4), 256, 0, ctx->stream>>>(
         start, count, (const uint32_t*)ctx->pool2.p, (const uint64_t*)ctx->set_start2.p,
@@ -2955,16 +2970,13 @@ int tim_sample_multi(tim_ctx* owner, MultiQuery* qs, int nq, uint64_t seed) {
             total_ic += count;
         total += count;
         if (qs[i].req.flags & SAMPLE_EMIT) {
+            open_store(c);
             uint64_t cap_sets = 1024;
             while (cap_sets < count + 1) cap_sets <<= 1;
             TIM_TRY(tim_ensure(c, c->set_start, cap_sets * sizeof(uint64_t)));
             TIM_TRY(tim_ensure(c, c->set_len, cap_sets * sizeof(uint32_t)));
             TIM_TRY(tim_ensure(c, c->set_width, cap_sets * sizeof(uint64_t)));
-            const uint64_t want = cap_sets * 8 + 4096;
-            if (c->pool.bytes < want * sizeof(uint32_t)) {
-                TIM_TRY(tim_ensure(c, c->pool, want * sizeof(uint32_t)));
-                TIM_TRY(tim_ensure(c, c->pool_sid, want * sizeof(uint32_t)));
-            }
+            TIM_TRY(ensure_pool(c, cap_sets * 8 + 4096));
         }
     }
     prefix[nq] = total_ic;
@@ -3061,7 +3073,7 @@ int tim_sample_multi(tim_ctx* owner, MultiQuery* qs, int nq, uint64_t seed) {
             const bool emit = r.flags & SAMPLE_EMIT;
             d.pool = emit ? (uint32_t*)c->pool.p : nullptr;
             d.pool_sid = emit ? (uint32_t*)c->pool_sid.p : nullptr;
-            d.pool_cap = emit ? c->pool.bytes / sizeof(uint32_t) : 0;
+            d.pool_cap = emit ? pool_entries(c) : 0;
             d.set_start = (uint64_t*)c->set_start.p;
             d.set_len = (uint32_t*)c->set_len.p;
             d.set_width = (uint64_t*)c->set_width.p;
@@ -3139,12 +3151,7 @@ int tim_sample_multi(tim_ctx* owner, MultiQuery* qs, int nq, uint64_t seed) {
         bool regrow = false;
         for (int i = 0; i < nq; i++) {
             if (h_scal[i].err & TIM_DEV_ERR_POOL) {
-                tim_ctx* c = qs[i].ctx;
-                const uint64_t need = h_scal[i].pool_used + h_scal[i].pool_used / 16 + 4096;
-                tim_free(c->pool);
-                tim_free(c->pool_sid);
-                TIM_TRY(tim_ensure(c, c->pool, need * sizeof(uint32_t)));
-                TIM_TRY(tim_ensure(c, c->pool_sid, need * sizeof(uint32_t)));
+                TIM_TRY(regrow_pool(qs[i].ctx, h_scal[i].pool_used));
                 regrow = true;
             } else if (h_scal[i].err) {
                 h_err |= h_scal[i].err;

@@ -1137,6 +1137,9 @@ int tim_greedy_begin(tim_ctx* ctx) {
 int tim_greedy_take(tim_ctx* ctx, int32_t v, uint64_t* newly_covered) {
     // the key cover_kernel decodes: any count, node v
     const unsigned long long key = (1ull << 32) | (unsigned long long)(~(uint32_t)v);
+    // (a selection between the steps that ran out of memory may have given these back)
+    TIM_TRY(tim_ensure(ctx, ctx->best, sizeof(unsigned long long)));
+    TIM_TRY(tim_ensure(ctx, ctx->seeds_dev, sizeof(int32_t)));
     TIM_TRY(tim_zero_scalars(ctx));
     DevScalars* ds = tim_dscal(ctx);
     set_key_kernel<<<1, 1, 0, ctx->stream>>>((unsigned long long*)ctx->best.p, key);

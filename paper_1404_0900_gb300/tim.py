@@ -130,6 +130,8 @@ _SIGS = {
     "tim_set_team_factor": (C.c_int, [_P, C.c_int]),
     "tim_set_pass1_capacity": (C.c_int, [_P, C.c_int]),
     "tim_set_wait_limit": (C.c_int, [_P, C.c_uint32]),
+    "tim_set_memory_limit": (C.c_int, [_P, C.c_uint64]),
+    "tim_memory_held": (C.c_uint64, [_P]),
     "tim_set_pass2_budget": (C.c_int, [_P, C.c_uint64]),
     "tim_set_heavy_pass": (C.c_int, [_P, C.c_int]),
     "tim_set_query_tag": (C.c_int, [_P, C.c_uint32]),
@@ -497,6 +499,14 @@ def tim_set_pass2_budget(ctx, budget: int):
 
 def tim_set_wait_limit(ctx, polls: int):
     _check(ctx, lib().tim_set_wait_limit(ctx, polls))
+
+
+def tim_set_memory_limit(ctx, limit: int):
+    _check(ctx, lib().tim_set_memory_limit(ctx, limit))
+
+
+def tim_memory_held(ctx) -> int:
+    return int(lib().tim_memory_held(ctx))
 
 
 def tim_set_heavy_pass(ctx, stepped: bool):

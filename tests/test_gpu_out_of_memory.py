@@ -1,0 +1,94 @@
+"""Calls that run out of device memory at any of their allocations (a limit on what the context
+holds stands in for a full device): TIM_ERR_OOM, an empty RR-set store, and a context whose next
+calls are right. RR sets equal the oracle's."""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_1404_0900_gb300 import inputs, tim
+
+pytestmark = pytest.mark.gpu
+FREE = 2 ** 64 - 1
+
+
+def _case(model):
+    g = inputs.chung_lu(3_001, 30_000, 2.1, seed=3)
+    if model == tim.TIM_IC:
+        w = inputs.weighted_cascade(g)
+    else:
+        w = inputs.lt_random_normalised(g, seed=4)
+    return g, w, O.load_graph(g.n, g.rowptr, g.dst, w, model)
+
+
+def _load(eng, g, w, model):
+    tim.tim_load_graph(eng.ctx, g.n, g.rowptr, g.dst, w, model)
+
+
+def _sorted(off, mem):
+    return [np.sort(mem[off[i]:off[i + 1]]) for i in range(len(off) - 1)]
+
+
+@pytest.mark.parametrize("model", [tim.TIM_IC, tim.TIM_LT])
+def test_sampling_without_room(model):
+    g, w, og = _case(model)
+    sid, few, many = O.make_sid(1, 5, 0), 500, 100_000
+    off, mem, wid = O.sample(og, 3, sid, many)
+    sets = _sorted(off, mem)
+
+    def check(eng, count):
+        o, m, x = tim.tim_get_rr(eng.ctx)
+        assert np.array_equal(o, off[:count + 1]) and np.array_equal(x, wid[:count])
+        assert all(np.array_equal(a, b) for a, b in zip(_sorted(o, m), sets))
+
+    with tim.Engine(0) as eng:
+        _load(eng, g, w, model)
+        tim.tim_sample_rr(eng.ctx, many, 3, sid)
+        full = tim.tim_memory_held(eng.ctx)
+    failed = 0
+    with tim.Engine(0) as eng:
+        _load(eng, g, w, model)
+        tim.tim_sample_rr(eng.ctx, few, 3, sid)
+        first = tim.tim_memory_held(eng.ctx)
+        assert first < full
+        for limit in np.linspace(first, full, 60).astype(np.int64):
+            tim.tim_sample_rr(eng.ctx, few, 3, sid)
+            tim.tim_kpt_estimate(eng.ctx, 3, 1.0, 3)
+            tim.tim_sample_rr(eng.ctx, few, 3, sid)
+            tim.tim_set_memory_limit(eng.ctx, int(limit))
+            try:
+                tim.tim_sample_rr(eng.ctx, many, 3, sid)
+                check(eng, many)
+            except tim.TimError as e:
+                assert e.code == tim.TIM_ERR_OOM
+                failed += 1
+                assert tim.tim_rr_size(eng.ctx) == (0, 0)
+            tim.tim_set_memory_limit(eng.ctx, FREE)
+            if tim.tim_rr_size(eng.ctx) == (0, 0):
+                assert not tim.tim_coverage_counts(eng.ctx, g.n).any()
+                seeds, _, cov = tim.tim_node_select(eng.ctx, 3)
+                assert seeds.tolist() == [0, 1, 2] and cov == 0
+                with pytest.raises(tim.TimError):
+                    tim.tim_refine_kpt(eng.ctx, 3, 1.0, 0.3, 3)
+                tim.tim_sample_rr(eng.ctx, few, 3, sid)
+                check(eng, few)
+        tim.tim_sample_rr(eng.ctx, many, 3, sid)
+        check(eng, many)
+    assert failed > 0
+
+
+def test_steps_after_a_selection_without_room():
+    g, w, og = _case(tim.TIM_IC)
+    sid = O.make_sid(1, 5, 0)
+    off, mem, _ = O.sample(og, 3, sid, 2000)
+    counts = np.bincount(mem, minlength=g.n)
+    v = int(np.argmax(counts))
+    with tim.Engine(0) as eng:
+        _load(eng, g, w, tim.TIM_IC)
+        tim.tim_sample_rr(eng.ctx, 2000, 3, sid)
+        tim.tim_select_begin(eng.ctx)
+        tim.tim_set_memory_limit(eng.ctx, 0)
+        with pytest.raises(tim.TimError):
+            tim.tim_node_select(eng.ctx, g.n)
+        tim.tim_set_memory_limit(eng.ctx, FREE)
+        assert np.array_equal(tim.tim_select_counts(eng.ctx, g.n), counts)
+        assert tim.tim_select_take(eng.ctx, v) == counts[v]
