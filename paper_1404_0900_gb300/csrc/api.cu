@@ -49,9 +49,14 @@ int tim_ensure(tim_ctx* ctx, DevBuf& b, size_t bytes) {
     // Allocation is stream-ordered with respect to previous work only through the
     // device-wide synchronisation of cudaMalloc/cudaFree.
     void* p = nullptr;
-    const bool room = bytes <= ctx->mem_limit && ctx->mem_held <= ctx->mem_limit - bytes;
-    if (!room || cudaMalloc(&p, bytes) != cudaSuccess) {
+    auto allocate = [&] {
+        if (bytes > ctx->mem_limit || ctx->mem_held > ctx->mem_limit - bytes) return false;
+        if (cudaMalloc(&p, bytes) == cudaSuccess) return true;
         cudaGetLastError();
+        return false;
+    };
+    // the second store only saves calls: it makes room for what is needed
+    if (!allocate() && (ctx->rounds_kept || !tim_drop_rounds(ctx, false) || !allocate())) {
         char buf[128];
         snprintf(buf, sizeof buf, "cudaMalloc of %zu bytes failed", bytes);
         return tim_fail(ctx, TIM_ERR_OOM, buf);
@@ -776,21 +781,22 @@ static void kpt_keep_state(tim_ctx* c, const KptJob& J, uint64_t seed) {
 // together; after them a call takes every round that stops only if the mean turns out at
 // least twice ktot / ctot + 4 / ctot (kappa lies in [0, 1], so that few sets leave the mean
 // that uncertain), and, while that is at most KPT_GROUP_SETS sets in all, the rounds up to
-// the expected stop. Sets past the stop are wasted, which this bounds; the rounds that are
-// reported and kept are Algorithm 2's. Algorithm 2 one round per call and grouped: R-MAT 20,
+// the expected stop. Sets past the stop are wasted, which this bounds, and a call of more than
+// KPT_CALL_SETS gains nothing from more; the rounds that are reported and kept are Algorithm 2's. Algorithm 2 one round per call and grouped: R-MAT 20,
 // weighted cascade, k = 50 (5 rounds) 6.7 -> 3.3 ms; Chung-Lu 4.16M nodes, trivalency (14
 // rounds) 24.5 -> 18.4 ms; R-MAT 14, k = 10 (4 rounds) 1.35 -> 0.84 ms.
-constexpr uint64_t KPT_GROUP_SETS = 16384;
+constexpr uint64_t KPT_GROUP_SETS = 16384, KPT_CALL_SETS = 1 << 22;
 
 static int kpt_group(int64_t n, double ell, int i, int rounds, double ktot, double ctot) {
-    if (i == 1) return std::min(2, rounds);
+    if (i == 1)
+        return rounds > 1 && tim_host_c_i(n, ell, 1) + tim_host_c_i(n, ell, 2) <= KPT_GROUP_SETS ? 2 : 1;
     auto round_of = [](double mean) { return mean > 0.0 ? (int)floor(-log2(mean)) : 62; };
     const int sure = round_of((ktot + 4.0) / ctot) - 1, stop = round_of(ktot / ctot) + 1;
     int g = 1;
     uint64_t total = tim_host_c_i(n, ell, i);
     while (i + g <= rounds && g < SID_ROUNDS) {
         const uint64_t more = total + tim_host_c_i(n, ell, i + g);
-        if (i + g > stop || more > 0x7FFFFFFFull || (i + g > sure && more > KPT_GROUP_SETS)) break;
+        if (i + g > stop || more > (i + g > sure ? KPT_GROUP_SETS : KPT_CALL_SETS)) break;
         total = more;
         g++;
     }
@@ -815,12 +821,13 @@ int tim_kpt_estimate(tim_ctx* ctx, int k, double ell, uint64_t seed, double* kpt
     ctx->kpt_width = 0;
     ctx->n_sets = ctx->members = 0;
     double ktot = 0.0, ctot = 0.0;  // kappa sum and sets so far
+    bool group = true;              // until there is no memory for several rounds
     for (int i = 1; i <= rounds && !ctx->kpt_round;) {
         SampleRequest req;
         req.seed = seed;
         req.sid0 = make_sid(1, (uint64_t)i, (uint64_t)ctx->query_tag << 32);
         req.k = k;
-        const int g = kpt_group(ctx->n, ell, i, rounds, ktot, ctot);
+        const int g = group ? kpt_group(ctx->n, ell, i, rounds, ktot, ctot) : 1;
         uint64_t c[SID_ROUNDS], start = 0;
         RoundSums sum[SID_ROUNDS];
         for (int r = 0; r < g; r++) c[r] = tim_host_c_i(ctx->n, ell, i + r);
@@ -833,7 +840,13 @@ int tim_kpt_estimate(tim_ctx* ctx, int k, double ell, uint64_t seed, double* kpt
             sum[0].lo = (unsigned long long)res.ksum;
             sum[0].width = res.wsum;
         } else {
-            TIM_TRY(tim_sample_rounds(ctx, req, c, g, sum));
+            const int rc = tim_sample_rounds(ctx, req, c, g, sum);
+            if (rc == TIM_ERR_OOM) {
+                tim_drop_rounds(ctx, true);
+                group = false;
+                continue;
+            }
+            TIM_TRY(rc);
         }
         for (int r = 0; r < g && !ctx->kpt_round; r++) {
             const unsigned __int128 S = ((unsigned __int128)sum[r].hi << 64) | sum[r].lo;
@@ -846,8 +859,17 @@ int tim_kpt_estimate(tim_ctx* ctx, int k, double ell, uint64_t seed, double* kpt
                 ctx->kpt_round = i + r;
             }
             // the stopping or last round's sets become the store
-            if (g > 1 && (ctx->kpt_round || i + r == rounds))
-                TIM_TRY(tim_keep_round(ctx, start, c[r], sum[r].members));
+            if (g > 1 && (ctx->kpt_round || i + r == rounds)) {
+                int rc = tim_keep_round(ctx, start, c[r], sum[r].members);
+                if (rc == TIM_ERR_OOM) {  // sampled again into the only store
+                    tim_drop_rounds(ctx, true);
+                    req.sid0 += (uint64_t)r << 48;
+                    req.count = c[r];
+                    req.flags = SAMPLE_EMIT;
+                    rc = tim_sample(ctx, req, nullptr);
+                }
+                TIM_TRY(rc);
+            }
             start += c[r];
             ktot += ldexp((double)S, -63);
             ctot += (double)c[r];

@@ -83,6 +83,7 @@ struct tim_ctx {
     DevBuf set_width;  // uint64[n_sets]
     // second store: the rounds of Algorithm 2 sampled in one call, and their sums
     DevBuf pool2, pool_sid2, set_start2, set_len2, set_width2, round_sums;
+    bool rounds_kept = false;  // tim_keep_round may still take one of them
 
     // greedy / index
     DevBuf counts;     // int32[n]
@@ -301,6 +302,9 @@ int tim_sample_rounds(tim_ctx* ctx, SampleRequest req, const uint64_t* counts, i
 // Makes round r of the last tim_sample_rounds (the sets [start, start + count), `members` of
 // them in all) the RR-set store.
 int tim_keep_round(tim_ctx* ctx, uint64_t start, uint64_t count, uint64_t members);
+// Gives the second store back, and (all) the sampler's workspaces that grow with a call's sets.
+// Returns whether the second store held any memory.
+bool tim_drop_rounds(tim_ctx* ctx, bool all);
 // Third tier for the heavy IC sets list[0 .. count) (sample_bulk.cu). With hand (may be
 // null), the set at list position i < hcap starts from the state pass 2 left at
 // hand + i hw: queue length, position of the batch to redo, then the queue.

@@ -2533,6 +2533,7 @@ static void open_store(tim_ctx* ctx) {
     ctx->n_sets = ctx->members = 0;
     ctx->select_open = false;
     ctx->have_kpt = false;
+    ctx->rounds_kept = false;
 }
 
 int tim_sample(tim_ctx* ctx, const SampleRequest& req, SampleResult* res) {
@@ -2819,6 +2820,21 @@ void swap_stores(tim_ctx* ctx) {
 
 }  // namespace
 
+bool tim_drop_rounds(tim_ctx* ctx, bool all) {
+    bool any = false;
+    for (DevBuf* b : {&ctx->pool2, &ctx->pool_sid2, &ctx->set_start2, &ctx->set_len2,
+                      &ctx->set_width2}) {
+        any = any || b->p;
+        tim_free(*b);
+    }
+    if (all)
+        for (DevBuf* b : {&ctx->ovf_list, &ctx->ovf_list2, &ctx->hand, &ctx->hand2,
+                          &ctx->bulk_bitmap, &ctx->bulk_slot})
+            tim_free(*b);
+    ctx->rounds_kept = false;
+    return any;
+}
+
 int tim_sample_rounds(tim_ctx* ctx, SampleRequest req, const uint64_t* counts, int rounds,
                       RoundSums* sums) {
     req.rounds = rounds;
@@ -2834,6 +2850,7 @@ int tim_sample_rounds(tim_ctx* ctx, SampleRequest req, const uint64_t* counts, i
     swap_stores(ctx);
     ctx->n_sets = ctx->members = 0;
     TIM_TRY(rc);
+    ctx->rounds_kept = true;
     TIM_TRY(tim_ensure(ctx, ctx->round_sums, SID_ROUNDS * sizeof(RoundSums)));
     CUDA_TRY(ctx, cudaMemsetAsync(ctx->round_sums.p, 0, rounds * sizeof(RoundSums), ctx->stream));
     round_sums_kernel<<<dim3(ctx->num_sms, rounds), 128, 0, ctx->stream>>>(
@@ -2859,6 +2876,7 @@ int tim_keep_round(tim_ctx* ctx, uint64_t start, uint64_t count, uint64_t member
     LAUNCH_CHECK(ctx, "keep_round_kernel");
     ctx->n_sets = count;
     ctx->members = members;
+    ctx->rounds_kept = false;
     return TIM_OK;
 }
 

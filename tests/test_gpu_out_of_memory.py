@@ -92,3 +92,53 @@ def test_steps_after_a_selection_without_room():
         tim.tim_set_memory_limit(eng.ctx, FREE)
         assert np.array_equal(tim.tim_select_counts(eng.ctx, g.n), counts)
         assert tim.tim_select_take(eng.ctx, v) == counts[v]
+
+
+@pytest.mark.parametrize("ell,dense", [(1.0, False), (300.0, False), (1.0, True), (8000.0, True)])
+def test_algorithm_2_in_the_memory_of_its_largest_round(ell, dense):
+    """Several rounds in one call are for speed only: in the memory that its rounds take one
+    after another Algorithm 2 gives the same estimate and leaves the same store."""
+    k, seed = 2, 3
+    if dense:  # stops in round 1 or 2
+        g = inputs.complete(60)
+        w = inputs.constant(g, 0.5)
+    else:
+        g = inputs.chung_lu(3_001, 12_000, 2.1, seed=3)
+        w = inputs.constant(g, 0.01)
+    with tim.Engine(0) as eng:
+        _load(eng, g, w, tim.TIM_IC)
+        want = tim.tim_kpt_estimate(eng.ctx, k, ell, seed)
+        off, mem, wid = tim.tim_get_rr(eng.ctx)
+    last = want[1] or O.kpt_rounds(g.n)
+    assert (last <= 2) == dense
+    with tim.Engine(0) as eng:
+        _load(eng, g, w, tim.TIM_IC)
+        for i in range(1, last + 1):
+            tim.tim_sample_rr(eng.ctx, O.c_i(g.n, ell, i), seed, O.make_sid(1, i, 0))
+        room = tim.tim_memory_held(eng.ctx)
+    with tim.Engine(0) as eng:
+        _load(eng, g, w, tim.TIM_IC)
+        tim.tim_set_memory_limit(eng.ctx, room + (64 << 10))
+        assert tim.tim_kpt_estimate(eng.ctx, k, ell, seed) == want
+        o, m, x = tim.tim_get_rr(eng.ctx)
+        assert np.array_equal(o, off) and np.array_equal(x, wid)
+        assert all(np.array_equal(a, b) for a, b in zip(_sorted(o, m), _sorted(off, mem)))
+
+
+def test_the_second_store_makes_room():
+    """What Algorithm 2 keeps for its grouped rounds does not take memory from a larger call."""
+    g, w, og = _case(tim.TIM_IC)
+    sid, count = O.make_sid(1, 5, 0), 60_000
+    with tim.Engine(0) as eng:
+        _load(eng, g, w, tim.TIM_IC)
+        tim.tim_sample_rr(eng.ctx, count, 3, sid)
+        off, mem, _ = tim.tim_get_rr(eng.ctx)
+        room = tim.tim_memory_held(eng.ctx)
+    with tim.Engine(0) as eng:
+        _load(eng, g, w, tim.TIM_IC)
+        tim.tim_kpt_estimate(eng.ctx, 2, 1.0, 3)
+        tim.tim_set_memory_limit(eng.ctx, room + (64 << 10))
+        tim.tim_sample_rr(eng.ctx, count, 3, sid)
+        o, m, _ = tim.tim_get_rr(eng.ctx)
+        assert np.array_equal(o, off)
+        assert all(np.array_equal(a, b) for a, b in zip(_sorted(o, m), _sorted(off, mem)))
