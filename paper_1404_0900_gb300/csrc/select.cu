@@ -17,6 +17,7 @@
 #include <stddef.h>
 
 #include <algorithm>
+#include <utility>
 #include <vector>
 
 #include "common.cuh"
@@ -1007,6 +1008,21 @@ int tim_greedy(tim_ctx* ctx, int k, int32_t* host_seeds, uint64_t* covered) {
         }
         cand = nb > 0;
     }
+    unsigned long long chunk_cap = 2 * (members / CG_CHUNK) + 1;
+    if (cand) {  // what the full index does without; it also does where this has no room
+        const std::pair<DevBuf*, size_t> need[] = {
+            {&ctx->set_rec, (ctx->n_sets + 1) * sizeof(uint4)},
+            {&ctx->cand, sizeof(CandState)},
+            {&ctx->greedy_chunks, chunk_cap * sizeof(unsigned long long)},
+            {&ctx->node_sets, (members + 1) * sizeof(uint32_t)}};
+        for (const auto& b : need) {
+            const int rc = cand ? tim_ensure(ctx, *b.first, b.second) : TIM_OK;
+            if (rc != TIM_OK && rc != TIM_ERR_OOM) return rc;
+            cand = cand && rc == TIM_OK;
+        }
+        if (!cand)
+            for (DevBuf* b : {&ctx->set_rec, &ctx->cand, &ctx->greedy_chunks}) tim_free(*b);
+    }
     if (!cand) {
         TIM_TRY(tim_build_index(ctx));
         return greedy_full(ctx, k, 0, host_seeds, covered);
@@ -1014,11 +1030,7 @@ int tim_greedy(tim_ctx* ctx, int k, int32_t* host_seeds, uint64_t* covered) {
     TIM_TRY(tim_ensure(ctx, ctx->covered, ctx->n_sets + 1));
     TIM_TRY(tim_ensure(ctx, ctx->chosen, n + 1));
     TIM_TRY(tim_ensure(ctx, ctx->seeds_dev, (size_t)k * sizeof(int32_t)));
-    TIM_TRY(tim_ensure(ctx, ctx->node_sets, (members + 1) * sizeof(uint32_t)));
     TIM_TRY(tim_ensure(ctx, ctx->greedy_bar, sizeof(GridBarrier)));
-    TIM_TRY(tim_ensure(ctx, ctx->cand, sizeof(CandState)));
-    unsigned long long chunk_cap = 2 * (members / CG_CHUNK) + 1;
-    TIM_TRY(tim_ensure(ctx, ctx->greedy_chunks, chunk_cap * sizeof(unsigned long long)));
     TIM_TRY(tim_ensure(ctx, ctx->greedy_nchunk, (size_t)k * sizeof(unsigned long long)));
     CUDA_TRY(ctx, cudaMemsetAsync(ctx->covered.p, 0, ctx->n_sets + 1, ctx->stream));
     CUDA_TRY(ctx, cudaMemsetAsync(ctx->chosen.p, 0, n + 1, ctx->stream));
@@ -1036,7 +1048,6 @@ int tim_greedy(tim_ctx* ctx, int k, int32_t* host_seeds, uint64_t* covered) {
         members <= CAND_SOLO
             ? 1u
             : (unsigned)std::min<uint64_t>(members / 8192 + 1, (uint64_t)ctx->num_sms);
-    TIM_TRY(tim_ensure(ctx, ctx->set_rec, (ctx->n_sets + 1) * sizeof(uint4)));
     if (ctx->n_sets) {
         set_rec_kernel<<<(unsigned)std::min<uint64_t>(ctx->n_sets / 256 + 1,
                                                       (uint64_t)ctx->num_sms * 8),

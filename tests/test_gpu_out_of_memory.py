@@ -142,3 +142,27 @@ def test_the_second_store_makes_room():
         o, m, _ = tim.tim_get_rr(eng.ctx)
         assert np.array_equal(o, off)
         assert all(np.array_equal(a, b) for a, b in zip(_sorted(o, m), _sorted(off, mem)))
+
+
+@pytest.mark.parametrize("k", [1, 40])
+def test_selection_in_the_memory_of_the_full_index(k):
+    """The greedy over candidates gives way to the full index where it has no room."""
+    g, w, og = _case(tim.TIM_IC)
+    sid, count = O.make_sid(1, 5, 0), 60_000
+    with tim.Engine(0) as eng:
+        _load(eng, g, w, tim.TIM_IC)
+        tim.tim_sample_rr(eng.ctx, count, 3, sid)
+        tim.tim_select_begin(eng.ctx)  # an open selection keeps to the full index
+        want = tim.tim_node_select(eng.ctx, k)
+        room = tim.tim_memory_held(eng.ctx)
+    with tim.Engine(0) as eng:
+        _load(eng, g, w, tim.TIM_IC)
+        tim.tim_sample_rr(eng.ctx, count, 3, sid)
+        tim.tim_set_memory_limit(eng.ctx, room + (4 << 10))
+        got = tim.tim_node_select(eng.ctx, k)
+        assert np.array_equal(got[0], want[0]) and got[1:] == want[1:]
+        tim.tim_set_memory_limit(eng.ctx, FREE)
+        got = tim.tim_node_select(eng.ctx, k)
+        assert np.array_equal(got[0], want[0]) and got[1:] == want[1:]
+    off, mem, _ = O.sample(og, 3, sid, count)
+    assert np.array_equal(want[0], O.greedy(g.n, off, mem, k)[0])
