@@ -210,7 +210,7 @@ int tim_destroy(tim_ctx* ctx) {
                       &ctx->ld_in_w,
                       &ctx->bulk_F,    &ctx->bulk_M,    &ctx->bulk_ng,   &ctx->bulk_gp,
                       &ctx->bulk_scal, &ctx->batch,     &ctx->greedy_batch,
-                      &ctx->out_rowptr, &ctx->out_row, &ctx->out_rec,  &ctx->out_pos,  &ctx->mc_bitmap,
+                      &ctx->out_row, &ctx->out_rec,  &ctx->out_pos,  &ctx->mc_bitmap,
                       &ctx->mc_queue,  &ctx->mc_live,
                       &ctx->mc_counts, &ctx->mc_seeds,  &ctx->mc_scal};
     for (DevBuf* b : bufs) tim_free(*b);

@@ -156,9 +156,10 @@ struct tim_ctx {
     // built from G^T on first use, with the out-record of every in-CSR position;
     // per-block visited bitmaps (kept all-zero between calls), queues and live-edge bits;
     // cascade counts, seeds, counters
-    DevBuf out_rowptr, out_row, out_rec, out_pos, mc_bitmap, mc_queue, mc_live, mc_counts, mc_seeds,
+    DevBuf out_row, out_rec, out_pos, mc_bitmap, mc_queue, mc_live, mc_counts, mc_seeds,
         mc_scal;
     bool have_out = false, mc_clean = false;
+    bool mc_walk_only = false;  // this graph's worlds found no room
 
     // generic scratch for scans and sorts
     DevBuf scratch_a, scratch_b, scratch_c, scratch_d, scratch_e, scratch_f;

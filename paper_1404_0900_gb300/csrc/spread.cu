@@ -522,7 +522,9 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) mc_cascade_kernel(McArgs a) {
 int build_out_records(tim_ctx* ctx, bool draws) {
     if (ctx->have_out) return TIM_OK;
     const uint64_t n = (uint64_t)ctx->n, m = (uint64_t)ctx->m;
-    TIM_TRY(tim_ensure(ctx, ctx->out_rowptr, (n + 1) * sizeof(uint64_t)));
+    // (the 64-bit offsets are needed here alone)
+    TIM_TRY(tim_ensure(ctx, ctx->scratch_d, (n + 1) * sizeof(uint64_t)));
+    auto* off = (uint64_t*)ctx->scratch_d.p;
     TIM_TRY(tim_ensure(ctx, ctx->out_rec, std::max<uint64_t>(m, 1) * sizeof(uint2)));
     if (draws)
         TIM_TRY(tim_ensure(ctx, ctx->out_pos, std::max<uint64_t>(m, 1) * sizeof(uint32_t)));
@@ -534,16 +536,15 @@ int build_out_records(tim_ctx* ctx, bool draws) {
         out_count_kernel<<<G, 256, 0, ctx->stream>>>((const uint32_t*)ctx->src.p, m, cnt);
         LAUNCH_CHECK(ctx, "out_count_kernel");
     }
-    TIM_TRY(tim_scan_u32_to_u64(ctx, cnt, (uint64_t*)ctx->out_rowptr.p, n));
+    TIM_TRY(tim_scan_u32_to_u64(ctx, cnt, off, n));
     TIM_TRY(tim_ensure(ctx, ctx->out_row, n * sizeof(uint2)));
-    out_rows_kernel<<<G, 256, 0, ctx->stream>>>((const uint64_t*)ctx->out_rowptr.p, n,
-                                                (uint2*)ctx->out_row.p);
+    out_rows_kernel<<<G, 256, 0, ctx->stream>>>(off, n, (uint2*)ctx->out_row.p);
     LAUNCH_CHECK(ctx, "out_rows_kernel");
     CUDA_TRY(ctx, cudaMemsetAsync(cnt, 0, (n + 1) * sizeof(uint32_t), ctx->stream));
     if (m) {
         out_scatter_kernel<<<G, 256, 0, ctx->stream>>>(
-            (const uint64_t*)ctx->rowptr.p, (const uint32_t*)ctx->src.p, n,
-            (const uint64_t*)ctx->out_rowptr.p, cnt, (uint2*)ctx->out_rec.p,
+            (const uint64_t*)ctx->rowptr.p, (const uint32_t*)ctx->src.p, n, off, cnt,
+            (uint2*)ctx->out_rec.p,
             draws ? (uint32_t*)ctx->out_pos.p : nullptr);
         LAUNCH_CHECK(ctx, "out_scatter_kernel");
     }
@@ -586,16 +587,32 @@ extern "C" int tim_spread_mc(tim_ctx* ctx, const int32_t* seeds, int k, uint64_t
     CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, threads, smem));
     nb = std::max(nb, 1);
     // queue, live bits and (outside shared memory) bitmap per resident block, within
-    // ~4 GiB; worlds are drawn when that leaves at least a block per SM
+    // ~4 GiB; worlds are drawn when that leaves at least a block per SM and the device has room
+    // for them
     const uint64_t budget = 4ull << 30;
     const uint64_t live_words = ((uint64_t)ctx->m + 127) / 128 * 4;
     const uint64_t base = n * 4 + (sm ? 0 : words * 4);
-    const bool draws = budget / (base + live_words * 4) >= (uint64_t)ctx->num_sms;
-    TIM_TRY(build_out_records(ctx, draws));
-    const uint64_t per_slot = base + (draws ? live_words * 4 : 0);
-    uint64_t slots = std::max<uint64_t>(1, budget / per_slot);
-    slots = std::min<uint64_t>(slots, (uint64_t)ctx->num_sms * nb);
-    slots = std::min<uint64_t>(slots, count);
+    bool draws = !ctx->mc_walk_only && budget / (base + live_words * 4) >= (uint64_t)ctx->num_sms;
+    uint64_t slots = 0;
+    // the records, queues and live bits of as many blocks as the budget holds
+    auto prepare = [&]() -> int {
+        TIM_TRY(build_out_records(ctx, draws));
+        const uint64_t per_slot = base + (draws ? live_words * 4 : 0);
+        slots = std::max<uint64_t>(1, budget / per_slot);
+        slots = std::min<uint64_t>(slots, (uint64_t)ctx->num_sms * nb);
+        slots = std::min<uint64_t>(slots, count);
+        TIM_TRY(tim_ensure(ctx, ctx->mc_queue, slots * n * 4));
+        return tim_ensure(ctx, ctx->mc_live, draws ? slots * live_words * 4 : 16);
+    };
+    int rc = prepare();
+    if (rc == TIM_ERR_OOM && draws) {
+        tim_free(ctx->out_pos);
+        tim_free(ctx->mc_live);
+        ctx->have_out = draws = false;
+        rc = prepare();
+        ctx->mc_walk_only = rc == TIM_OK;
+    }
+    TIM_TRY(rc);
     if (!sm) {
         const uint64_t made = ctx->mc_bitmap.made;
         TIM_TRY(tim_ensure(ctx, ctx->mc_bitmap, slots * words * 4));
@@ -604,8 +621,6 @@ extern "C" int tim_spread_mc(tim_ctx* ctx, const int32_t* seeds, int k, uint64_t
             ctx->mc_clean = true;
         }
     }
-    TIM_TRY(tim_ensure(ctx, ctx->mc_queue, slots * n * 4));
-    TIM_TRY(tim_ensure(ctx, ctx->mc_live, draws ? slots * live_words * 4 : 16));
     TIM_TRY(tim_ensure(ctx, ctx->mc_counts, count * 4));
     TIM_TRY(tim_ensure(ctx, ctx->mc_seeds, std::max(k, 1) * sizeof(int32_t)));
     TIM_TRY(tim_ensure(ctx, ctx->mc_scal, 2 * sizeof(unsigned long long)));

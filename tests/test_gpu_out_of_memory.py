@@ -166,3 +166,30 @@ def test_selection_in_the_memory_of_the_full_index(k):
         assert np.array_equal(got[0], want[0]) and got[1:] == want[1:]
     off, mem, _ = O.sample(og, 3, sid, count)
     assert np.array_equal(want[0], O.greedy(g.n, off, mem, k)[0])
+
+
+@pytest.mark.parametrize("model", [tim.TIM_IC, tim.TIM_LT])
+def test_cascades_without_room_for_worlds(model):
+    """Cascades need the out-records, a queue per block and the counts; whole worlds (the
+    out-record of every in-edge, a bit per out-record and block) only where there is room."""
+    g, w, og = _case(model)
+    count, seeds = 400, np.arange(30, dtype=np.int32)
+    counts, total = O.spread_mc(og, seeds, count, 3, 0)
+    with tim.Engine(0) as eng:
+        _load(eng, g, w, model)
+        one = tim.tim_spread_mc(eng.ctx, seeds, count, 3, 0, want_counts=True)
+        full = tim.tim_memory_held(eng.ctx)
+    with tim.Engine(0) as eng:
+        _load(eng, g, w, model)
+        blocks = min(count, 2 * 160)
+        room = tim.tim_memory_held(eng.ctx) + 4 * blocks * g.n + 12 * (g.n + 1) + 8 * g.m + 4 * count
+        assert room + (64 << 10) < full
+        tim.tim_set_memory_limit(eng.ctx, room + (64 << 10))
+        for _ in range(2):
+            got = tim.tim_spread_mc(eng.ctx, seeds, count, 3, 0, want_counts=True)
+            assert got[1] == one[1] == total
+            assert np.array_equal(got[2], counts) and np.array_equal(one[2], counts)
+        tim.tim_set_memory_limit(eng.ctx, FREE)
+        _load(eng, g, w, model)
+        got = tim.tim_spread_mc(eng.ctx, seeds, count, 3, 0, want_counts=True)
+        assert got[1] == total and np.array_equal(got[2], counts)
