@@ -212,7 +212,7 @@ int tim_destroy(tim_ctx* ctx) {
                       &ctx->bulk_scal, &ctx->batch,     &ctx->greedy_batch,
                       &ctx->out_row, &ctx->out_rec,  &ctx->out_pos,  &ctx->mc_bitmap,
                       &ctx->mc_queue,  &ctx->mc_live,
-                      &ctx->mc_counts, &ctx->mc_seeds,  &ctx->mc_scal};
+                      &ctx->mc_counts, &ctx->mc_seeds,  &ctx->mc_scal, &ctx->mc_list};
     for (DevBuf* b : bufs) tim_free(*b);
     if (ctx->h_scal) cudaFreeHost(ctx->h_scal);
     for (int i = 0; i < 8; i++)

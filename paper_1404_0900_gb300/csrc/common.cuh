@@ -157,7 +157,7 @@ struct tim_ctx {
     // per-block visited bitmaps (kept all-zero between calls), queues and live-edge bits;
     // cascade counts, seeds, counters
     DevBuf out_row, out_rec, out_pos, mc_bitmap, mc_queue, mc_live, mc_counts, mc_seeds,
-        mc_scal;
+        mc_scal, mc_list;
     bool have_out = false, mc_clean = false;
     bool mc_walk_only = false;  // this graph's worlds found no room
 

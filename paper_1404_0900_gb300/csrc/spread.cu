@@ -13,8 +13,9 @@
 //
 // The walk needs G itself: out-records {in-CSR position, destination} grouped by
 // source, and the inverse (out-record index of every in-CSR position), built from G^T on
-// first use. One block per cascade. Its visited bitmap (n bits) sits in shared memory
-// when it fits there, its queue (the activated nodes, n slots) and the live-edge bits
+// first use. A block per cascade, after a pass of a warp per cascade over calls of many (the
+// small ones end there, mc_light_kernel). The visited bitmap (n bits) sits in shared memory
+// when it fits there, the queue (the activated nodes, n slots) and the live-edge bits
 // (below) in global memory, one set per resident block. A round expands the nodes the
 // round before added; a round that adds nothing ends the cascade.
 //
@@ -24,10 +25,10 @@
 // four consecutive in-CSR positions with one Philox block and 16 contiguous bytes of
 // thresholds, LT and triggering models make one pick per unvisited node, and every live
 // edge sets one bit at its out-record; from then on a node's live out-edges are read 32
-// to a word. A cascade starts walking and draws its world as soon as the out-edges it
+// to a word. A cascade starts walking and draws its world when the out-edges it
 // would have walked by the end of the next round pass a fixed share (MC_WALK) of the draws
-// that the world takes (m / 4 blocks for IC, n picks otherwise): small cascades never pay
-// for a world, large ones walk little before they do. Against walking alone (one 256-thread
+// that the world takes (m / 4 blocks for IC, n picks otherwise) and it grows: small cascades
+// never pay for a world, large ones walk little before they do. Against walking alone (one 256-thread
 // block per cascade, one warp per node): 50 seeds on R-MAT 18, 2000 IC cascades 42.2 -> 10.9
 // ms, 1000 LT cascades 70.4 -> 7.4 ms. Drawing is bound by issue (Philox) and by the one L1
 // sector per clock of scattered out-record indexes and bit updates, the rounds by their
@@ -96,7 +97,8 @@ struct McArgs {
     uint64_t live_words;          // a multiple of 4
     unsigned long long draw_at;   // out-edges a cascade walks at most; ~0: never draws
     uint32_t* counts;              // per cascade
-    unsigned long long* scal;      // [0] next cascade, [1] total activated
+    unsigned long long* scal;      // [0] next cascade, [1] total activated, [2] cascades listed
+    uint32_t* list;                // cascades that the warps left to the blocks; null: all
     // triggering model: options per node, cumulative thresholds, sorted in-CSR positions
     const uint64_t* node_opt;
     const uint32_t* opt_cum;
@@ -166,6 +168,13 @@ __device__ __forceinline__ void set_live(const McArgs& a, uint32_t* live, uint64
 // goes on (MC_WALK 2, 4, 12, 24: 50 seeds on R-MAT 18, IC, 16.0, 15.0, 11.1, 11.1 ms; one
 // seed on a 200,001-node Chung-Lu graph, 1000 cascades, 6.2, 4.9, 3.7, 3.6 ms).
 constexpr unsigned MC_WALK = 12;
+// It goes on walking, up to MC_SURE times that share, while its rounds are small (a world costs
+// 20 of them or more) and do not grow: a cascade that neither grows nor dies out walks a
+// fraction of what its world takes. Growing: the next round has an eighth of the out-edges of all
+// rounds before it and half as many again as their average. (Random graph of 600,001 nodes, 38M
+// edges, p = 0.0155, 500 cascades of 200 seeds: drawing at the share alone 25.3 ms, walking alone
+// 14.2, here 14.8; 60,001 nodes, 2000 of 10 seeds 2.74, 1.81, 1.24.)
+constexpr float MC_SURE = 6.f;
 
 // Live in-CSR positions a warp collects (in shared memory) before it sets their bits, four
 // per lane in flight: setting each one as it is found would wait for its out-record index
@@ -199,11 +208,10 @@ __device__ __forceinline__ void draw_world(const McArgs& a, uint32_t s0, uint32_
     if (a.model == TIM_IC) {
         const uint4* thr4 = reinterpret_cast<const uint4*>(a.thr);
         const uint32_t groups = (uint32_t)((a.m + 3) >> 2);  // thr is zero past its end
-        // four groups per thread and step: their loads overlap, and the live in-edges of all
-        // four (about one in sixteen coins under weighted cascade) share one loop
         uint32_t* st = stage + (threadIdx.x >> 5) * MC_STAGE;
         uint32_t held = 0;
-        // four groups per thread and step, so that their loads overlap
+        // four groups per thread and step: their loads overlap, and the live in-edges of all
+        // four (about one in sixteen coins under weighted cascade) share one loop
         for (uint32_t gw = threadIdx.x & ~31u; gw < groups; gw += 4 * blockDim.x) {
             const uint32_t g0 = gw + lane;
             uint32_t lm = 0;
@@ -292,30 +300,131 @@ __device__ __forceinline__ void draw_world(const McArgs& a, uint32_t s0, uint32_
     __syncthreads();
 }
 
+// Cascades that stay small, a warp each: members and their hash in shared memory, walked edge by
+// edge. One that outgrows LIGHT_Q members or LIGHT_EDGES out-edges is listed and starts over in
+// a block of mc_cascade_kernel. What such a cascade takes is its chain of dependent loads, so what
+// counts is how many are in flight: 7,296 warps, against 152 or 304 blocks, each of which
+// also has barriers to pass and a bitmap to clear. Used for calls of more than four times as many
+// cascades as blocks (with fewer the blocks are faster) from at most LIGHT_Q / 2 seeds.
+// (20,000 weighted-cascade cascades of one node of low out-degree, Chung-Lu 600,001 and 1,000,003
+// nodes, R-MAT 16: a block of 256 threads each 0.19, 0.20, 1.47 ms; the large blocks alone 0.37,
+// 0.68, 0.77; here 0.12, 0.14, 0.53. LIGHT_Q 256 with 2048 out-edges: within 10 % either way.)
+constexpr int LIGHT_THREADS = 256, LIGHT_BLOCKS = 6;
+constexpr int LIGHT_Q = 128;
+constexpr int LIGHT_LOG2H = 8;  // 256 slots for at most LIGHT_Q + 31 nodes
+constexpr uint32_t LIGHT_EDGES = 1024;
+
+__global__ void __launch_bounds__(LIGHT_THREADS, LIGHT_BLOCKS) mc_light_kernel(McArgs a) {
+    constexpr uint32_t H = 1u << LIGHT_LOG2H, NONE = 0xFFFFFFFFu;
+    __shared__ uint32_t s_hash[LIGHT_THREADS / 32][H], s_queue[LIGHT_THREADS / 32][LIGHT_Q];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint32_t *hash = s_hash[wid], *q = s_queue[wid];
+    for (uint32_t i = lane; i < H; i += 32) hash[i] = NONE;
+    __syncwarp();
+    const uint64_t nw = (uint64_t)gridDim.x * (LIGHT_THREADS / 32);
+    unsigned long long all = 0;
+    for (uint64_t c = blockIdx.x * (uint64_t)(LIGHT_THREADS / 32) + wid; c < a.count; c += nw) {
+        const uint64_t sid = a.sid0 + c;
+        const uint32_t s0 = (uint32_t)sid, s1 = (uint32_t)(sid >> 32);
+        int tail = 0;
+        bool heavy = false;
+        auto add = [&](bool want, uint32_t v) {
+            bool fresh = false;
+            if (want) {
+                uint32_t h = (v * 0x9E3779B1u) >> (32 - LIGHT_LOG2H);
+                for (uint32_t p = 0; p < H; p++) {
+                    const uint32_t old = atomicCAS(&hash[h], NONE, v);
+                    fresh = old == NONE;
+                    if (fresh || old == v) break;
+                    h = (h + 1) & (H - 1);
+                }
+            }
+            const uint32_t fm = __ballot_sync(0xffffffffu, fresh);
+            const int at = tail + __popc(fm & ((1u << lane) - 1u));
+            if (fresh && at < LIGHT_Q) q[at] = v;
+            tail += __popc(fm);
+            heavy = tail > LIGHT_Q;
+            __syncwarp();
+        };
+        for (int i = 0; i < a.k && !heavy; i += 32)
+            add(i + lane < a.k, i + lane < a.k ? (uint32_t)a.seeds[i + lane] : 0u);
+        uint32_t edges = 0;
+        for (int head = 0; head < tail && !heavy;) {
+            const int nb = min(32, tail - head);
+            uint2 row = make_uint2(0u, 0u);
+            if (lane < nb) row = __ldg(a.out_row + q[head + lane]);
+            head += nb;
+            uint32_t incl = row.y - row.x;  // distinct rows: fewer than 2^32 edges together
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+            heavy = total > LIGHT_EDGES - edges;
+            if (heavy) break;
+            edges += total;
+            const uint32_t first = row.x - (incl - (row.y - row.x));
+            for (uint32_t base = 0; base < total && !heavy; base += 32) {
+                const uint32_t t = base + lane;
+                int own = 0;  // number of lanes whose inclusive count is <= t
+#pragma unroll
+                for (int sft = 16; sft > 0; sft >>= 1) {
+                    const uint32_t ic = __shfl_sync(0xffffffffu, incl, own + sft - 1);
+                    if (ic <= t) own += sft;
+                }
+                const uint32_t at = __shfl_sync(0xffffffffu, first, own) + t;
+                uint2 r = make_uint2(0u, 0u);
+                if (t < total) r = __ldg(a.out_rec + at);
+                add(t < total && edge_kept(a, s0, s1, r.y, r.x), r.y);
+            }
+        }
+        for (uint32_t i = lane; i < H; i += 32) hash[i] = NONE;
+        __syncwarp();
+        if (lane == 0 && heavy) {
+            a.list[atomicAdd(&a.scal[2], 1ull)] = (uint32_t)c;
+        } else if (lane == 0) {
+            a.counts[c] = (uint32_t)tail;
+            all += tail;
+        }
+    }
+    if (lane == 0 && all) atomicAdd(&a.scal[1], all);
+}
+
+// With the bitmap in shared memory: members up to which it is cleared through the queue (clearing
+// all of its words takes about as long as this many stores).
+constexpr uint32_t MC_LIST = 4096;
+
 // SM: the visited bitmap in shared memory (n bits of dynamic shared memory).
 template <bool SM, int THREADS, int BLOCKS>
 __global__ void __launch_bounds__(THREADS, BLOCKS) mc_cascade_kernel(McArgs a) {
     extern __shared__ uint32_t s_bm[];
     __shared__ uint32_t s_stage[THREADS / 32 * MC_STAGE];
     __shared__ unsigned long long s_c, s_edges;
-    __shared__ uint32_t s_tail, s_next;
+    // round r expands s_tail[r % 3] nodes, claimed through s_next[r % 2], and counts the next
+    // round's in s_tail[(r + 1) % 3]; the third and the other are cleared meanwhile
+    __shared__ uint32_t s_tail[3], s_next[2], s_draw;
+    const uint32_t count = (uint32_t)(a.list ? __ldcg(&a.scal[2]) : a.count);
+    if (blockIdx.x >= count) return;
     const int lane = threadIdx.x & 31;
+    constexpr uint32_t W = THREADS / 32;
     uint32_t* bm = SM ? s_bm : a.bitmap + (uint64_t)blockIdx.x * a.words;
     uint32_t* q = a.queue + (uint64_t)blockIdx.x * a.n;
     uint32_t* live = a.live + (uint64_t)blockIdx.x * a.live_words;
     uint32_t* st = s_stage + (threadIdx.x >> 5) * MC_STAGE;
     if (SM)
         for (uint32_t w = threadIdx.x; w < (uint32_t)a.words; w += blockDim.x) bm[w] = 0u;
-    // The round's nodes are q[cur .. ] and the next round's q[nxt .. ], step +1 or -1. With
-    // the bitmap in shared memory the rounds fill the queue from its two ends in turn (the
-    // nodes of two rounds are distinct, so they fit), which keeps its lines in L2; without,
-    // they follow one another, so that the bitmap can be cleared through the queue.
-    int64_t cur = 0, nxt = 0;
-    int dcur = 1, dnxt = 1;
+    // The round's nodes are q[cur .. ] and the next round's q[nxt .. ], step +1 or -1. The
+    // rounds follow one another, so that the bitmap can be cleared through the queue. With the
+    // bitmap in shared memory the rounds of a cascade of more than MC_LIST nodes fill the queue
+    // from its two ends in turn (the nodes of two rounds are distinct, so they fit), which
+    // keeps its lines in L2.
+    int cur = 0, nxt = 0, dcur = 1, dnxt = 1;
+    uint32_t to = 0;  // the next round's nodes are counted in s_tail[to]
     auto add = [&](uint32_t v) {
         const uint32_t b = 1u << (v & 31);
         if (!(atomicOr(&bm[v >> 5], b) & b))
-            q[nxt + dnxt * (int64_t)atomicAdd(&s_tail, 1u)] = v;
+            q[nxt + dnxt * (int)atomicAdd(&s_tail[to], 1u)] = v;
     };
     // a plain read first: a stale zero only costs a draw or an atomic
     auto seen = [&](uint32_t v) {
@@ -324,62 +433,92 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) mc_cascade_kernel(McArgs a) {
     for (;;) {
         __syncthreads();
         if (threadIdx.x == 0) {
-            s_c = atomicAdd(&a.scal[0], 1ull);
-            s_tail = 0;
+            const unsigned long long i = atomicAdd(&a.scal[0], 1ull);
+            s_c = i >= count ? ~0ull : a.list ? __ldcg(a.list + i) : i;
+            s_tail[0] = s_tail[1] = s_next[0] = s_draw = 0u;
         }
         __syncthreads();
         const unsigned long long c = s_c;
-        if (c >= a.count) break;
+        if (c == ~0ull) break;
         const uint64_t sid = a.sid0 + c;
         const uint32_t s0 = (uint32_t)sid, s1 = (uint32_t)(sid >> 32);
         nxt = 0;
         dnxt = 1;
+        to = 0;
+        bool ends = false;
         for (int i = threadIdx.x; i < a.k; i += blockDim.x) add((uint32_t)a.seeds[i]);
         __syncthreads();
         uint32_t act = 0;  // nodes of the rounds before
         bool drawn = false;
-        unsigned long long walked = 0;
+        float walked = 0.f;  // out-edges of the rounds before
         // every round either adds a node or ends the cascade: at most n + 1 rounds
-        for (uint64_t round = 0; round <= a.n; round++) {
-            const uint32_t f = s_tail;
+        for (uint32_t round = 0; round <= (uint32_t)a.n; round++) {
+            const uint32_t f = s_tail[to];
             if (f == 0) break;
             cur = nxt;
             dcur = dnxt;
-            if (SM) {
-                nxt = cur ? 0 : (int64_t)a.n - 1;
-                dnxt = -dcur;
+            if (SM && act + f > MC_LIST) {
+                nxt = ends && dcur < 0 ? 0 : (int)a.n - 1;
+                dnxt = ends ? -dcur : -1;
+                ends = true;
             } else {
-                nxt = cur + f;
+                nxt = cur + (int)f;
             }
             act += f;
-            __syncthreads();  // every thread has read s_tail
+            to = to == 2 ? 0 : to + 1;
             if (threadIdx.x == 0) {
-                s_next = 0;
-                s_edges = 0;
-                s_tail = 0;
+                s_tail[to == 2 ? 0 : to + 1] = 0;
+                s_next[(round + 1) & 1] = 0;
             }
-            __syncthreads();
+            // a round of at most 32 nodes: every warp holds all their rows and takes its share of
+            // their edges, without claims. One barrier ends such a round (three when its nodes
+            // are more; with four a round and rows claimed one by one: 500 cascades of 600 nodes in
+            // fifty rounds 0.44 ms, here 0.37; one hub on R-MAT 18, 1000 cascades, 3.93 -> 3.15)
+            const bool few = f <= 32;
+            uint2 rows = make_uint2(0u, 0u);
+            if (few && (uint32_t)lane < f)
+                rows = __ldg(a.out_row + __ldcg(q + (cur + dcur * lane)));
             if (!drawn && a.draw_at != ~0ull) {
-                unsigned long long d = 0;
-                for (uint32_t i = threadIdx.x; i < f; i += blockDim.x) {
-                    const uint32_t u = __ldcg(q + cur + dcur * (int64_t)i);
-                    const uint2 row = __ldg(a.out_row + u);
-                    d += row.y - row.x;
-                }
+                float out;  // of this round
+                if (few) {
+                    out = (float)__reduce_add_sync(0xffffffffu, rows.y - rows.x);
+                } else {
+                    if (threadIdx.x == 0) s_edges = 0;
+                    __syncthreads();
+                    unsigned long long d = 0;
+                    for (uint32_t i = threadIdx.x; i < f; i += THREADS) {
+                        const uint32_t u = __ldcg(q + (cur + dcur * (int)i));
+                        const uint2 row = __ldg(a.out_row + u);
+                        d += row.y - row.x;
+                    }
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-                if (lane == 0 && d) atomicAdd(&s_edges, d);
-                __syncthreads();
-                walked += s_edges;
-                if (walked > a.draw_at) {
-                    draw_world(a, s0, s1, bm, live, s_stage);
-                    drawn = true;
+                    for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+                    if (lane == 0 && d) atomicAdd(&s_edges, d);
+                    __syncthreads();
+                    out = (float)s_edges;
+                }
+                const float at = (float)a.draw_at;
+                const bool grows = 5.f * out >= at ||
+                                   (8.f * out >= walked && 2.f * (float)round * out >= 3.f * walked);
+                walked += out;
+                if (walked > at && (grows || walked > MC_SURE * at)) {
+                    if (threadIdx.x == 0) s_draw = 1u;
+                    __syncthreads();
                 }
             }
-            // warps claim the round's nodes, up to 32 at a time (fewer when the round has
-            // few nodes for its warps), and flatten their rows over the lanes: one out-edge
+            // (decided by shared memory alone, as the set id comes from it: so that the branch and
+            // the id are known to be the same for the whole block. The drawing takes a quarter
+            // to 40 % longer otherwise: 1000 cascades of 50 seeds on R-MAT 18 3.4 -> 4.3 to 4.8 ms)
+            if (s_draw) {
+                draw_world(a, s0, s1, bm, live, s_stage);
+                drawn = true;
+                if (threadIdx.x == 0) s_draw = 0u;
+            }
+            // otherwise warps claim the round's nodes, up to 32 at a time (fewer when the round
+            // has few nodes for its warps). Rows are flattened over the lanes: one out-edge
             // per lane, or one word of 32 live bits
-            const uint32_t per = min(32u, max(1u, f / (blockDim.x >> 5)));
+            const uint32_t per = min(32u, max(1u, f / W));
+            const uint32_t start = few ? threadIdx.x & ~31u : 0u, half = few ? W * 32u : 32u;
             uint32_t held = 0;  // live out-records staged by this warp
             // destinations of the staged records, four per lane in flight; the new ones join
             // the queue with one counter update per warp
@@ -400,21 +539,23 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) mc_cascade_kernel(McArgs a) {
                         const uint32_t fm = __ballot_sync(0xffffffffu, fresh);
                         if (!fm) continue;
                         uint32_t base = 0;
-                        if (lane == 0) base = atomicAdd(&s_tail, (uint32_t)__popc(fm));
+                        if (lane == 0) base = atomicAdd(&s_tail[to], (uint32_t)__popc(fm));
                         base = __shfl_sync(0xffffffffu, base, 0) + __popc(fm & ((1u << lane) - 1u));
-                        if (fresh) q[nxt + dnxt * (int64_t)base] = v[k];
+                        if (fresh) q[nxt + dnxt * (int)base] = v[k];
                     }
                 }
                 __syncwarp();
             };
-            for (;;) {
-                uint32_t i0 = 0;
-                if (lane == 0) i0 = atomicAdd(&s_next, per);
-                i0 = __shfl_sync(0xffffffffu, i0, 0);
-                if (i0 >= f) break;
-                uint2 row = make_uint2(0u, 0u);
-                if ((uint32_t)lane < per && i0 + lane < f)
-                    row = __ldg(a.out_row + __ldcg(q + cur + dcur * (int64_t)(i0 + lane)));
+            do {
+                uint2 row = rows;
+                if (!few) {
+                    uint32_t i0 = 0;
+                    if (lane == 0) i0 = atomicAdd(&s_next[round & 1], per);
+                    i0 = __shfl_sync(0xffffffffu, i0, 0);
+                    if (i0 >= f) break;
+                    if ((uint32_t)lane < per && i0 + lane < f)
+                        row = __ldg(a.out_row + __ldcg(q + (cur + dcur * (int)(i0 + lane))));
+                }
                 // m < 2^32: a warp's distinct rows have fewer than 2^32 edges together
                 const uint32_t n32 = row.y - row.x;
                 const uint32_t r0 = drawn ? row.x >> 5 : row.x;
@@ -438,11 +579,11 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) mc_cascade_kernel(McArgs a) {
                     return own;
                 };
                 if (!drawn) {
-                    for (uint32_t base = 0; base < total; base += 64) {
+                    for (uint32_t base = start; base < total; base += min(2 * half, total - base)) {
                         uint2 r[2];
 #pragma unroll
                         for (int i = 0; i < 2; i++) {
-                            const uint32_t t = base + 32 * i + lane;
+                            const uint32_t t = base + half * i + lane;
                             const int own = owner(t);
                             const uint32_t at = __shfl_sync(0xffffffffu, r0, own) +
                                                 (t - __shfl_sync(0xffffffffu, excl, own));
@@ -454,13 +595,13 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) mc_cascade_kernel(McArgs a) {
                                 edge_kept(a, s0, s1, r[i].y, r[i].x))
                                 add(r[i].y);
                     }
-                    continue;
+                    continue;  // (few: the last turn)
                 }
-                for (uint32_t base = 0; base < total; base += 64) {
+                for (uint32_t base = start; base < total; base += min(2 * half, total - base)) {
                     uint32_t at[2], w[2];
 #pragma unroll
                     for (int i = 0; i < 2; i++) {
-                        const uint32_t t = base + 32 * i + lane;
+                        const uint32_t t = base + half * i + lane;
                         const int own = owner(t);
                         at[i] = __shfl_sync(0xffffffffu, r0, own) +
                                 (t - __shfl_sync(0xffffffffu, excl, own));
@@ -501,7 +642,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) mc_cascade_kernel(McArgs a) {
                         }
                     if (fits) held += wt;
                 }
-            }
+            } while (!few);
             take();
             held = 0;
             __syncthreads();
@@ -511,7 +652,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) mc_cascade_kernel(McArgs a) {
             atomicAdd(&a.scal[1], (unsigned long long)act);
         }
         // leave the bitmap all-zero
-        if (SM)
+        if (SM && ends)
             for (uint32_t w = threadIdx.x; w < (uint32_t)a.words; w += blockDim.x) bm[w] = 0u;
         else  // every set bit belongs to a queued node
             for (uint32_t i = threadIdx.x; i < act; i += blockDim.x) bm[__ldcg(q + i) >> 5] = 0u;
@@ -623,11 +764,14 @@ extern "C" int tim_spread_mc(tim_ctx* ctx, const int32_t* seeds, int k, uint64_t
     }
     TIM_TRY(tim_ensure(ctx, ctx->mc_counts, count * 4));
     TIM_TRY(tim_ensure(ctx, ctx->mc_seeds, std::max(k, 1) * sizeof(int32_t)));
-    TIM_TRY(tim_ensure(ctx, ctx->mc_scal, 2 * sizeof(unsigned long long)));
+    TIM_TRY(tim_ensure(ctx, ctx->mc_scal, 3 * sizeof(unsigned long long)));
+    // by warps first where there are several times more cascades than blocks at once
+    const bool light = k <= LIGHT_Q / 2 && count > 4 * (uint64_t)ctx->num_sms * nb &&
+                       tim_ensure(ctx, ctx->mc_list, count * sizeof(uint32_t)) == TIM_OK;
     if (k > 0)
         CUDA_TRY(ctx, cudaMemcpyAsync(ctx->mc_seeds.p, seeds, (size_t)k * sizeof(int32_t),
                                       cudaMemcpyHostToDevice, ctx->stream));
-    CUDA_TRY(ctx, cudaMemsetAsync(ctx->mc_scal.p, 0, 2 * sizeof(unsigned long long), ctx->stream));
+    CUDA_TRY(ctx, cudaMemsetAsync(ctx->mc_scal.p, 0, 3 * sizeof(unsigned long long), ctx->stream));
     McArgs a;
     a.node = (const uint4*)ctx->node.p;
     a.thr = (const uint32_t*)ctx->thr.p;
@@ -655,6 +799,13 @@ extern "C" int tim_spread_mc(tim_ctx* ctx, const int32_t* seeds, int k, uint64_t
     a.opt_cum = (const uint32_t*)ctx->opt_cum.p;
     a.opt_off = (const uint64_t*)ctx->opt_off.p;
     a.opt_pos = (const uint32_t*)ctx->opt_pos.p;
+    a.list = light ? (uint32_t*)ctx->mc_list.p : nullptr;
+    if (light) {
+        const uint64_t blocks = (count + LIGHT_THREADS / 32 - 1) / (LIGHT_THREADS / 32);
+        mc_light_kernel<<<(unsigned)std::min<uint64_t>(blocks, (uint64_t)ctx->num_sms * LIGHT_BLOCKS),
+                          LIGHT_THREADS, 0, ctx->stream>>>(a);
+        LAUNCH_CHECK(ctx, "mc_light_kernel");
+    }
     if (!sm) ctx->mc_clean = false;
     void* args[] = {&a};
     CUDA_TRY(ctx, cudaLaunchKernel(kernel, dim3((unsigned)slots), dim3(threads), args, smem, ctx->stream));
