@@ -356,16 +356,19 @@ __global__ void __launch_bounds__(256) count_bins_kernel(const uint32_t* __restr
 }
 
 // tau = the smallest bin floor that leaves at most CAND nodes at or above it (every block
-// finds it from the bins), and the nodes there, in the order of descending bins.
+// finds it from the bins), and the nodes there, in the order of descending bins. tau = 0, no
+// candidates: there are more than CAND in the highest bin, or fewer than `need` among more nodes
+// that have sets.
 __global__ void __launch_bounds__(256) candidates_kernel(const uint32_t* __restrict__ counts,
-                                                         uint64_t n, CandState* st) {
+                                                         uint64_t n, uint32_t need,
+                                                         CandState* st) {
     __shared__ uint32_t sfx[256];
-    __shared__ uint32_t s_bin;
+    __shared__ uint32_t s_bin, s_cand;
     // thread t owns bins 4 t .. 4 t + 3; sfx[t] = nodes in its bins and above
     uint32_t b[4], sum = 0;
     for (int i = 0; i < 4; i++) sum += b[i] = st->bins[threadIdx.x * 4 + i];
     sfx[threadIdx.x] = sum;
-    if (threadIdx.x == 0) s_bin = CAND_BINS;
+    if (threadIdx.x == 0) s_bin = CAND_BINS, s_cand = 0u;
     __syncthreads();
     for (int o = 1; o < 256; o <<= 1) {
         const uint32_t y = threadIdx.x + o < 256 ? sfx[threadIdx.x + o] : 0u;
@@ -380,7 +383,14 @@ __global__ void __launch_bounds__(256) candidates_kernel(const uint32_t* __restr
         if (bin >= 1 && above <= CAND) atomicMin(&s_bin, (uint32_t)bin);
     }
     __syncthreads();
-    const uint32_t tau = s_bin < CAND_BINS ? bin_floor(s_bin) : 0u;
+    above = sfx[threadIdx.x] - sum;
+    for (int i = 3; i >= 0; i--) {
+        above += b[i];
+        if (threadIdx.x * 4 + i == (int)s_bin) s_cand = above;
+    }
+    __syncthreads();
+    const uint32_t tau =
+        s_bin == 1u || (s_bin < CAND_BINS && s_cand >= need) ? bin_floor(s_bin) : 0u;
     if (blockIdx.x == 0 && threadIdx.x == 0) st->tau = tau;
     if (tau == 0u) return;
     // a bin's candidates follow those of the bins above it
@@ -389,8 +399,8 @@ __global__ void __launch_bounds__(256) candidates_kernel(const uint32_t* __restr
     for (int i = 3; i >= 0; i--) {
         first[threadIdx.x * 4 + i] = above;
         above += b[i];
-        if (blockIdx.x == 0 && threadIdx.x * 4 + i == (int)s_bin) st->ncand = above;
     }
+    if (blockIdx.x == 0 && threadIdx.x == 0) st->ncand = s_cand;
     __syncthreads();
     const int lane = threadIdx.x & 31;
     for (uint64_t v0 = blockIdx.x * 256ull + (threadIdx.x & ~31u); v0 < n;
@@ -412,6 +422,7 @@ __device__ __forceinline__ uint32_t cand_hash(uint32_t u) { return u * 0x9E3779B
 // entry).
 __global__ void __launch_bounds__(1024) cand_table_kernel(CandState* st) {
     __shared__ uint32_t wsum[32];
+    if (st->tau == 0u) return;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const uint32_t nc = min(st->ncand, CAND);
     constexpr uint32_t PER = CAND / 1024;
@@ -497,6 +508,7 @@ cand_index_kernel(const uint32_t* __restrict__ pool, const uint32_t* __restrict_
                   const uint8_t* __restrict__ covered, uint64_t members, CandState* st,
                   uint32_t* __restrict__ sets) {
     extern __shared__ __align__(16) uint32_t sm[];
+    if (st->tau == 0u) return;
     const CandTable tab = load_table(st, sm);
     uint32_t* num = sm + TABLE_SMEM / 4;  // [CAND]
     constexpr uint64_t TILE = (uint64_t)CG_THREADS * TILE_ITEMS;
@@ -605,6 +617,10 @@ cand_rounds_kernel(CandState* st, const uint32_t* __restrict__ sets,
     __shared__ unsigned long long wbest[CG_THREADS / 32];
     __shared__ uint32_t wcand[CG_THREADS / 32];
     __shared__ unsigned long long wsum[CG_THREADS / 32];
+    if (st->tau == 0u) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) *done = (uint32_t)r0;
+        return;
+    }
     const CandTable tab = load_table(st, sm);
     int* cnt = reinterpret_cast<int*>(sm + TABLE_SMEM / 4);               // [CAND]
     uint32_t* dec = reinterpret_cast<uint32_t*>(cnt + CAND);              // [CAND]
@@ -859,11 +875,12 @@ static int count_members(tim_ctx* ctx, bool live) {
 
 int tim_count_members(tim_ctx* ctx) { return count_members(ctx, false); }
 
-int tim_build_index(tim_ctx* ctx) {
+// counted: the counts are already those of the store.
+static int build_index(tim_ctx* ctx, bool counted) {
     const uint64_t n = (uint64_t)ctx->n, members = ctx->members;
     TIM_TRY(tim_ensure(ctx, ctx->node_off, (n + 2) * sizeof(uint64_t)));
     TIM_TRY(tim_ensure(ctx, ctx->node_sets, (members + 1) * sizeof(uint32_t)));
-    TIM_TRY(count_members(ctx, false));
+    if (!counted) TIM_TRY(count_members(ctx, false));
     CUDA_TRY(ctx, cudaMemsetAsync(ctx->node_off.p, 0, sizeof(uint64_t), ctx->stream));
     const unsigned G = (unsigned)(ctx->num_sms * 8);
     // node_off[v + 1] = start of node v's sets (node_off[0] = 0); the scatter turns it
@@ -878,6 +895,8 @@ int tim_build_index(tim_ctx* ctx) {
     }
     return TIM_OK;
 }
+
+int tim_build_index(tim_ctx* ctx) { return build_index(ctx, false); }
 
 // Rounds r0 .. k - 1 over the full index; with r0 > 0 the flags of the sets and nodes and the
 // covered counter are those of the rounds before, and counts holds the uncovered sets'.
@@ -983,6 +1002,15 @@ __global__ void fill_seeds_kernel(int r0, int k, uint64_t n, uint8_t* __restrict
 // is a pass over the members that counts, one that indexes the candidates, and the rounds: an
 // epoch that did not do CAND_MIN_ROUNDS hands the rest to the full index.
 constexpr int CAND_MIN_ROUNDS = 8;
+// The candidates cost some 50 us before the first round and save some 4 us a round: selections of
+// at most CAND_MIN_K seeds from stores of at most CAND_MIN_MEMBERS take the full index. (One, five
+// and eight seeds, candidates / full index: 107,497 members, 8,192 nodes 0.145 / 0.093, 0.170 /
+// 0.142, 0.194 / 0.177 ms; 498,451, 262,144 nodes 0.158 / 0.115, 0.194 / 0.187, 0.218 / 0.237;
+// 1,048,301, 8,192 nodes 0.157 / 0.189, 0.186 / 0.251, 0.213 / 0.290.)
+constexpr int CAND_MIN_K = 6;
+constexpr uint64_t CAND_MIN_MEMBERS = 1'000'000;
+// an epoch needs a candidate for every round left, or this many
+constexpr int CAND_NEED = 128;
 
 int tim_greedy(tim_ctx* ctx, int k, int32_t* host_seeds, uint64_t* covered) {
     const uint64_t n = (uint64_t)ctx->n, members = ctx->members;
@@ -990,7 +1018,8 @@ int tim_greedy(tim_ctx* ctx, int k, int32_t* host_seeds, uint64_t* covered) {
     int coop = 0, nb = 0;
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, ctx->device);
     // 32-bit offsets and counts; an open stepwise selection keeps the full index's counts
-    bool cand = coop && !ctx->select_open && members < 0xFFFFFFFFull && ctx->n_sets < 0x7FFFFFFFull;
+    bool cand = coop && !ctx->select_open && members < 0xFFFFFFFFull &&
+                ctx->n_sets < 0x7FFFFFFFull && (k > CAND_MIN_K || members > CAND_MIN_MEMBERS);
     if (cand) {
         CUDA_TRY(ctx, cudaFuncSetAttribute(cand_rounds_kernel,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1064,7 +1093,8 @@ int tim_greedy(tim_ctx* ctx, int k, int32_t* host_seeds, uint64_t* covered) {
         CUDA_TRY(ctx, cudaMemsetAsync(ctx->greedy_bar.p, 0, sizeof(GridBarrier), ctx->stream));
         count_bins_kernel<<<GN, 256, 0, ctx->stream>>>((const uint32_t*)ctx->counts.p, n, st);
         LAUNCH_CHECK(ctx, "count_bins_kernel");
-        candidates_kernel<<<GN, 256, 0, ctx->stream>>>((const uint32_t*)ctx->counts.p, n, st);
+        candidates_kernel<<<GN, 256, 0, ctx->stream>>>((const uint32_t*)ctx->counts.p, n,
+                                                    (uint32_t)std::min(k - r, CAND_NEED), st);
         LAUNCH_CHECK(ctx, "candidates_kernel");
         cand_table_kernel<<<1, 1024, 0, ctx->stream>>>(st);
         LAUNCH_CHECK(ctx, "cand_table_kernel");
@@ -1111,7 +1141,7 @@ int tim_greedy(tim_ctx* ctx, int k, int32_t* host_seeds, uint64_t* covered) {
                                               cudaMemcpyDeviceToHost, ctx->stream));
             TIM_TRY(tim_sync(ctx));
         } else if (done < k && done - r < CAND_MIN_ROUNDS) {
-            TIM_TRY(tim_build_index(ctx));
+            TIM_TRY(build_index(ctx, !live));
             if (done > 0) TIM_TRY(count_members(ctx, true));
             return greedy_full(ctx, k, done, host_seeds, covered);
         } else if (done < k) {

@@ -82,3 +82,12 @@ def test_beside_an_open_stepwise_selection():
         hit[sid[np.isin(mem, rseeds)]] = True
         assert cov == hit.sum()
         assert np.array_equal(left, np.bincount(mem[~hit[sid]], minlength=g.n))
+
+
+@pytest.mark.parametrize("n,theta,ks", [
+    (30_000, 1_000_000, (3, 6, 7)), (30_000, 1_000_001, (3, 6, 7)),  # the largest small store
+    (2_000_000, 12_000, (6, 7, 30, 45, 127, 128, 129, 300))])  # some 36 nodes in two sets
+def test_few_seeds_and_few_candidates(n, theta, ks):
+    # every set is its root alone
+    g = inputs.from_edges(n, [(0, 1)])
+    _run(g, inputs.constant(g, 0.0), O.IC, theta, ks)
