@@ -314,8 +314,8 @@ int tim_set_pass1_capacity(tim_ctx* ctx, int members);
  * set to the heavy-set pass, whose warps spread each in-list over the whole GPU, once
  * the in-edges the team would examine exceed `budget` (default 2^64 - 1). Sets that outgrow
  * the queue, or whose coins in long in-lists (512 in-edges or more, outside the
- * geometric-skip rule) would pass a fixed number, go there whatever the budget. Results do
- * not change. */
+ * geometric-skip rule) would pass a number that depends on the call's sets and the graph's
+ * edges, go there whatever the budget. Results do not change. */
 int tim_set_pass2_budget(tim_ctx* ctx, uint64_t budget);
 
 /* Polls a block makes at a grid barrier of a persistent kernel (the heavy-set pass of

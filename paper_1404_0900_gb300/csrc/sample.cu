@@ -50,7 +50,13 @@ constexpr int BIG_THREADS = 256;  // tier 3 LT CTA size
 // trivalency on Chung-Lu graphs of 100,001 nodes 9.4 9.4 9.1 9.4 9.8 10.9 12.0 ms, 700,001
 // nodes 18.9 19.1 19.5 20.4 22.1 29.5 44.7, 4.16M nodes 38.1 38.5 38.8 40.2 42.4 59.4 83.5,
 // 41.6M nodes - 225.9 224.0 220.3 220.1 229.6 247.3.
-constexpr unsigned long long LONG_BUDGET2 = 6144;
+// A call of few sets, or on a graph of few edges, has a larger one: a launch of the heavy-set pass
+// takes 0.2 ms or more, a set waits for at most its graph's edges, and where many sets are heavy
+// the teams have enough of them (trivalency, 6144 -> 24576: 1000 sets of the 100,001 nodes 0.37 ->
+// 0.17 ms; 10,000 of 20,001 nodes, 378K edges, 0.37 -> 0.17, TIM+ 3.3 -> 2.5; 200,000 of R-MAT 14,
+// 228K edges, 30.0 -> 13.9, TIM+ 121 -> 60; but 1000 of R-MAT 14 0.53 -> 0.67).
+constexpr unsigned long long LONG_BUDGET2 = 6144, LONG_BUDGET2_FEW = 24576;
+constexpr uint64_t LONG_FEW_SETS = 2048, LONG_FEW_EDGES = 2'000'000;
 
 // Queue capacity Q and hash size 2^LOG2H (>= 2Q) of one warp's set. With BM the visited set is
 // a bitmap (bit 0: a member) instead of the hash, in the hash's place or in shared memory; like
@@ -2625,7 +2631,8 @@ int tim_sample(tim_ctx* ctx, const SampleRequest& req, SampleResult* res) {
     a.set_width = (uint64_t*)ctx->set_width.p;
     a.width_budget = ctx->width_budget;
     a.width_budget2 = ctx->width_budget2;
-    a.long_budget2 = LONG_BUDGET2;
+    a.long_budget2 = count <= LONG_FEW_SETS || (uint64_t)ctx->m <= LONG_FEW_EDGES
+                         ? LONG_BUDGET2_FEW : LONG_BUDGET2;
     a.chunk = std::max(1, ctx->chunk);
     a.inflight = plan.inflight;
     // IC: room for the pass-1 state of up to count / 2 + 4096 handed-over sets (at most

@@ -91,3 +91,19 @@ def test_batch_of_many_small_queries():
         assert st["kpt_star"] == ref.kpt.kpt_star and st["theta"] == ref.theta
     for e in engines:
         e.close()
+
+
+@pytest.mark.parametrize("count", [2048, 2049])
+def test_long_lists_of_few_and_many_sets(count):
+    """Sets with coins in long in-lists of their own thresholds, on both sides of the number of
+    sets from which on the heavy-set pass takes them earlier; more than two million edges."""
+    g = inputs.chung_lu(60_001, 2_300_000, 2.1, seed=8)
+    assert g.m > 2_000_000
+    w = inputs.trivalency(g, seed=2)
+    sid = O.make_sid(1, 4, 0)
+    off, _, wid = O.sample(O.load_graph(g.n, g.rowptr, g.dst, w, O.IC), 3, sid, count)
+    with tim.Engine(0) as eng:
+        tim.tim_load_graph(eng.ctx, g.n, g.rowptr, g.dst, w, tim.TIM_IC)
+        tim.tim_sample_rr(eng.ctx, count, 3, sid)
+        o, _, x = tim.tim_get_rr(eng.ctx)
+        assert np.array_equal(o, off) and np.array_equal(x, wid)
