@@ -41,3 +41,26 @@ def test_runs_split_and_match_the_gradient(n, d):
             assert np.array_equal(tim.tim_mlp_get_params(eng.ctx, net), end)
         finally:
             tim.tim_mlp_destroy(net)
+
+
+@pytest.mark.parametrize("n,d", [(1, 1), (32, 12), (33, 5), (500, 32), (4865, 12), (9728, 12)])
+def test_one_launch_equals_launches_per_step(n, d):
+    # runs of one step are two launches, longer ones one
+    rng = np.random.default_rng(3 * n + d)
+    x = rng.normal(size=(n, d)).astype(np.float32)
+    y = rng.normal(size=n).astype(np.float32)
+    with tim.Engine(0) as eng:
+        net, p = _net(eng, d, 9)
+        try:
+            out = []
+            for runs in ((12,), (1,) * 12, (3, 1, 2, 6)):
+                tim.tim_mlp_set_params(eng.ctx, net, p)
+                before = tim.tim_launch_count(eng.ctx)
+                h = np.concatenate([tim.tim_mlp_train(eng.ctx, net, x, y, s, 1e-2) for s in runs])
+                out.append((h, tim.tim_mlp_get_params(eng.ctx, net)))
+                launches = tim.tim_launch_count(eng.ctx) - before
+                assert launches == sum(1 if s > 1 else 2 for s in runs)
+            for h, q in out[1:]:
+                assert np.array_equal(h, out[0][0]) and np.array_equal(q, out[0][1])
+        finally:
+            tim.tim_mlp_destroy(net)
