@@ -54,9 +54,10 @@ constexpr int BIG_THREADS = 256;  // tier 3 LT CTA size
 // takes 0.2 ms or more, a set waits for at most its graph's edges, and where many sets are heavy
 // the teams have enough of them (trivalency, 6144 -> 24576: 1000 sets of the 100,001 nodes 0.37 ->
 // 0.17 ms; 10,000 of 20,001 nodes, 378K edges, 0.37 -> 0.17, TIM+ 3.3 -> 2.5; 200,000 of R-MAT 14,
-// 228K edges, 30.0 -> 13.9, TIM+ 121 -> 60; but 1000 of R-MAT 14 0.53 -> 0.67).
+// 228K edges, 30.0 -> 13.9, TIM+ 121 -> 60; but 1000 of R-MAT 14 0.53 -> 0.67; R-MAT 16, 956K
+// edges, the same within 3 %).
 constexpr unsigned long long LONG_BUDGET2 = 6144, LONG_BUDGET2_FEW = 24576;
-constexpr uint64_t LONG_FEW_SETS = 2048, LONG_FEW_EDGES = 2'000'000;
+constexpr uint64_t LONG_FEW_SETS = 2048, LONG_FEW_EDGES = 400'000;
 
 // Queue capacity Q and hash size 2^LOG2H (>= 2Q) of one warp's set. With BM the visited set is
 // a bitmap (bit 0: a member) instead of the hash, in the hash's place or in shared memory; like
@@ -541,7 +542,7 @@ __device__ __forceinline__ int team_rr(const A& a, const PhiloxKeys& K, uint64_t
                 const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
                 if (lane >= o) incl += y;
             }
-            const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);  
+            const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
             const uint32_t excl = ngs ? incl - ngs : ~0u;
             const uint32_t lists = __ballot_sync(0xffffffffu, ngs != 0u);
             if (ngs)
