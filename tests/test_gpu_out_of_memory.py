@@ -94,7 +94,7 @@ def test_steps_after_a_selection_without_room():
         assert tim.tim_select_take(eng.ctx, v) == counts[v]
 
 
-@pytest.mark.parametrize("ell,dense", [(1.0, False), (300.0, False), (1.0, True), (8000.0, True)])
+@pytest.mark.parametrize("ell,dense", [(1.0, False), (20.0, False), (1.0, True), (8000.0, True)])
 def test_algorithm_2_in_the_memory_of_its_largest_round(ell, dense):
     """Several rounds in one call are for speed only: in the memory that its rounds take one
     after another Algorithm 2 gives the same estimate and leaves the same store."""
