@@ -40,7 +40,7 @@ PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 # one launch is scaled from it by members. None where no capture of the current kernel
 # exists.
 DRAM_BYTES_PER_MEMBER = {
-    "c3": {1: None, 2: None, 3: None},
+    "c3": {1: 328.2, 2: 540.5, 3: 510.8},
     "c2": {1: None, 2: None, 3: None},
 }
 FALLBACK_HBM_GBS = 6800.0
@@ -376,8 +376,8 @@ def sampler_roofline(p: dict, workload: str) -> dict:
         return max(p["pass3_batches"] if i == 3 and p.get("pass3_batches")
                    else p[f"pass{i}_launches"], 1)
     dom = max((1, 2, 3), key=kernel_ms)
-    names = {1: "rr_team_kernel<IC, Cap<256,9>, pass 1> (shared-memory hash, warp per set)",
-             2: "rr_team_kernel<IC, Cap<8192,14>, pass 2> (global-arena hash, team per set)",
+    names = {1: "rr_pack_kernel (pass 1: eight sets per warp, shared-memory hashes)",
+             2: "rr_team_kernel<IC, Cap<8192,14>, pass 2> (arena hash or bitmap, team per set)",
              3: "bulk_levels_kernel (heavy sets: all BFS levels of a batch in one "
                 "persistent cooperative launch)"}
     alg = sampler_bytes(p, dom)

@@ -306,8 +306,9 @@ int tim_set_team_factor(tim_ctx* ctx, int factor);
 
 /* IC sampler tuning: pass 1's queue capacity per RR set, 128, 256 (default) or 512
  * members per warp, of which each of its eight sets has an eighth (the visited hash has
- * twice as many slots; both sit in shared memory). Larger sets move on to pass 2. Results
- * do not change. */
+ * twice as many slots; both sit in shared memory); in a call of no more sets than warps a
+ * set has 16 members whatever the capacity. Larger sets move on to pass 2. Results do not
+ * change. */
 int tim_set_pass1_capacity(tim_ctx* ctx, int members);
 
 /* IC sampler tuning: pass 2 (a team of warps per RR set, queue of 8192 members) hands a
@@ -319,9 +320,10 @@ int tim_set_pass1_capacity(tim_ctx* ctx, int members);
 int tim_set_pass2_budget(tim_ctx* ctx, uint64_t budget);
 
 /* Polls a block makes at a grid barrier of a persistent kernel (the heavy-set pass of
- * the IC sampler, the greedy of Algorithm 1; a training run waits at least the default) before it gives up; default 2^24 (about a
- * second). When one block gives up, every block of the launch stops and the call
- * returns TIM_ERR_TIMEOUT; the context stays usable. Results do not change. */
+ * the IC sampler, the greedy of Algorithm 1) before it gives up; default 2^24 (about a
+ * second). A training run waits at least the default. When one block gives up, every block
+ * of the launch stops and the call returns TIM_ERR_TIMEOUT; the context stays usable.
+ * Results do not change. */
 int tim_set_wait_limit(tim_ctx* ctx, uint32_t polls);
 
 /* Device memory that the context's buffers may take in all (default: no limit); an
@@ -380,7 +382,10 @@ int tim_get_profile(tim_ctx* ctx, tim_profile* out, int reset);
  *   d_covered   device uint64[1] (output): number of sets the seeds cover
  * Returns TIM_ERR_ARG, without running anything, for sizes beyond these limits, and
  * after the run if a member or an offset was out of range; TIM_ERR_TIMEOUT if the blocks
- * of its one cooperative launch waited too long for each other. Every call copies d_off[0]
+ * of its one cooperative launch waited too long for each other. That launch starts when all
+ * of its blocks (at most one per SM, 512 threads and 33 KB of shared memory each) find room at
+ * once: beside other streams' kernels that fill every SM it waits for theirs to end (an
+ * 8192^3 GEMM after another beside it: 1.2 ms instead of 0.7). Every call copies d_off[0]
  * and d_off[n_sets] to the host and waits for the stream before its kernels, and
  * waits again before it returns. Scratch is one __device__ array of about 13.3 MiB
  * that every GPU holds once the library is loaded; the first call on a device also
@@ -522,13 +527,13 @@ uint64_t tim_launch_count(tim_ctx* ctx);
  * also in in-lists that RR sampling skips geometrically); LT node v keeps the in-edge
  * picked by word 0 of Philox(seed; sid, v, TAG_LT), and under a general triggering
  * model (tim_load_graph_triggering) the in-edges of the option that word picks. Where
- * no in-list is skipped (LT, triggering models, or IC lists outside the skip rule) the RR set of sid is the set of nodes that reach
- * its root in that world, so root in cascade(S) <=> RR set meets S, world by world.
+ * no in-list is skipped (LT, triggering models, or IC lists outside the skip rule) the RR
+ * set of sid is the set of nodes that reach its root in that world, so root in cascade(S) <=> RR set meets S, world by world.
  * Outputs (each may be NULL): *total = sum over cascades of the activated nodes
  * (seeds included; exact), *mean = total / count in FP64, counts_out = host
  * uint32[count] of per-cascade counts. G as out-records (8 B per node and per edge,
- * and 4 B per edge more once whole worlds are drawn) is built from G^T on the first call
- * after a load and kept. Errors: TIM_ERR_STATE without a graph,
+ * and 4 B per edge more once whole worlds are drawn, which they are where the device has
+ * room) is built from G^T on the first call after a load and kept. Errors: TIM_ERR_STATE without a graph,
  * TIM_ERR_ARG for a seed out of range or count >= 2^32, TIM_ERR_OOM. */
 int tim_spread_mc(tim_ctx* ctx, const int32_t* seeds, int k, uint64_t count, uint64_t seed,
                   uint64_t first_set_id, uint64_t* total, double* mean, uint32_t* counts_out);

@@ -782,14 +782,19 @@ static void kpt_keep_state(tim_ctx* c, const KptJob& J, uint64_t seed) {
 // least twice ktot / ctot + 4 / ctot (kappa lies in [0, 1], so that few sets leave the mean
 // that uncertain), and, while that is at most KPT_GROUP_SETS sets in all, the rounds up to
 // the expected stop. Sets past the stop are wasted, which this bounds, and a call of more than
-// KPT_CALL_SETS gains nothing from more; the rounds that are reported and kept are Algorithm 2's. Algorithm 2 one round per call and grouped: R-MAT 20,
-// weighted cascade, k = 50 (5 rounds) 6.7 -> 3.3 ms; Chung-Lu 4.16M nodes, trivalency (14
-// rounds) 24.5 -> 18.4 ms; R-MAT 14, k = 10 (4 rounds) 1.35 -> 0.84 ms.
+// KPT_CALL_SETS gains nothing from more; the rounds that are reported and kept are Algorithm
+// 2's. Algorithm 2 one round per call and grouped: R-MAT 20, weighted cascade, k = 50 (5 rounds)
+// 6.7 -> 3.3 ms; Chung-Lu 4.16M nodes, trivalency (14 rounds) 24.5 -> 18.4 ms; R-MAT 14, k = 10 (4
+// rounds) 1.35 -> 0.84 ms. KPT_GROUP_SETS 4096, 16384, 65536: R-MAT 14, k = 1, 1.34, 0.87, 0.68
+// ms; R-MAT 20, LT, k = 1, 2.50, 2.47, 1.49; 700,001 nodes, trivalency, k = 50, 6.41, 6.41, 5.64; others
+// within 5 %, but the sets past the stop count too.
 constexpr uint64_t KPT_GROUP_SETS = 16384, KPT_CALL_SETS = 1 << 22;
 
 static int kpt_group(int64_t n, double ell, int i, int rounds, double ktot, double ctot) {
-    if (i == 1)
-        return rounds > 1 && tim_host_c_i(n, ell, 1) + tim_host_c_i(n, ell, 2) <= KPT_GROUP_SETS ? 2 : 1;
+    if (i == 1) {
+        const uint64_t two = tim_host_c_i(n, ell, 1) + tim_host_c_i(n, ell, 2);
+        return rounds > 1 && two <= KPT_GROUP_SETS ? 2 : 1;
+    }
     auto round_of = [](double mean) { return mean > 0.0 ? (int)floor(-log2(mean)) : 62; };
     const int sure = round_of((ktot + 4.0) / ctot) - 1, stop = round_of(ktot / ctot) + 1;
     int g = 1;

@@ -131,7 +131,8 @@ struct tim_ctx {
     // the smallest T with listed * team_factor >= resident warps / T (at most 8)
     int team_size = 0;
     int team_factor = 2;
-    // IC tier 1: queue capacity of one warp's set (128, 256 or 512 members)
+    // IC tier 1: queue capacity of a warp (128, 256 or 512 members), an eighth for each of its
+    // sets; 16 members per set in calls of no more sets than warps
     int cap1 = 256;
     // sets claimed per work-counter increment in tiers 1 and 2
     int chunk = 2;
@@ -475,10 +476,10 @@ __device__ __forceinline__ const unsigned long long* skip_table(const unsigned l
 }
 
 // Live in-edges of a list under the rule, warp-cooperatively: lane b decides digit b
-// of each gap (T_b from the node's table) and lane B whether the gap is 2^B or more (Q_B), one
-// ballot gives G; a lane's draw for gap 2i also serves gap 2i + 1. visit(j) runs on every lane with the same in-CSR position j
-// of each live in-edge, in increasing order, and returns true to stop early. All 32
-// lanes must call it with the same arguments.
+// of each gap (T_b from the node's table) and lane B whether the gap is 2^B or more (Q_B),
+// one ballot gives G; a lane's draw for gap 2i also serves gap 2i + 1. visit(j) runs on
+// every lane with the same in-CSR position j of each live in-edge, in increasing order, and
+// returns true to stop early. All 32 lanes must call it with the same arguments.
 template <class Visit>
 __device__ __forceinline__ void skip_live_warp(uint32_t s0, uint32_t s1, const PhiloxKeys& K,
                                                uint32_t beg, uint32_t d,
@@ -600,8 +601,8 @@ __device__ __forceinline__ unsigned long long kappa_fixed(double kappa) {
     return __double2ull_rz(__dmul_rn(kappa, 9223372036854775808.0));
 }
 
-// Barrier over all blocks (or the first `blocks`) of a co-resident (cooperative) launch: sense reversal on a
-// generation counter, which the host zeroes before each launch. The wait is bounded:
+// Barrier over all blocks (or the first `blocks`) of a co-resident (cooperative) launch: sense
+// reversal on a generation counter, which the host zeroes before each launch. The wait is bounded:
 // after `limit` polls a block sets TIM_DEV_ERR_TIMEOUT in *err and the barrier returns
 // false; it also returns false once any block has set that bit, so every block of the
 // launch stops within one barrier of the first timeout.

@@ -37,7 +37,7 @@ constexpr uint64_t OFF_COVERED = al(OFF_NODE_SETS + 4 * NA_MAX_MEMBERS);     // 
 constexpr uint64_t OFF_CHOSEN = al(OFF_COVERED + NA_MAX_SETS);               // u8[n]
 constexpr uint64_t OFF_BEST = al(OFF_CHOSEN + NA_MAX_NODES);                 // u64[k]
 constexpr uint64_t OFF_SUMS = al(OFF_BEST + 8 * NA_MAX_K);                   // u64[blocks]
-constexpr uint64_t OFF_FLAGS = al(OFF_SUMS + 8 * NA_MAX_BLOCKS);            // u64[8]
+constexpr uint64_t OFF_FLAGS = al(OFF_SUMS + 8 * NA_MAX_BLOCKS);             // u64[8]
 constexpr uint64_t NA_SCRATCH_BYTES = al(OFF_FLAGS + 64);
 
 static __device__ __align__(256) unsigned char na_scratch[NA_SCRATCH_BYTES];
@@ -51,7 +51,8 @@ struct NaView {
     uint8_t* chosen;
     unsigned long long* best;
     unsigned long long* sums;
-    unsigned long long* flags;  // [0] covered count, [1] error bits, [2] barrier, [3] barrier error, [4] the rounds' barrier
+    unsigned long long* flags;  // [0] covered count, [1] error bits, [2] barrier, [3] its error,
+                                // [4] the rounds' barrier
 };
 
 NaView view_of(unsigned char* base) {
