@@ -1008,13 +1008,14 @@ __global__ void fill_seeds_kernel(int r0, int k, uint64_t n, uint8_t* __restrict
 // is a pass over the members that counts, one that indexes the candidates, and the rounds: an
 // epoch that did not do CAND_MIN_ROUNDS hands the rest to the full index.
 constexpr int CAND_MIN_ROUNDS = 8;
-// The candidates cost some 50 us before the first round and save some 4 us a round: selections of
-// at most CAND_MIN_K seeds from stores of at most CAND_MIN_MEMBERS take the full index. (One, five
-// and eight seeds, candidates / full index: 107,497 members, 8,192 nodes 0.145 / 0.093, 0.170 /
-// 0.142, 0.194 / 0.177 ms; 498,451, 262,144 nodes 0.158 / 0.115, 0.194 / 0.187, 0.218 / 0.237;
-// 1,048,301, 8,192 nodes 0.157 / 0.189, 0.186 / 0.251, 0.213 / 0.290.)
-constexpr int CAND_MIN_K = 6;
-constexpr uint64_t CAND_MIN_MEMBERS = 1'000'000;
+// The candidates cost some 50 us before the first round and save some 4 us a round, and more the
+// more members there are: selections of at most CAND_MIN_K seeds from stores of at most
+// CAND_MIN_MEMBERS take the full index. (One, three and six seeds, candidates / full index, Chung-Lu
+// 20,001 nodes: 113,528 members 0.140 / 0.110, 0.160 / 0.134, 0.185 / 0.166 ms; 226,602 0.152 / 0.135,
+// 0.163 / 0.162, 0.187 / 0.195; 458,240 0.153 / 0.188, 0.166 / 0.220, 0.191 / 0.257. 5,001 nodes cross
+// at 200,000 members, R-MAT 19 at a million for one seed and, at any size, between three and six.)
+constexpr int CAND_MIN_K = 5;
+constexpr uint64_t CAND_MIN_MEMBERS = 150'000;
 // an epoch needs a candidate for every round left, or this many
 constexpr int CAND_NEED = 128;
 

@@ -85,8 +85,8 @@ def test_beside_an_open_stepwise_selection():
 
 
 @pytest.mark.parametrize("n,theta,ks", [
-    (30_000, 1_000_000, (3, 6, 7)), (30_000, 1_000_001, (3, 6, 7)),  # the largest small store
-    (2_000_000, 12_000, (6, 7, 30, 45, 127, 128, 129, 300))])  # some 36 nodes in two sets
+    (30_000, 150_000, (3, 5, 6)), (30_000, 150_001, (3, 5, 6)),  # the largest small store
+    (2_000_000, 12_000, (5, 6, 30, 45, 127, 128, 129, 300))])  # some 36 nodes in two sets
 def test_few_seeds_and_few_candidates(n, theta, ks):
     # every set is its root alone
     g = inputs.from_edges(n, [(0, 1)])
